@@ -143,13 +143,14 @@ const char *tm_status_string(tm_status s);
  *        must not overlap in.
  * Asynchronous on `stream`, except that with the automatic histogram path
  * (TM_OPT_HIST_PATH = 0, the default) the first call for an image size and
- * dtype pair times both paths and synchronises `stream` once. The context's
+ * dtype pair that the compact integral histogram does not take (see there)
+ * times the two other paths and synchronises `stream` once. The context's
  * workspace is reused, so calls on one context must be ordered (same stream,
- * or synchronised). On the fused path, an (in, out) pair of descriptors that
- * comes back is captured in a CUDA graph of the context and replayed while
- * the same descriptors are passed (a replay reads the current pixel
- * contents); not with debug exports, stage timing or streaming range reuse
- * on. The context keeps six such graphs (batches' included). */
+ * or synchronised). On the fused and compact paths, an (in, out) pair of
+ * descriptors that comes back is captured in a CUDA graph of the context and
+ * replayed while the same descriptors are passed (a replay reads the current
+ * pixel contents); not with debug exports, stage timing or streaming range
+ * reuse on. The context keeps six such graphs (batches' included). */
 tm_status tm_forward(tm_ctx *ctx, const tm_image *in, const tm_image *out,
                      void *stream);
 
@@ -179,11 +180,15 @@ tm_status tm_forward_host(tm_ctx *ctx, const tm_image *in_host,
 tm_status tm_forward_host_async(tm_ctx *ctx, const tm_image *in_host,
                                 const tm_image *out_host, void *stream);
 
-/* Forward over n images of possibly different sizes. Images whose fields do
- * not fit the fused sweep take the materialised integral histogram; the
- * others take TM_OPT_HIST_PATH's path (automatic: the first batch of a given
- * list of sizes and dtype pairs times both batched passes on those images,
- * synchronising `stream` once, and keeps the faster for later batches).
+/* Forward over n images of possibly different sizes. With the automatic
+ * histogram path a batch whose images all fit the compact integral histogram
+ * runs on it as one batched pass: the range, bin and integral-image stages
+ * once for all of them, then the histograms and lookups of a group of images
+ * at a time (32 images, 8 GiB). Otherwise, images whose fields do not fit the
+ * fused sweep take the materialised integral histogram; the others take
+ * TM_OPT_HIST_PATH's path (automatic: the first batch of a given list of sizes
+ * and dtype pairs times both batched passes on those images, synchronising
+ * `stream` once, and keeps the faster for later batches).
  * The images on the fused path run as one batched pass: one launch per
  * stage, the sweep as one persistent launch over a shared queue of (image,
  * strip, row band) tiles. Those on the materialised path run as another:
@@ -318,13 +323,18 @@ tm_status tm_debug_export(tm_ctx *ctx, int32_t what, void *dst, size_t bytes,
 /* Tuning options.
  *   TM_OPT_HIST_PATH     0 = automatic (default), 1 = fused sliding sweep,
  *                        2 = materialised bin-major integral histogram.
- *                        Automatic: the first single-image forward of each
- *                        (width, height, input dtype, output dtype) on a
- *                        context runs both paths twice, timing the second
- *                        runs (it synchronises its stream once), and keeps
- *                        the faster; later forwards of that size take it
- *                        directly. Batches and tm_backward take the fused
- *                        path where it fits.
+ *                        Automatic: the compact integral histogram (per
+ *                        32-column chunk instead of per column) for images
+ *                        of at least two bins, at most 65535 columns and
+ *                        rows and under 24 GiB of it (0.4 GB for 12 MP with
+ *                        16 bins, 1.8 GB with 64). For others, and once its
+ *                        memory could not be had, the first single-image
+ *                        forward of each (width, height, input dtype, output
+ *                        dtype) on a context runs paths 1 and 2 twice, timing
+ *                        the second runs (it synchronises its stream once),
+ *                        and keeps the faster. All paths give the same
+ *                        outputs bit for bit. tm_backward takes the fields
+ *                        that fit the fused sweep.
  *   TM_OPT_STAGE_TIMING  1 = record a CUDA event after every stage of each
  *                        forward/backward call on its stream (see
  *                        tm_stage_times); 0 = off (default).

@@ -72,6 +72,7 @@ struct tm_ctx {
   int hist_path = 0;
   int sweep_tiles = 0;  // TM_OPT_SWEEP_TILES (0: one wave of the sweep's CTAs per image share)
   int sweep_width = 0;  // TM_OPT_SWEEP_WIDTH (0: automatic)
+  bool no_compact = false;  // the compact integral histogram's memory could not be had
   int64_t launches = 0;
   int num_sms = 0;
   size_t smem_optin = 0;
@@ -129,6 +130,7 @@ struct tm_ctx {
     int64_t launches = 0;
     std::vector<Job> jobs;
     uint64_t used = 0;
+    int path = 0;  // kPathSweep or kPathCompact
   };
   std::vector<FusedGraph> graphs;
   uint64_t calls = 0;  // forward calls so far (FusedGraph::used counts in them)
@@ -586,20 +588,50 @@ tm_status forward_materialised(tm_ctx *c, const tm_image *in, const tm_image *ou
   return TM_OK;
 }
 
-// The fused path over a batch of images: one launch per stage for the whole
-// batch, the sweep as a persistent kernel over a queue of (image, strip, row
-// band) tiles. `graph`: capture the batch into a CUDA graph of the context's
-// cache and replay it while the batch is unchanged. Returns TM_EUNSUPPORTED
-// if some image cannot be swept.
+// How the Eq. 1 numerators come about: from the fused sweep, from the
+// materialised planes, or from the compact integral histogram.
+enum Path { kPathSweep = 1, kPathMaterialised = 2, kPathCompact = 3 };
+
+// The compact integral histograms of a group of images stay below this (or
+// hold one image's); the groups of a batch run one after another on the same
+// buffers. One image's may take kCompactMax.
+constexpr size_t kCompactGroup = size_t(8) << 30, kCompactMax = size_t(24) << 30;
+
+size_t compact_bytes(const CompactPlan &C) {
+  return align256(C.rec_bytes) + align256(C.vec_bytes) + align256(C.row_bytes);
+}
+
+// Whether the fused sweep fits image `in` under the context's fields.
+bool sweep_fits(tm_ctx *c, const tm_image *in) {
+  SweepPlan plan;
+  return plan_sweep(dev_params(c->p, 0), in->width, in->height, 1,
+                    std::min(c->smem_optin - 2048, (size_t)110 * 1024), 256, plan);
+}
+
+// Whether the compact integral histogram takes image `im` under the context's
+// fields and bins.
+bool compact_fits(const tm_ctx *c, const tm_image *im) {
+  CompactPlan C;
+  return !c->no_compact && plan_compact(dev_params(c->p, 0), im->width, im->height, C) && compact_bytes(C) <= kCompactMax;
+}
+
+// The batched path over images that share it: one launch per stage for the
+// whole batch. path: kPathSweep, the sweep as a persistent kernel over a queue
+// of (image, strip, row band) tiles (TM_EUNSUPPORTED if some image cannot be
+// swept); or kPathCompact, the compact integral histogram, built and looked
+// up per group of images (every image has to fit it). `graph`: capture the
+// batch into a CUDA graph of the context's cache and replay it while the batch
+// is unchanged.
 tm_status finish_fused(tm_ctx *c, int nimg, const tm_image *in, const std::vector<Job> &jobs, int64_t n,
                        bool run_range, std::vector<Job> *jobs_out);
 
 tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image *out, cudaStream_t s,
-                        bool graph, bool do_lookup = true, std::vector<Job> *jobs_out = nullptr) {
+                        bool graph, Path path, bool do_lookup = true, std::vector<Job> *jobs_out = nullptr) {
+  const bool compact = path == kPathCompact;
   tm_status st;
   if (graph)
     for (auto &G : c->graphs) {
-      if (!same_images(G.in, in, nimg) || !same_images(G.out, out, nimg)) continue;
+      if (G.path != path || !same_images(G.in, in, nimg) || !same_images(G.out, out, nimg)) continue;
       c->fwd_valid = false;
       TM_CUDA(c, cudaGraphLaunch(G.exec, s));
       G.used = c->calls;
@@ -613,13 +645,13 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   for (int i = 0; i < nimg; ++i) total_px += (double)in[i].width * in[i].height;
   std::vector<Job> jobs((size_t)nimg);
   std::vector<JobLayout> lays((size_t)nimg);
-  std::vector<size_t> offs((size_t)nimg);
+  std::vector<size_t> offs((size_t)nimg), coffs((size_t)nimg);
   // strips of 512 own columns (one CTA per SM, with all of its shared memory)
   // where every image fits them, else 256 (two CTAs per SM)
   const DevParams P0 = dev_params(c->p, 0);
   int width = c->sweep_width == 256 ? 256 : 512;
   size_t smem_limit = 0, smem = 0;
-  for (int pass = 0; pass < 2; ++pass) {
+  for (int pass = 0; pass < 2 && !compact; ++pass) {
     smem_limit = width == 512 ? c->smem_optin - 2048 : std::min(c->smem_optin - 2048, (size_t)110 * 1024);
     smem = 0;
     bool ok = true;
@@ -633,8 +665,24 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     if (width == 256) return TM_EUNSUPPORTED;
     width = 256;
   }
-  const int cps = std::max(1, sweep_ctas_per_sm(c->p.n_fields, smem, width));
+  const int cps = compact ? 1 : std::max(1, sweep_ctas_per_sm(c->p.n_fields, smem, width));
   const int wave = c->num_sms * cps;
+  // the compact path's groups of images: their first images, and their blocks
+  struct Group {
+    int first, rows, cols, look;
+  };
+  std::vector<Group> groups;
+  std::vector<CompactPlan> cplans((size_t)nimg);
+  size_t c_used = 0, c_total = 0;
+  bool c_wide = false;  // 32-bit vectors for every image if one needs them
+  for (int i = 0; i < nimg && compact; ++i) {
+    CompactPlan &C = cplans[(size_t)i];
+    if (!plan_compact(P0, in[i].width, in[i].height, C))
+      return fail(c, TM_EUNSUPPORTED, "image %d is outside the compact path", i);
+    c_wide = c_wide || C.wide;
+  }
+  const int K = c->p.n_bins - 1;
+  const int look_rows = (int)std::min(8.0, std::max(1.0, total_px / (c->num_sms * 128.0 * 40)));
   size_t ws_total = 0;
   int b_range = 0, b_prep = 0, b_rows = 0, b_cols = 0, b_look = 0;
   std::vector<std::pair<double, int>> order;  // (work of one tile, image)
@@ -642,15 +690,50 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     const int W = in[i].width, H = in[i].height;
     const double share = nimg == 1 ? 1.0 : std::max(1.0 / c->num_sms, W * (double)H / total_px);
     Job &J = jobs[(size_t)i];
+    if (compact) memset(&J, 0, sizeof J);
     J.qbits = choose_qbits(c->p, W, H);
-    // one wave of segments, shared among a batch's images by pixel count (the
-    // segments' band claims even out the CTAs' work; two waves of them were
-    // slower on 16 x 1 MP: 1.33 against 1.28 ms)
-    const int target = c->sweep_tiles > 0 ? c->sweep_tiles : std::max(1, (int)std::lround(wave * share));
-    plan_sweep(P0, W, H, target, smem_limit, width, J.plan);
     integral_layout(W, H, SIZE_MAX, J.nseg, J.seg_rows);
-    const size_t cnt_bytes = sweep_count_bytes(P0, J.plan, J.cnt_off);
-    J.cnt_wide = J.plan.cnt_wide;
+    size_t cnt_bytes = 0;
+    if (compact) {
+      CompactPlan &C = cplans[(size_t)i];
+      if (c_wide && !C.wide) C.vec_bytes *= 2;
+      const size_t b = compact_bytes(C);
+      if (groups.empty() || c_used + b > kCompactGroup || i - groups.back().first >= kCompactImages) {
+        groups.push_back({i, 0, 0, 0});
+        c_used = 0;
+      }
+      coffs[(size_t)i] = c_used;
+      c_used += b;
+      c_total = std::max(c_total, c_used);
+      Group &g = groups.back();
+      J.b0[kStCRows] = g.rows;
+      g.rows += compact_row_blocks(H, K);
+      J.b0[kStCCols] = g.cols;
+      g.cols += compact_col_blocks(W, K);
+      J.b0[kStLook] = g.look;
+      g.look += compact_look_blocks(W, H, look_rows);
+      J.c_shift = C.shift;
+      // count planes only for the backward
+      J.plan.W = W, J.plan.H = H, J.plan.cnt_wide = (1 << c->p.n_fields) - 1;
+      J.cnt_wide = J.plan.cnt_wide;
+      if (keep_mom || !do_lookup) cnt_bytes = sweep_count_bytes(P0, J.plan, J.cnt_off);
+    } else {
+      // one wave of segments, shared among a batch's images by pixel count (the
+      // segments' band claims even out the CTAs' work; two waves of them were
+      // slower on 16 x 1 MP: 1.33 against 1.28 ms)
+      const int target = c->sweep_tiles > 0 ? c->sweep_tiles : std::max(1, (int)std::lround(wave * share));
+      plan_sweep(P0, W, H, target, smem_limit, width, J.plan);
+      cnt_bytes = sweep_count_bytes(P0, J.plan, J.cnt_off);
+      J.cnt_wide = J.plan.cnt_wide;
+      J.b0[kStLook] = b_look;
+      b_look += lookup_blocks(W, H);
+      J.nitemA = J.plan.tiles_x * ((J.plan.tiles_y + J.plan.K - 1) / J.plan.K);
+      J.nitemB = J.plan.tiles_x * J.plan.tiles_y - J.nitemA;
+      const double seg = (double)J.plan.K * J.plan.TY;  // rows of a segment
+      const double rows = std::min(seg + 2.0 * J.plan.Ry + 1, H + 1.0);
+      const double cols = std::min(J.plan.TX + 2.0 * J.plan.Rx + 2, W + 1.0);
+      order.push_back({rows * (cols * 0.05 + 100.0) + 6.0 * J.plan.TX * seg, i});
+    }
     lays[(size_t)i] = job_layout(c->p, W, H, J.nseg, cnt_bytes, debug, keep_mom, J.plan.tiles_x * J.plan.tiles_y);
     offs[(size_t)i] = ws_total;
     ws_total += lays[(size_t)i].total;
@@ -662,14 +745,6 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     b_rows += integral_tile_blocks(W, J.nseg);
     J.b0[kStCols] = b_cols;
     b_cols += integral_col_blocks(W);
-    J.b0[kStLook] = b_look;
-    b_look += lookup_blocks(W, H);
-    J.nitemA = J.plan.tiles_x * ((J.plan.tiles_y + J.plan.K - 1) / J.plan.K);
-    J.nitemB = J.plan.tiles_x * J.plan.tiles_y - J.nitemA;
-    const double seg = (double)J.plan.K * J.plan.TY;  // rows of a segment
-    const double rows = std::min(seg + 2.0 * J.plan.Ry + 1, H + 1.0);
-    const double cols = std::min(J.plan.TX + 2.0 * J.plan.Rx + 2, W + 1.0);
-    order.push_back({rows * (cols * 0.05 + 100.0) + 6.0 * J.plan.TX * seg, i});
   }
   // the queue holds each image's tiles together, the images with the
   // costliest tiles first
@@ -685,7 +760,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     nitems += jobs[(size_t)o.second].nitemB;
   }
   if ((st = ensure_stats(c, nimg))) return st;
-  if ((st = grow_device(c, &c->ws, &c->ws_bytes, ws_total))) return st;
+  if ((st = grow_device(c, &c->ws, &c->ws_bytes, ws_total + c_total))) return st;
   if (graph && c->graphs.size() >= kFusedGraphs) {  // room for the graph captured below
     auto lru = std::min_element(c->graphs.begin(), c->graphs.end(),
                                 [](const tm_ctx::FusedGraph &a, const tm_ctx::FusedGraph &b) { return a.used < b.used; });
@@ -713,9 +788,17 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     J.s2 = J.s1 + 1;
     J.s_pair = 1;
     J.segtot = reinterpret_cast<long long *>(b + L.segtot);
-    J.cnt = reinterpret_cast<unsigned char *>(b + L.cnt);
+    if (compact) {
+      char *cb = ws + ws_total + coffs[(size_t)i];
+      J.c_rec = reinterpret_cast<uint2 *>(cb);
+      J.c_vec = cb + align256(cplans[(size_t)i].rec_bytes);
+      J.c_row = reinterpret_cast<uint16_t *>(cb + align256(cplans[(size_t)i].rec_bytes) +
+                                             align256(cplans[(size_t)i].vec_bytes));
+    }
+    // (the compact path has count planes only where the backward reads them)
+    J.cnt = !compact || keep_mom || !do_lookup ? reinterpret_cast<unsigned char *>(b + L.cnt) : nullptr;
     J.grp = reinterpret_cast<uint16_t *>(b + L.grp);
-    J.claim = reinterpret_cast<int *>(b + L.claim);
+    J.claim = compact ? nullptr : reinterpret_cast<int *>(b + L.claim);
     J.mom = keep_mom ? reinterpret_cast<float2 *>(b + L.mom) : nullptr;
     if (debug) {
       J.dbg.cnt = reinterpret_cast<unsigned *>(b + L.dcnt);
@@ -750,7 +833,8 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   const int in_dt = input_dtype(jobs.data(), nimg);
   if (run_range) launch_range(dj, nimg, b_range, c->p.n_bins, in_dt, s);
   if (!graph) mark(c, s, ST_RANGE);
-  launch_prep(dj, nimg, b_prep, c->p.n_bins, c->p.flags, c->p.n_fields, in_dt, s);
+  // (the sweep accumulates into count planes that the prep stage clears)
+  launch_prep(dj, nimg, b_prep, c->p.n_bins, c->p.flags, compact ? 0 : c->p.n_fields, in_dt, s);
   const int m_prep = graph ? -1 : mark(c, s, ST_PREP);
   // the sweep (high priority, launched first, so its CTAs take the SMs) and
   // the integral images (low priority) side by side, each timed from the end
@@ -758,9 +842,15 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   TM_CUDA(c, cudaEventRecord(c->ov_fork, s));
   TM_CUDA(c, cudaStreamWaitEvent(c->sweep_stream, c->ov_fork, 0));
   TM_CUDA(c, cudaStreamWaitEvent(c->int_stream, c->ov_fork, 0));
-  const int ls = launch_sweep(P, dj, nimg, nitems, queue, smem, ctas, width, c->sweep_stream);
-  if (!graph) mark(c, c->sweep_stream, ST_SWEEP, m_prep);
-  n += 1 + launch_integral_jobs(dj, nimg, b_rows, b_cols, c->int_stream);
+  const auto group_end = [&](size_t k) { return k + 1 < groups.size() ? groups[k + 1].first : nimg; };
+  const auto build = [&](size_t k, cudaStream_t q) {
+    const Group &g = groups[k];
+    return launch_compact_build(dj + g.first, group_end(k) - g.first, g.rows, g.cols, K, c_wide, q);
+  };
+  int ls = compact ? build(0, c->sweep_stream)
+                   : launch_sweep(P, dj, nimg, nitems, queue, smem, ctas, width, c->sweep_stream);
+  if (!graph) mark(c, c->sweep_stream, compact ? ST_HIST : ST_SWEEP, m_prep);
+  n += std::max(ls, 0) + launch_integral_jobs(dj, nimg, b_rows, b_cols, c->int_stream);
   if (!graph) mark(c, c->int_stream, ST_INTEGRAL, m_prep);
   n += run_range ? 2 : 1;
   TM_CUDA(c, cudaEventRecord(c->ov_sweep, c->sweep_stream));
@@ -768,7 +858,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   TM_CUDA(c, cudaStreamWaitEvent(s, c->ov_sweep, 0));
   TM_CUDA(c, cudaStreamWaitEvent(s, c->ov_int, 0));
   if (!graph) mark(c, s, kNoStage);  // the join: the lookup is timed from here
-  if (do_lookup) {
+  if (compact || do_lookup) {
     // the lookup variant: without debug planes, with or without the moments,
     // and for one dtype of every input and output when they share it
     bool wide = true;
@@ -777,7 +867,20 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
       wide = wide && J.cnt_wide == (1 << c->p.n_fields) - 1;
       if (J.in.dtype != dt || J.out.dtype != dt) dt = -1;
     }
-    n += launch_lookup_counts(P, dj, nimg, b_look, !debug && wide, keep_mom, dt, s);
+    if (compact) {
+      for (size_t k = 0; k < groups.size(); ++k) {
+        const Group &g = groups[k];
+        if (k > 0) {
+          const int r = build(k, s);
+          ls = std::min(ls, r);
+          n += std::max(r, 0);
+        }
+        n += launch_lookup_compact(P, jobs.data() + g.first, group_end(k) - g.first, g.look, look_rows, c_wide, !debug, keep_mom,
+                                   !do_lookup, dt, s);
+      }
+    } else {
+      n += launch_lookup_counts(P, dj, nimg, b_look, !debug && wide, keep_mom, dt, s);
+    }
     if (!graph) mark(c, s, ST_LOOKUP);
   }
   if (graph) {
@@ -797,10 +900,11 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     G.launches = n;
     G.jobs = jobs;
     G.used = c->calls;
+    G.path = path;
     c->graphs.push_back(std::move(G));
     TM_CUDA(c, cudaGraphLaunch(c->graphs.back().exec, caller));
   } else if (ls < 0) {
-    return check_launch(c, "sweep shared-memory attribute");
+    return check_launch(c, "histogram shared-memory attribute");
   }
   if ((st = check_launch(c, "forward launch"))) return st;
   return finish_fused(c, nimg, in, jobs, n, run_range, jobs_out);
@@ -958,7 +1062,7 @@ tm_status choose_path(tm_ctx *c, const tm_image *in, const tm_image *out, cudaSt
   for (int path = 1; path <= 2 && !st; ++path) {
     for (int rep = 0; rep < 2 && !st; ++rep) {
       cudaEventRecord(e0, s);
-      st = path == 1 ? forward_fused(c, 1, in, out, s, false) : forward_materialised(c, in, out, s);
+      st = path == 1 ? forward_fused(c, 1, in, out, s, false, kPathSweep) : forward_materialised(c, in, out, s);
       if (path == 1 && st == TM_EUNSUPPORTED) {
         fused_ok = false;
         st = TM_OK;
@@ -989,10 +1093,10 @@ tm_status choose_path(tm_ctx *c, const tm_image *in, const tm_image *out, cudaSt
 constexpr uint64_t kGraphStale = 64;
 constexpr size_t kGraphSeen = 16;
 
-bool single_graph_ok(tm_ctx *c, const tm_image *in, const tm_image *out) {
+bool single_graph_ok(tm_ctx *c, const tm_image *in, const tm_image *out, Path path) {
   const std::vector<tm_image> pair{*in, *out};
   for (const auto &G : c->graphs)
-    if (same_images(G.in, in, 1) && same_images(G.out, out, 1)) return true;
+    if (G.path == path && same_images(G.in, in, 1) && same_images(G.out, out, 1)) return true;
   auto seen = std::find_if(c->graph_seen.begin(), c->graph_seen.end(), [&](const auto &e) {
     return same_images(e.first, pair.data(), 2);
   });
@@ -1017,7 +1121,13 @@ tm_status forward_device(tm_ctx *c, const tm_image *in, const tm_image *out, cud
   if (st) return st;
   ++c->calls;
   int path = c->hist_path;
-  if (c->p.n_bins < 2) path = 2;  // no thresholds: nothing to sweep
+  if (c->p.n_bins < 2) path = kPathMaterialised;  // no thresholds: nothing to count
+  if (path == 0 && compact_fits(c, in)) {
+    const bool graph = !c->stage_timing && !c->debug && !c->reuse_range && single_graph_ok(c, in, out, kPathCompact);
+    st = forward_fused(c, 1, in, out, s, graph, kPathCompact);
+    if (st != TM_ENOMEM) return st;
+    c->no_compact = true;  // the other paths need less memory
+  }
   if (path == 0) {
     const auto key = std::make_tuple((int)in->width, (int)in->height, (int)in->dtype, (int)out->dtype);
     auto it = c->path_choice.find(key);
@@ -1029,8 +1139,8 @@ tm_status forward_device(tm_ctx *c, const tm_image *in, const tm_image *out, cud
   }
   if (path == 1) {
     // a cached CUDA graph per image pair unless a per-call feature is on
-    const bool graph = !c->stage_timing && !c->debug && !c->reuse_range && single_graph_ok(c, in, out);
-    st = forward_fused(c, 1, in, out, s, graph);
+    const bool graph = !c->stage_timing && !c->debug && !c->reuse_range && single_graph_ok(c, in, out, kPathSweep);
+    st = forward_fused(c, 1, in, out, s, graph, kPathSweep);
     if (st != TM_EUNSUPPORTED) return st;
     if (c->hist_path == 1)
       return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit these fields (use the materialised path)");
@@ -1133,11 +1243,20 @@ tm_status backward_images(tm_ctx *c, int n, const tm_image *in, const tm_image *
   need += head;
   std::vector<Job> jobs;
   int64_t launches = 0;
+  // the backward takes the fields that the sweep fits, whatever path counts
+  bool compact = c->hist_path == 0;
+  for (int i = 0; i < n; ++i) {
+    if (!sweep_fits(c, &in[i])) return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit these fields");
+    compact = compact && compact_fits(c, &in[i]);
+  }
   if (c->bwd_reuse && c->fwd_valid && (int)c->fwd_in.size() == n && same_images(c->fwd_in, in, n)) {
     jobs = c->fwd_jobs;  // the last forward's intermediates of these images are in the workspace
   } else {
-    st = forward_fused(c, n, in, in, s, false, false, &jobs);
-    if (st == TM_EUNSUPPORTED) return fail(c, st, "fused sweep does not fit these fields");
+    st = forward_fused(c, n, in, in, s, false, compact ? kPathCompact : kPathSweep, false, &jobs);
+    if (st == TM_ENOMEM && compact) {
+      c->no_compact = true;
+      st = forward_fused(c, n, in, in, s, false, kPathSweep, false, &jobs);
+    }
     if (st) return st;
     launches = c->launches;
   }
@@ -1245,13 +1364,6 @@ tm_status leave_caller(tm_ctx *c, cudaStream_t s, tm_status st) {
   return TM_OK;
 }
 
-// Whether the fused sweep fits image `in` under the context's fields.
-bool sweep_fits(tm_ctx *c, const tm_image *in) {
-  SweepPlan plan;
-  return plan_sweep(dev_params(c->p, 0), in->width, in->height, 1,
-                    std::min(c->smem_optin - 2048, (size_t)110 * 1024), 256, plan);
-}
-
 // Automatic path of a batch's images that fit the sweep: run the batched
 // fused pass and the batched materialised pass twice each on them (without
 // graphs) and time the second runs with events (synchronising the stream);
@@ -1264,7 +1376,7 @@ tm_status choose_batch_path(tm_ctx *c, int n, const tm_image *in, const tm_image
   tm_status st = TM_OK;
   for (int rep = 0; rep < 2 && !st; ++rep) {
     cudaEventRecord(e[0], s);
-    st = forward_fused(c, n, in, out, s, false);
+    st = forward_fused(c, n, in, out, s, false, kPathSweep);
     cudaEventRecord(e[1], s);
     if (!st) st = forward_materialised_batch(c, n, in, out, s, false, stats0);
     cudaEventRecord(e[2], s);
@@ -1283,15 +1395,18 @@ tm_status choose_batch_path(tm_ctx *c, int n, const tm_image *in, const tm_image
   return TM_OK;
 }
 
-// tm_forward_batch on validated arguments, n >= 1. Images whose fields do not
-// fit the sweep take the materialised path; with TM_OPT_HIST_PATH = 0 the
-// others take the path measured faster for this batch (cached per context by
-// the images' sizes and dtype pairs). The images of each path run as one
-// batched pass captured in a graph of its own.
+// tm_forward_batch on validated arguments, n >= 1. With TM_OPT_HIST_PATH = 0
+// the batch runs on the compact integral histogram as one pass (stage "batch",
+// or "batch_materialised" if some image's fields are too wide for the sweep)
+// where every image fits it. Otherwise images whose fields do not fit the
+// sweep take the materialised path, and the others the path measured faster
+// for this batch (cached per context by the images' sizes and dtype pairs),
+// each path's images as one batched pass. Every pass is captured in a graph.
 tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *out, cudaStream_t st) {
   tm_status s = ensure_device_info(c);
   if (s) return s;
   std::vector<tm_image> fin, fout, min_, mout;
+  bool compact = c->hist_path == 0;
   for (int i = 0; i < n; ++i) {
     bool fused = c->p.n_bins > 1 && c->hist_path != 2;
     if (fused && !sweep_fits(c, &in[i])) {
@@ -1299,10 +1414,19 @@ tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *ou
         return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit image %d's fields (use the materialised path)", i);
       fused = false;
     }
+    compact = compact && compact_fits(c, &in[i]);
     (fused ? fin : min_).push_back(in[i]);
     (fused ? fout : mout).push_back(out[i]);
   }
   if ((s = ensure_stats(c, n))) return s;
+  if (compact) {
+    ++c->calls;
+    mark(c, st, -1);
+    s = forward_fused(c, n, in, out, st, true, kPathCompact);
+    if (!s) mark(c, st, min_.empty() ? ST_BATCH : ST_BATCH_MAT);
+    if (s != TM_ENOMEM) return s;
+    c->no_compact = true;  // the other paths need less memory
+  }
   if (!fin.empty() && c->hist_path == 0) {
     std::vector<std::tuple<int, int, int, int>> key;
     for (size_t i = 0; i < fin.size(); ++i)
@@ -1325,7 +1449,7 @@ tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *ou
   ++c->calls;
   if (!fin.empty()) {
     mark(c, st, -1);
-    s = forward_fused(c, (int)fin.size(), fin.data(), fout.data(), st, true);
+    s = forward_fused(c, (int)fin.size(), fin.data(), fout.data(), st, true, kPathSweep);
     if (s) return s;
     total += c->launches;
     mark(c, st, ST_BATCH);

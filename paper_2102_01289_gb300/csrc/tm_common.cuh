@@ -91,9 +91,16 @@ struct SweepPlan {
   size_t smem;                    // dynamic shared memory bytes
 };
 
+// Sizes of one image's compact integral histogram (plan_compact).
+struct CompactPlan {
+  int shift;                           // log2 of the thresholds per group
+  bool wide;                           // 32-bit vectors (a window taller than 65535 / 31 rows)
+  size_t rec_bytes, vec_bytes, row_bytes;
+};
+
 // Batched stages; every stage kernel of a batch maps its blocks to images
 // through the per-image first-block offsets b0[stage].
-enum StageId { kStRange = 0, kStPrep, kStRows, kStCols, kStLook, kNumStages };
+enum StageId { kStRange = 0, kStPrep, kStRows, kStCols, kStLook, kStCRows, kStCCols, kNumStages };
 
 // One image of a batch: its buffers and its share of every batched launch.
 // 16-byte aligned, so that kernels can copy it with 16-byte loads.
@@ -121,6 +128,11 @@ struct alignas(16) Job {
   int itemA0, nitemA;       // the sweep queue's slots of this job's group starts (first phase)
   int itemB0, nitemB;       // and of its other bands (second phase)
   int *claim;               // tiles_x x tiles_y band claims (cleared by the prep stage)
+  uint2 *c_rec;             // compact integral histogram (tm_compact.cu): records, threshold groups x
+                            //   (W / 32 + 1) chunks x (H + 1) positions x 2^c_shift thresholds
+  void *c_vec;              // in-chunk vectors, (W / 32 + 1) x (n - 1) x (H + 1) slots x 32 columns
+  uint16_t *c_row;          // row prefixes over the chunks, groups x (W / 32 + 1) x H x 2^c_shift
+  int c_shift;              // log2 of the thresholds per group
   SweepPlan plan;           // sweep tiling of this image
 };
 
@@ -349,7 +361,8 @@ __device__ __forceinline__ float window_variance(long long s1, long long s2, uns
   // |mean| <= 2^(Q-1) <= 2^23: the nearest integer fits 32 bits
   const int m = sm ? __float2int_rn(__int2float_rn((int)(s1 >> 10)) * (rN * 1024.f))
                    : __float2int_rn(__ll2float_rn(s1) * rN);
-  const long long d = s1 - (long long)m * (long long)N;
+  // small: |d| < 2^31, so 32 bits hold it
+  const long long d = sm ? (long long)(int)((unsigned)s1 - (unsigned)m * (unsigned)N) : s1 - (long long)m * (long long)N;
   const unsigned long long T = (unsigned long long)s2 - (unsigned long long)((long long)m * (s1 + d));
   const float df = sm ? __int2float_rn((int)d) : __ll2float_rn(d);
   const float v = fmaf(-df * rN, df, __ull2float_rn(T)) * rN;

@@ -1,0 +1,562 @@
+// tm_compact.cu -- the Eq. 1 numerators from a compact form of the cumulative
+// integral histogram.
+//
+// For a threshold k let C_k(u, p) be the integral histogram in cumulative form
+// (Eq. 7-8 summed over the bins below k): the pixels of the first p rows and
+// first u columns whose bin is below k. Eq. 9 takes four of its values per
+// field and pixel. Written out it is n - 1 planes of the image's size (3 GB at
+// 12 MP with 64 bins); here it is kept per 32-column chunk instead, as
+//     C_k(u, p) = PT + o m + B[o]          c = u / 32, o = u mod 32,
+// a record per (chunk c, row position p, threshold k) with
+//     PT  the pixels below k of the first p rows in the chunks left of c,
+//     m   the rows (of the first p) in which all of chunk c lies below k, and
+//     the count j of the rows in which chunk c holds bins on both sides of k
+//     ("mixed" rows), which names the vector
+//     B[o] (slot j of the chunk and threshold): the sum over those rows of the
+//         chunk's pixels below k left of column o.
+// A vector is written only at a mixed row, so column work is paid only where a
+// bin edge crosses a chunk: at 12 MP, 64 bins, the records are 192 MB and the
+// vectors of one photograph-like scene about 40 MB. Against the sweep this
+// takes a 12 MP forward from 758 to 588 us, a 1080p float16 one from 206 to
+// 131; white noise (every chunk row mixed for every threshold) is its worst
+// case. Differences between two
+// rows are taken modulo the width of m and B, so B is 16 bits wide unless a
+// window is taller than 65535 / 31 rows.
+//
+// Three launches per group of images:
+//   1. k_compact_rows: the prefix over the chunks of each row's counts below k
+//      (lanes = thresholds, walking along the row);
+//   2. k_compact_cols, a cluster of four CTAs per chunk and group of
+//      thresholds: its warps take consecutive row segments twice (lanes =
+//      thresholds, walking down the rows), once for the segments' totals and,
+//      after a scan of the totals over the segments, to write records and
+//      vectors;
+//   3. k_lookup_compact, a thread per column and a few rows: four records and
+//      up to four vector entries per field and pixel, then the lookup's
+//      arithmetic.
+// Thresholds come in groups of KL (32, or 4, 8, 16 where n - 1 is no larger):
+// a warp holds 32 / KL rows (launch 1) or row segments (launch 2) at once.
+// The bin ranges of the chunks come from the group summary of the bin pass.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "tm_kernels.cuh"
+#include "tm_lookup.cuh"
+
+namespace tmk {
+namespace {
+
+constexpr int kRowWarps = 8;  // warps of a k_compact_rows block
+constexpr int kCluster = 4;   // CTAs that share a chunk's rows
+
+template <int KL>
+struct Shape {
+  static constexpr int Sub = 32 / KL;                    // rows or segments of a warp
+  static constexpr int Step = KL == 32 ? 4 : KL == 16 ? 2 : 1;  // rows or chunks in flight together
+  static constexpr int ColWarps = KL == 32 ? 16 : KL == 16 ? 8 : 4;
+  static constexpr int Segs = ColWarps * Sub;            // row segments of a CTA
+};
+
+// Whether a chunk row with bins in [g & 255, g >> 8] has bins on both sides of
+// some threshold of the group (k0 + 1 .. k0 + KL).
+template <int KL>
+__device__ __forceinline__ bool mixed_range(unsigned g, int k0) {
+  return max((int)(g & 0xffu), k0) < min((int)(g >> 8), k0 + KL);
+}
+
+constexpr unsigned kNoRow = 0xffffu;  // a bin range on no threshold's lower side
+
+// Rows: lane = (row, threshold k0 + 1 + j), walking along the rows' chunks.
+template <int KL>
+__global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(const Job *__restrict__ jobs, int njobs, int K) {
+  using S = Shape<KL>;
+  const Job &J = jobs[find_job(jobs, njobs, kStCRows, blockIdx.x)];
+  const int lane = threadIdx.x & 31, sub = lane / KL, j = lane % KL;
+  const int W = J.in.W, H = J.in.H, G = (W + 31) >> 5, Gp = (W >> 5) + 1;
+  const int rb = (H + kRowWarps * S::Sub - 1) / (kRowWarps * S::Sub);
+  const int lb = blockIdx.x - J.b0[kStCRows];
+  const int kg = lb / rb, k0 = KL * kg;
+  const int v0 = ((lb - kg * rb) * kRowWarps + (threadIdx.x >> 5)) * S::Sub;  // the warp's first row
+  if (v0 >= H) return;
+  const bool own = v0 + sub < H;
+  const int v = min(v0 + sub, H - 1);  // the lane's row (past the last: read, not written)
+  const unsigned k = (unsigned)(k0 + 1 + j), k8 = k << 8;
+  const uint8_t *__restrict__ bins = J.bins + (size_t)v0 * W + lane;
+  const uint16_t *__restrict__ grow = J.grp + (size_t)v * G;
+  const size_t cstride = (size_t)H * KL;
+  uint16_t *__restrict__ dst = J.c_row + ((size_t)kg * Gp * H + v) * KL + j;
+  unsigned run = 0;
+  for (int cb = 0; cb < Gp; cb += KL) {
+    const unsigned gl = cb + j < G && own ? (unsigned)__ldg(grow + cb + j) : kNoRow;
+    const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit (sub, chunk of the batch)
+    const int n = min(KL, Gp - cb);
+    for (int i = 0; i < n; i += S::Step) {
+      int b[S::Step][S::Sub];
+#pragma unroll
+      for (int u = 0; u < S::Step; ++u)
+#pragma unroll
+        for (int q = 0; q < S::Sub; ++q) {
+          const int col = 32 * (cb + i + u);
+          b[u][q] = 256;
+          if (((mixed >> (q * KL + ((i + u) & (KL - 1)))) & 1u) && col + lane < W)
+            b[u][q] = (int)__ldg(bins + (size_t)q * W + col);
+        }
+#pragma unroll
+      for (int u = 0; u < S::Step; ++u) {
+        if (i + u >= n) break;
+        const unsigned g = __shfl_sync(0xffffffffu, gl, sub * KL + i + u);
+        if (own) *dst = (uint16_t)run;
+        dst += cstride;
+        unsigned cc = g < k8 ? 32u : 0u;  // every bin of the chunk below k
+        unsigned ball = 0;
+        if (S::Sub > 1 || ((mixed >> (i + u)) & 1u)) ball = __ballot_sync(0xffffffffu, (g & 0xffu) < k && k8 <= g);
+#pragma unroll
+        for (int q = 0; q < S::Sub; ++q) {
+          unsigned part = S::Sub == 1 ? ball : (ball >> (q * KL)) & ((1u << (KL & 31)) - 1u);
+          while (part) {
+            const int t = __ffs(part) - 1;
+            part &= part - 1;
+            const unsigned mask = __ballot_sync(0xffffffffu, b[u][q] <= k0 + t);  // bins below k0 + 1 + t
+            if (lane == q * KL + t) cc = (unsigned)__popc(mask);
+          }
+        }
+        run += cc;
+      }
+    }
+  }
+}
+
+// A warp's pass over its row segments of chunk c: lane = (segment sub,
+// threshold k0 + 1 + j) with rows row0 .. of segment 0, each segment `per`
+// rows, the last ending before rend. The lane's state is pt and mc = m |
+// (mixed rows) << 16.
+// kWrite: write records and vectors; sB[(sub, j)][o] holds the vectors (lane =
+// column o there). Else sB counts, per (sub, j) and column, the pixels of the
+// mixed rows with bin k0 + j (k0 or less for j = 0), and mh the mixed rows
+// wholly below the lane's threshold.
+template <int KL, class BT, bool kWrite>
+__device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int row0, int per, int rend, BT *sB,
+                                         unsigned &pt, unsigned &mc, unsigned &mh) {
+  using S = Shape<KL>;
+  const int lane = threadIdx.x & 31, sub = lane / KL, j = lane % KL;
+  const int W = J.in.W, H = J.in.H, G = (W + 31) >> 5, Gp = (W >> 5) + 1;
+  const int k0 = KL * kg;
+  const unsigned k = (unsigned)(k0 + 1 + j), k8 = k << 8;
+  const int mine = row0 + sub * per;
+  int left = min(per, rend - mine);  // the lane's rows still to come
+  const unsigned lt = (1u << lane) - 1u;
+  const bool colok = 32 * c + lane < W;
+  const uint8_t *__restrict__ bins = J.bins + (size_t)row0 * W + 32 * c + lane;
+  const uint16_t *__restrict__ grp = J.grp + (size_t)(mine + j) * G + c;
+  const size_t plane = (size_t)kg * Gp + c;
+  const uint16_t *__restrict__ row = J.c_row + (plane * H + mine) * KL + j;
+  uint2 *__restrict__ rec = J.c_rec + (plane * (H + 1) + mine + 1) * KL + j;
+  BT *__restrict__ vec = static_cast<BT *>(J.c_vec) + ((size_t)c * K + k0) * (H + 1) * 32 + lane;
+  const unsigned vstep = (unsigned)(H + 1);
+  for (int ib = 0; ib < per; ib += KL) {
+    const unsigned gl = c < G && j < left ? (unsigned)__ldg(grp) : kNoRow;
+    grp += (size_t)KL * G;
+    const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit (sub, row of the batch)
+    const int n = min(KL, per - ib);
+    for (int i = 0; i < n; i += S::Step) {
+      unsigned rp[S::Step];
+      int b[S::Step][S::Sub];
+#pragma unroll
+      for (int u = 0; u < S::Step; ++u) {
+        rp[u] = u < left ? (unsigned)__ldg(row + u * KL) : 0u;
+#pragma unroll
+        for (int q = 0; q < S::Sub; ++q) {
+          b[u][q] = 256;
+          if (((mixed >> (q * KL + ((i + u) & (KL - 1)))) & 1u) && colok)
+            b[u][q] = (int)__ldg(bins + (size_t)(unsigned)(q * per + u) * W);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < S::Step; ++u) {
+        // (rows past the segment have no bins below or on both sides)
+        const unsigned g = __shfl_sync(0xffffffffu, gl, sub * KL + ((i + u) & (KL - 1)));
+        pt += rp[u];
+        if (g < k8) ++mc;
+        if (S::Sub > 1 || ((mixed >> ((i + u) & (KL - 1))) & 1u)) {
+          const bool both = (g & 0xffu) < k && k8 <= g;
+          if (both) mc += 0x10000u;
+          if (!kWrite) {
+            if (g < k8 && mixed_range<KL>(g, k0)) ++mh;
+#pragma unroll
+            for (int q = 0; q < S::Sub; ++q) {
+              const int h = max(b[u][q] - k0, 0);
+              if (h < KL) {
+                BT *const s = sB + (q * KL + h) * 32 + lane;
+                *s = (BT)(*s + 1);
+              }
+            }
+          } else {
+            const unsigned ball = __ballot_sync(0xffffffffu, both);
+#pragma unroll
+            for (int q = 0; q < S::Sub; ++q) {
+              unsigned part = S::Sub == 1 ? ball : (ball >> (q * KL)) & ((1u << (KL & 31)) - 1u);
+              while (part) {
+                const int t = __ffs(part) - 1;  // threshold k0 + 1 + t
+                part &= part - 1;
+                const unsigned mask = __ballot_sync(0xffffffffu, b[u][q] <= k0 + t);
+                const unsigned slot = __shfl_sync(0xffffffffu, mc, q * KL + t) >> 16;
+                BT *const s = sB + (q * KL + t) * 32 + lane;
+                const BT val = (BT)(*s + __popc(mask & lt));
+                *s = val;
+                vec[(size_t)((unsigned)t * vstep + slot) * 32] = val;
+              }
+            }
+          }
+        }
+        if (kWrite && u < left) rec[u * KL] = make_uint2(pt, mc);
+      }
+      row += S::Step * KL;
+      rec += S::Step * KL;
+      bins += (size_t)S::Step * W;
+      left -= S::Step;
+    }
+  }
+}
+
+// Columns: cluster -> (image, chunk, threshold group), CTA -> a quarter of the
+// rows, cut into Segs segments.
+template <int KL, class BT>
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(32 * Shape<KL>::ColWarps, KL == 32 ? 3 : 8)
+    k_compact_cols(const Job *__restrict__ jobs, int njobs, int K) {
+  using S = Shape<KL>;
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) unsigned char smem[];
+  BT *const sB = reinterpret_cast<BT *>(smem);                  // [Segs][KL][32]
+  BT *const sT = sB + S::Segs * KL * 32;                        // [KL][32]: the CTA's totals
+  uint2 *const tot = reinterpret_cast<uint2 *>(sT + KL * 32);   // [Segs + 1][KL], the last: the CTA's totals
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const Job &J = jobs[find_job(jobs, njobs, kStCCols, blockIdx.x)];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, sub = lane / KL, j = lane % KL;
+  const int H = J.in.H, Gp = (J.in.W >> 5) + 1;
+  const int lb = (blockIdx.x - J.b0[kStCCols]) / kCluster;
+  const int kg = lb / Gp, c = lb - kg * Gp;
+  const int share = (H + kCluster - 1) / kCluster, per = (share + S::Segs - 1) / S::Segs;
+  const int row0 = rank * share + wid * S::Sub * per, rend = min((rank + 1) * share, H);
+  BT *const mine = sB + wid * S::Sub * KL * 32;
+  for (int i = lane; i < S::Sub * KL * 32; i += 32) mine[i] = 0;
+  __syncwarp();
+  unsigned pt = 0, mc = 0, mh = 0;
+  col_pass<KL, BT, false>(J, c, kg, K, row0, per, rend, mine, pt, mc, mh);
+  tot[(wid * S::Sub + sub) * KL + j] = make_uint2(pt, mc);
+  // per segment: the vectors' totals from the column counts (the pixels of
+  // mixed rows below k, less those of rows wholly below it, left of o)
+  const unsigned any = __ballot_sync(0xffffffffu, mc >> 16);
+  if (any) {
+    __syncwarp();
+#pragma unroll 1
+    for (int q = 0; q < S::Sub; ++q) {
+      unsigned below = 0;
+#pragma unroll 4
+      for (int t = 0; t < KL; ++t) {
+        BT *const s = mine + (q * KL + t) * 32 + lane;
+        below += *s;
+        unsigned e = 0;
+        if ((any >> (q * KL + t)) & 1u) {
+          const unsigned v = below - __shfl_sync(0xffffffffu, mh, q * KL + t);
+          e = v;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, e, o);
+            if (lane >= o) e += y;
+          }
+          e -= v;
+        }
+        *s = (BT)e;
+      }
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < KL * 32; e += 32 * S::ColWarps) {
+    unsigned t = 0;
+#pragma unroll 4
+    for (int w = 0; w < S::Segs; ++w) t += sB[w * KL * 32 + e];
+    sT[e] = (BT)t;
+  }
+  if (tid < KL) {
+    uint2 t = make_uint2(0u, 0u);
+    for (int w = 0; w < S::Segs; ++w) {
+      const uint2 x = tot[w * KL + tid];
+      t.x += x.x, t.y += x.y;
+    }
+    tot[S::Segs * KL + tid] = t;
+  }
+  cluster.sync();
+  // exclusive scans over the cluster's segments
+  for (int e = tid; e < KL * 32; e += 32 * S::ColWarps) {
+    unsigned run = 0;
+    for (int r = 0; r < rank; ++r) run += cluster.map_shared_rank(sT, r)[e];
+#pragma unroll 4
+    for (int w = 0; w < S::Segs; ++w) {
+      BT *const s = sB + w * KL * 32 + e;
+      const unsigned v = *s;
+      *s = (BT)run;
+      run += v;
+    }
+  }
+  if (tid < KL) {
+    uint2 run = make_uint2(0u, 0u);
+    for (int r = 0; r < rank; ++r) {
+      const uint2 x = cluster.map_shared_rank(tot, r)[S::Segs * KL + tid];
+      run.x += x.x, run.y += x.y;
+    }
+    for (int w = 0; w < S::Segs; ++w) {
+      const uint2 x = tot[w * KL + tid];
+      tot[w * KL + tid] = run;
+      run.x += x.x, run.y += x.y;
+    }
+  }
+  cluster.sync();  // also: no CTA ends while another reads its totals
+  if (rank == 0 && wid == 0) {
+    if (lane < KL) J.c_rec[((size_t)kg * Gp + c) * (H + 1) * KL + lane] = make_uint2(0u, 0u);
+    // slot 0 of every threshold: no mixed row yet
+    BT *vec = static_cast<BT *>(J.c_vec) + (size_t)c * K * (H + 1) * 32 + lane;
+    for (int t = KL * kg; t < min(KL * kg + KL, K); ++t) vec[(size_t)t * (H + 1) * 32] = 0;
+  }
+  const uint2 t = tot[(wid * S::Sub + sub) * KL + j];
+  pt = t.x;
+  mc = t.y;
+  col_pass<KL, BT, true>(J, c, kg, K, row0, per, rend, mine, pt, mc, mh);
+}
+
+// What a launch does beside writing the output image.
+enum { kOut = 0, kOutKeep = 1, kCountsOnly = 2 };
+
+// The images of a lookup launch travel as kernel parameters: every block reads
+// its image's pointers and sizes from constant memory, as uniform values.
+struct LookJob {
+  Image in, out;
+  const uint8_t *bins;
+  const uint2 *rec;
+  const void *vec;
+  const longlong2 *s12;
+  unsigned *cnt;      // count planes (or null), field f's at cnt + f * cnt_step
+  float2 *mom;        // window moments (or null)
+  DebugPlanes dbg;
+  long long cnt_step;
+  int qbits, shift, b0, pad;
+};
+struct LookPack {
+  LookJob j[kCompactImages];
+  int n, rows;
+};
+
+// A block covers 128 columns x `rows` rows, a thread one column: what depends
+// on the column (the windows' left and right edges, their chunks) is formed
+// once for its rows, and what depends on the row is uniform. kPlain: no debug
+// planes and the literal area is off; kSmall as for window_variance; kDt as
+// for k_lookup_counts. kMode: kOut the output only; kOutKeep also the count
+// planes and window moments for the backward; kCountsOnly only the count
+// planes.
+// Bound by load latency and issue. At 12 MP, three fields, eight blocks per SM
+// (64 registers) and three fields' loads in flight took 273 us; 10 and 12
+// blocks 298 and 311; one field at a time at 10 and 16 blocks 313 and 334;
+// descriptors read from global memory instead of the parameters 372 (at 8).
+constexpr int kLookCols = 128;
+constexpr int kFieldBatch = 3;
+
+template <int NF, class BT, bool kPlain, int kSmall, int kDt, int kMode>
+__global__ void __launch_bounds__(kLookCols, 8)
+    k_lookup_compact(const __grid_constant__ DevParams P, const __grid_constant__ LookPack L) {
+  int jb = 0;
+  while (jb + 1 < L.n && L.j[jb + 1].b0 <= (int)blockIdx.x) ++jb;
+  const LookJob &J = L.j[jb];
+  const int W = J.in.W, H = J.in.H;
+  const int bx = (W + kLookCols - 1) / kLookCols;
+  const int lb = blockIdx.x - J.b0, by = lb / bx;
+  const int x = (lb - by * bx) * kLookCols + (int)threadIdx.x;
+  if (x >= W) return;
+  const int K = P.n_bins - 1, incl = (P.flags & kFlagCdfIncl) ? 1 : 0, shift = J.shift;
+  const unsigned cstep = (unsigned)(H + 1) << shift;         // records per chunk
+  const unsigned gstep = ((unsigned)(W >> 5) + 1u) * cstep;  // per threshold group
+  const unsigned slots = (unsigned)(H + 1);                  // vectors per threshold
+  const uint2 *__restrict__ rec = J.rec;
+  const BT *__restrict__ vec = static_cast<const BT *>(J.vec);
+  const float inv_scale = ldexpf(1.f, -J.qbits);
+  const float inv_scale2 = inv_scale * inv_scale;
+  const int y0 = by * L.rows, yend = min(y0 + L.rows, H);
+#pragma unroll 1
+  for (int y = y0; y < yend; ++y) {
+    const unsigned pix = (unsigned)y * (unsigned)W + (unsigned)x;
+    const int t = (int)__ldg(J.bins + pix) + incl;
+    const bool look = t > 0 && t <= K;
+    const unsigned k = look ? (unsigned)(t - 1) : 0u;
+    const unsigned kofs = (k >> 5) * gstep + (k & 31u);  // (one group below 32 thresholds)
+    Fusion fu;
+    // fields in batches whose loads are in flight together: all records, then
+    // all vector entries (slot 0 where no row is mixed), then the moments
+#pragma unroll
+    for (int f0 = 0; f0 < NF; f0 += kFieldBatch) {
+      unsigned cnt[kFieldBatch];
+      if (look) {
+        uint2 r[kFieldBatch][4];
+        unsigned e[kFieldBatch][4];
+#pragma unroll
+        for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
+          const int f = f0 + i;
+          const unsigned ul = (unsigned)max(x - P.rx[f], 0), ur = (unsigned)min(x + P.rx[f], W - 1) + 1u;
+          const unsigned p0 = (unsigned)max(y - P.ry[f], 0), p1 = (unsigned)min(y + P.ry[f], H - 1) + 1u;
+          const unsigned cl = (ul >> 5) * cstep + kofs, cr = (ur >> 5) * cstep + kofs;
+          const uint2 *ra = rec + (size_t)(p0 << shift), *rb = rec + (size_t)(p1 << shift);
+          r[i][0] = __ldg(ra + cl);
+          r[i][1] = __ldg(rb + cl);
+          r[i][2] = __ldg(ra + cr);
+          r[i][3] = __ldg(rb + cr);
+        }
+#pragma unroll
+        for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
+          const int f = f0 + i;
+          const unsigned ul = (unsigned)max(x - P.rx[f], 0), ur = (unsigned)min(x + P.rx[f], W - 1) + 1u;
+          const unsigned ol = ul & 31u, orr = ur & 31u;
+          // C(ur, p1) - C(ur, p0) - (C(ul, p1) - C(ul, p0))
+          cnt[i] = (r[i][3].x - r[i][2].x) - (r[i][1].x - r[i][0].x) + orr * ((r[i][3].y - r[i][2].y) & 0xffffu) -
+                   ol * ((r[i][1].y - r[i][0].y) & 0xffffu);
+          const unsigned vl = ((ul >> 5) * (unsigned)K + k) * slots, vr = ((ur >> 5) * (unsigned)K + k) * slots;
+          const BT *pl = vec + ol, *pr = vec + orr;
+          e[i][0] = __ldg(pl + (size_t)(vl + (r[i][0].y >> 16)) * 32);
+          e[i][1] = __ldg(pl + (size_t)(vl + (r[i][1].y >> 16)) * 32);
+          e[i][2] = __ldg(pr + (size_t)(vr + (r[i][2].y >> 16)) * 32);
+          e[i][3] = __ldg(pr + (size_t)(vr + (r[i][3].y >> 16)) * 32);
+        }
+#pragma unroll
+        for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i)
+          cnt[i] += (unsigned)(BT)(e[i][3] - e[i][2]) - (unsigned)(BT)(e[i][1] - e[i][0]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
+          const Win w = window_of(P, f0 + i, x, y, W, H);  // threshold n: the whole window
+          cnt[i] = t > 0 ? (unsigned)((w.x1 - w.x0 + 1) * (w.y1 - w.y0 + 1)) : 0u;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
+        const int f = f0 + i;
+        if (kMode == kCountsOnly || (kPlain ? kMode == kOutKeep : J.cnt != nullptr))
+          J.cnt[f * J.cnt_step + pix] = cnt[i];
+        if (kMode != kCountsOnly)
+          fold_field<kPlain, kMode == kOutKeep, kSmall>(P, f, x, y, W, H, cnt[i], J.s12, J.qbits, inv_scale2, fu,
+                                                        J.dbg, J.mom, inv_scale);
+      }
+    }
+    if (kMode != kCountsOnly) finish_pixel<kPlain, kDt>(J.in, J.out, P, x, y, fu, J.dbg);
+  }
+}
+
+template <int KL, class BT>
+int launch_cols(const Job *jobs, int njobs, int blocks, int K, cudaStream_t s) {
+  using S = Shape<KL>;
+  const size_t smem = (size_t)(S::Segs + 1) * KL * (32 * sizeof(BT) + sizeof(uint2));
+  if (cudaFuncSetAttribute(k_compact_cols<KL, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+      cudaSuccess)
+    return -1;
+  k_compact_cols<KL, BT><<<blocks, 32 * S::ColWarps, smem, s>>>(jobs, njobs, K);
+  return 1;
+}
+
+template <int KL>
+int launch_build(const Job *jobs, int njobs, int row_blocks, int col_blocks, int K, bool wide, cudaStream_t s) {
+  k_compact_rows<KL><<<row_blocks, 32 * kRowWarps, 0, s>>>(jobs, njobs, K);
+  const int r = wide ? launch_cols<KL, uint32_t>(jobs, njobs, col_blocks, K, s)
+                     : launch_cols<KL, uint16_t>(jobs, njobs, col_blocks, K, s);
+  return r < 0 ? -1 : 2;
+}
+
+// Thresholds per group for K of them (log2).
+int group_shift(int K) { return K <= 4 ? 2 : K <= 8 ? 3 : K <= 16 ? 4 : 5; }
+
+}  // namespace
+
+bool plan_compact(const DevParams &P, int W, int H, CompactPlan &C) {
+  if (P.n_bins < 2 || W > 65535 || H > 65535) return false;
+  const long long K = P.n_bins - 1, Gp = W / 32 + 1;
+  int tall = 0;
+  for (int f = 0; f < P.n_fields; ++f) tall = std::max(tall, std::min(2 * P.ry[f] + 1, H));
+  C.shift = group_shift((int)K);
+  C.wide = 31LL * tall > 65535;
+  const long long KL = 1LL << C.shift, groups = (K + KL - 1) >> C.shift;
+  const long long recs = groups * Gp * (H + 1) * KL, slots = Gp * K * (H + 1);
+  if (recs >= (1LL << 31) || slots >= (1LL << 31)) return false;  // 32-bit indices in the lookup
+  C.rec_bytes = sizeof(uint2) * (size_t)recs;
+  C.row_bytes = sizeof(uint16_t) * (size_t)(groups * Gp * H * KL);
+  C.vec_bytes = (size_t)slots * 32 * (C.wide ? 4 : 2);
+  return true;
+}
+
+int compact_row_blocks(int H, int K) {
+  const int sh = group_shift(K), per = kRowWarps * (32 >> sh);
+  return (H + per - 1) / per * ((K + (1 << sh) - 1) >> sh);
+}
+
+int compact_col_blocks(int W, int K) {
+  const int sh = group_shift(K);
+  return kCluster * (W / 32 + 1) * ((K + (1 << sh) - 1) >> sh);
+}
+
+int launch_compact_build(const Job *jobs, int njobs, int row_blocks, int col_blocks, int K, bool wide,
+                         cudaStream_t s) {
+  switch (group_shift(K)) {
+    case 2: return launch_build<4>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
+    case 3: return launch_build<8>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
+    case 4: return launch_build<16>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
+    default: return launch_build<32>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
+  }
+}
+
+int compact_look_blocks(int W, int H, int rows) {
+  return (W + kLookCols - 1) / kLookCols * ((H + rows - 1) / rows);
+}
+
+template <class BT, bool kPlain, int kSmall, int kDt, int kMode>
+static void launch_look(const DevParams &P, const LookPack &L, int blocks, cudaStream_t s) {
+  switch (P.n_fields) {
+#define TM_LOOK(nf)                                                                                            \
+  case nf: k_lookup_compact<nf, BT, kPlain, kSmall, kDt, kMode><<<blocks, kLookCols, 0, s>>>(P, L); break;
+    TM_LOOK(1) TM_LOOK(2) TM_LOOK(3) TM_LOOK(4) TM_LOOK(5) TM_LOOK(6) TM_LOOK(7) TM_LOOK(8)
+#undef TM_LOOK
+  }
+}
+
+template <class BT, int kSmall>
+static void launch_look_dtype(const DevParams &P, const LookPack &L, int blocks, int dtype, cudaStream_t s) {
+  if (dtype == kF32) launch_look<BT, true, kSmall, kF32, kOut>(P, L, blocks, s);
+  else if (dtype == kF16) launch_look<BT, true, kSmall, kF16, kOut>(P, L, blocks, s);
+  else launch_look<BT, true, kSmall, -1, kOut>(P, L, blocks, s);
+}
+
+int launch_lookup_compact(const DevParams &P, const Job *jobs, int njobs, int blocks, int rows, bool wide,
+                          bool plain, bool keep, bool counts_only, int dtype, cudaStream_t s) {
+  const bool general = !plain || (P.flags & kFlagAreaLit) || (keep && (wide || !P.small_win || dtype != kF32));
+  LookPack L{};
+  L.n = njobs;
+  L.rows = rows;
+  for (int i = 0; i < njobs; ++i) {
+    const Job &J = jobs[i];
+    L.j[i] = {J.in, J.out, J.bins, J.c_rec, J.c_vec, reinterpret_cast<const longlong2 *>(J.s1),
+              reinterpret_cast<unsigned *>(J.cnt), J.mom, J.dbg, J.cnt_off[1] / 4, J.qbits, J.c_shift,
+              J.b0[kStLook], 0};
+  }
+  if (counts_only) {
+    if (wide) launch_look<uint32_t, true, -1, -1, kCountsOnly>(P, L, blocks, s);
+    else launch_look<uint16_t, true, -1, -1, kCountsOnly>(P, L, blocks, s);
+  } else if (general) {
+    if (wide) launch_look<uint32_t, false, -1, -1, kOut>(P, L, blocks, s);
+    else launch_look<uint16_t, false, -1, -1, kOut>(P, L, blocks, s);
+  } else if (keep) {
+    launch_look<uint16_t, true, 1, kF32, kOutKeep>(P, L, blocks, s);
+  } else if (wide) {
+    launch_look_dtype<uint32_t, -1>(P, L, blocks, dtype, s);
+  } else if (P.small_win) {
+    launch_look_dtype<uint16_t, 1>(P, L, blocks, dtype, s);
+  } else {
+    launch_look_dtype<uint16_t, -1>(P, L, blocks, dtype, s);
+  }
+  return 1;
+}
+
+}  // namespace tmk

@@ -88,6 +88,27 @@ int sweep_ctas_per_sm(int n_fields, size_t smem, int width);
 int launch_sweep(const DevParams &P, const Job *jobs, int njobs, int nitems, int *queue, size_t smem, int ctas,
                  int width, cudaStream_t s);
 
+// Stage a3'': the compact integral histogram (tm_compact.cu). plan_compact: its
+// sizes for one image (false if the image is outside its index ranges). The
+// build over a group of jobs of n - 1 = K thresholds, from their bin maps and
+// group summaries (J.b0[kStCRows], J.b0[kStCCols]: the job's first blocks;
+// wide: CompactPlan::wide of any job; returns its launches, -1 on error).
+bool plan_compact(const DevParams &P, int W, int H, CompactPlan &C);
+int compact_row_blocks(int H, int K);
+int compact_col_blocks(int W, int K);
+int launch_compact_build(const Job *jobs, int njobs, int row_blocks, int col_blocks, int K, bool wide,
+                         cudaStream_t s);
+// The lookup from it (jobs: HOST descriptors of at most kCompactImages images,
+// which travel as kernel parameters): blocks of `rows` rows (compact_look_blocks of an image,
+// first block J.b0[kStLook]). plain: no job has debug planes
+// to write; keep: every job also gets its count planes (J.cnt, uint32) and
+// window moments (J.mom); counts_only: only its count planes; dtype as for
+// launch_lookup_counts.
+constexpr int kCompactImages = 32;
+int compact_look_blocks(int W, int H, int rows);
+int launch_lookup_compact(const DevParams &P, const Job *jobs, int njobs, int blocks, int rows, bool wide,
+                          bool plain, bool keep, bool counts_only, int dtype, cudaStream_t s);
+
 // Stage a4: per-pixel lookup, tone curve, fusion and colour restoration.
 int lookup_blocks(int W, int H);
 // plain: no job has debug planes to write and every job's count planes are
