@@ -709,7 +709,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
       J.b0[kStCRows] = g.rows;
       g.rows += compact_row_blocks(H, K);
       J.b0[kStCCols] = g.cols;
-      g.cols += compact_col_blocks(W, K);
+      g.cols += compact_col_units(W, K);
       J.b0[kStLook] = g.look;
       g.look += compact_look_blocks(W, H, look_rows);
       J.c_shift = C.shift;

@@ -26,7 +26,7 @@
 // Three launches per group of images:
 //   1. k_compact_rows: the prefix over the chunks of each row's counts below k
 //      (lanes = thresholds, walking along the row);
-//   2. k_compact_cols, a cluster of four CTAs per chunk and group of
+//   2. k_compact_cols, a cluster of CTAs per chunk and group of
 //      thresholds: its warps take consecutive row segments twice (lanes =
 //      thresholds, walking down the rows), once for the segments' totals and,
 //      after a scan of the totals over the segments, to write records and
@@ -34,8 +34,9 @@
 //   3. k_lookup_compact, a thread per column and a few rows: four records and
 //      up to four vector entries per field and pixel, then the lookup's
 //      arithmetic.
-// Thresholds come in groups of KL (32, or 4, 8, 16 where n - 1 is no larger):
-// a warp holds 32 / KL rows (launch 1) or row segments (launch 2) at once.
+// Thresholds come in groups of KL (64, or 4, 8, 16, 32 where n - 1 is no
+// larger), a group of 64 two adjacent ones to a lane; a warp holds the rows
+// (launch 1) or row segments (launch 2) that its 32 lanes take at once.
 // The bin ranges of the chunks come from the group summary of the bin pass.
 #include <cooperative_groups.h>
 
@@ -48,14 +49,22 @@ namespace tmk {
 namespace {
 
 constexpr int kRowWarps = 8;  // warps of a k_compact_rows block
-constexpr int kCluster = 4;   // CTAs that share a chunk's rows
-
+// A group of KL thresholds takes KL / T lanes of T adjacent thresholds each.
 template <int KL>
 struct Shape {
-  static constexpr int Sub = 32 / KL;                    // rows or segments of a warp
-  static constexpr int Step = KL == 32 ? 4 : KL == 16 ? 2 : 1;  // rows or chunks in flight together
-  static constexpr int ColWarps = KL == 32 ? 16 : KL == 16 ? 8 : 4;
+  static constexpr int T = KL == 64 ? 2 : 1;
+  static constexpr int Lanes = KL / T;                   // lanes of a row
+  static constexpr int Sub = 32 / Lanes;                 // rows or segments of a warp
+  static constexpr int Step = Sub == 1 ? 4 : Sub == 2 ? 2 : 1;  // rows or chunks in flight together
+  static constexpr int ColWarps = KL >= 32 ? 16 : KL == 16 ? 8 : 4;
+  static constexpr int MinBlocks = 32 / ColWarps;        // 64 registers
   static constexpr int Segs = ColWarps * Sub;            // row segments of a CTA
+  // column CTAs share a chunk's rows until the launch has this many warps.
+  // 12 MP, 63 thresholds, a forward with clusters of 2, 4, 8: 549, 536, 563
+  // us; 1080p, 31 thresholds, 4 and 8: 127 and 133; 32 1080p images in one
+  // launch, 1 and 4: 9.49 and 9.75 ms per 120 (short segments pay more for
+  // their totals, long ones leave the rows of a vertical edge to one warp).
+  static constexpr int Fill = KL == 64 ? 4864 : 3600;
 };
 
 // Whether a chunk row with bins in [g & 255, g >> 8] has bins on both sides of
@@ -65,14 +74,39 @@ __device__ __forceinline__ bool mixed_range(unsigned g, int k0) {
   return max((int)(g & 0xffu), k0) < min((int)(g >> 8), k0 + KL);
 }
 
+// Its thresholds k0 + 1 + t are t0 <= t < t1.
+template <int KL>
+__device__ __forceinline__ void mixed_thresholds(unsigned g, int k0, int &t0, int &t1) {
+  t0 = max((int)(g & 0xffu) - k0, 0);
+  t1 = min((int)(g >> 8) - k0, KL);
+}
+
 constexpr unsigned kNoRow = 0xffffu;  // a bin range on no threshold's lower side
 
-// Rows: lane = (row, threshold k0 + 1 + j), walking along the rows' chunks.
+// T adjacent uint16 as one load, and T records as one store.
+template <int T>
+__device__ __forceinline__ void load_prefix(const uint16_t *p, unsigned *v) {
+  if (T == 2) {
+    const unsigned w = __ldg(reinterpret_cast<const unsigned *>(p));
+    v[0] = w & 0xffffu;
+    v[T - 1] = w >> 16;
+  } else {
+    v[0] = __ldg(p);
+  }
+}
+template <int T>
+__device__ __forceinline__ void store_records(uint2 *p, const unsigned *pt, const unsigned *mc) {
+  if (T == 2) *reinterpret_cast<uint4 *>(p) = make_uint4(pt[0], mc[0], pt[T - 1], mc[T - 1]);
+  else *p = make_uint2(pt[0], mc[0]);
+}
+
+// Rows: lane = (row, T thresholds), walking along the rows' chunks.
 template <int KL>
 __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(const Job *__restrict__ jobs, int njobs, int K) {
   using S = Shape<KL>;
+  constexpr int T = S::T, NL = S::Lanes;
   const Job &J = jobs[find_job(jobs, njobs, kStCRows, blockIdx.x)];
-  const int lane = threadIdx.x & 31, sub = lane / KL, j = lane % KL;
+  const int lane = threadIdx.x & 31, sub = lane / NL, j = lane % NL;
   const int W = J.in.W, H = J.in.H, G = (W + 31) >> 5, Gp = (W >> 5) + 1;
   const int rb = (H + kRowWarps * S::Sub - 1) / (kRowWarps * S::Sub);
   const int lb = blockIdx.x - J.b0[kStCRows];
@@ -81,16 +115,18 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(const Job *__re
   if (v0 >= H) return;
   const bool own = v0 + sub < H;
   const int v = min(v0 + sub, H - 1);  // the lane's row (past the last: read, not written)
-  const unsigned k = (unsigned)(k0 + 1 + j), k8 = k << 8;
+  const unsigned k8 = (unsigned)(k0 + 1 + T * j) << 8;  // the lane's first threshold
   const uint8_t *__restrict__ bins = J.bins + (size_t)v0 * W + lane;
   const uint16_t *__restrict__ grow = J.grp + (size_t)v * G;
   const size_t cstride = (size_t)H * KL;
-  uint16_t *__restrict__ dst = J.c_row + ((size_t)kg * Gp * H + v) * KL + j;
-  unsigned run = 0;
-  for (int cb = 0; cb < Gp; cb += KL) {
+  uint16_t *__restrict__ dst = J.c_row + ((size_t)kg * Gp * H + v) * KL + T * j;
+  unsigned run[T];
+#pragma unroll
+  for (int z = 0; z < T; ++z) run[z] = 0;
+  for (int cb = 0; cb < Gp; cb += NL) {
     const unsigned gl = cb + j < G && own ? (unsigned)__ldg(grow + cb + j) : kNoRow;
     const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit (sub, chunk of the batch)
-    const int n = min(KL, Gp - cb);
+    const int n = min(NL, Gp - cb);
     for (int i = 0; i < n; i += S::Step) {
       int b[S::Step][S::Sub];
 #pragma unroll
@@ -99,50 +135,62 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(const Job *__re
         for (int q = 0; q < S::Sub; ++q) {
           const int col = 32 * (cb + i + u);
           b[u][q] = 256;
-          if (((mixed >> (q * KL + ((i + u) & (KL - 1)))) & 1u) && col + lane < W)
+          if (((mixed >> (q * NL + ((i + u) & (NL - 1)))) & 1u) && col + lane < W)
             b[u][q] = (int)__ldg(bins + (size_t)q * W + col);
         }
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
         if (i + u >= n) break;
-        const unsigned g = __shfl_sync(0xffffffffu, gl, sub * KL + i + u);
-        if (own) *dst = (uint16_t)run;
+        const unsigned g = __shfl_sync(0xffffffffu, gl, sub * NL + i + u);
+        if (own) {
+          if (T == 2) *reinterpret_cast<unsigned *>(dst) = run[0] | (run[T - 1] << 16);
+          else *dst = (uint16_t)run[0];
+        }
         dst += cstride;
-        unsigned cc = g < k8 ? 32u : 0u;  // every bin of the chunk below k
-        unsigned ball = 0;
-        if (S::Sub > 1 || ((mixed >> (i + u)) & 1u)) ball = __ballot_sync(0xffffffffu, (g & 0xffu) < k && k8 <= g);
+        unsigned cc[T];
+#pragma unroll
+        for (int z = 0; z < T; ++z) cc[z] = g < k8 + 256u * z ? 32u : 0u;  // every bin of the chunk below k
 #pragma unroll
         for (int q = 0; q < S::Sub; ++q) {
-          unsigned part = S::Sub == 1 ? ball : (ball >> (q * KL)) & ((1u << (KL & 31)) - 1u);
-          while (part) {
-            const int t = __ffs(part) - 1;
-            part &= part - 1;
-            const unsigned mask = __ballot_sync(0xffffffffu, b[u][q] <= k0 + t);  // bins below k0 + 1 + t
-            if (lane == q * KL + t) cc = (unsigned)__popc(mask);
+          if (!((mixed >> (q * NL + i + u)) & 1u)) continue;
+          int t0, t1;
+          mixed_thresholds<KL>(S::Sub == 1 ? g : __shfl_sync(0xffffffffu, gl, q * NL + i + u), k0, t0, t1);
+          for (int t = t0 / T * T; t < t1; t += T) {
+#pragma unroll
+            for (int z = 0; z < T; ++z) {
+              const unsigned mask = __ballot_sync(0xffffffffu, b[u][q] <= k0 + t + z);  // bins below k0 + 1 + t + z
+              if (lane == q * NL + t / T) cc[z] = (unsigned)__popc(mask);
+            }
           }
         }
-        run += cc;
+#pragma unroll
+        for (int z = 0; z < T; ++z) run[z] += cc[z];
       }
     }
   }
 }
 
-// A warp's pass over its row segments of chunk c: lane = (segment sub,
-// threshold k0 + 1 + j) with rows row0 .. of segment 0, each segment `per`
-// rows, the last ending before rend. The lane's state is pt and mc = m |
-// (mixed rows) << 16.
-// kWrite: write records and vectors; sB[(sub, j)][o] holds the vectors (lane =
-// column o there). Else sB counts, per (sub, j) and column, the pixels of the
-// mixed rows with bin k0 + j (k0 or less for j = 0), and mh the mixed rows
-// wholly below the lane's threshold.
+// The lane's state over its rows: T thresholds' pt and mc = m | (mixed rows)
+// << 16, and mh, the mixed rows wholly below the threshold (first pass only).
+template <int T>
+struct ColState {
+  unsigned pt[T], mc[T], mh[T];
+};
+
+// A warp's pass over its row segments of chunk c: lane = (segment, T
+// thresholds) with rows row0 .. of segment 0, each segment `per` rows, the
+// last ending before rend. kWrite: write records and vectors; sB[(sub, t)][o]
+// holds the vectors (lane = column o there). Else sB counts, per (sub, t) and
+// column, the pixels of the mixed rows with bin k0 + t (k0 or less for t = 0).
 template <int KL, class BT, bool kWrite>
 __device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int row0, int per, int rend, BT *sB,
-                                         unsigned &pt, unsigned &mc, unsigned &mh) {
+                                         ColState<Shape<KL>::T> &st) {
   using S = Shape<KL>;
-  const int lane = threadIdx.x & 31, sub = lane / KL, j = lane % KL;
+  constexpr int T = S::T, NL = S::Lanes;
+  const int lane = threadIdx.x & 31, sub = lane / NL, j = lane % NL;
   const int W = J.in.W, H = J.in.H, G = (W + 31) >> 5, Gp = (W >> 5) + 1;
   const int k0 = KL * kg;
-  const unsigned k = (unsigned)(k0 + 1 + j), k8 = k << 8;
+  const unsigned k8 = (unsigned)(k0 + 1 + T * j) << 8;
   const int mine = row0 + sub * per;
   int left = min(per, rend - mine);  // the lane's rows still to come
   const unsigned lt = (1u << lane) - 1u;
@@ -150,66 +198,78 @@ __device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int
   const uint8_t *__restrict__ bins = J.bins + (size_t)row0 * W + 32 * c + lane;
   const uint16_t *__restrict__ grp = J.grp + (size_t)(mine + j) * G + c;
   const size_t plane = (size_t)kg * Gp + c;
-  const uint16_t *__restrict__ row = J.c_row + (plane * H + mine) * KL + j;
-  uint2 *__restrict__ rec = J.c_rec + (plane * (H + 1) + mine + 1) * KL + j;
+  const uint16_t *__restrict__ row = J.c_row + (plane * H + mine) * KL + T * j;
+  uint2 *__restrict__ rec = J.c_rec + (plane * (H + 1) + mine + 1) * KL + T * j;
   BT *__restrict__ vec = static_cast<BT *>(J.c_vec) + ((size_t)c * K + k0) * (H + 1) * 32 + lane;
   const unsigned vstep = (unsigned)(H + 1);
-  for (int ib = 0; ib < per; ib += KL) {
+  for (int ib = 0; ib < per; ib += NL) {
     const unsigned gl = c < G && j < left ? (unsigned)__ldg(grp) : kNoRow;
-    grp += (size_t)KL * G;
+    grp += (size_t)NL * G;
     const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit (sub, row of the batch)
-    const int n = min(KL, per - ib);
+    const int n = min(NL, per - ib);
     for (int i = 0; i < n; i += S::Step) {
-      unsigned rp[S::Step];
+      unsigned rp[S::Step][T];
       int b[S::Step][S::Sub];
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
-        rp[u] = u < left ? (unsigned)__ldg(row + u * KL) : 0u;
+#pragma unroll
+        for (int z = 0; z < T; ++z) rp[u][z] = 0;
+        if (u < left) load_prefix<T>(row + u * KL, rp[u]);
 #pragma unroll
         for (int q = 0; q < S::Sub; ++q) {
           b[u][q] = 256;
-          if (((mixed >> (q * KL + ((i + u) & (KL - 1)))) & 1u) && colok)
+          if (((mixed >> (q * NL + ((i + u) & (NL - 1)))) & 1u) && colok)
             b[u][q] = (int)__ldg(bins + (size_t)(unsigned)(q * per + u) * W);
         }
       }
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
         // (rows past the segment have no bins below or on both sides)
-        const unsigned g = __shfl_sync(0xffffffffu, gl, sub * KL + ((i + u) & (KL - 1)));
-        pt += rp[u];
-        if (g < k8) ++mc;
-        if (S::Sub > 1 || ((mixed >> ((i + u) & (KL - 1))) & 1u)) {
-          const bool both = (g & 0xffu) < k && k8 <= g;
-          if (both) mc += 0x10000u;
-          if (!kWrite) {
-            if (g < k8 && mixed_range<KL>(g, k0)) ++mh;
+        const unsigned g = __shfl_sync(0xffffffffu, gl, sub * NL + ((i + u) & (NL - 1)));
 #pragma unroll
-            for (int q = 0; q < S::Sub; ++q) {
-              const int h = max(b[u][q] - k0, 0);
-              if (h < KL) {
-                BT *const s = sB + (q * KL + h) * 32 + lane;
-                *s = (BT)(*s + 1);
-              }
+        for (int z = 0; z < T; ++z) {
+          st.pt[z] += rp[u][z];
+          if (g < k8 + 256u * z) ++st.mc[z];
+        }
+#pragma unroll
+        for (int z = 0; z < T; ++z) {
+          const unsigned kz = k8 + 256u * z;
+          if (g >= kz && ((g & 0xffu) << 8) < kz) st.mc[z] += 0x10000u;  // bins on both sides
+          if (!kWrite && g < kz && mixed_range<KL>(g, k0)) ++st.mh[z];
+        }
+#pragma unroll
+        for (int q = 0; q < S::Sub; ++q) {
+          if (!((mixed >> (q * NL + ((i + u) & (NL - 1)))) & 1u)) continue;
+          if (!kWrite) {
+            const int h = max(b[u][q] - k0, 0);
+            if (h < KL) {
+              BT *const s = sB + (q * KL + h) * 32 + lane;
+              *s = (BT)(*s + 1);
             }
           } else {
-            const unsigned ball = __ballot_sync(0xffffffffu, both);
+            int t0, t1;
+            mixed_thresholds<KL>(S::Sub == 1 ? g : __shfl_sync(0xffffffffu, gl, q * NL + ((i + u) & (NL - 1))), k0,
+                                 t0, t1);
+            for (int t = t0 / T * T; t < t1; t += T) {
+              BT *const s = sB + (q * KL + t) * 32 + lane;
+              unsigned slot[T];
+              BT val[T];
 #pragma unroll
-            for (int q = 0; q < S::Sub; ++q) {
-              unsigned part = S::Sub == 1 ? ball : (ball >> (q * KL)) & ((1u << (KL & 31)) - 1u);
-              while (part) {
-                const int t = __ffs(part) - 1;  // threshold k0 + 1 + t
-                part &= part - 1;
-                const unsigned mask = __ballot_sync(0xffffffffu, b[u][q] <= k0 + t);
-                const unsigned slot = __shfl_sync(0xffffffffu, mc, q * KL + t) >> 16;
-                BT *const s = sB + (q * KL + t) * 32 + lane;
-                const BT val = (BT)(*s + __popc(mask & lt));
-                *s = val;
-                vec[(size_t)((unsigned)t * vstep + slot) * 32] = val;
+              for (int z = 0; z < T; ++z) {
+                const unsigned mask = __ballot_sync(0xffffffffu, b[u][q] <= k0 + t + z);
+                slot[z] = __shfl_sync(0xffffffffu, st.mc[z], q * NL + t / T) >> 16;
+                val[z] = (BT)(s[z * 32] + __popc(mask & lt));
               }
+#pragma unroll
+              for (int z = 0; z < T; ++z)
+                if (t + z >= t0 && t + z < t1) {
+                  s[z * 32] = val[z];
+                  vec[(size_t)((unsigned)(t + z) * vstep + slot[z]) * 32] = val[z];
+                }
             }
           }
         }
-        if (kWrite && u < left) rec[u * KL] = make_uint2(pt, mc);
+        if (kWrite && u < left) store_records<T>(rec + u * KL, st.pt, st.mc);
       }
       row += S::Step * KL;
       rec += S::Step * KL;
@@ -219,56 +279,64 @@ __device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int
   }
 }
 
-// Columns: cluster -> (image, chunk, threshold group), CTA -> a quarter of the
+// Columns: cluster -> (image, chunk, threshold group), CTA -> a share of the
 // rows, cut into Segs segments.
 template <int KL, class BT>
-__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(32 * Shape<KL>::ColWarps, KL == 32 ? 3 : 8)
+__global__ void __launch_bounds__(32 * Shape<KL>::ColWarps, sizeof(BT) == 2 ? Shape<KL>::MinBlocks : 1)
     k_compact_cols(const Job *__restrict__ jobs, int njobs, int K) {
   using S = Shape<KL>;
+  constexpr int T = S::T, NL = S::Lanes;
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char smem[];
   BT *const sB = reinterpret_cast<BT *>(smem);                  // [Segs][KL][32]
   BT *const sT = sB + S::Segs * KL * 32;                        // [KL][32]: the CTA's totals
   uint2 *const tot = reinterpret_cast<uint2 *>(sT + KL * 32);   // [Segs + 1][KL], the last: the CTA's totals
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const Job &J = jobs[find_job(jobs, njobs, kStCCols, blockIdx.x)];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, sub = lane / KL, j = lane % KL;
+  const int rank = (int)cluster.block_rank(), nc = (int)cluster.num_blocks();
+  const Job &J = jobs[find_job(jobs, njobs, kStCCols, blockIdx.x / nc)];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, sub = lane / NL, j = lane % NL;
   const int H = J.in.H, Gp = (J.in.W >> 5) + 1;
-  const int lb = (blockIdx.x - J.b0[kStCCols]) / kCluster;
+  const int lb = blockIdx.x / nc - J.b0[kStCCols];
   const int kg = lb / Gp, c = lb - kg * Gp;
-  const int share = (H + kCluster - 1) / kCluster, per = (share + S::Segs - 1) / S::Segs;
+  const int share = (H + nc - 1) / nc, per = (share + S::Segs - 1) / S::Segs;
   const int row0 = rank * share + wid * S::Sub * per, rend = min((rank + 1) * share, H);
   BT *const mine = sB + wid * S::Sub * KL * 32;
-  for (int i = lane; i < S::Sub * KL * 32; i += 32) mine[i] = 0;
+  for (int i = lane; i < S::Sub * KL * 32 * (int)sizeof(BT) / 4; i += 32) reinterpret_cast<unsigned *>(mine)[i] = 0;
   __syncwarp();
-  unsigned pt = 0, mc = 0, mh = 0;
-  col_pass<KL, BT, false>(J, c, kg, K, row0, per, rend, mine, pt, mc, mh);
-  tot[(wid * S::Sub + sub) * KL + j] = make_uint2(pt, mc);
+  ColState<T> st{};
+  col_pass<KL, BT, false>(J, c, kg, K, row0, per, rend, mine, st);
+  uint2 *const mytot = tot + (wid * S::Sub + sub) * KL + T * j;
+#pragma unroll
+  for (int z = 0; z < T; ++z) mytot[z] = make_uint2(st.pt[z], st.mc[z]);
   // per segment: the vectors' totals from the column counts (the pixels of
   // mixed rows below k, less those of rows wholly below it, left of o)
-  const unsigned any = __ballot_sync(0xffffffffu, mc >> 16);
-  if (any) {
+  unsigned any[T];
+#pragma unroll
+  for (int z = 0; z < T; ++z) any[z] = __ballot_sync(0xffffffffu, st.mc[z] >> 16);
+  if (any[0] | any[T - 1]) {
     __syncwarp();
 #pragma unroll 1
     for (int q = 0; q < S::Sub; ++q) {
       unsigned below = 0;
-#pragma unroll 4
-      for (int t = 0; t < KL; ++t) {
-        BT *const s = mine + (q * KL + t) * 32 + lane;
-        below += *s;
-        unsigned e = 0;
-        if ((any >> (q * KL + t)) & 1u) {
-          const unsigned v = below - __shfl_sync(0xffffffffu, mh, q * KL + t);
-          e = v;
+#pragma unroll 2
+      for (int t = 0; t < NL; ++t) {
 #pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, e, o);
-            if (lane >= o) e += y;
+        for (int z = 0; z < T; ++z) {
+          BT *const s = mine + (q * KL + T * t + z) * 32 + lane;
+          below += *s;
+          unsigned e = 0;
+          if ((any[z] >> (q * NL + t)) & 1u) {
+            const unsigned v = below - __shfl_sync(0xffffffffu, st.mh[z], q * NL + t);
+            e = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const unsigned y = __shfl_up_sync(0xffffffffu, e, o);
+              if (lane >= o) e += y;
+            }
+            e -= v;
           }
-          e -= v;
+          *s = (BT)e;
         }
-        *s = (BT)e;
       }
     }
   }
@@ -314,15 +382,19 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(32 * Shape<KL
   }
   cluster.sync();  // also: no CTA ends while another reads its totals
   if (rank == 0 && wid == 0) {
-    if (lane < KL) J.c_rec[((size_t)kg * Gp + c) * (H + 1) * KL + lane] = make_uint2(0u, 0u);
+    uint2 *const rec = J.c_rec + ((size_t)kg * Gp + c) * (H + 1) * KL;
+    for (int t = lane; t < KL; t += 32) rec[t] = make_uint2(0u, 0u);
     // slot 0 of every threshold: no mixed row yet
     BT *vec = static_cast<BT *>(J.c_vec) + (size_t)c * K * (H + 1) * 32 + lane;
     for (int t = KL * kg; t < min(KL * kg + KL, K); ++t) vec[(size_t)t * (H + 1) * 32] = 0;
   }
-  const uint2 t = tot[(wid * S::Sub + sub) * KL + j];
-  pt = t.x;
-  mc = t.y;
-  col_pass<KL, BT, true>(J, c, kg, K, row0, per, rend, mine, pt, mc, mh);
+#pragma unroll
+  for (int z = 0; z < T; ++z) {
+    const uint2 x = mytot[z];
+    st.pt[z] = x.x;
+    st.mc[z] = x.y;
+  }
+  col_pass<KL, BT, true>(J, c, kg, K, row0, per, rend, mine, st);
 }
 
 // What a launch does beside writing the output image.
@@ -387,7 +459,7 @@ __global__ void __launch_bounds__(kLookCols, 8)
     const int t = (int)__ldg(J.bins + pix) + incl;
     const bool look = t > 0 && t <= K;
     const unsigned k = look ? (unsigned)(t - 1) : 0u;
-    const unsigned kofs = (k >> 5) * gstep + (k & 31u);  // (one group below 32 thresholds)
+    const unsigned kofs = (k >> 6) * gstep + (k & 63u);  // (one group up to 64 thresholds)
     Fusion fu;
     // fields in batches whose loads are in flight together: all records, then
     // all vector entries (slot 0 where no row is mixed), then the moments
@@ -455,8 +527,20 @@ int launch_cols(const Job *jobs, int njobs, int blocks, int K, cudaStream_t s) {
   if (cudaFuncSetAttribute(k_compact_cols<KL, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return -1;
-  k_compact_cols<KL, BT><<<blocks, 32 * S::ColWarps, smem, s>>>(jobs, njobs, K);
-  return 1;
+  int nc = 1;  // CTAs that share a chunk's rows
+  while (nc < 8 && blocks * S::ColWarps * nc < S::Fill) nc *= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(blocks * nc));
+  cfg.blockDim = dim3(32 * S::ColWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)nc;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_compact_cols<KL, BT>, jobs, njobs, K) == cudaSuccess ? 1 : -1;
 }
 
 template <int KL>
@@ -468,7 +552,7 @@ int launch_build(const Job *jobs, int njobs, int row_blocks, int col_blocks, int
 }
 
 // Thresholds per group for K of them (log2).
-int group_shift(int K) { return K <= 4 ? 2 : K <= 8 ? 3 : K <= 16 ? 4 : 5; }
+int group_shift(int K) { return K <= 4 ? 2 : K <= 8 ? 3 : K <= 16 ? 4 : K <= 32 ? 5 : 6; }
 
 }  // namespace
 
@@ -489,13 +573,13 @@ bool plan_compact(const DevParams &P, int W, int H, CompactPlan &C) {
 }
 
 int compact_row_blocks(int H, int K) {
-  const int sh = group_shift(K), per = kRowWarps * (32 >> sh);
+  const int sh = group_shift(K), lanes = sh == 6 ? 32 : 1 << sh, per = kRowWarps * (32 / lanes);
   return (H + per - 1) / per * ((K + (1 << sh) - 1) >> sh);
 }
 
-int compact_col_blocks(int W, int K) {
+int compact_col_units(int W, int K) {
   const int sh = group_shift(K);
-  return kCluster * (W / 32 + 1) * ((K + (1 << sh) - 1) >> sh);
+  return (W / 32 + 1) * ((K + (1 << sh) - 1) >> sh);
 }
 
 int launch_compact_build(const Job *jobs, int njobs, int row_blocks, int col_blocks, int K, bool wide,
@@ -504,7 +588,8 @@ int launch_compact_build(const Job *jobs, int njobs, int row_blocks, int col_blo
     case 2: return launch_build<4>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
     case 3: return launch_build<8>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
     case 4: return launch_build<16>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
-    default: return launch_build<32>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
+    case 5: return launch_build<32>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
+    default: return launch_build<64>(jobs, njobs, row_blocks, col_blocks, K, wide, s);
   }
 }
 

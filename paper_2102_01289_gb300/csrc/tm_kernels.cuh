@@ -91,12 +91,12 @@ int launch_sweep(const DevParams &P, const Job *jobs, int njobs, int nitems, int
 // Stage a3'': the compact integral histogram (tm_compact.cu). plan_compact: its
 // sizes for one image (false if the image is outside its index ranges). The
 // build over a group of jobs of n - 1 = K thresholds, from their bin maps and
-// group summaries (J.b0[kStCRows], J.b0[kStCCols]: the job's first blocks;
-// wide: CompactPlan::wide of any job; returns its launches, -1 on error).
+// group summaries (J.b0[kStCRows], J.b0[kStCCols]: the job's first block and
+// its first unit of the column launch; wide: CompactPlan::wide of any job; returns its launches, -1 on error).
 bool plan_compact(const DevParams &P, int W, int H, CompactPlan &C);
 int compact_row_blocks(int H, int K);
-int compact_col_blocks(int W, int K);
-int launch_compact_build(const Job *jobs, int njobs, int row_blocks, int col_blocks, int K, bool wide,
+int compact_col_units(int W, int K);
+int launch_compact_build(const Job *jobs, int njobs, int row_blocks, int col_units, int K, bool wide,
                          cudaStream_t s);
 // The lookup from it (jobs: HOST descriptors of at most kCompactImages images,
 // which travel as kernel parameters): blocks of `rows` rows (compact_look_blocks of an image,
