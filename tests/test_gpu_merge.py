@@ -84,3 +84,27 @@ def test_merge_then_tone_map_matches_oracle(orc):
     ref, _ = orc.forward(gpu_merged, op)  # the forward on the GPU's own WDR image
     got = out.cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - ref) <= 1e-4 * np.maximum(np.abs(ref), 1e-3))
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 8])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
+def test_merge_vector_and_scalar_paths_agree(n, dtype):
+    """Gapless images (four pixels at a time over the whole image, odd widths
+    and a ragged end included) against the same pixels with padded rows and
+    unaligned bases (one pixel at a time): bit-identical."""
+    rng = np.random.default_rng(n)
+    g = synth.camera_log_response()
+    times = [float(np.float32(2.0 ** -k)) for k in range(n)]
+    for H, W in ((1, 1), (5, 3), (37, 129), (64, 260)):
+        ldr = [torch.from_numpy(rng.integers(0, 256, size=(H, W, 3)).astype(np.uint8)).cuda() for _ in range(n)]
+        for a in ldr:
+            a.view(-1)[: 3 * W // 2] = 255  # saturated in every exposure
+        out = torch.empty((H, W, 3), dtype=dtype, device="cuda")
+        tm.tm_merge_exposures(ldr, times, g, out)
+        pad = [torch.zeros(H * (W + 1) * 3 + 1, dtype=torch.uint8, device="cuda")[1:].view(H, W + 1, 3)[:, :W] for _ in ldr]
+        for a, b in zip(pad, ldr):
+            a.copy_(b)
+        ref = torch.zeros((H, W + 1, 3), dtype=dtype, device="cuda")[:, :W]
+        tm.tm_merge_exposures(pad, times, g, ref)
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
