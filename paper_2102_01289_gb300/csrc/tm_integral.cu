@@ -10,9 +10,8 @@
 //   3. per tile: the row prefixes again, offset by the chunks to the left, and
 //      accumulated down the tile from the column's offset, written once.
 // The same tile kernels, templated on the source of their two planes, build
-// the backward's fixed-point integral planes of (u_f, v_f) and the integral
-// histograms (indicator planes of the bin map, two thresholds per tile
-// task). Integer arithmetic is modular (2^64 in the sums, 2^32 in the
+// the backward's fixed-point integral planes of (u_f, v_f). The integral
+// histograms have kernels of their own (k_hist_*). Integer arithmetic is modular (2^64 in the sums, 2^32 in the
 // histogram planes), so box sums (Eq. 6, Eq. 9) are exact whatever the image
 // size or summation order.
 #include <algorithm>
@@ -150,20 +149,6 @@ __device__ __forceinline__ FixSource fix_source_of(const float *u, const float *
                    ldexpf(1.f, sb - sb / 2)};
 }
 
-// Values of the planes: indicators of a bin map for thresholds k0 and k0 + 1,
-// [b < k] (cumulative) or [b == k]; raw -1 stands for no pixel.
-struct BinSource {
-  using Raw = int;
-  const uint8_t *bins;
-  int W, k0, eq;
-  __device__ __forceinline__ Raw load(int r, int c) const { return __ldg(bins + (long long)r * W + c); }
-  __device__ __forceinline__ Raw zero() const { return -1; }
-  __device__ __forceinline__ void values(Raw x, long long &a, long long &b) const {
-    a = x >= 0 && (eq ? x == k0 : x < k0);
-    b = x >= 0 && (eq ? x == k0 + 1 : x < k0 + 1);
-  }
-};
-
 // Exclusive block scan of a pair of values with one set of barriers.
 __device__ __forceinline__ void block_scan_pair(long long v1, long long v2, long long (*wt)[kINT / 32],
                                                 long long &e1, long long &e2, long long &t1, long long &t2) {
@@ -235,93 +220,10 @@ __device__ __forceinline__ void chunk_row_prefix(const Src &src, const typename 
 // rows are only summed down each column and across each row (warp sums, no
 // barrier per row); one block scan over the columns ends the tile. The row
 // and tile totals of the last chunk column are read by no later launch (they
-// only offset the chunks to their right), so its tiles skip them.
+// only offset the chunks to their right), so its tiles skip them. Each thread
+// owns four consecutive columns of the chunk and keeps kFSRows rows of loads
+// in flight, 16 bytes at a time where the rows are 16-byte aligned.
 constexpr int kRowGroup = 16;  // rows whose warp partial sums are combined together
-struct StatsSmem {
-  long long col[2][kIC / 8 * 9];            // the tile's column sums, padded for the scan
-  long long row[kRowGroup][2][kINT / 32];   // warp partial sums of a group of rows
-  long long wt[2][kINT / 32];               // block scan
-};
-
-template <class Src>
-__device__ __forceinline__ void int_stats_tile(const IntTask &X, const Src &src, int seg, int k, StatsSmem &sm) {
-  const int W = X.W, H = X.H;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int R0 = seg * X.seg_rows, R1 = min(R0 + X.seg_rows, H), C0 = k * kIC, nc = min(kIC, W - C0);
-  const bool totals = k + 1 < X.nchunk;  // block-uniform
-  long long c1[kItems], c2[kItems];  // sums down the thread's strided columns threadIdx.x + m kINT
-#pragma unroll
-  for (int m = 0; m < kItems; ++m) c1[m] = c2[m] = 0;
-  typename Src::Raw cur[kItems], nxt[kItems];
-  load_chunk_row(src, R0, C0, nc, cur);
-  for (int r = R0; r < R1; ++r) {
-    if (r + 1 < R1) load_chunk_row(src, r + 1, C0, nc, nxt);  // in flight meanwhile
-    long long s1 = 0, s2 = 0;
-#pragma unroll
-    for (int m = 0; m < kItems; ++m) {
-      long long x1, x2;
-      src.values(cur[m], x1, x2);
-      c1[m] += x1;
-      c2[m] += x2;
-      s1 += x1;
-      s2 += x2;
-      cur[m] = nxt[m];
-    }
-    if (!totals) continue;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-    const int g = (r - R0) % kRowGroup;
-    if (lane == 0) {
-      sm.row[g][0][wid] = s1;
-      sm.row[g][1][wid] = s2;
-    }
-    if (g == kRowGroup - 1 || r == R1 - 1) {  // the group's row totals
-      __syncthreads();
-      if ((int)threadIdx.x <= g) {
-        const int rr = r - g + (int)threadIdx.x;
-        long long t1 = 0, t2 = 0;
-#pragma unroll
-        for (int w = 0; w < kINT / 32; ++w) t1 += sm.row[threadIdx.x][0][w], t2 += sm.row[threadIdx.x][1][w];
-        X.rowsum[(long long)rr * X.nchunk + k] = t1;
-        X.rowsum[((long long)H + rr) * X.nchunk + k] = t2;
-      }
-      __syncthreads();  // sm.row is rewritten by the next group
-    }
-  }
-  // chunk-local column prefixes of the column sums: consecutive columns per thread
-#pragma unroll
-  for (int m = 0; m < kItems; ++m) {
-    sm.col[0][pad9(threadIdx.x + m * kINT)] = c1[m];
-    sm.col[1][pad9(threadIdx.x + m * kINT)] = c2[m];
-  }
-  __syncthreads();
-  long long l1[kItems], l2[kItems], a1 = 0, a2 = 0;
-#pragma unroll
-  for (int i = 0; i < kItems; ++i) {
-    a1 += sm.col[0][threadIdx.x * 9 + i];
-    a2 += sm.col[1][threadIdx.x * 9 + i];
-    l1[i] = a1;
-    l2[i] = a2;
-  }
-  long long e1, e2, t1, t2;
-  block_scan_pair(a1, a2, sm.wt, e1, e2, t1, t2);
-#pragma unroll
-  for (int i = 0; i < kItems; ++i) {
-    const int c = C0 + threadIdx.x * kItems + i;
-    if (c < W) {
-      X.colsum[(long long)seg * W + c] = e1 + l1[i];
-      X.colsum[((long long)X.nseg + seg) * W + c] = e2 + l2[i];
-    }
-  }
-  if (threadIdx.x == 0 && totals) {
-    X.tiletot[(long long)seg * X.nchunk + k] = t1;
-    X.tiletot[((long long)X.nseg + seg) * X.nchunk + k] = t2;
-  }
-}
-
 // Launch 2: for columns c0 .. c0 + kMidCols - 1 (of the image, one chunk),
 // replace each segment's column sum by the plane value just above the
 // segment: the sum, over the segments above, of their column sums plus the
@@ -459,10 +361,6 @@ __device__ __forceinline__ void int_write_tile(const IntTask &X, const Src &src,
   }
 }
 
-// Launch 1 with each thread owning four consecutive columns of the chunk and
-// kFSRows rows of loads in flight, 16 bytes at a time where the rows are
-// 16-byte aligned: plain column sums down the segment, then one block scan
-// over the columns; the same outputs as int_stats_tile.
 constexpr int kFS = 256;    // threads of a four-column stats block
 constexpr int kFSRows = 4;  // rows in flight per thread
 static_assert(kFS * 4 == kIC, "a four-column stats block spans one chunk");
@@ -474,7 +372,7 @@ __device__ __forceinline__ void int_stats4_tile(const IntTask &X, const Src &src
   const int R0 = seg * X.seg_rows, R1 = min(R0 + X.seg_rows, H);
   const int c = k * kIC + 4 * (int)threadIdx.x;
   const bool vec = src.vec_ok();
-  const bool totals = k + 1 < X.nchunk;  // block-uniform; see int_stats_tile
+  const bool totals = k + 1 < X.nchunk;  // block-uniform
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   long long cu[4] = {0, 0, 0, 0}, cv[4] = {0, 0, 0, 0};
   for (int r0 = R0; r0 < R1; r0 += kFSRows) {
@@ -651,48 +549,186 @@ __global__ void __launch_bounds__(kINT, 4) k_fix_write(const FixJob *__restrict_
                                              out1, out2, wt);
 }
 
-// Integral histogram planes (uint32, modulo 2^32) of a bin map over the same
-// tiles: pair p = pair0 + blockIdx.y holds planes 2p and 2p + 1 of `planes`
-// (thresholds k_begin + 2p and + 1; the second is skipped past n_planes),
-// scratch per grid row.
-struct HistPairs {
+// Integral histogram planes (uint32, modulo 2^32) of a bin map. The rows are
+// cut into segments of seg_rows (a multiple of 32) and the columns into strips
+// of 128, one warp each:
+//   1. k_hist_cols counts, per segment, plane and column, the pixels the plane
+//      indicates;
+//   2. k_hist_mid replaces the counts by those of the segments above;
+//   3. k_hist_write, a block per segment and plane, walks the strips of the
+//      image eight at a time. A warp's accumulators start from the column
+//      counts above, summed along the strip; per row, ballots give the
+//      indicator masks and the popcounts of their low bits the row prefixes.
+//      What lies left of a strip comes from the strips' row totals, exchanged
+//      once per 32 rows.
+// Bound by the writes (4 bytes per element; the bin map stays in L2) and by
+// issue (105 warp instructions per strip row and plane). 32 planes of 1080p
+// (265 MB) took 230 us over the int64 tiles of the integral images and take 100
+// (counts 13, mid 10, writes 77).
+constexpr int kHW = 8;                  // strips (warps) of a block's pass
+constexpr int kHStrip = 128;            // columns of a strip
+constexpr int kHCols = kHW * kHStrip;   // columns of a pass
+
+struct HistPlanes {
   const uint8_t *bins;
   uint32_t *planes;
-  long long *scratch;
-  size_t scratch_stride;
-  int W, H, nseg, seg_rows, k_begin, n_planes, eq, pair0;
+  uint32_t *counts;  // nseg x n_planes x W column counts
+  int W, H, nseg, seg_rows, n_planes, k_begin, eq;
 };
 
-__device__ __forceinline__ IntTask hist_task(const HistPairs &Q) {
-  return int_task(Q.W, Q.H, Q.nseg, Q.seg_rows, Q.scratch + (long long)blockIdx.y * Q.scratch_stride);
+// Plane p indicates [b == k] (eq) or [b < k], k = k_begin + p.
+__global__ void __launch_bounds__(kHStrip) k_hist_cols(const __grid_constant__ HistPlanes Q) {
+  extern __shared__ unsigned hcount[];  // [n_planes][kHStrip]
+  const int c = blockIdx.x * kHStrip + threadIdx.x, seg = blockIdx.y;
+  for (int p = 0; p < Q.n_planes; ++p) hcount[p * kHStrip + threadIdx.x] = 0;
+  if (c >= Q.W) return;  // (a thread only touches its own column)
+  const int r0 = seg * Q.seg_rows, r1 = min(r0 + Q.seg_rows, Q.H);
+  const uint8_t *b = Q.bins + (size_t)r0 * Q.W + c;
+  for (int r = r0; r < r1; r += 8) {
+    int v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = r + u < r1 ? (int)__ldg(b + (size_t)u * Q.W) : 256;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (v[u] < Q.n_planes) ++hcount[v[u] * kHStrip + threadIdx.x];
+    b += (size_t)8 * Q.W;
+  }
+  uint32_t *o = Q.counts + (size_t)seg * Q.n_planes * Q.W + c;
+  unsigned run = 0;
+  for (int p = 0; p < Q.n_planes; ++p) {
+    const unsigned h = hcount[p * kHStrip + threadIdx.x];
+    run += h;
+    o[(size_t)p * Q.W] = Q.eq ? h : run;  // [b < k_begin + p] with k_begin = 1: the bins 0 .. p
+  }
 }
 
-__device__ __forceinline__ BinSource hist_source(const HistPairs &Q) {
-  return BinSource{Q.bins, Q.W, Q.k_begin + 2 * (Q.pair0 + (int)blockIdx.y), Q.eq};
+__global__ void __launch_bounds__(128) k_hist_mid(const __grid_constant__ HistPlanes Q) {
+  const size_t n = (size_t)Q.n_planes * Q.W, i = (size_t)blockIdx.x * 128 + threadIdx.x;
+  if (i >= n) return;
+  uint32_t *o = Q.counts + i;
+  unsigned run = 0;
+  for (int s = 0; s < Q.nseg; s += 8, o += 8 * n) {
+    unsigned v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = s + u < Q.nseg ? o[u * n] : 0u;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (s + u < Q.nseg) o[u * n] = run;
+      run += v[u];
+    }
+  }
 }
 
-__global__ void __launch_bounds__(kINT, 4) k_hist_stats(HistPairs Q) {
-  __shared__ StatsSmem sm;
-  const IntTask X = hist_task(Q);
-  int_stats_tile(X, hist_source(Q), blockIdx.x / X.nchunk, blockIdx.x % X.nchunk, sm);
+__device__ __forceinline__ unsigned warp_inclusive(unsigned v) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) >= (unsigned)o) v += y;
+  }
+  return v;
 }
 
-__global__ void __launch_bounds__(kMidCols * kMidGroups) k_hist_mid(HistPairs Q) {
-  __shared__ long long part[2][kMidGroups][kMidCols];
-  __shared__ long long leftT[2][kMidBatch];
-  int_mid_cols(hist_task(Q), blockIdx.x * kMidCols, part, leftT);
-}
-
-__global__ void __launch_bounds__(kINT, 4) k_hist_write(HistPairs Q) {
-  __shared__ int tile[kIC / 8 * 9];
-  __shared__ long long out1[kIC / 8 * 9], out2[kIC / 8 * 9];
-  __shared__ long long wt[2][kINT / 32];
-  const IntTask X = hist_task(Q);
-  const long long plane = ((long long)Q.W + 1) * ((long long)Q.H + 1);
-  const int p = Q.pair0 + (int)blockIdx.y;
-  uint32_t *a = Q.planes + 2LL * p * plane;
-  uint32_t *b = 2 * p + 1 < Q.n_planes ? a + plane : nullptr;
-  int_write_tile(X, hist_source(Q), a, b, blockIdx.x / X.nchunk, blockIdx.x % X.nchunk, tile, out1, out2, wt);
+// kEq: Q.eq.
+template <bool kEq>
+__global__ void __launch_bounds__(32 * kHW, 5) k_hist_write(const __grid_constant__ HistPlanes Q) {
+  // [2][seg_rows]: the rows' totals of the passes before, read by one pass
+  // while it writes the next one's (only where the image takes several)
+  extern __shared__ unsigned left[];
+  __shared__ uint4 mask[kHW][32];          // indicator masks of a strip's row, four words of 32 columns
+  __shared__ unsigned part[kHW][32];       // and the counts of the first one, two and three words, a byte each
+  __shared__ unsigned tot[2][kHW][32];     // row totals of the strips, per batch of 32 rows
+  __shared__ unsigned above[kHW];          // totals of the strips in the segments above
+  const int W = Q.W, H = Q.H, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int p = blockIdx.x % Q.n_planes, seg = blockIdx.x / Q.n_planes;
+  const int k = Q.k_begin + p;
+  const int r0 = seg * Q.seg_rows, r1 = min(r0 + Q.seg_rows, H);
+  const size_t W1 = (size_t)W + 1;
+  uint32_t *const plane = Q.planes + (size_t)p * W1 * ((size_t)H + 1);
+  const bool passes = W > kHCols;
+  for (int r = threadIdx.x; r < Q.seg_rows && passes; r += 32 * kHW) left[r] = 0;
+  if (seg == 0)
+    for (int c = threadIdx.x; c <= W; c += 32 * kHW) plane[c] = 0;
+  for (int r = r0 + (int)threadIdx.x; r < r1; r += 32 * kHW) plane[(size_t)(r + 1) * W1] = 0;
+  unsigned carry = 0;  // the passes before: their columns' total in the segments above
+  const unsigned le = 0xffffffffu >> (31 - lane);
+  int flip = 0, par = 0;
+  for (int C0 = 0; C0 < W; C0 += kHCols, par ^= 1) {
+    const int c0 = C0 + wid * kHStrip;  // the warp's strip
+    unsigned acc[4];                    // columns c0 + 32 m + lane
+    bool ok[4];
+    const uint32_t *cnt = Q.counts + ((size_t)seg * Q.n_planes + p) * W + c0 + lane;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      ok[m] = c0 + 32 * m + lane < W;
+      acc[m] = ok[m] ? __ldg(cnt + 32 * m) : 0u;
+    }
+    unsigned run = 0;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      acc[m] = warp_inclusive(acc[m]) + run;
+      run = __shfl_sync(0xffffffffu, acc[m], 31);
+    }
+    __syncthreads();  // the pass before has read above (and left is cleared)
+    if (lane == 0) above[wid] = run;
+    __syncthreads();
+    unsigned base = carry;  // P: everything left of the strip, down to the row
+    for (int w = 0; w < kHW; ++w) {
+      if (w < wid) base += above[w];
+      carry += above[w];
+    }
+    for (int rb = r0; rb < r1; rb += 32, flip ^= 1) {
+      const int n = min(32, r1 - rb);
+      const uint8_t *b = Q.bins + (size_t)rb * W + c0 + lane;
+      uint4 rw = make_uint4(0u, 0u, 0u, 0u);  // lane = row: its masks
+      for (int i = 0; i < n; i += 4) {
+        int v[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int m = 0; m < 4; ++m) v[u][m] = i + u < n && ok[m] ? (int)__ldg(b + (size_t)u * W + 32 * m) : 256;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          uint4 w;
+          w.x = __ballot_sync(0xffffffffu, kEq ? v[u][0] == k : v[u][0] < k);
+          w.y = __ballot_sync(0xffffffffu, kEq ? v[u][1] == k : v[u][1] < k);
+          w.z = __ballot_sync(0xffffffffu, kEq ? v[u][2] == k : v[u][2] < k);
+          w.w = __ballot_sync(0xffffffffu, kEq ? v[u][3] == k : v[u][3] < k);
+          if (lane == i + u) rw = w;
+        }
+        b += (size_t)4 * W;
+      }
+      mask[wid][lane] = rw;
+      const unsigned t0 = __popc(rw.x), t1 = t0 + __popc(rw.y), t2 = t1 + __popc(rw.z);
+      part[wid][lane] = t0 | (t1 << 8) | (t2 << 16);
+      const unsigned mine = t2 + __popc(rw.w);
+      tot[flip][wid][lane] = mine;
+      __syncthreads();  // (tot is double buffered: one barrier per batch)
+      unsigned row = passes && lane < n ? left[par * Q.seg_rows + rb - r0 + lane] : 0u, all = row;
+      for (int w = 0; w < kHW; ++w) {
+        const unsigned t = tot[flip][w][lane];
+        if (w < wid) row += t;
+        all += t;
+      }
+      const unsigned P = warp_inclusive(row) + base;
+      base = __shfl_sync(0xffffffffu, P, 31);
+      uint32_t *o = plane + (size_t)(rb + 1) * W1 + c0 + 1 + lane;
+#pragma unroll 4
+      for (int i = 0; i < n; ++i) {
+        const uint4 w = mask[wid][i];
+        const unsigned t = part[wid][i], off = __shfl_sync(0xffffffffu, P, i);
+        acc[0] += __popc(w.x & le);
+        acc[1] += (t & 0xffu) + __popc(w.y & le);
+        acc[2] += ((t >> 8) & 0xffu) + __popc(w.z & le);
+        acc[3] += (t >> 16) + __popc(w.w & le);
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+          if (ok[m]) o[32 * m] = acc[m] + off;
+        o += W1;
+      }
+      __syncwarp();  // mask is rewritten by the next batch
+      if (passes && wid == 0 && lane < n) left[(par ^ 1) * Q.seg_rows + rb - r0 + lane] = all;
+    }
+  }
 }
 
 }  // namespace
@@ -747,42 +783,42 @@ int launch_integral_jobs(const Job *jobs, int njobs, int tile_blocks, int col_bl
   return 3;
 }
 
-constexpr int kHistPairs = 8;  // plane pairs per launch of the histogram tiles
+// Segments of 64 rows, longer (a multiple of 32) where there would be more
+// than 4096 of them.
+static void hist_layout(int H, int &nseg, int &seg_rows) {
+  seg_rows = 64;
+  const long long most = 4096LL * 64;
+  if (H > most) seg_rows = (int)(((long long)H + 4095) / 4096 + 31) / 32 * 32;
+  nseg = (H + seg_rows - 1) / seg_rows;
+}
 
 size_t hist_scratch_bytes(int W, int H, int planes) {
   int nseg, seg_rows;
-  integral_layout(W, H, SIZE_MAX, nseg, seg_rows);
-  const int pairs = std::min((planes + 1) / 2, kHistPairs);
-  return 8 * (size_t)std::max(pairs, 1) * integral_scratch_elems(W, H, nseg);
+  hist_layout(H, nseg, seg_rows);
+  return sizeof(uint32_t) * (size_t)std::max(planes, 1) * nseg * W;
 }
 
 int launch_integral_histogram(const uint8_t *bins, int W, int H, int n_bins, bool cumulative,
                               uint32_t *planes, void *scratch, cudaStream_t s) {
-  const int k_begin = cumulative ? 1 : 0;
-  const int n_planes = cumulative ? n_bins - 1 : n_bins;
-  if (n_planes <= 0) return 0;
-  HistPairs Q{};
+  HistPlanes Q{};
   Q.bins = bins;
   Q.planes = planes;
-  Q.scratch = static_cast<long long *>(scratch);
+  Q.counts = static_cast<uint32_t *>(scratch);
   Q.W = W;
   Q.H = H;
-  integral_layout(W, H, SIZE_MAX, Q.nseg, Q.seg_rows);
-  Q.scratch_stride = integral_scratch_elems(W, H, Q.nseg);
-  Q.k_begin = k_begin;
-  Q.n_planes = n_planes;
+  Q.k_begin = cumulative ? 1 : 0;
+  Q.n_planes = cumulative ? n_bins - 1 : n_bins;
   Q.eq = cumulative ? 0 : 1;
-  const int pairs = (n_planes + 1) / 2;
-  int n = 0;
-  for (Q.pair0 = 0; Q.pair0 < pairs; Q.pair0 += kHistPairs) {  // groups share the scratch in turn
-    const int g = std::min(kHistPairs, pairs - Q.pair0);
-    const dim3 tiles(integral_tile_blocks(W, Q.nseg), g), cols(integral_col_blocks(W), g);
-    k_hist_stats<<<tiles, kINT, 0, s>>>(Q);
-    k_hist_mid<<<cols, kMidCols * kMidGroups, 0, s>>>(Q);
-    k_hist_write<<<tiles, kINT, 0, s>>>(Q);
-    n += 3;
-  }
-  return n;
+  if (Q.n_planes <= 0) return 0;
+  hist_layout(H, Q.nseg, Q.seg_rows);
+  const size_t smem = sizeof(unsigned) * kHStrip * (size_t)Q.n_planes;  // at most 128 KB
+  cudaFuncSetAttribute(k_hist_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)(sizeof(unsigned) * kHStrip * kMaxBins));
+  k_hist_cols<<<dim3((unsigned)((W + kHStrip - 1) / kHStrip), (unsigned)Q.nseg), kHStrip, smem, s>>>(Q);
+  k_hist_mid<<<(unsigned)(((size_t)Q.n_planes * W + 127) / 128), 128, 0, s>>>(Q);
+  auto *const write = cumulative ? k_hist_write<false> : k_hist_write<true>;
+  write<<<(unsigned)(Q.nseg * Q.n_planes), 32 * kHW, W > kHCols ? 2 * sizeof(unsigned) * Q.seg_rows : 0, s>>>(Q);
+  return 3;
 }
 
 }  // namespace tmk

@@ -66,7 +66,7 @@ int launch_fix_integrals(const FixJob *jobs, int n, int tile_blocks, int col_blo
 
 // Stage a3 (Eq. 7-8), materialised: integral histogram planes,
 // (H+1) x (W+1) uint32 each (modulo 2^32, zero first row and column), over
-// the integral images' tiles, two planes per tile task. cumulative = true:
+// row segments x 128-column strips. cumulative = true:
 // planes k = 1..n-1 hold the integral of [b < k]; cumulative = false: planes
 // k = 0..n-1 the integral of [b == k]. `scratch` holds at least
 // hist_scratch_bytes(W, H, planes) bytes. Returns the number of launches.
