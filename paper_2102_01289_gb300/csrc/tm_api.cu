@@ -342,6 +342,9 @@ DevParams dev_params(const tm_params &p, int qbits) {
   bool small = true;  // every unclipped window below 2^18 pixels
   for (int f = 0; f < p.n_fields; ++f) small = small && (2LL * p.rx[f] + 1) * (2LL * p.ry[f] + 1) < (1LL << 18);
   d.small_win = small ? 1 : 0;
+  bool fast = p.sat <= 0.9f;
+  for (int f = 0; f < p.n_fields; ++f) fast = fast && p.eps[f] >= 1e-30f;
+  d.fast = fast ? 1 : 0;
   return d;
 }
 

@@ -32,6 +32,7 @@ struct DevParams {
   int qbits;                // Q: q = round(2^Q lhat) - 2^(Q-1)
   int flags;                // TM_FLAG_* reading variants
   int small_win;            // 1: every unclipped window holds fewer than 2^18 pixels
+  int fast;                 // 1: every eps >= 1e-30 and sat <= 0.9 (no denormals in Eq. 4's divisor and Eq. 12)
 };
 
 // Reading variants (the TM_FLAG_* bits of tm_params.flags).
@@ -223,15 +224,49 @@ __device__ __forceinline__ void store_rgb(const Image &im, int x, int y, float r
   }
 }
 
-// Bin of a luminance (Section II-A): the number of edges at or below it. The
-// first guess comes from the fast base-2 log, scaled to bins; the compares
-// against the exact edges then settle it, so the result does not depend on
-// the guess.
-__device__ __forceinline__ int bin_of(float i, const float *thr, int n, float lg_min, float bin_scale) {
-  int k = (int)((__log2f(i) - lg_min) * bin_scale);
+// 1 / x, log2 x and 2^x on the special-function unit for arguments and results
+// in the normal range: the flush-to-zero forms of the approximations behind
+// __fdividef, __log2f and exp2f, without the instructions that rescale
+// denormals (the same bits there).
+__device__ __forceinline__ float rcp_normal(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float log2_normal(float x) {
+  float r;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float exp2_normal(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Exponent and base-2 logarithm of the significand (in [1, 2)) of a normal
+// positive float; the logarithm's absolute error is near 2^-22.
+struct LogParts {
+  int e;
+  float lm;
+};
+__device__ __forceinline__ LogParts log_parts(float lum) {
+  const unsigned bits = __float_as_uint(lum);
+  return {(int)(bits >> 23) - 127, log2_normal(__uint_as_float((bits & 0x7fffffu) | 0x3f800000u))};
+}
+
+// Bin of a luminance (Section II-A): the number of edges at or below it
+// (edge[1 .. n - 1], between -inf at edge[0] and +inf at edge[n]). The first
+// guess comes from the fast base-2 log, scaled to bins; the compares against
+// the exact edges then settle it, so the result does not depend on the guess.
+__device__ __forceinline__ int bin_of(float i, const LogParts &p, const float *edge, int n, float lg_min,
+                                      float bin_scale) {
+  int k = (int)(((float)p.e + p.lm - lg_min) * bin_scale);
   k = min(max(k, 0), n - 1);
-  while (k > 0 && i < thr[k - 1]) --k;
-  while (k < n - 1 && i >= thr[k]) ++k;
+  if (i < edge[k] || i >= edge[k + 1]) {
+    while (k > 0 && i < edge[k]) --k;
+    while (k < n - 1 && i >= edge[k + 1]) ++k;
+  }
   return k;
 }
 
@@ -240,12 +275,9 @@ __device__ __forceinline__ int bin_of(float i, const float *thr, int n, float lg
 // logs is formed as exponent difference + significand-log difference and the
 // product with the scale is kept as a float pair, so q is accurate to about
 // one unit of 2^-Q.
-__device__ __forceinline__ int quantise_log(float lum, const Stats &st, int qbits) {
-  unsigned bits = __float_as_uint(lum);
-  int e = (int)(bits >> 23) - 127;
-  float m = __uint_as_float((bits & 0x7fffffu) | 0x3f800000u);
-  float f = __log2f(m) - st.c0;  // m in [1, 2): absolute error near 2^-22
-  float de = (float)(e - st.e0);
+__device__ __forceinline__ int quantise_log(const LogParts &lp, const Stats &st, int qbits) {
+  float f = lp.lm - st.c0;
+  float de = (float)(lp.e - st.e0);
   float d_hi = de + f;                       // TwoSum(de, f)
   float bv = d_hi - de;
   float d_lo = (de - (d_hi - bv)) + (f - bv);
@@ -416,7 +448,7 @@ __device__ __forceinline__ WinMoments window_moments(const DevParams &P, int f, 
                              (unsigned long long)a.y);
   if (kLit) literal_area(P, f, qbits, q1, q2, N);
   WinMoments m;
-  m.rarea = __fdividef(1.f, (float)(unsigned)N);  // N <= 65535^2 < 2^32
+  m.rarea = rcp_normal((float)(unsigned)N);  // N <= 65535^2 < 2^32
   m.var = window_variance<kSmall>(q1, q2, N, m.rarea, inv_scale2, P.small_win != 0);
   m.q1 = q1;
   return m;

@@ -426,15 +426,18 @@ struct LookPack {
 // for k_lookup_counts. kMode: kOut the output only; kOutKeep also the count
 // planes and window moments for the backward; kCountsOnly only the count
 // planes.
-// Bound by load latency and issue. At 12 MP, three fields, eight blocks per SM
-// (64 registers) and three fields' loads in flight took 273 us; 10 and 12
-// blocks 298 and 311; one field at a time at 10 and 16 blocks 313 and 334;
-// descriptors read from global memory instead of the parameters 372 (at 8).
+// Bound by issue (72 % of the active cycles), the L1's wavefronts (63 %) and
+// load latency; a pixel takes 12 record, 12 vector and 12 corner loads. At
+// 12 MP, three fields, seven blocks per SM (72 registers) and three fields'
+// loads in flight took 252 us; 6, 8, 9 and 10 blocks 290, 265, 265 and 298; two
+// fields at a time 283. Before the moments moved between the records and the
+// vectors and the powers behind the vectors' loads it took 272, with
+// descriptors read from global memory instead of the parameters 372.
 constexpr int kLookCols = 128;
 constexpr int kFieldBatch = 3;
 
 template <int NF, class BT, bool kPlain, int kSmall, int kDt, int kMode>
-__global__ void __launch_bounds__(kLookCols, 8)
+__global__ void __launch_bounds__(kLookCols, 7)
     k_lookup_compact(const __grid_constant__ DevParams P, const __grid_constant__ LookPack L) {
   int jb = 0;
   while (jb + 1 < L.n && L.j[jb + 1].b0 <= (int)blockIdx.x) ++jb;
@@ -453,70 +456,100 @@ __global__ void __launch_bounds__(kLookCols, 8)
   const float inv_scale = ldexpf(1.f, -J.qbits);
   const float inv_scale2 = inv_scale * inv_scale;
   const int y0 = by * L.rows, yend = min(y0 + L.rows, H);
+  int t = (int)__ldg(J.bins + ((unsigned)y0 * (unsigned)W + (unsigned)x)) + incl;
 #pragma unroll 1
   for (int y = y0; y < yend; ++y) {
     const unsigned pix = (unsigned)y * (unsigned)W + (unsigned)x;
-    const int t = (int)__ldg(J.bins + pix) + incl;
     const bool look = t > 0 && t <= K;
-    const unsigned k = look ? (unsigned)(t - 1) : 0u;
+    const unsigned k = look ? (unsigned)(t - 1) : 0u;  // (record and vector loads of threshold 1 where none is needed)
+    const bool whole = t > K;
+    if (y + 1 < yend) t = (int)__ldg(J.bins + pix + W) + incl;
     const unsigned kofs = (k >> 6) * gstep + (k & 63u);  // (one group up to 64 thresholds)
+    float rgb[3], pw[3];
+    unsigned black = 0;
+    if (kMode != kCountsOnly) load_rgb<kDt>(J.in, x, y, rgb[0], rgb[1], rgb[2]);
     Fusion fu;
-    // fields in batches whose loads are in flight together: all records, then
-    // all vector entries (slot 0 where no row is mixed), then the moments
+    // fields in batches whose loads are in flight together: all records, the
+    // moments while they arrive, all vector entries (slot 0 where no row is
+    // mixed), and the colour powers while those arrive
 #pragma unroll
     for (int f0 = 0; f0 < NF; f0 += kFieldBatch) {
       unsigned cnt[kFieldBatch];
-      if (look) {
-        uint2 r[kFieldBatch][4];
-        unsigned e[kFieldBatch][4];
+      uint2 r[kFieldBatch][4];
+      unsigned e[kFieldBatch][4];
+      float var[kFieldBatch], rarea[kFieldBatch];
+#pragma unroll
+      for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
+        const int f = f0 + i;
+        const unsigned ul = (unsigned)max(x - P.rx[f], 0), ur = (unsigned)min(x + P.rx[f], W - 1) + 1u;
+        const unsigned p0 = (unsigned)max(y - P.ry[f], 0), p1 = (unsigned)min(y + P.ry[f], H - 1) + 1u;
+        const unsigned cl = (ul >> 5) * cstep + kofs, cr = (ur >> 5) * cstep + kofs;
+        const uint2 *ra = rec + (size_t)(p0 << shift), *rb = rec + (size_t)(p1 << shift);
+        r[i][0] = __ldg(ra + cl);
+        r[i][1] = __ldg(rb + cl);
+        r[i][2] = __ldg(ra + cr);
+        r[i][3] = __ldg(rb + cr);
+      }
+      if (kMode != kCountsOnly) {
 #pragma unroll
         for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
-          const int f = f0 + i;
-          const unsigned ul = (unsigned)max(x - P.rx[f], 0), ur = (unsigned)min(x + P.rx[f], W - 1) + 1u;
-          const unsigned p0 = (unsigned)max(y - P.ry[f], 0), p1 = (unsigned)min(y + P.ry[f], H - 1) + 1u;
-          const unsigned cl = (ul >> 5) * cstep + kofs, cr = (ur >> 5) * cstep + kofs;
-          const uint2 *ra = rec + (size_t)(p0 << shift), *rb = rec + (size_t)(p1 << shift);
-          r[i][0] = __ldg(ra + cl);
-          r[i][1] = __ldg(rb + cl);
-          r[i][2] = __ldg(ra + cr);
-          r[i][3] = __ldg(rb + cr);
-        }
-#pragma unroll
-        for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
-          const int f = f0 + i;
-          const unsigned ul = (unsigned)max(x - P.rx[f], 0), ur = (unsigned)min(x + P.rx[f], W - 1) + 1u;
-          const unsigned ol = ul & 31u, orr = ur & 31u;
-          // C(ur, p1) - C(ur, p0) - (C(ul, p1) - C(ul, p0))
-          cnt[i] = (r[i][3].x - r[i][2].x) - (r[i][1].x - r[i][0].x) + orr * ((r[i][3].y - r[i][2].y) & 0xffffu) -
-                   ol * ((r[i][1].y - r[i][0].y) & 0xffffu);
-          const unsigned vl = ((ul >> 5) * (unsigned)K + k) * slots, vr = ((ur >> 5) * (unsigned)K + k) * slots;
-          const BT *pl = vec + ol, *pr = vec + orr;
-          e[i][0] = __ldg(pl + (size_t)(vl + (r[i][0].y >> 16)) * 32);
-          e[i][1] = __ldg(pl + (size_t)(vl + (r[i][1].y >> 16)) * 32);
-          e[i][2] = __ldg(pr + (size_t)(vr + (r[i][2].y >> 16)) * 32);
-          e[i][3] = __ldg(pr + (size_t)(vr + (r[i][3].y >> 16)) * 32);
-        }
-#pragma unroll
-        for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i)
-          cnt[i] += (unsigned)(BT)(e[i][3] - e[i][2]) - (unsigned)(BT)(e[i][1] - e[i][0]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
-          const Win w = window_of(P, f0 + i, x, y, W, H);  // threshold n: the whole window
-          cnt[i] = t > 0 ? (unsigned)((w.x1 - w.x0 + 1) * (w.y1 - w.y0 + 1)) : 0u;
+          const WinMoments m = window_moments<!kPlain, kSmall>(P, f0 + i, x, y, W, H, J.s12, J.qbits, inv_scale2);
+          var[i] = m.var;
+          rarea[i] = m.rarea;
+          if (kPlain ? kMode == kOutKeep : J.mom != nullptr)
+            J.mom[(size_t)(f0 + i) * W * H + pix] = make_float2(m.var, window_mean(m.q1, m.rarea, inv_scale));
         }
       }
 #pragma unroll
       for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
         const int f = f0 + i;
+        const unsigned ul = (unsigned)max(x - P.rx[f], 0), ur = (unsigned)min(x + P.rx[f], W - 1) + 1u;
+        const unsigned ol = ul & 31u, orr = ur & 31u;
+        // C(ur, p1) - C(ur, p0) - (C(ul, p1) - C(ul, p0))
+        cnt[i] = (r[i][3].x - r[i][2].x) - (r[i][1].x - r[i][0].x) + orr * ((r[i][3].y - r[i][2].y) & 0xffffu) -
+                 ol * ((r[i][1].y - r[i][0].y) & 0xffffu);
+        const unsigned vl = ((ul >> 5) * (unsigned)K + k) * slots, vr = ((ur >> 5) * (unsigned)K + k) * slots;
+        const BT *pl = vec + (size_t)vl * 32 + ol, *pr = vec + (size_t)vr * 32 + orr;
+        e[i][0] = __ldg(pl + (r[i][0].y >> 16) * 32);
+        e[i][1] = __ldg(pl + (r[i][1].y >> 16) * 32);
+        e[i][2] = __ldg(pr + (r[i][2].y >> 16) * 32);
+        e[i][3] = __ldg(pr + (r[i][3].y >> 16) * 32);
+      }
+      if (f0 == 0 && kMode != kCountsOnly) black = colour_powers<kPlain>(P, rgb, pw);
+#pragma unroll
+      for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
+        const int f = f0 + i;
+        cnt[i] += (unsigned)(BT)(e[i][3] - e[i][2]) - (unsigned)(BT)(e[i][1] - e[i][0]);
+        if (!look) {  // threshold n takes the whole window, threshold 0 nothing
+          const Win w = window_of(P, f, x, y, W, H);
+          cnt[i] = whole ? (unsigned)((w.x1 - w.x0 + 1) * (w.y1 - w.y0 + 1)) : 0u;
+        }
         if (kMode == kCountsOnly || (kPlain ? kMode == kOutKeep : J.cnt != nullptr))
           J.cnt[f * J.cnt_step + pix] = cnt[i];
-        if (kMode != kCountsOnly)
-          fold_field<kPlain, kMode == kOutKeep, kSmall>(P, f, x, y, W, H, cnt[i], J.s12, J.qbits, inv_scale2, fu,
-                                                        J.dbg, J.mom, inv_scale);
+        if (kMode != kCountsOnly) {
+          float Wf, Lf;
+          fuse_field<kPlain>(P, f, cnt[i], rarea[i], var[i], fu, Wf, Lf);
+          if (!kPlain && J.dbg.l) {
+            const size_t N = (size_t)W * H;
+            J.dbg.cnt[f * N + pix] = cnt[i];
+            J.dbg.sigma2[f * N + pix] = var[i];
+            J.dbg.weight[f * N + pix] = Wf;
+            J.dbg.lf[f * N + pix] = Lf;
+          }
+        }
       }
     }
-    if (kMode != kCountsOnly) finish_pixel<kPlain, kDt>(J.in, J.out, P, x, y, fu, J.dbg);
+    if (kMode != kCountsOnly) {
+      const float Lc = fused_value(P, fu);
+      rgb[0] = pw[0] * Lc, rgb[1] = pw[1] * Lc, rgb[2] = pw[2] * Lc;
+      if (black) {
+        if (black & 1u) rgb[0] = 0.f;
+        if (black & 2u) rgb[1] = 0.f;
+        if (black & 4u) rgb[2] = 0.f;
+      }
+      store_rgb<kDt>(J.out, x, y, rgb[0], rgb[1], rgb[2], (P.flags & kFlagSrgb) != 0);
+      if (!kPlain && J.dbg.l) J.dbg.l[pix] = Lc;
+    }
   }
 }
 
@@ -616,7 +649,7 @@ static void launch_look_dtype(const DevParams &P, const LookPack &L, int blocks,
 
 int launch_lookup_compact(const DevParams &P, const Job *jobs, int njobs, int blocks, int rows, bool wide,
                           bool plain, bool keep, bool counts_only, int dtype, cudaStream_t s) {
-  const bool general = !plain || (P.flags & kFlagAreaLit) || (keep && (wide || !P.small_win || dtype != kF32));
+  const bool general = !plain || !P.fast || (P.flags & kFlagAreaLit) || (keep && (wide || !P.small_win || dtype != kF32));
   LookPack L{};
   L.n = njobs;
   L.rows = rows;

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(256) k_range(const Job *__restrict__ jobs, int
 // kLin: TM_FLAG_VAR_LINEAR; kDt as in k_range.
 template <bool kLin, int kDt>
 __global__ void __launch_bounds__(256) k_prep(const Job *__restrict__ jobs, int njobs, int n_bins, int n_fields) {
-  __shared__ float thr[kMaxBins];
+  __shared__ float edge[kMaxBins + 1];  // bin k is [edge[k], edge[k + 1])
   const int j = find_job(jobs, njobs, kStPrep, blockIdx.x);
   const Job &J = jobs[j];
   const int lb = blockIdx.x - J.b0[kStPrep];
@@ -209,7 +209,8 @@ __global__ void __launch_bounds__(256) k_prep(const Job *__restrict__ jobs, int 
   const Image in = J.in;
   const bool vec = vec_ok(in);
   const Stats *st = J.st;
-  for (int k = threadIdx.x; k < n_bins - 1; k += blockDim.x) thr[k] = st->thr[k];
+  for (int k = threadIdx.x; k <= n_bins; k += blockDim.x)
+    edge[k] = k == 0 ? -__int_as_float(0x7f800000) : k == n_bins ? __int_as_float(0x7f800000) : st->thr[k - 1];
   Stats sst;  // only the three constants quantise_log reads
   sst.c0 = __ldg(&st->c0);
   sst.e0 = __ldg(&st->e0);
@@ -227,9 +228,10 @@ __global__ void __launch_bounds__(256) k_prep(const Job *__restrict__ jobs, int 
   unsigned bmin = 0x7f800000u, bmax = 0u;  // this image's own range (streaming reuse)
   // whole warps iterate together (the group shuffles need all lanes)
   for (int g0 = lb * blockDim.x + (threadIdx.x & ~31); g0 < ng; g0 += nb * blockDim.x) {
-    const int gi = g0 + lane;
-    const int y = gi / gpr, x = (gi - y * gpr) * 4;
-    const int n = gi < ng ? max(0, min(4, W - x)) : 0;
+    // from the image's end: what the range pass read last is still in L2
+    const int gi = ng - 32 - g0 + lane;  // (whole groups of 32 pixels: ng is a multiple of 8)
+    const int y = gi >= 0 ? gi / gpr : 0, x = (gi - y * gpr) * 4;
+    const int n = gi >= 0 ? max(0, min(4, W - x)) : 0;
     int kmin = 256, kmax = -1;
     if (n > 0) {
       float r[4], g[4], b[4];
@@ -239,9 +241,10 @@ __global__ void __launch_bounds__(256) k_prep(const Job *__restrict__ jobs, int 
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const float l = luminance(r[i], g[i], b[i]);
-        const int bi = bin_of(l, thr, n_bins, lg_min, bin_scale);
+        const LogParts p = log_parts(l);
+        const int bi = bin_of(l, p, edge, n_bins, lg_min, bin_scale);
         bq |= (unsigned)bi << (8 * i);
-        qq[i] = kLin ? quantise_lin(l, sst, qbits) : quantise_log(l, sst, qbits);
+        qq[i] = kLin ? quantise_lin(l, sst, qbits) : quantise_log(p, sst, qbits);
         if (i < n) {
           bmin = min(bmin, __float_as_uint(l));
           bmax = max(bmax, __float_as_uint(l));
