@@ -35,8 +35,7 @@
 //      up to four vector entries per field and pixel, then the lookup's
 //      arithmetic.
 // Thresholds come in groups of KL (64, or 4, 8, 16, 32 where n - 1 is no
-// larger), a group of 64 two adjacent ones to a lane; a warp holds the rows
-// (launch 1) or row segments (launch 2) that its 32 lanes take at once.
+// larger), a group of 64 two adjacent ones to a lane.
 // The bin ranges of the chunks come from the group summary of the bin pass.
 #include <cooperative_groups.h>
 
@@ -49,22 +48,22 @@ namespace tmk {
 namespace {
 
 constexpr int kRowWarps = 8;  // warps of a k_compact_rows block
-// A group of KL thresholds takes KL / T lanes of T adjacent thresholds each.
+// A group of KL thresholds takes T adjacent ones per lane (lanes past KL / T
+// hold none).
 template <int KL>
 struct Shape {
   static constexpr int T = KL == 64 ? 2 : 1;
-  static constexpr int Lanes = KL / T;                   // lanes of a row
-  static constexpr int Sub = 32 / Lanes;                 // rows or segments of a warp
-  static constexpr int Step = Sub == 1 ? 4 : Sub == 2 ? 2 : 1;  // rows or chunks in flight together
-  static constexpr int ColWarps = KL >= 32 ? 16 : KL == 16 ? 8 : 4;
-  static constexpr int MinBlocks = 32 / ColWarps;        // 64 registers
-  static constexpr int Segs = ColWarps * Sub;            // row segments of a CTA
+  static constexpr int Step = 4;                         // rows or chunks in flight together
+  static constexpr int ColWarps = 16;                    // row segments of a CTA
+  static constexpr int MinBlocks = 2;                    // 64 registers
   // column CTAs share a chunk's rows until the launch has this many warps.
   // 12 MP, 63 thresholds, a forward with clusters of 2, 4, 8: 549, 536, 563
   // us; 1080p, 31 thresholds, 4 and 8: 127 and 133; 32 1080p images in one
   // launch, 1 and 4: 9.49 and 9.75 ms per 120 (short segments pay more for
-  // their totals, long ones leave the rows of a vertical edge to one warp).
-  static constexpr int Fill = KL == 64 ? 4864 : 3600;
+  // their totals, long ones leave the rows of a vertical edge to one warp);
+  // the pyramid at 12 MP, 4 thresholds, up to 4000, 8000 and 16000 warps: the
+  // build 89, 81 and 87 us (125 with eight segments to a warp).
+  static constexpr int Fill = KL == 64 ? 4864 : KL == 32 ? 3600 : 8000;
 };
 
 // Whether a chunk row with bins in [g & 255, g >> 8] has bins on both sides of
@@ -100,48 +99,44 @@ __device__ __forceinline__ void store_records(uint2 *p, const unsigned *pt, cons
   else *p = make_uint2(pt[0], mc[0]);
 }
 
-// Rows: lane = (row, T thresholds), walking along the rows' chunks.
+// Rows: a warp per row, lane = T thresholds, walking along the row's chunks.
 template <int KL>
 __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(const Job *__restrict__ jobs, int njobs, int K) {
   using S = Shape<KL>;
-  constexpr int T = S::T, NL = S::Lanes;
+  constexpr int T = S::T;
   const Job &J = jobs[find_job(jobs, njobs, kStCRows, blockIdx.x)];
-  const int lane = threadIdx.x & 31, sub = lane / NL, j = lane % NL;
+  const int lane = threadIdx.x & 31;
   const int W = J.in.W, H = J.in.H, G = (W + 31) >> 5, Gp = (W >> 5) + 1;
-  const int rb = (H + kRowWarps * S::Sub - 1) / (kRowWarps * S::Sub);
+  const int rb = (H + kRowWarps - 1) / kRowWarps;
   const int lb = blockIdx.x - J.b0[kStCRows];
   const int kg = lb / rb, k0 = KL * kg;
-  const int v0 = ((lb - kg * rb) * kRowWarps + (threadIdx.x >> 5)) * S::Sub;  // the warp's first row
-  if (v0 >= H) return;
-  const bool own = v0 + sub < H;
-  const int v = min(v0 + sub, H - 1);  // the lane's row (past the last: read, not written)
-  const unsigned k8 = (unsigned)(k0 + 1 + T * j) << 8;  // the lane's first threshold
-  const uint8_t *__restrict__ bins = J.bins + (size_t)v0 * W + lane;
+  const int v = (lb - kg * rb) * kRowWarps + (threadIdx.x >> 5);
+  if (v >= H) return;
+  const bool own = T * lane < KL;
+  const unsigned k8 = (unsigned)(k0 + 1 + T * lane) << 8;  // the lane's first threshold
+  const uint8_t *__restrict__ bins = J.bins + (size_t)v * W + lane;
   const uint16_t *__restrict__ grow = J.grp + (size_t)v * G;
   const size_t cstride = (size_t)H * KL;
-  uint16_t *__restrict__ dst = J.c_row + ((size_t)kg * Gp * H + v) * KL + T * j;
+  uint16_t *__restrict__ dst = J.c_row + ((size_t)kg * Gp * H + v) * KL + T * lane;
   unsigned run[T];
 #pragma unroll
   for (int z = 0; z < T; ++z) run[z] = 0;
-  for (int cb = 0; cb < Gp; cb += NL) {
-    const unsigned gl = cb + j < G && own ? (unsigned)__ldg(grow + cb + j) : kNoRow;
-    const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit (sub, chunk of the batch)
-    const int n = min(NL, Gp - cb);
+  for (int cb = 0; cb < Gp; cb += 32) {
+    const unsigned gl = cb + lane < G ? (unsigned)__ldg(grow + cb + lane) : kNoRow;
+    const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit = chunk of the batch
+    const int n = min(32, Gp - cb);
     for (int i = 0; i < n; i += S::Step) {
-      int b[S::Step][S::Sub];
+      int b[S::Step];
 #pragma unroll
-      for (int u = 0; u < S::Step; ++u)
-#pragma unroll
-        for (int q = 0; q < S::Sub; ++q) {
-          const int col = 32 * (cb + i + u);
-          b[u][q] = 256;
-          if (((mixed >> (q * NL + ((i + u) & (NL - 1)))) & 1u) && col + lane < W)
-            b[u][q] = (int)__ldg(bins + (size_t)q * W + col);
-        }
+      for (int u = 0; u < S::Step; ++u) {
+        const int col = 32 * (cb + i + u);
+        b[u] = 256;
+        if (((mixed >> (i + u)) & 1u) && col + lane < W) b[u] = (int)__ldg(bins + col);
+      }
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
         if (i + u >= n) break;
-        const unsigned g = __shfl_sync(0xffffffffu, gl, sub * NL + i + u);
+        const unsigned g = __shfl_sync(0xffffffffu, gl, i + u);
         if (own) {
           if (T == 2) *reinterpret_cast<unsigned *>(dst) = run[0] | (run[T - 1] << 16);
           else *dst = (uint16_t)run[0];
@@ -150,16 +145,14 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(const Job *__re
         unsigned cc[T];
 #pragma unroll
         for (int z = 0; z < T; ++z) cc[z] = g < k8 + 256u * z ? 32u : 0u;  // every bin of the chunk below k
-#pragma unroll
-        for (int q = 0; q < S::Sub; ++q) {
-          if (!((mixed >> (q * NL + i + u)) & 1u)) continue;
+        if ((mixed >> (i + u)) & 1u) {
           int t0, t1;
-          mixed_thresholds<KL>(S::Sub == 1 ? g : __shfl_sync(0xffffffffu, gl, q * NL + i + u), k0, t0, t1);
+          mixed_thresholds<KL>(g, k0, t0, t1);
           for (int t = t0 / T * T; t < t1; t += T) {
 #pragma unroll
             for (int z = 0; z < T; ++z) {
-              const unsigned mask = __ballot_sync(0xffffffffu, b[u][q] <= k0 + t + z);  // bins below k0 + 1 + t + z
-              if (lane == q * NL + t / T) cc[z] = (unsigned)__popc(mask);
+              const unsigned mask = __ballot_sync(0xffffffffu, b[u] <= k0 + t + z);  // bins below k0 + 1 + t + z
+              if (lane == t / T) cc[z] = (unsigned)__popc(mask);
             }
           }
         }
@@ -177,87 +170,78 @@ struct ColState {
   unsigned pt[T], mc[T], mh[T];
 };
 
-// A warp's pass over its row segments of chunk c: lane = (segment, T
-// thresholds) with rows row0 .. of segment 0, each segment `per` rows, the
-// last ending before rend. kWrite: write records and vectors; sB[(sub, t)][o]
-// holds the vectors (lane = column o there). Else sB counts, per (sub, t) and
-// column, the pixels of the mixed rows with bin k0 + t (k0 or less for t = 0).
+// A warp's pass over rows [row0, rend) of chunk c: lane = T thresholds. kWrite:
+// write records and vectors; sB[t][o] holds the vectors (lane = column o
+// there). Else sB counts, per t and column, the pixels of the mixed rows with
+// bin k0 + t (k0 or less for t = 0).
 template <int KL, class BT, bool kWrite>
-__device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int row0, int per, int rend, BT *sB,
+__device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int row0, int rend, BT *sB,
                                          ColState<Shape<KL>::T> &st) {
   using S = Shape<KL>;
-  constexpr int T = S::T, NL = S::Lanes;
-  const int lane = threadIdx.x & 31, sub = lane / NL, j = lane % NL;
+  constexpr int T = S::T;
+  const int lane = threadIdx.x & 31;
   const int W = J.in.W, H = J.in.H, G = (W + 31) >> 5, Gp = (W >> 5) + 1;
   const int k0 = KL * kg;
-  const unsigned k8 = (unsigned)(k0 + 1 + T * j) << 8;
-  const int mine = row0 + sub * per;
-  int left = min(per, rend - mine);  // the lane's rows still to come
+  const unsigned k8 = (unsigned)(k0 + 1 + T * lane) << 8;
+  const bool own = T * lane < KL;
   const unsigned lt = (1u << lane) - 1u;
   const bool colok = 32 * c + lane < W;
   const uint8_t *__restrict__ bins = J.bins + (size_t)row0 * W + 32 * c + lane;
-  const uint16_t *__restrict__ grp = J.grp + (size_t)(mine + j) * G + c;
+  const uint16_t *__restrict__ grp = J.grp + (size_t)(row0 + lane) * G + c;
   const size_t plane = (size_t)kg * Gp + c;
-  const uint16_t *__restrict__ row = J.c_row + (plane * H + mine) * KL + T * j;
-  uint2 *__restrict__ rec = J.c_rec + (plane * (H + 1) + mine + 1) * KL + T * j;
+  const uint16_t *__restrict__ row = J.c_row + (plane * H + row0) * KL + T * lane;
+  uint2 *__restrict__ rec = J.c_rec + (plane * (H + 1) + row0 + 1) * KL + T * lane;
   BT *__restrict__ vec = static_cast<BT *>(J.c_vec) + ((size_t)c * K + k0) * (H + 1) * 32 + lane;
   const unsigned vstep = (unsigned)(H + 1);
-  for (int ib = 0; ib < per; ib += NL) {
-    const unsigned gl = c < G && j < left ? (unsigned)__ldg(grp) : kNoRow;
-    grp += (size_t)NL * G;
-    const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit (sub, row of the batch)
-    const int n = min(NL, per - ib);
+  for (int rb = row0; rb < rend; rb += 32) {
+    const int n = min(32, rend - rb);
+    const unsigned gl = c < G && lane < n ? (unsigned)__ldg(grp) : kNoRow;
+    grp += (size_t)32 * G;
+    const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit = row of the batch
     for (int i = 0; i < n; i += S::Step) {
       unsigned rp[S::Step][T];
-      int b[S::Step][S::Sub];
+      int b[S::Step];
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
 #pragma unroll
         for (int z = 0; z < T; ++z) rp[u][z] = 0;
-        if (u < left) load_prefix<T>(row + u * KL, rp[u]);
-#pragma unroll
-        for (int q = 0; q < S::Sub; ++q) {
-          b[u][q] = 256;
-          if (((mixed >> (q * NL + ((i + u) & (NL - 1)))) & 1u) && colok)
-            b[u][q] = (int)__ldg(bins + (size_t)(unsigned)(q * per + u) * W);
-        }
+        if (own && i + u < n) load_prefix<T>(row + u * KL, rp[u]);
+        b[u] = 256;
+        if (((mixed >> (i + u)) & 1u) && colok) b[u] = (int)__ldg(bins + (size_t)u * W);
       }
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
         // (rows past the segment have no bins below or on both sides)
-        const unsigned g = __shfl_sync(0xffffffffu, gl, sub * NL + ((i + u) & (NL - 1)));
+        const unsigned g = __shfl_sync(0xffffffffu, gl, i + u);
 #pragma unroll
         for (int z = 0; z < T; ++z) {
           st.pt[z] += rp[u][z];
           if (g < k8 + 256u * z) ++st.mc[z];
         }
+        if ((mixed >> (i + u)) & 1u) {
 #pragma unroll
-        for (int z = 0; z < T; ++z) {
-          const unsigned kz = k8 + 256u * z;
-          if (g >= kz && ((g & 0xffu) << 8) < kz) st.mc[z] += 0x10000u;  // bins on both sides
-          if (!kWrite && g < kz && mixed_range<KL>(g, k0)) ++st.mh[z];
-        }
-#pragma unroll
-        for (int q = 0; q < S::Sub; ++q) {
-          if (!((mixed >> (q * NL + ((i + u) & (NL - 1)))) & 1u)) continue;
+          for (int z = 0; z < T; ++z) {
+            const unsigned kz = k8 + 256u * z;
+            if (g >= kz && ((g & 0xffu) << 8) < kz) st.mc[z] += 0x10000u;  // bins on both sides
+            if (!kWrite && g < kz) ++st.mh[z];
+          }
           if (!kWrite) {
-            const int h = max(b[u][q] - k0, 0);
+            const int h = max(b[u] - k0, 0);
             if (h < KL) {
-              BT *const s = sB + (q * KL + h) * 32 + lane;
+              BT *const s = sB + h * 32 + lane;
               *s = (BT)(*s + 1);
             }
           } else {
             int t0, t1;
-            mixed_thresholds<KL>(S::Sub == 1 ? g : __shfl_sync(0xffffffffu, gl, q * NL + ((i + u) & (NL - 1))), k0,
-                                 t0, t1);
+            mixed_thresholds<KL>(g, k0, t0, t1);
             for (int t = t0 / T * T; t < t1; t += T) {
-              BT *const s = sB + (q * KL + t) * 32 + lane;
+              BT *const s = sB + t * 32 + lane;
               unsigned slot[T];
               BT val[T];
 #pragma unroll
               for (int z = 0; z < T; ++z) {
-                const unsigned mask = __ballot_sync(0xffffffffu, b[u][q] <= k0 + t + z);
-                slot[z] = __shfl_sync(0xffffffffu, st.mc[z], q * NL + t / T) >> 16;
+                const unsigned mask = __ballot_sync(0xffffffffu, b[u] <= k0 + t + z);
+                slot[z] = __shfl_sync(0xffffffffu, st.mc[z], t / T) >> 16;
                 val[z] = (BT)(s[z * 32] + __popc(mask & lt));
               }
 #pragma unroll
@@ -269,99 +253,97 @@ __device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int
             }
           }
         }
-        if (kWrite && u < left) store_records<T>(rec + u * KL, st.pt, st.mc);
+        if (kWrite && own && i + u < n) store_records<T>(rec + u * KL, st.pt, st.mc);
       }
       row += S::Step * KL;
       rec += S::Step * KL;
       bins += (size_t)S::Step * W;
-      left -= S::Step;
     }
   }
 }
 
 // Columns: cluster -> (image, chunk, threshold group), CTA -> a share of the
-// rows, cut into Segs segments.
+// rows, a segment of them per warp.
 template <int KL, class BT>
-__global__ void __launch_bounds__(32 * Shape<KL>::ColWarps, sizeof(BT) == 2 ? Shape<KL>::MinBlocks : 1)
+__global__ void __launch_bounds__(32 * Shape<KL>::ColWarps, KL == 64 && sizeof(BT) == 4 ? 1 : Shape<KL>::MinBlocks)
     k_compact_cols(const Job *__restrict__ jobs, int njobs, int K) {
   using S = Shape<KL>;
-  constexpr int T = S::T, NL = S::Lanes;
+  constexpr int T = S::T, NW = S::ColWarps;
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char smem[];
-  BT *const sB = reinterpret_cast<BT *>(smem);                  // [Segs][KL][32]
-  BT *const sT = sB + S::Segs * KL * 32;                        // [KL][32]: the CTA's totals
-  uint2 *const tot = reinterpret_cast<uint2 *>(sT + KL * 32);   // [Segs + 1][KL], the last: the CTA's totals
+  BT *const sB = reinterpret_cast<BT *>(smem);                  // [NW][KL][32]
+  BT *const sT = sB + NW * KL * 32;                             // [KL][32]: the CTA's totals
+  uint2 *const tot = reinterpret_cast<uint2 *>(sT + KL * 32);   // [NW + 1][KL], the last: the CTA's totals
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), nc = (int)cluster.num_blocks();
   const Job &J = jobs[find_job(jobs, njobs, kStCCols, blockIdx.x / nc)];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, sub = lane / NL, j = lane % NL;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int H = J.in.H, Gp = (J.in.W >> 5) + 1;
   const int lb = blockIdx.x / nc - J.b0[kStCCols];
   const int kg = lb / Gp, c = lb - kg * Gp;
-  const int share = (H + nc - 1) / nc, per = (share + S::Segs - 1) / S::Segs;
-  const int row0 = rank * share + wid * S::Sub * per, rend = min((rank + 1) * share, H);
-  BT *const mine = sB + wid * S::Sub * KL * 32;
-  for (int i = lane; i < S::Sub * KL * 32 * (int)sizeof(BT) / 4; i += 32) reinterpret_cast<unsigned *>(mine)[i] = 0;
+  const bool own = T * lane < KL;
+  const int share = (H + nc - 1) / nc, per = (share + NW - 1) / NW;
+  const int row0 = rank * share + wid * per, rend = min(min(row0 + per, (rank + 1) * share), H);
+  BT *const mine = sB + wid * KL * 32;
+  for (int i = lane; i < KL * 32 * (int)sizeof(BT) / 4; i += 32) reinterpret_cast<unsigned *>(mine)[i] = 0;
   __syncwarp();
   ColState<T> st{};
-  col_pass<KL, BT, false>(J, c, kg, K, row0, per, rend, mine, st);
-  uint2 *const mytot = tot + (wid * S::Sub + sub) * KL + T * j;
+  col_pass<KL, BT, false>(J, c, kg, K, row0, rend, mine, st);
+  uint2 *const mytot = tot + wid * KL + T * lane;
 #pragma unroll
-  for (int z = 0; z < T; ++z) mytot[z] = make_uint2(st.pt[z], st.mc[z]);
+  for (int z = 0; z < T; ++z)
+    if (own) mytot[z] = make_uint2(st.pt[z], st.mc[z]);
   // per segment: the vectors' totals from the column counts (the pixels of
   // mixed rows below k, less those of rows wholly below it, left of o)
   unsigned any[T];
 #pragma unroll
-  for (int z = 0; z < T; ++z) any[z] = __ballot_sync(0xffffffffu, st.mc[z] >> 16);
+  for (int z = 0; z < T; ++z) any[z] = __ballot_sync(0xffffffffu, own && (st.mc[z] >> 16));
   if (any[0] | any[T - 1]) {
     __syncwarp();
-#pragma unroll 1
-    for (int q = 0; q < S::Sub; ++q) {
-      unsigned below = 0;
+    unsigned below = 0;
 #pragma unroll 2
-      for (int t = 0; t < NL; ++t) {
+    for (int t = 0; t < KL / T; ++t) {
 #pragma unroll
-        for (int z = 0; z < T; ++z) {
-          BT *const s = mine + (q * KL + T * t + z) * 32 + lane;
-          below += *s;
-          unsigned e = 0;
-          if ((any[z] >> (q * NL + t)) & 1u) {
-            const unsigned v = below - __shfl_sync(0xffffffffu, st.mh[z], q * NL + t);
-            e = v;
+      for (int z = 0; z < T; ++z) {
+        BT *const s = mine + (T * t + z) * 32 + lane;
+        below += *s;
+        unsigned e = 0;
+        if ((any[z] >> t) & 1u) {
+          const unsigned v = below - __shfl_sync(0xffffffffu, st.mh[z], t);
+          e = v;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-              const unsigned y = __shfl_up_sync(0xffffffffu, e, o);
-              if (lane >= o) e += y;
-            }
-            e -= v;
+          for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, e, o);
+            if (lane >= o) e += y;
           }
-          *s = (BT)e;
+          e -= v;
         }
+        *s = (BT)e;
       }
     }
   }
   __syncthreads();
-  for (int e = tid; e < KL * 32; e += 32 * S::ColWarps) {
+  for (int e = tid; e < KL * 32; e += 32 * NW) {
     unsigned t = 0;
 #pragma unroll 4
-    for (int w = 0; w < S::Segs; ++w) t += sB[w * KL * 32 + e];
+    for (int w = 0; w < NW; ++w) t += sB[w * KL * 32 + e];
     sT[e] = (BT)t;
   }
   if (tid < KL) {
     uint2 t = make_uint2(0u, 0u);
-    for (int w = 0; w < S::Segs; ++w) {
+    for (int w = 0; w < NW; ++w) {
       const uint2 x = tot[w * KL + tid];
       t.x += x.x, t.y += x.y;
     }
-    tot[S::Segs * KL + tid] = t;
+    tot[NW * KL + tid] = t;
   }
   cluster.sync();
   // exclusive scans over the cluster's segments
-  for (int e = tid; e < KL * 32; e += 32 * S::ColWarps) {
+  for (int e = tid; e < KL * 32; e += 32 * NW) {
     unsigned run = 0;
     for (int r = 0; r < rank; ++r) run += cluster.map_shared_rank(sT, r)[e];
 #pragma unroll 4
-    for (int w = 0; w < S::Segs; ++w) {
+    for (int w = 0; w < NW; ++w) {
       BT *const s = sB + w * KL * 32 + e;
       const unsigned v = *s;
       *s = (BT)run;
@@ -371,10 +353,10 @@ __global__ void __launch_bounds__(32 * Shape<KL>::ColWarps, sizeof(BT) == 2 ? Sh
   if (tid < KL) {
     uint2 run = make_uint2(0u, 0u);
     for (int r = 0; r < rank; ++r) {
-      const uint2 x = cluster.map_shared_rank(tot, r)[S::Segs * KL + tid];
+      const uint2 x = cluster.map_shared_rank(tot, r)[NW * KL + tid];
       run.x += x.x, run.y += x.y;
     }
-    for (int w = 0; w < S::Segs; ++w) {
+    for (int w = 0; w < NW; ++w) {
       const uint2 x = tot[w * KL + tid];
       tot[w * KL + tid] = run;
       run.x += x.x, run.y += x.y;
@@ -390,11 +372,11 @@ __global__ void __launch_bounds__(32 * Shape<KL>::ColWarps, sizeof(BT) == 2 ? Sh
   }
 #pragma unroll
   for (int z = 0; z < T; ++z) {
-    const uint2 x = mytot[z];
+    const uint2 x = own ? mytot[z] : make_uint2(0u, 0u);
     st.pt[z] = x.x;
     st.mc[z] = x.y;
   }
-  col_pass<KL, BT, true>(J, c, kg, K, row0, per, rend, mine, st);
+  col_pass<KL, BT, true>(J, c, kg, K, row0, rend, mine, st);
 }
 
 // What a launch does beside writing the output image.
@@ -556,7 +538,7 @@ __global__ void __launch_bounds__(kLookCols, 7)
 template <int KL, class BT>
 int launch_cols(const Job *jobs, int njobs, int blocks, int K, cudaStream_t s) {
   using S = Shape<KL>;
-  const size_t smem = (size_t)(S::Segs + 1) * KL * (32 * sizeof(BT) + sizeof(uint2));
+  const size_t smem = (size_t)(S::ColWarps + 1) * KL * (32 * sizeof(BT) + sizeof(uint2));
   if (cudaFuncSetAttribute(k_compact_cols<KL, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return -1;
@@ -606,8 +588,8 @@ bool plan_compact(const DevParams &P, int W, int H, CompactPlan &C) {
 }
 
 int compact_row_blocks(int H, int K) {
-  const int sh = group_shift(K), lanes = sh == 6 ? 32 : 1 << sh, per = kRowWarps * (32 / lanes);
-  return (H + per - 1) / per * ((K + (1 << sh) - 1) >> sh);
+  const int sh = group_shift(K);
+  return (H + kRowWarps - 1) / kRowWarps * ((K + (1 << sh) - 1) >> sh);
 }
 
 int compact_col_units(int W, int K) {
