@@ -171,22 +171,28 @@ def make_params(n_bins: int, radii: Sequence, eps=0.1, alpha=1.0, ld_min=0.0, ld
 
 
 # ------------------------------------------------------------------ images --
-def _dtype_code(t) -> int:
-    import torch
+_DTYPE_CODES = {}  # torch dtype -> tm_dtype, filled on first use (importing works without torch)
 
-    m = {torch.float32: TM_F32, torch.float16: TM_F16, torch.uint8: TM_U8}
-    if t.dtype not in m:
+
+def _dtype_code(t) -> int:
+    if not _DTYPE_CODES:
+        import torch
+
+        _DTYPE_CODES.update({torch.float32: TM_F32, torch.float16: TM_F16, torch.uint8: TM_U8})
+    code = _DTYPE_CODES.get(t.dtype)
+    if code is None:
         raise TypeError(f"unsupported dtype {t.dtype}")
-    return m[t.dtype]
+    return code
 
 
 def image_of(t) -> TmImage:
     """Descriptor of an (H, W, 3) tensor whose rows are dense RGB."""
-    if t.dim() != 3 or t.shape[2] != 3:
+    shape, stride = t.shape, t.stride()
+    if len(shape) != 3 or shape[2] != 3:
         raise ValueError("image tensors are (H, W, 3)")
-    if t.stride(2) != 1 or t.stride(1) != 3:
+    if stride[2] != 1 or stride[1] != 3:
         raise ValueError("image rows must be dense interleaved RGB")
-    return TmImage(t.data_ptr(), int(t.shape[1]), int(t.shape[0]), int(t.stride(0)), _dtype_code(t))
+    return TmImage(t.data_ptr(), shape[1], shape[0], stride[0], _dtype_code(t))
 
 
 def image_of_numpy(a) -> TmImage:
@@ -379,7 +385,7 @@ class _CtxCache:
         self.ctxs = {}
 
     def get(self, t):
-        key = tuple(round(float(x), 9) for x in t.detach().cpu().reshape(-1))
+        key = tuple([round(x, 9) for x in t.detach().cpu().reshape(-1).tolist()])
         if key not in self.ctxs:
             c = tm_create(params_from_tensor(self.template, t))
             # the autograd function keeps its input saved and unchanged between

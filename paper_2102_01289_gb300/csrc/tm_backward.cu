@@ -229,39 +229,36 @@ __global__ void __launch_bounds__(kBT, kMinBlocksPix) k_bwd_pixel(DevParams P, c
   }
 }
 
-// Range terms at each image's argmin / argmax pixels (block j: image j), and
-// the parameter gradients (block 0).
-__global__ void k_bwd_finish(DevParams P, const BwdJob *__restrict__ jobs, const double *gsum,
-                             float *grad_params) {
-  if (threadIdx.x == 0) {
-    const BwdJob &J = jobs[blockIdx.x];
-    const int W = J.in.W;
-    const float imin = J.st->imin, imax = J.st->imax;
-    const bool range = imax > imin && J.grad_in.p;
-    const unsigned long long idx[2] = {J.acc->argmin, J.acc->argmax};
-    const double gterm[2] = {J.acc->lmin / (double)imin, J.acc->lmax / (double)imax};
-    for (int k = 0; k < 2 && range; ++k) {
-      if (idx[k] >= (unsigned long long)W * (unsigned long long)J.in.H) continue;  // no pixel held it
-      const long long pix = (long long)idx[k];
-      const int y = (int)(pix / W), x = (int)(pix - (long long)y * W);
-      float r, g, b;
-      load_rgb(J.in, x, y, r, g, b);
-      const float raw = __fadd_rn(__fadd_rn(__fmul_rn(0.2126f, r), __fmul_rn(0.7152f, g)), __fmul_rn(0.0722f, b));
-      if (!(raw > kLumFloor)) continue;
-      float *gin = static_cast<float *>(J.grad_in.p) + (long long)y * J.grad_in.pitch + 3LL * x;
-      gin[0] += (float)(0.2126 * gterm[k]);
-      gin[1] += (float)(0.7152 * gterm[k]);
-      gin[2] += (float)(0.0722 * gterm[k]);
-    }
-  }
-  if (grad_params && blockIdx.x == 0 && threadIdx.x == 0) {
-    const int nf = P.n_fields;
-    for (int k = 0; k < 3; ++k) grad_params[k] = (float)gsum[k];
-    for (int f = 0; f < nf; ++f) {
-      grad_params[3 + f] = (float)gsum[3 + f];
-      grad_params[3 + nf + f] = (float)gsum[3 + kMaxFields + f];
-    }
-  }
+// Range terms at each image's argmin / argmax pixels (block j: image j, lanes
+// 0 and 1; imin < imax, so the pixels differ), and the parameter gradients
+// (block 0, a lane each). Bound by the latency of its dependent loads: with one
+// thread for everything it took 9 us.
+__global__ void __launch_bounds__(32) k_bwd_finish(DevParams P, const BwdJob *__restrict__ jobs, const double *gsum,
+                                                   float *grad_params) {
+  const int nf = P.n_fields;
+  const int t = threadIdx.x;
+  if (grad_params && blockIdx.x == 0 && t < 3 + 2 * nf)
+    grad_params[t] = (float)gsum[t < 3 + nf ? t : kMaxFields + t - nf];
+  if (t > 1) return;
+  const BwdJob &J = jobs[blockIdx.x];
+  const int W = J.in.W;
+  const float imin = J.st->imin, imax = J.st->imax;
+  const unsigned long long idx = t ? J.acc->argmax : J.acc->argmin;
+  const double sum = t ? J.acc->lmax : J.acc->lmin;
+  if (!(imax > imin) || !J.grad_in.p) return;
+  if (idx >= (unsigned long long)W * (unsigned long long)J.in.H) return;  // no pixel held it
+  const long long pix = (long long)idx;
+  const int y = (int)(pix / W), x = (int)(pix - (long long)y * W);
+  float r, g, b;
+  load_rgb(J.in, x, y, r, g, b);
+  float *gin = static_cast<float *>(J.grad_in.p) + (long long)y * J.grad_in.pitch + 3LL * x;
+  const float g0 = gin[0], g1 = gin[1], g2 = gin[2];
+  const double gterm = sum / (double)(t ? imax : imin);
+  const float raw = __fadd_rn(__fadd_rn(__fmul_rn(0.2126f, r), __fmul_rn(0.7152f, g)), __fmul_rn(0.0722f, b));
+  if (!(raw > kLumFloor)) return;
+  gin[0] = g0 + (float)(0.2126 * gterm);
+  gin[1] = g1 + (float)(0.7152 * gterm);
+  gin[2] = g2 + (float)(0.0722 * gterm);
 }
 
 // Per pixel: the adjoint of the window variances, through the normalised log,
