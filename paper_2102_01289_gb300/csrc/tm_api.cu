@@ -642,8 +642,6 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     }
   c->fwd_valid = false;  // the workspace is rewritten below
   const bool debug = c->debug != 0 && nimg == 1 && !graph;
-  // under TM_OPT_BACKWARD_REUSE the lookup also keeps the window moments
-  const bool keep_mom = c->bwd_reuse != 0 && do_lookup;
   double total_px = 0;
   for (int i = 0; i < nimg; ++i) total_px += (double)in[i].width * in[i].height;
   std::vector<Job> jobs((size_t)nimg);
@@ -684,6 +682,11 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
       return fail(c, TM_EUNSUPPORTED, "image %d is outside the compact path", i);
     c_wide = c_wide || C.wide;
   }
+  // under TM_OPT_BACKWARD_REUSE the lookup also keeps the window moments; a
+  // recomputation for the backward keeps them where the compact lookup's plain
+  // variant forms them beside the counts
+  const bool keep_mom = do_lookup ? c->bwd_reuse != 0
+                                  : compact && !c_wide && P0.small_win && !(c->p.flags & TM_FLAG_AREA_LITERAL);
   const int K = c->p.n_bins - 1;
   const int look_rows = (int)std::min(8.0, std::max(1.0, total_px / (c->num_sms * 128.0 * 40)));
   size_t ws_total = 0;
@@ -1281,12 +1284,12 @@ tm_status backward_images(tm_ctx *c, int n, const tm_image *in, const tm_image *
     FixJob *dfj = reinterpret_cast<FixJob *>(desc + sizeof(BwdJob) * (size_t)m);
     char *o = b + head;
     int pix = 0, inb = 0, tiles = 0, cols = 0;
-    bool plain = true;  // float32 inputs and uint32 count planes throughout the group
+    int plain = jobs[(size_t)i0].in.dtype;  // one input dtype and uint32 count planes throughout the group
     for (int r = 0; r < m; ++r) {
       const int i = i0 + r;
       const Job &J = jobs[(size_t)i];
       const int W = J.in.W, H = J.in.H;
-      plain = plain && J.in.dtype == kF32 && J.cnt_wide == (1 << nf) - 1;
+      if (J.in.dtype != plain || J.cnt_wide != (1 << nf) - 1) plain = -1;
       const size_t N = (size_t)W * H, plane = (size_t)(W + 1) * (H + 1);
       BwdJob &B = bj[(size_t)r];
       B = BwdJob{};

@@ -380,7 +380,10 @@ __global__ void __launch_bounds__(32 * Shape<KL>::ColWarps, KL == 64 && sizeof(B
 }
 
 // What a launch does beside writing the output image.
-enum { kOut = 0, kOutKeep = 1, kCountsOnly = 2 };
+// kOut: nothing; kOutKeep: also the count planes and window moments for the
+// backward; kCountsOnly: only the count planes, no output; kCountsMom: the
+// count planes and moments, no output.
+enum { kOut = 0, kOutKeep = 1, kCountsOnly = 2, kCountsMom = 3 };
 
 // The images of a lookup launch travel as kernel parameters: every block reads
 // its image's pointers and sizes from constant memory, as uniform values.
@@ -449,7 +452,7 @@ __global__ void __launch_bounds__(kLookCols, 7)
     const unsigned kofs = (k >> 6) * gstep + (k & 63u);  // (one group up to 64 thresholds)
     float rgb[3], pw[3];
     unsigned black = 0;
-    if (kMode != kCountsOnly) load_rgb<kDt>(J.in, x, y, rgb[0], rgb[1], rgb[2]);
+    if (kMode < kCountsOnly) load_rgb<kDt>(J.in, x, y, rgb[0], rgb[1], rgb[2]);
     Fusion fu;
     // fields in batches whose loads are in flight together: all records, the
     // moments while they arrive, all vector entries (slot 0 where no row is
@@ -478,7 +481,7 @@ __global__ void __launch_bounds__(kLookCols, 7)
           const WinMoments m = window_moments<!kPlain, kSmall>(P, f0 + i, x, y, W, H, J.s12, J.qbits, inv_scale2);
           var[i] = m.var;
           rarea[i] = m.rarea;
-          if (kPlain ? kMode == kOutKeep : J.mom != nullptr)
+          if (kPlain ? kMode == kOutKeep || kMode == kCountsMom : J.mom != nullptr)
             J.mom[(size_t)(f0 + i) * W * H + pix] = make_float2(m.var, window_mean(m.q1, m.rarea, inv_scale));
         }
       }
@@ -497,7 +500,7 @@ __global__ void __launch_bounds__(kLookCols, 7)
         e[i][2] = __ldg(pr + (r[i][2].y >> 16) * 32);
         e[i][3] = __ldg(pr + (r[i][3].y >> 16) * 32);
       }
-      if (f0 == 0 && kMode != kCountsOnly) black = colour_powers<kPlain>(P, rgb, pw);
+      if (f0 == 0 && kMode < kCountsOnly) black = colour_powers<kPlain>(P, rgb, pw);
 #pragma unroll
       for (int i = 0; i < kFieldBatch && f0 + i < NF; ++i) {
         const int f = f0 + i;
@@ -506,9 +509,9 @@ __global__ void __launch_bounds__(kLookCols, 7)
           const Win w = window_of(P, f, x, y, W, H);
           cnt[i] = whole ? (unsigned)((w.x1 - w.x0 + 1) * (w.y1 - w.y0 + 1)) : 0u;
         }
-        if (kMode == kCountsOnly || (kPlain ? kMode == kOutKeep : J.cnt != nullptr))
+        if (kMode >= kCountsOnly || (kPlain ? kMode == kOutKeep : J.cnt != nullptr))
           J.cnt[f * J.cnt_step + pix] = cnt[i];
-        if (kMode != kCountsOnly) {
+        if (kMode < kCountsOnly) {
           float Wf, Lf;
           fuse_field<kPlain>(P, f, cnt[i], rarea[i], var[i], fu, Wf, Lf);
           if (!kPlain && J.dbg.l) {
@@ -521,7 +524,7 @@ __global__ void __launch_bounds__(kLookCols, 7)
         }
       }
     }
-    if (kMode != kCountsOnly) {
+    if (kMode < kCountsOnly) {
       const float Lc = fused_value(P, fu);
       rgb[0] = pw[0] * Lc, rgb[1] = pw[1] * Lc, rgb[2] = pw[2] * Lc;
       if (black) {
@@ -641,7 +644,9 @@ int launch_lookup_compact(const DevParams &P, const Job *jobs, int njobs, int bl
               reinterpret_cast<unsigned *>(J.cnt), J.mom, J.dbg, J.cnt_off[1] / 4, J.qbits, J.c_shift,
               J.b0[kStLook], 0};
   }
-  if (counts_only) {
+  if (counts_only && keep) {
+    launch_look<uint16_t, true, 1, -1, kCountsMom>(P, L, blocks, s);
+  } else if (counts_only) {
     if (wide) launch_look<uint32_t, true, -1, -1, kCountsOnly>(P, L, blocks, s);
     else launch_look<uint16_t, true, -1, -1, kCountsOnly>(P, L, blocks, s);
   } else if (general) {

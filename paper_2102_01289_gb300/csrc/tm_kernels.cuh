@@ -102,7 +102,8 @@ int launch_compact_build(const Job *jobs, int njobs, int row_blocks, int col_uni
 // which travel as kernel parameters): blocks of `rows` rows (compact_look_blocks of an image,
 // first block J.b0[kStLook]). plain: no job has debug planes
 // to write; keep: every job also gets its count planes (J.cnt, uint32) and
-// window moments (J.mom); counts_only: only its count planes; dtype as for
+// window moments (J.mom); counts_only: no output (with keep: 16-bit vectors and
+// small windows without the literal area only); dtype as for
 // launch_lookup_counts.
 constexpr int kCompactImages = 32;
 int compact_look_blocks(int W, int H, int rows);
