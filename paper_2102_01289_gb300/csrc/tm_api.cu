@@ -670,7 +670,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   const int wave = c->num_sms * cps;
   // the compact path's groups of images: their first images, and their blocks
   struct Group {
-    int first, rows, cols, look;
+    int first, rows, cols, look, tall;
   };
   std::vector<Group> groups;
   std::vector<CompactPlan> cplans((size_t)nimg);
@@ -705,13 +705,14 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
       if (c_wide && !C.wide) C.vec_bytes *= 2;
       const size_t b = compact_bytes(C);
       if (groups.empty() || c_used + b > kCompactGroup || i - groups.back().first >= kCompactImages) {
-        groups.push_back({i, 0, 0, 0});
+        groups.push_back({i, 0, 0, 0, 0});
         c_used = 0;
       }
       coffs[(size_t)i] = c_used;
       c_used += b;
       c_total = std::max(c_total, c_used);
       Group &g = groups.back();
+      g.tall = std::max(g.tall, H);
       J.b0[kStCRows] = g.rows;
       g.rows += compact_row_blocks(H, K);
       J.b0[kStCCols] = g.cols;
@@ -851,7 +852,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   const auto group_end = [&](size_t k) { return k + 1 < groups.size() ? groups[k + 1].first : nimg; };
   const auto build = [&](size_t k, cudaStream_t q) {
     const Group &g = groups[k];
-    return launch_compact_build(dj + g.first, group_end(k) - g.first, g.rows, g.cols, K, c_wide, q);
+    return launch_compact_build(dj + g.first, group_end(k) - g.first, g.rows, g.cols, g.tall, K, c_wide, q);
   };
   int ls = compact ? build(0, c->sweep_stream)
                    : launch_sweep(P, dj, nimg, nitems, queue, smem, ctas, width, c->sweep_stream);
