@@ -58,6 +58,10 @@ template <int KL>
 struct Shape {
   static constexpr int T = KL == 64 ? 2 : 1;
   static constexpr int Step = 4;                         // rows or chunks in flight together
+  // the column pass loads the next rows while it works on these, where the
+  // registers allow (31 thresholds, 1080p: the build 55 -> 50 us; 63, 12 MP:
+  // spills, 194 -> 214)
+  static constexpr bool Ahead = T == 1;
   static constexpr int ColWarps = 16;                    // row segments of a CTA
   static constexpr int MinBlocks = 2;                    // 64 registers
   // column CTAs share a chunk's rows until the launch has this many warps.
@@ -129,14 +133,21 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(const Job *__re
     const unsigned gl = cb + lane < G ? (unsigned)__ldg(grow + cb + lane) : kNoRow;
     const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit = chunk of the batch
     const int n = min(32, Gp - cb);
-    for (int i = 0; i < n; i += S::Step) {
-      int b[S::Step];
+    const auto fetch = [&](int i, int *b) {  // the lane's bins of chunks i .. of the batch, where they are mixed
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
         const int col = 32 * (cb + i + u);
         b[u] = 256;
-        if (((mixed >> (i + u)) & 1u) && col + lane < W) b[u] = (int)__ldg(bins + col);
+        if (i + u < 32 && ((mixed >> ((i + u) & 31)) & 1u) && col + lane < W) b[u] = (int)__ldg(bins + col);
       }
+    };
+    int nb[S::Step];
+    fetch(0, nb);
+    for (int i = 0; i < n; i += S::Step) {
+      int b[S::Step];
+#pragma unroll
+      for (int u = 0; u < S::Step; ++u) b[u] = nb[u];
+      fetch(i + S::Step, nb);  // in flight meanwhile
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
         if (i + u >= n) break;
@@ -202,16 +213,32 @@ __device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int
     const unsigned gl = c < G && lane < n ? (unsigned)__ldg(grp) : kNoRow;
     grp += (size_t)32 * G;
     const unsigned mixed = __ballot_sync(0xffffffffu, mixed_range<KL>(gl, k0));  // bit = row of the batch
-    for (int i = 0; i < n; i += S::Step) {
-      unsigned rp[S::Step][T];
-      int b[S::Step];
+    const auto fetch = [&](int i, unsigned (*rp)[T], int *b) {  // rows i .. of the batch: prefixes, mixed rows' bins
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
 #pragma unroll
         for (int z = 0; z < T; ++z) rp[u][z] = 0;
-        if (own && i + u < n) load_prefix<T>(row + u * KL, rp[u]);
+        if (own && i + u < n) load_prefix<T>(row + (i + u) * KL, rp[u]);
         b[u] = 256;
-        if (((mixed >> (i + u)) & 1u) && colok) b[u] = (int)__ldg(bins + (size_t)u * W);
+        if (i + u < 32 && ((mixed >> ((i + u) & 31)) & 1u) && colok) b[u] = (int)__ldg(bins + (size_t)(unsigned)(i + u) * W);
+      }
+    };
+    unsigned nrp[S::Step][T];
+    int nb[S::Step];
+    if (S::Ahead) fetch(0, nrp, nb);
+    for (int i = 0; i < n; i += S::Step) {
+      unsigned rp[S::Step][T];
+      int b[S::Step];
+      if (S::Ahead) {
+#pragma unroll
+        for (int u = 0; u < S::Step; ++u) {
+#pragma unroll
+          for (int z = 0; z < T; ++z) rp[u][z] = nrp[u][z];
+          b[u] = nb[u];
+        }
+        fetch(i + S::Step, nrp, nb);
+      } else {
+        fetch(i, rp, b);
       }
 #pragma unroll
       for (int u = 0; u < S::Step; ++u) {
@@ -259,10 +286,10 @@ __device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int
         }
         if (kWrite && own && i + u < n) store_records<T>(rec + u * KL, st.pt, st.mc);
       }
-      row += S::Step * KL;
       rec += S::Step * KL;
-      bins += (size_t)S::Step * W;
     }
+    row += 32 * KL;
+    bins += (size_t)32 * W;
   }
 }
 
