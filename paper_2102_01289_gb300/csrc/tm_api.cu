@@ -83,14 +83,15 @@ struct tm_ctx {
   int stats_n = 0;
   // job descriptors: written to a device buffer at the start of each call by
   // put_jobs (the sweep queue is written on the device); stream-ordered like
-  // the workspace. The cached batch graph has its own device buffers, written
-  // by its own nodes at every replay.
+  // the workspace. Each cached graph has its own copy, written once before its
+  // first launch.
   Job *djobs = nullptr;    // device copy of the job array (calls outside the graph)
   int4 *ditems = nullptr;  // sweep queue: the pop counter
   size_t djobs_bytes = 0, ditems_bytes = 0;
-  Job *gdjobs = nullptr;   // device buffers written by the cached graph
-  int4 *gditems = nullptr;
-  size_t gdjobs_bytes = 0, gditems_bytes = 0;
+  int4 *gditems = nullptr;  // the queue of the cached graphs (cleared by their own nodes)
+  size_t gditems_bytes = 0;
+  Job *gspare = nullptr;    // descriptor buffer of a replaced graph, or of one being captured
+  int gspare_n = 0;
   // backward workspace
   void *bws = nullptr;
   size_t bws_bytes = 0;
@@ -121,7 +122,7 @@ struct tm_ctx {
   // CUDA graphs of the last fused forwards (batches, or the images of a batch
   // taking the fused path, and single images), each replayed while its images
   // are unchanged; the least recently used is replaced. They share the
-  // workspace and gdjobs / gditems, which each replay rewrites first. And the
+  // workspace and gditems; each has descriptors of its own. And the
   // graph of the last batch's images taking the materialised path, with that
   // pass's own workspace and descriptors.
   struct FusedGraph {
@@ -129,6 +130,8 @@ struct tm_ctx {
     std::vector<tm_image> in, out;
     int64_t launches = 0;
     std::vector<Job> jobs;
+    Job *djobs = nullptr;  // its own device copy of jobs, written when it was captured
+    int djobs_n = 0;
     uint64_t used = 0;
     int path = 0;  // kPathSweep or kPathCompact
   };
@@ -378,8 +381,10 @@ tm_status ensure_side_streams(tm_ctx *c) {
 constexpr size_t kFusedGraphs = 6;
 
 void drop_graph(tm_ctx *c) {
-  for (auto &g : c->graphs)
+  for (auto &g : c->graphs) {
     if (g.exec) cudaGraphExecDestroy(g.exec);
+    if (g.djobs) cudaFree(g.djobs);  // (after the replays in flight)
+  }
   c->graphs.clear();
   if (c->mgraph) cudaGraphExecDestroy(c->mgraph);
   c->mgraph = nullptr;
@@ -519,7 +524,7 @@ tm_status forward_materialised(tm_ctx *c, const tm_image *in, const tm_image *ou
   const int qbits = choose_qbits(c->p, W, H);
   DevParams P = dev_params(c->p, qbits);
   int nseg, seg_rows;
-  integral_layout(W, H, SIZE_MAX, nseg, seg_rows);
+  integral_layout(W, H, SIZE_MAX, 2 * c->num_sms, nseg, seg_rows);
   JobLayout L = job_layout(c->p, W, H, nseg, 0, c->debug != 0);
   const size_t plane = (size_t)(W + 1) * (H + 1);
   size_t off_cpl = align256(L.total), off_hscr = 0, total = off_cpl;
@@ -698,7 +703,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     Job &J = jobs[(size_t)i];
     if (compact) memset(&J, 0, sizeof J);
     J.qbits = choose_qbits(c->p, W, H);
-    integral_layout(W, H, SIZE_MAX, J.nseg, J.seg_rows);
+    integral_layout(W, H, SIZE_MAX, (int)(2 * c->num_sms * share), J.nseg, J.seg_rows);
     size_t cnt_bytes = 0;
     if (compact) {
       CompactPlan &C = cplans[(size_t)i];
@@ -772,12 +777,26 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     auto lru = std::min_element(c->graphs.begin(), c->graphs.end(),
                                 [](const tm_ctx::FusedGraph &a, const tm_ctx::FusedGraph &b) { return a.used < b.used; });
     cudaGraphExecDestroy(lru->exec);
+    if (c->gspare) cudaFree(c->gspare);
+    c->gspare = lru->djobs;
+    c->gspare_n = lru->djobs_n;
     c->graphs.erase(lru);
   }
-  Job **djobs = graph ? &c->gdjobs : &c->djobs;
   int4 **ditems = graph ? &c->gditems : &c->ditems;
-  if ((st = grow_device(c, (void **)djobs, graph ? &c->gdjobs_bytes : &c->djobs_bytes, sizeof(Job) * nimg)))
+  if (graph) {
+    if (c->gspare_n < nimg) {
+      if (c->gspare) cudaFree(c->gspare);
+      c->gspare = nullptr;
+      c->gspare_n = 0;
+      if (cudaMalloc(&c->gspare, sizeof(Job) * (size_t)nimg) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, TM_ENOMEM, "device allocation of %zu bytes", sizeof(Job) * (size_t)nimg);
+      }
+      c->gspare_n = nimg;
+    }
+  } else if ((st = grow_device(c, (void **)&c->djobs, &c->djobs_bytes, sizeof(Job) * nimg))) {
     return st;
+  }
   if ((st = grow_device(c, (void **)ditems, graph ? &c->gditems_bytes : &c->ditems_bytes, sizeof(int4))))
     return st;
   char *ws = static_cast<char *>(c->ws);
@@ -823,19 +842,22 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     run_range = own;
   }
   const DevParams P = dev_params(c->p, jobs[0].qbits);  // qbits is per job
-  Job *dj = *djobs;
+  Job *dj = graph ? c->gspare : c->djobs;
   int *queue = reinterpret_cast<int *>(*ditems);
   const int ctas = std::min(nitems, wave);
   // a batch is captured on the context's own stream (capture is not allowed on
   // the legacy default stream) and the graph is then launched on the caller's
   const cudaStream_t caller = s;
   if ((st = ensure_side_streams(c))) return st;  // before any capture begins
+  // a graph's descriptors are written once, ahead of it (a replay saves the
+  // launch: 2 us of a forward's 41 at 512 x 384)
+  const int64_t puts = put_jobs(jobs.data(), nimg, dj, s);
   if (graph) {
     if (!c->graph_stream) TM_CUDA(c, cudaStreamCreateWithFlags(&c->graph_stream, cudaStreamNonBlocking));
     s = c->graph_stream;
     TM_CUDA(c, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
   }
-  int64_t n = put_jobs(jobs.data(), nimg, dj, s);
+  int64_t n = graph ? 0 : puts;
   if (!graph) mark(c, s, -1);
   const int in_dt = input_dtype(jobs.data(), nimg);
   if (run_range) launch_range(dj, nimg, b_range, c->p.n_bins, in_dt, s);
@@ -908,13 +930,17 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     G.jobs = jobs;
     G.used = c->calls;
     G.path = path;
+    G.djobs = c->gspare;
+    G.djobs_n = c->gspare_n;
+    c->gspare = nullptr;
+    c->gspare_n = 0;
     c->graphs.push_back(std::move(G));
     TM_CUDA(c, cudaGraphLaunch(c->graphs.back().exec, caller));
   } else if (ls < 0) {
     return check_launch(c, "histogram shared-memory attribute");
   }
   if ((st = check_launch(c, "forward launch"))) return st;
-  return finish_fused(c, nimg, in, jobs, n, run_range, jobs_out);
+  return finish_fused(c, nimg, in, jobs, graph ? n + puts : n, run_range, jobs_out);
 }
 
 // Bookkeeping after a fused forward over `jobs` (n launches), launched or
@@ -971,7 +997,7 @@ tm_status forward_materialised_batch(tm_ctx *c, int nimg, const tm_image *in, co
     Job &J = jobs[(size_t)i];
     memset(&J, 0, sizeof J);
     J.qbits = choose_qbits(c->p, W, H);
-    integral_layout(W, H, SIZE_MAX, J.nseg, J.seg_rows);
+    integral_layout(W, H, SIZE_MAX, (int)(2 * c->num_sms * share), J.nseg, J.seg_rows);
     lays[(size_t)i] = job_layout(c->p, W, H, J.nseg, 0, false);
     offs[(size_t)i] = ws_total;
     ws_total += lays[(size_t)i].total;
@@ -1521,7 +1547,7 @@ tm_status tm_create(const tm_params *params, tm_ctx **out) {
 
 void tm_destroy(tm_ctx *c) {
   if (!c) return;
-  if (c->ws || c->mws || c->stats || c->rr_stats || c->stage || c->djobs || c->gdjobs || !c->graphs.empty() || c->mgraph ||
+  if (c->ws || c->mws || c->stats || c->rr_stats || c->stage || c->djobs || c->gspare || !c->graphs.empty() || c->mgraph ||
       c->hslot[0])
     cudaDeviceSynchronize();
   drop_graph(c);
@@ -1550,7 +1576,7 @@ void tm_destroy(tm_ctx *c) {
     if (q) cudaStreamDestroy(q);
   for (cudaEvent_t e : {c->ov_fork, c->ov_sweep, c->ov_int})
     if (e) cudaEventDestroy(e);
-  if (c->gdjobs) cudaFree(c->gdjobs);
+  if (c->gspare) cudaFree(c->gspare);
   if (c->gditems) cudaFree(c->gditems);
   if (c->mws) cudaFree(c->mws);
   if (c->mdjobs) cudaFree(c->mdjobs);
@@ -1795,7 +1821,7 @@ tm_status tm_integral_image(const int32_t *q, int32_t width, int32_t height, int
   J.q = const_cast<int32_t *>(q);
   J.s1 = reinterpret_cast<long long *>(s1);
   J.s2 = reinterpret_cast<long long *>(s2);
-  integral_layout(width, height, SIZE_MAX, J.nseg, J.seg_rows);
+  integral_layout(width, height, SIZE_MAX, 304, J.nseg, J.seg_rows);
   const size_t seg_bytes = 8 * integral_scratch_elems(width, height, J.nseg);
   void *scr = nullptr;
   cudaError_t e = cudaMallocAsync(&scr, align256(sizeof(Job)) + seg_bytes, st);

@@ -733,9 +733,14 @@ __global__ void __launch_bounds__(32 * kHW, 5) k_hist_write(const __grid_constan
 
 }  // namespace
 
-void integral_layout(int W, int H, size_t max_scratch_elems, int &nseg, int &seg_rows) {
-  // the shortest segments (most tiles) whose scratch fits, at least kIR rows
+void integral_layout(int W, int H, size_t max_scratch_elems, int tiles, int &nseg, int &seg_rows) {
+  // the shortest segments (most tiles) whose scratch fits, at least kIR rows;
+  // fewer, down to four, where that gives no more than `tiles` tiles: a tile's
+  // rows are a serial chain of barriers (16 rows 15 us, of 45 for a forward at
+  // 512 x 384)
   seg_rows = kIR;
+  const long long chunks = (W + kIC - 1) / kIC;
+  while (seg_rows > 4 && (H + seg_rows / 2 - 1) / (seg_rows / 2) * chunks <= tiles) seg_rows /= 2;
   for (;;) {
     nseg = (H + seg_rows - 1) / seg_rows;
     if (integral_scratch_elems(W, H, nseg) <= max_scratch_elems || seg_rows >= H) return;

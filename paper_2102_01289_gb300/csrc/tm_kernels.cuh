@@ -26,12 +26,13 @@ int prep_blocks(int W, int H, int num_sms, double share);
 // Stage a2 (Eq. 5): integral images of q and q^2, (H+1) x (W+1) int64, over
 // tiles of row segments x column chunks. integral_layout picks the segments
 // (J.nseg of J.seg_rows rows) whose scratch fits max_scratch_elems (the
-// shortest such, at least 16 rows; at worst one segment). Per image:
+// shortest such, at least 16 rows, or down to 4 while the image then has no
+// more than `tiles` tiles; at worst one segment). Per image:
 // integral_tile_blocks(W, nseg) blocks of the tile launches (first block
 // J.b0[kStRows]), integral_col_blocks(W) of the column-prefix launch
 // (J.b0[kStCols]), and integral_scratch_elems(W, H, nseg) int64 elements of
 // scratch at J.segtot. Returns the number of launches.
-void integral_layout(int W, int H, size_t max_scratch_elems, int &nseg, int &seg_rows);
+void integral_layout(int W, int H, size_t max_scratch_elems, int tiles, int &nseg, int &seg_rows);
 size_t integral_scratch_elems(int W, int H, int nseg);
 int integral_tile_blocks(int W, int nseg);
 int integral_col_blocks(int W);

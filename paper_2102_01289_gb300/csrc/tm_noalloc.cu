@@ -34,7 +34,7 @@ extern "C" tm_status tm_integral_image_noalloc(const int32_t *q, int32_t width, 
     return fail_noctx(TM_EINVAL, "tm_integral_image_noalloc: width and height must be >= 1, below 2^31 pixels");
   const size_t job_bytes = round256(sizeof(Job));
   int nseg = 1, seg_rows = 1;
-  integral_layout(width, height, (kScratchBytes - job_bytes) / 8, nseg, seg_rows);
+  integral_layout(width, height, (kScratchBytes - job_bytes) / 8, 0, nseg, seg_rows);
   const size_t need = job_bytes + 8 * integral_scratch_elems(width, height, nseg);
   if (need > kScratchBytes)
     return fail_noctx(TM_EINVAL, "tm_integral_image_noalloc: the image needs more than the 8 MiB static scratch "
