@@ -109,23 +109,21 @@ __device__ void commit_range(Stats *st, unsigned bmin, unsigned bmax, int nb, in
   const float imin = __uint_as_float(vs->min_bits);
   const float imax = __uint_as_float(vs->max_bits);
   const bool degenerate = !(imax > imin);
-  // the FP64 logarithms, one warp each, so that their latencies overlap (the
-  // FP64 pipe is slow on this part and this block is the kernel's tail)
+  // This block is the kernel's tail, and the FP64 pipe is slow on this part (a
+  // warp instruction holds it for 16 cycles however many lanes take part): the
+  // natural logarithms are two lanes of one warp and the base-2 ones three of
+  // another; then one warp's lanes form the quotients while the others form
+  // the edges. A warp per logarithm and one thread for the quotients took 2 us
+  // more.
   __shared__ double lg[5];
   const unsigned bits = __float_as_uint(imin);
-  if ((threadIdx.x & 31) == 0) {
-    switch (threadIdx.x >> 5) {
-      case 0: lg[0] = log((double)imin); break;
-      case 1: lg[1] = log((double)imax); break;
-      case 2: lg[2] = log2((double)imin); break;
-      case 3: lg[3] = log2((double)imax); break;
-      case 4: lg[4] = log2((double)__uint_as_float((bits & 0x7fffffu) | 0x3f800000u)); break;
-      default: break;
-    }
-  }
+  if (wid == 0 && lane < 2) lg[lane] = log((double)(lane ? imax : imin));
+  if (wid == 1 && lane < 3)
+    lg[2 + lane] = log2((double)(lane == 0 ? imin : lane == 1 ? imax : __uint_as_float((bits & 0x7fffffu) | 0x3f800000u)));
   __syncthreads();
   const double lmin = lg[0], lmax = lg[1];
-  for (int k = 1 + threadIdx.x; k < n_bins; k += blockDim.x) {
+  const int last_warp = (int)(blockDim.x >> 5) - 1;
+  for (int k = 1 + threadIdx.x; k < n_bins && wid < last_warp; k += 32 * last_warp) {
     float edge = __int_as_float(0x7f800000);
     if (!degenerate) {
       const double t = exp(lmin + (lmax - lmin) * ((double)k / (double)n_bins));
@@ -133,14 +131,17 @@ __device__ void commit_range(Stats *st, unsigned bmin, unsigned bmax, int nb, in
     }
     st->thr[k - 1] = edge;
   }
-  if (threadIdx.x == 0) {
-    const double l2min = lg[2], l2max = lg[3];
+  if (wid == last_warp && lane < 3) {
+    const double span = lg[3] - lg[2];
+    const float r = (float)((lane == 2 ? (double)n_bins : ldexp(1.0, qbits)) / (lane == 1 ? (double)imax : span));
+    if (lane == 0) st->log2_scale = degenerate ? 0.f : r;
+    if (lane == 1) st->lin_scale = r;
+    if (lane == 2) st->bin_scale = degenerate ? 0.f : r;
+  }
+  if (wid == last_warp && lane == 3) {
     st->e0 = (int)(bits >> 23) - 127;
     st->c0 = (float)lg[4];
-    st->log2_scale = degenerate ? 0.f : (float)(ldexp(1.0, qbits) / (l2max - l2min));
-    st->lin_scale = (float)(ldexp(1.0, qbits) / (double)imax);
-    st->lg_min = (float)l2min;
-    st->bin_scale = degenerate ? 0.f : (float)((double)n_bins / (l2max - l2min));
+    st->lg_min = (float)lg[2];
     st->imin = imin;
     st->imax = imax;
     st->degenerate = degenerate ? 1 : 0;
