@@ -1190,10 +1190,12 @@ tm_status forward_device(tm_ctx *c, const tm_image *in, const tm_image *out, cud
 // the parameter sums and the descriptor arrays of the largest group, then per
 // image of a group its u / v planes, direct luminance gradient, fixed-point
 // pair planes and their scratch.
+size_t uv_pitch(int W) { return ((size_t)W + 3) & ~(size_t)3; }
+
 size_t backward_image_bytes(const tm_params &p, int W, int H, int nseg) {
   const size_t N = (size_t)W * H, plane = (size_t)(W + 1) * (H + 1);
   const int nf = p.n_fields;
-  return 2 * align256(4 * N * nf) + align256(4 * N) + align256(16 * plane * nf) +
+  return 2 * align256(4 * uv_pitch(W) * H * nf) + align256(4 * N) + align256(16 * plane * nf) +
          align256(8 * fix_integral_scratch_elems(W, H, nf, nseg));
 }
 
@@ -1337,9 +1339,11 @@ tm_status backward_images(tm_ctx *c, int n, const tm_image *in, const tm_image *
       B.cnt_wide = J.cnt_wide;
       B.qbits = J.qbits;
       B.U = reinterpret_cast<float *>(o);
-      B.V = reinterpret_cast<float *>(o + align256(4 * N * nf));
-      B.gi_direct = reinterpret_cast<float *>(o + 2 * align256(4 * N * nf));
-      char *iuv = o + 2 * align256(4 * N * nf) + align256(4 * N);
+      const size_t uv = align256(4 * uv_pitch(W) * H * nf);
+      B.V = reinterpret_cast<float *>(o + uv);
+      B.upitch = (int)uv_pitch(W);
+      B.gi_direct = reinterpret_cast<float *>(o + 2 * uv);
+      char *iuv = o + 2 * uv + align256(4 * N);
       B.IUV = reinterpret_cast<const longlong2 *>(iuv);
       B.acc = accs + r;
       B.b0 = pix;
@@ -1359,6 +1363,7 @@ tm_status backward_images(tm_ctx *c, int n, const tm_image *in, const tm_image *
       F.nseg = nseg[(size_t)i];
       F.seg_rows = seg_rows[(size_t)i];
       F.np = nf;
+      F.pitch = B.upitch;
       F.b0_tile = tiles;
       F.b0_col = cols;
       tiles += fix_tile_blocks(W, F.nseg, nf);

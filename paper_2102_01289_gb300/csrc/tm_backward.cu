@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kBT, kMinBlocksPix) k_bwd_pixel(DevParams P, c
   const int lb = blockIdx.x - J.b0, bx = (W + 31) / 32;
   const int x = (lb % bx) * 32 + (threadIdx.x & 31);
   const int ybase = (lb / bx) * (8 * kRowsPix) + (threadIdx.x >> 5);
-  const size_t N = (size_t)W * H;
+  const size_t N = (size_t)W * H, NU = (size_t)J.upitch * H;
   const float inv_scale = ldexpf(1.f, -J.qbits);
   const float inv_scale2 = inv_scale * inv_scale;
   const float imin = J.st->imin, imax = J.st->imax;
@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(kBT, kMinBlocksPix) k_bwd_pixel(DevParams P, c
       const int y = ybase + 8 * r;
       if (y >= H) break;
       const unsigned pix = (unsigned)y * (unsigned)W + (unsigned)x;
+      const size_t upix = (size_t)y * J.upitch + x;
       float Pf[NF], rarea[NF], var[NF], mu[NF], wv[NF], lf[NF];
       float wsum = 0.f, accL = 0.f, meanL = 0.f;
 #pragma unroll
@@ -187,8 +188,8 @@ __global__ void __launch_bounds__(kBT, kMinBlocksPix) k_bwd_pixel(DevParams P, c
         acc[3 + NF + f] += gW * v * ve * rden;
         const float u = 2.f * (gW * a * e * rden) * rarea[f];
         const float vv = u * mu[f];
-        J.U[f * N + pix] = u;
-        J.V[f * N + pix] = vv;
+        J.U[f * NU + upix] = u;
+        J.V[f * NU + upix] = vv;
         amax[f] = max(amax[f], __float_as_uint(fabsf(u)));
         amax[NF + f] = max(amax[NF + f], __float_as_uint(fabsf(vv)));
       }

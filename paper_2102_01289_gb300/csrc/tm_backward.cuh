@@ -32,7 +32,8 @@ struct alignas(16) BwdJob {
   long long cnt_off[kMaxFields];
   int cnt_wide;                 // bit f: plane f is uint32 (else uint16)
   int qbits;
-  float *U, *V;                 // s x H x W: u_f = 2 dLoss/ds_f / N_f and u_f * mu_f
+  int upitch;                   // W rounded up to 4, so that the fixed-point passes read whole vectors
+  float *U, *V;                 // s x H x upitch: u_f = 2 dLoss/ds_f / N_f and u_f * mu_f
   float *gi_direct;             // H x W: dLoss/di through Eq. 12 directly
   const longlong2 *IUV;         // s pair planes of (H+1)*(W+1) positions: the fixed-point
                                 //   integrals of u_f and v_f, interleaved

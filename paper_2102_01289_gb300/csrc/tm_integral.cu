@@ -106,15 +106,15 @@ struct QSource {
 struct FixSource {
   using Raw = float2;
   const float *u, *v;
-  int W;
+  int W, pitch;  // rows of pitch floats
   float a_hi, a_lo, b_hi, b_lo;
   __device__ __forceinline__ Raw load(int r, int c) const {
-    const long long o = (long long)r * W + c;
+    const long long o = (long long)r * pitch + c;
     return make_float2(__ldg(u + o), __ldg(v + o));
   }
   __device__ __forceinline__ Raw zero() const { return make_float2(0.f, 0.f); }
   __device__ __forceinline__ void load4(int r, int c, bool vec, Raw *x) const {
-    const size_t o = (size_t)r * W + c;
+    const size_t o = (size_t)r * pitch + c;
     if (vec && c + 3 < W) {
       const float4 a = __ldg(reinterpret_cast<const float4 *>(u + o));
       const float4 b = __ldg(reinterpret_cast<const float4 *>(v + o));
@@ -126,7 +126,7 @@ struct FixSource {
     }
   }
   __device__ __forceinline__ bool vec_ok() const {
-    return (W & 3) == 0 && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
+    return (pitch & 3) == 0 && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
   }
   __device__ __forceinline__ void warp_sums(long long &su, long long &sv) const {
 #pragma unroll
@@ -144,8 +144,8 @@ struct FixSource {
   }
 };
 
-__device__ __forceinline__ FixSource fix_source_of(const float *u, const float *v, int W, int sa, int sb) {
-  return FixSource{u, v, W, ldexpf(1.f, sa / 2), ldexpf(1.f, sa - sa / 2), ldexpf(1.f, sb / 2),
+__device__ __forceinline__ FixSource fix_source_of(const float *u, const float *v, int W, int pitch, int sa, int sb) {
+  return FixSource{u, v, W, pitch, ldexpf(1.f, sa / 2), ldexpf(1.f, sa - sa / 2), ldexpf(1.f, sb / 2),
                    ldexpf(1.f, sb - sb / 2)};
 }
 
@@ -511,8 +511,8 @@ __device__ __forceinline__ IntTask fix_task(const FixJob &F, int p) {
 }
 
 __device__ __forceinline__ FixSource fix_source(const FixJob &F, int p) {
-  const long long N = (long long)F.W * F.H;
-  return fix_source_of(F.u + p * N, F.v + p * N, F.W, fix_shift(__ldg(F.amax + p), F.nmax[p]),
+  const long long N = (long long)F.pitch * F.H;
+  return fix_source_of(F.u + p * N, F.v + p * N, F.W, F.pitch, fix_shift(__ldg(F.amax + p), F.nmax[p]),
                        fix_shift(__ldg(F.amax + kMaxFields + p), F.nmax[p]));
 }
 
@@ -758,11 +758,12 @@ int integral_tile_blocks(int W, int nseg) { return nseg * ((W + kIC - 1) / kIC);
 int integral_col_blocks(int W) { return (W + kMidCols - 1) / kMidCols; }
 
 // Row segments of an image's fixed-point pairs in a batch whose pairs, over
-// all images, number `batch_pairs`: short enough for about 2048 tiles over
-// the batch, 4 to kIR rows.
+// all images, number `batch_pairs`: short enough for about 512 tiles over the
+// batch, 4 to kIR rows (the three launches at 1599 x 1199, three pairs, for
+// 4096, 2048, 1024 and 512 tiles: 89, 89, 85 and 81 us).
 void fix_layout(int W, int H, long long batch_pairs, int &nseg, int &seg_rows) {
   const long long tiles_per_row = batch_pairs * ((W + kIC - 1) / kIC);
-  seg_rows = (int)std::min<long long>(kIR, std::max<long long>(4, H * tiles_per_row / 2048));
+  seg_rows = (int)std::min<long long>(kIR, std::max<long long>(4, H * tiles_per_row / 512));
   nseg = (H + seg_rows - 1) / seg_rows;
 }
 

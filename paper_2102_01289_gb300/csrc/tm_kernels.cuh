@@ -39,7 +39,7 @@ int integral_col_blocks(int W);
 int launch_integral_jobs(const Job *jobs, int njobs, int tile_blocks, int col_blocks, cudaStream_t s);
 
 // The backward's integral planes (64-bit fixed point) of one image's `np`
-// float plane pairs (u_p, v_p), each W x H: u_p scaled by 2^fix_shift(amax[p],
+// float plane pairs (u_p, v_p), each W x H in rows of `pitch` floats: u_p scaled by 2^fix_shift(amax[p],
 // nmax[p]) and v_p by 2^fix_shift(amax[kMaxFields + p], nmax[p]) (amax on the
 // device), interleaved into pair plane p of dst ((H+1) x (W+1) positions of
 // two int64). Over a batch: the image's first blocks in the tile and column
@@ -51,6 +51,7 @@ struct alignas(16) FixJob {
   long long *scratch;        // fix_integral_scratch_elems(W, H, np, nseg) int64
   long long scratch_stride;  // per pair
   int W, H, nseg, seg_rows, np;
+  int pitch;                 // floats from row to row of u and v
   int b0_tile, b0_col;
   float nmax[kMaxFields];
 };
