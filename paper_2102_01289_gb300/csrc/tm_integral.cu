@@ -554,7 +554,9 @@ __global__ void __launch_bounds__(kINT, 4) k_fix_write(const FixJob *__restrict_
 // of 128, one warp each:
 //   1. k_hist_cols counts, per segment, plane and column, the pixels the plane
 //      indicates;
-//   2. k_hist_mid replaces the counts by those of the segments above;
+//   2. k_hist_mid, where there are more than kHDirect segments, replaces the
+//      counts by those of the segments above (else the next launch adds them
+//      up itself: a launch less);
 //   3. k_hist_write, a block per segment and plane, walks the strips of the
 //      image eight at a time. A warp's accumulators start from the column
 //      counts above, summed along the strip; per row, ballots give the
@@ -568,12 +570,14 @@ __global__ void __launch_bounds__(kINT, 4) k_fix_write(const FixJob *__restrict_
 constexpr int kHW = 8;                  // strips (warps) of a block's pass
 constexpr int kHStrip = 128;            // columns of a strip
 constexpr int kHCols = kHW * kHStrip;   // columns of a pass
+constexpr int kHDirect = 32;            // segments whose counts the write pass adds up
 
 struct HistPlanes {
   const uint8_t *bins;
   uint32_t *planes;
   uint32_t *counts;  // nseg x n_planes x W column counts
   int W, H, nseg, seg_rows, n_planes, k_begin, eq;
+  int summed;        // the counts have been replaced by those of the segments above
 };
 
 // Plane p indicates [b == k] (eq) or [b < k], k = k_begin + p.
@@ -656,11 +660,17 @@ __global__ void __launch_bounds__(32 * kHW, 5) k_hist_write(const __grid_constan
     const int c0 = C0 + wid * kHStrip;  // the warp's strip
     unsigned acc[4];                    // columns c0 + 32 m + lane
     bool ok[4];
-    const uint32_t *cnt = Q.counts + ((size_t)seg * Q.n_planes + p) * W + c0 + lane;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       ok[m] = c0 + 32 * m + lane < W;
-      acc[m] = ok[m] ? __ldg(cnt + 32 * m) : 0u;
+      acc[m] = 0;
+    }
+#pragma unroll 4
+    for (int q = Q.summed ? seg : 0; q < seg + Q.summed; ++q) {
+      const uint32_t *cnt = Q.counts + ((size_t)q * Q.n_planes + p) * W + c0 + lane;
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        if (ok[m]) acc[m] += __ldg(cnt + 32 * m);
     }
     unsigned run = 0;
 #pragma unroll
@@ -821,10 +831,11 @@ int launch_integral_histogram(const uint8_t *bins, int W, int H, int n_bins, boo
   cudaFuncSetAttribute(k_hist_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)(sizeof(unsigned) * kHStrip * kMaxBins));
   k_hist_cols<<<dim3((unsigned)((W + kHStrip - 1) / kHStrip), (unsigned)Q.nseg), kHStrip, smem, s>>>(Q);
-  k_hist_mid<<<(unsigned)(((size_t)Q.n_planes * W + 127) / 128), 128, 0, s>>>(Q);
+  Q.summed = Q.nseg > kHDirect ? 1 : 0;
+  if (Q.summed) k_hist_mid<<<(unsigned)(((size_t)Q.n_planes * W + 127) / 128), 128, 0, s>>>(Q);
   auto *const write = cumulative ? k_hist_write<false> : k_hist_write<true>;
   write<<<(unsigned)(Q.nseg * Q.n_planes), 32 * kHW, W > kHCols ? 2 * sizeof(unsigned) * Q.seg_rows : 0, s>>>(Q);
-  return 3;
+  return 2 + Q.summed;
 }
 
 }  // namespace tmk
