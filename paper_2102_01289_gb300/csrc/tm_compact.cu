@@ -527,9 +527,10 @@ __global__ void __launch_bounds__(kLookCols, 7)
         const unsigned vl = ((ul >> 5) * (unsigned)K + k) * slots, vr = ((ur >> 5) * (unsigned)K + k) * slots;
         const BT *pl = vec + (size_t)vl * 32 + ol, *pr = vec + (size_t)vr * 32 + orr;
         // no vectors where no row is mixed between the two positions; checked
-        // where it pays: with 16-bit vectors at 12 MP 254 -> 249 us, with the
-        // pyramid's wide windows, which rarely skip, 433 -> 485
-        const bool check = sizeof(BT) == 2;
+        // where it pays: with 16-bit vectors at 12 MP 254 -> 249 us; with the
+        // pyramid's wide windows, which rarely skip, 433 -> 485, and where the
+        // moments are kept 16 MP 370 -> 395
+        const bool check = sizeof(BT) == 2 && kMode == kOut;
         e[i][0] = e[i][1] = e[i][2] = e[i][3] = 0;
         if (!check || (r[i][0].y ^ r[i][1].y) >> 16) {
           e[i][0] = __ldg(pl + (r[i][0].y >> 16) * 32);
