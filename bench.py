@@ -333,20 +333,26 @@ def run_ours(args):
     e2e_sync_s = max_over_ranks(time.perf_counter() - t0, world, dev)
 
     peak, peak_kind = load_peaks()
-    # on the fused path the integral images run beside the sweep, in the SMs
-    # its last segments leave idle: their stage time spans the sweep's tail and
-    # is not a kernel of its own, so the dominant kernel is taken among the others
-    own = {k: v for k, v in stages.items() if not (k == "integral_image" and "fused_sweep" in stages)}
+    hist_path = "fused" if "fused_sweep" in stages else "compact" if args.hist_path == "auto" else "materialised"
+    # the integral images run beside the sweep or the compact histogram's build
+    # (two launches): those stage times overlap and are not one kernel's, so
+    # the dominant kernel is taken among the others
+    beside = {"fused": ("integral_image",), "compact": ("integral_image", "integral_histogram")}.get(hist_path, ())
+    own = {k: v for k, v in stages.items() if k not in beside}
     dominant = max(own.items(), key=lambda kv: kv[1])[0] if own else None
     dom_ms = stages.get(dominant, 0.0) / args.steps if dominant else 0.0
     # the roofline of the dominant kernel takes the path's algorithmic bytes per
     # pixel times the pixels one launch processes, over that kernel's mean time
     bpp = PATH_BYTES_PER_PX
     achieved = bpp * npx / (dom_ms / 1e3) / 1e9 if dom_ms > 0 else None
-    traffic = load_traffic(dominant)
+    if dominant == "lookup" and hist_path == "compact":
+        dominant_profile = "lookup_compact"
+    else:
+        dominant_profile = dominant
+    traffic = load_traffic(dominant_profile)
     # the dominant kernel is limited by instruction issue, not HBM: its warp
     # instructions per launch (ncu) over the SMs' issue slots in its time
-    inst = load_profile(dominant, "warp_inst_per_launch")
+    inst = load_profile(dominant_profile, "warp_inst_per_launch")
     nsm = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = clk.get("sm_mhz") or None
     issue = None
@@ -361,7 +367,7 @@ def run_ours(args):
         "config": {"workload": wl["name"], "height": H, "width": W, "channels": 3, "input": "float32",
                    "n_bins": wl["n_bins"], "radii": wl["radii"], "parallelism": "replicas",
                    "l2": "inputs larger than L2 (two 144 MB images alternated)",
-                   "hist_path": "fused" if "fused_sweep" in stages else "materialised"},
+                   "hist_path": hist_path},
         "roofline": {"bound": "hbm", "kernel": dominant, "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": (achieved / peak) if achieved else None,
                      "traffic": traffic, "peak_kind": peak_kind,
@@ -606,7 +612,8 @@ def leg_paper_preset(args, dev, steps=None, warmup=None):
         "dtype": "f32",
         "config": {"workload": "wdr-12mp-paper-preset", "height": H, "width": W, "n_bins": 5,
                    "fields": [[int(params.rx[f]), int(params.ry[f])] for f in range(5)],
-                   "hist_path": "materialised" if "integral_histogram" in stages else "fused",
+                   "hist_path": "fused" if "fused_sweep" in stages
+                   else "compact" if args.hist_path == "auto" else "materialised",
                    "l2": "inputs larger than L2 (two 144 MB images alternated)",
                    "inputs": "rendered on the device (synth.wdr_device)"},
         "stages_ms_per_step": {k: v / steps for k, v in stages.items()},
@@ -666,7 +673,7 @@ def kernel_source_hash(kernel):
 
     import paper_2102_01289_gb300 as tm
 
-    srcs = {"fused_sweep": "tm_sweep.cu", "lookup": "tm_lookup.cu", "bwd_pixel": "tm_backward.cu",
+    srcs = {"fused_sweep": "tm_sweep.cu", "lookup": "tm_lookup.cu", "lookup_compact": "tm_compact.cu", "bwd_pixel": "tm_backward.cu",
             "bwd_input": "tm_backward.cu", "fix_stats": "tm_integral.cu", "fix_write": "tm_integral.cu",
             "integral_histogram": "tm_integral.cu", "integral_image": "tm_integral.cu",
             "prep": "tm_prepass.cu", "range": "tm_prepass.cu"}
