@@ -623,6 +623,23 @@ bool compact_fits(const tm_ctx *c, const tm_image *im) {
   return !c->no_compact && plan_compact(dev_params(c->p, 0), im->width, im->height, C) && compact_bytes(C) <= kCompactMax;
 }
 
+// Whether the images of a call are strips that the sweep takes faster than the
+// compact integral histogram, whose row pass is a chain along each row and
+// whose column pass, with at most 128 warps per 32 columns, one down each
+// column. One image, 64 bins, us, compact and sweep: 16384 x 64 (width x
+// height) 124 and 117, x 128 163 and 185, 4096 x 32 59 and 56; 32 x 4096 163
+// and 117, 256 x 16384 676 and 437, 37 x 60000 2141 and 1051. The images of a
+// batch share the SMs, and only wide ones stay behind (eight images, 32 bins:
+// 16384 x 16 261 and 212, x 64 477 and 557; 32 x 8192 377 and 862).
+bool strips(tm_ctx *c, int n, const tm_image *im) {
+  for (int i = 0; i < n; ++i) {
+    const long long W = im[i].width, H = im[i].height;
+    const bool strip = n > 1 ? W >= 256 * H : W > 128 * H || (H > 32 * W && H >= 4096);
+    if (!strip || !sweep_fits(c, &im[i])) return false;
+  }
+  return true;
+}
+
 // The batched path over images that share it: one launch per stage for the
 // whole batch. path: kPathSweep, the sweep as a persistent kernel over a queue
 // of (image, strip, row band) tiles (TM_EUNSUPPORTED if some image cannot be
@@ -1160,7 +1177,7 @@ tm_status forward_device(tm_ctx *c, const tm_image *in, const tm_image *out, cud
   ++c->calls;
   int path = c->hist_path;
   if (c->p.n_bins < 2) path = kPathMaterialised;  // no thresholds: nothing to count
-  if (path == 0 && compact_fits(c, in)) {
+  if (path == 0 && compact_fits(c, in) && !strips(c, 1, in)) {
     const bool graph = !c->stage_timing && !c->debug && !c->reuse_range && single_graph_ok(c, in, out, kPathCompact);
     st = forward_fused(c, 1, in, out, s, graph, kPathCompact);
     if (st != TM_ENOMEM) return st;
@@ -1284,7 +1301,7 @@ tm_status backward_images(tm_ctx *c, int n, const tm_image *in, const tm_image *
   std::vector<Job> jobs;
   int64_t launches = 0;
   // the backward takes the fields that the sweep fits, whatever path counts
-  bool compact = c->hist_path == 0;
+  bool compact = c->hist_path == 0 && !strips(c, n, in);
   for (int i = 0; i < n; ++i) {
     if (!sweep_fits(c, &in[i])) return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit these fields");
     compact = compact && compact_fits(c, &in[i]);
@@ -1449,7 +1466,7 @@ tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *ou
   tm_status s = ensure_device_info(c);
   if (s) return s;
   std::vector<tm_image> fin, fout, min_, mout;
-  bool compact = c->hist_path == 0;
+  bool compact = c->hist_path == 0 && !strips(c, n, in);
   for (int i = 0; i < n; ++i) {
     bool fused = c->p.n_bins > 1 && c->hist_path != 2;
     if (fused && !sweep_fits(c, &in[i])) {

@@ -139,3 +139,32 @@ def test_batch_of_16_and_32_bit_vectors():
             assert torch.equal(y, z)
     finally:
         tm.tm_destroy(ctx)
+
+
+# both sides of the rule that takes strips to the sweep: one image, and two
+@pytest.mark.parametrize("H,W,count", [
+    (8, 1024, 1), (8, 1025, 1), (4096, 128, 1), (4097, 128, 1), (4095, 20, 1), (4, 1023, 2), (4, 1024, 2),
+])
+def test_strips_equal_the_materialised_path(H, W, count):
+    p = tm.make_params(33, [2, (40, 3)])
+    xs = [torch.from_numpy(_image(H, W, 7 + k, "scene")).cuda() for k in range(count)]
+    gs = [torch.ones_like(x) for x in xs]
+    got = {}
+    for path in (0, 1, 2):
+        ys, gin = [torch.empty_like(x) for x in xs], [torch.empty_like(x) for x in xs]
+        ctx = tm.tm_create(p)
+        try:
+            tm.tm_set_option(ctx, tm.TM_OPT_HIST_PATH, path)
+            if count == 1:
+                tm.tm_forward(ctx, xs[0], ys[0])
+            else:
+                tm.tm_forward_batch(ctx, xs, ys)
+            if path != 2:  # the backward refuses the materialised path
+                tm.tm_backward_batch(ctx, xs, gs, gin, torch.empty(7, device="cuda"))
+            torch.cuda.synchronize()
+            got[path] = ys, gin
+        finally:
+            tm.tm_destroy(ctx)
+    for k in range(count):
+        assert torch.equal(got[0][0][k], got[2][0][k])
+        assert torch.equal(got[0][1][k], got[1][1][k])
