@@ -460,13 +460,15 @@ def leg_batch(args, dev, kind, steps=None, warmup=None):
     for _ in range(warmup):
         tm.tm_forward_batch(ctx, xs, ys, stream)
     launches = tm.tm_last_launch_count(ctx)
-    # which batched pass(es) the images took: the fused sweep and/or the
-    # materialised integral histogram (the per-size choice the library made)
+    # which batched pass(es) the images took: the compact integral histogram
+    # (automatic path), the fused sweep and/or the materialised one
     tm.tm_set_option(ctx, tm.TM_OPT_STAGE_TIMING, 1)
     tm.tm_stage_times(ctx)
     tm.tm_forward_batch(ctx, xs, ys, stream)
-    passes = sorted({"batch": "fused", "batch_materialised": "materialised"}[k]
-                    for k in tm.tm_stage_times(ctx) if k in ("batch", "batch_materialised"))
+    names = {"batch": "fused", "batch_materialised": "materialised"}
+    if args.hist_path == "auto":
+        names = dict.fromkeys(names, "compact")
+    passes = sorted({names[k] for k in tm.tm_stage_times(ctx) if k in names})
     tm.tm_set_option(ctx, tm.TM_OPT_STAGE_TIMING, 0)
     clocks.start()
     time.sleep(0.3)
@@ -694,7 +696,7 @@ def main():
     ap.add_argument("--no-legs", action="store_true",
                     help="skip the other legs of the metric (fwd+bwd, batches, paper preset)")
     ap.add_argument("--hist-path", choices=sorted(HIST_PATHS), default="auto",
-                    help="histogram path: auto (the library measures both once), fused or materialised")
+                    help="histogram path: auto (compact), fused or materialised")
     ap.add_argument("--ref-seconds", type=float, default=0.0,
                     help="oracle sample per step of the reference arm (default: sized so the run takes ~1 min)")
     ap.add_argument("--workload", default="fwd-12mp",
