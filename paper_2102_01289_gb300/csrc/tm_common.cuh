@@ -386,17 +386,26 @@ __device__ __forceinline__ long long float_to_i64_rn(float y) {
 // 2^10 / N + 4 of it; then |d| <= 4.5 N + 2^10 < 2^31. The float error of
 // T - d^2 / N grows to about 2^-24 (var + (m - mean)^2) unit^2, at most
 // 2^-4 unit^2 (one-pixel windows), below the quantisation step.
+// Other windows of a launch without the literal area (kSmall = 0) give the
+// same bits as the 64-bit conversions. N < 2^31 and N 2^(2Q-2) < 2^63, so
+// Q >= 17 and |s1| <= N 2^(Q-1) < 2^48: its upper part and its lower 24 bits
+// are exact floats, and one fused multiply-add rounds their sum. The estimate
+// of the mean is within 2.5 x 2^(Q-24) + 0.5 of it, so |d| < 2^31. (12 MP, the
+// five fields of the pyramid: the FP64 pipe 68 % busy with all three.)
 template <int kSmall = -1>
 __device__ __forceinline__ float window_variance(long long s1, long long s2, unsigned long long N,
                                                  float rN, float inv_scale2, bool small = false) {
   const bool sm = kSmall >= 0 ? kSmall != 0 : small;
   // |mean| <= 2^(Q-1) <= 2^23: the nearest integer fits 32 bits
   const int m = sm ? __float2int_rn(__int2float_rn((int)(s1 >> 10)) * (rN * 1024.f))
-                   : __float2int_rn(__ll2float_rn(s1) * rN);
+                   : __float2int_rn((kSmall == 0 ? fmaf(__int2float_rn((int)(s1 >> 24)), 16777216.f,
+                                                        __uint2float_rn((unsigned)s1 & 0xffffffu))
+                                                 : __ll2float_rn(s1)) * rN);
   // small: |d| < 2^31, so 32 bits hold it
-  const long long d = sm ? (long long)(int)((unsigned)s1 - (unsigned)m * (unsigned)N) : s1 - (long long)m * (long long)N;
+  const bool d32 = sm || kSmall == 0;
+  const long long d = d32 ? (long long)(int)((unsigned)s1 - (unsigned)m * (unsigned)N) : s1 - (long long)m * (long long)N;
   const unsigned long long T = (unsigned long long)s2 - (unsigned long long)((long long)m * (s1 + d));
-  const float df = sm ? __int2float_rn((int)d) : __ll2float_rn(d);
+  const float df = d32 ? __int2float_rn((int)d) : __ll2float_rn(d);
   const float v = fmaf(-df * rN, df, __ull2float_rn(T)) * rN;
   return fmaxf(v, 0.f) * inv_scale2;
 }

@@ -697,11 +697,11 @@ int launch_lookup_compact(const DevParams &P, const Job *jobs, int njobs, int bl
   } else if (keep) {
     launch_look<uint16_t, true, 1, kF32, kOutKeep>(P, L, blocks, s);
   } else if (wide) {
-    launch_look_dtype<uint32_t, -1>(P, L, blocks, dtype, s);
-  } else if (P.small_win) {
-    launch_look_dtype<uint16_t, 1>(P, L, blocks, dtype, s);
+    if (P.small_win) launch_look_dtype<uint32_t, 1>(P, L, blocks, dtype, s);
+    else launch_look_dtype<uint32_t, 0>(P, L, blocks, dtype, s);
   } else {
-    launch_look_dtype<uint16_t, -1>(P, L, blocks, dtype, s);
+    if (P.small_win) launch_look_dtype<uint16_t, 1>(P, L, blocks, dtype, s);
+    else launch_look_dtype<uint16_t, 0>(P, L, blocks, dtype, s);
   }
   return 1;
 }

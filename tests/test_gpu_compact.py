@@ -168,3 +168,25 @@ def test_strips_equal_the_materialised_path(H, W, count):
     for k in range(count):
         assert torch.equal(got[0][0][k], got[2][0][k])
         assert torch.equal(got[0][1][k], got[1][1][k])
+
+
+# the largest sums of a launch without small windows: windows of the whole
+# image, the luminance at both ends of the range, uneven halves
+@pytest.mark.parametrize("H,W,cut", [(513, 700, 350), (3000, 4000, 4000), (3000, 4000, 7), (3001, 3999, 2500)])
+def test_large_windows_equal_the_materialised_path(H, W, cut):
+    x = synth.wdr_device(H, W, seed=9, device="cuda")
+    x[:, :cut] = 1e-3
+    x[-1, -1] = 1e4
+    p = tm.make_params(6, [(W, H), (W // 2, H // 2), (W // 4, 60), 9])
+    got = []
+    for path in (0, 2):
+        y = torch.empty_like(x)
+        ctx = tm.tm_create(p)
+        try:
+            tm.tm_set_option(ctx, tm.TM_OPT_HIST_PATH, path)
+            tm.tm_forward(ctx, x, y)
+            torch.cuda.synchronize()
+            got.append(y)
+        finally:
+            tm.tm_destroy(ctx)
+    assert torch.equal(got[0], got[1])
