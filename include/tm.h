@@ -182,7 +182,7 @@ tm_status tm_forward_host_async(tm_ctx *ctx, const tm_image *in_host,
 
 /* Forward over n images of possibly different sizes. With the automatic
  * histogram path a batch whose images all fit the compact integral histogram
- * runs on it as one batched pass: the range, bin and integral-image stages
+ * (and are not all wide strips, see TM_OPT_HIST_PATH) runs on it as one batched pass: the range, bin and integral-image stages
  * once for all of them, then the histograms and lookups of a group of images
  * at a time (32 images, 8 GiB). Otherwise, images whose fields do not fit the
  * fused sweep take the materialised integral histogram; the others take
@@ -327,8 +327,11 @@ tm_status tm_debug_export(tm_ctx *ctx, int32_t what, void *dst, size_t bytes,
  *                        32-column chunk instead of per column) for images
  *                        of at least two bins, at most 65535 columns and
  *                        rows and under 24 GiB of it (0.4 GB for 12 MP with
- *                        16 bins, 1.8 GB with 64). For others, and once its
- *                        memory could not be had, the first single-image
+ *                        16 bins, 1.8 GB with 64). For others, for strips
+ *                        that the sweep takes faster (one image: width > 128
+ *                        heights, or height > 32 widths from 4096 rows; more:
+ *                        every width >= 256 heights), and once its memory
+ *                        could not be had, the first single-image
  *                        forward of each (width, height, input dtype, output
  *                        dtype) on a context runs paths 1 and 2 twice, timing
  *                        the second runs (it synchronises its stream once),

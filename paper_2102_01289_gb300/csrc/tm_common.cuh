@@ -391,7 +391,8 @@ __device__ __forceinline__ long long float_to_i64_rn(float y) {
 // Q >= 17 and |s1| <= N 2^(Q-1) < 2^48: its upper part and its lower 24 bits
 // are exact floats, and one fused multiply-add rounds their sum. The estimate
 // of the mean is within 2.5 x 2^(Q-24) + 0.5 of it, so |d| < 2^31. (12 MP, the
-// five fields of the pyramid: the FP64 pipe 68 % busy with all three.)
+// five fields of the pyramid: the FP64 pipe 68 % busy with all three, the
+// lookup 432 us; 403 so; 410 with T normalised by hand as well.)
 template <int kSmall = -1>
 __device__ __forceinline__ float window_variance(long long s1, long long s2, unsigned long long N,
                                                  float rN, float inv_scale2, bool small = false) {
