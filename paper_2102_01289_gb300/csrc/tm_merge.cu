@@ -195,7 +195,9 @@ extern "C" tm_status tm_merge_exposures(int32_t n, const uint8_t *const *ldr, co
   }
   const size_t align = out->dtype == TM_F32 ? 16 : 8, es = out->dtype == TM_F32 ? 4 : 2;
   bool vec = (o.H == 1 || (pitch % 4 == 0 && ((size_t)out->pitch * es) % align == 0)) && (uintptr_t)o.p % align == 0;
-  for (int j = 0; j < n; ++j) vec = vec && (uintptr_t)ldr[j] % 4 == 0;
+  // (an infinite exposure time makes sums infinite: the corrected quotient of
+  // the vector form would turn their limit, E = 0, into NaN)
+  for (int j = 0; j < n; ++j) vec = vec && (uintptr_t)ldr[j] % 4 == 0 && std::isfinite(a.neg_log_t[j]);
   for (const auto &ch : a.g)
     for (const float v : ch) vec = vec && std::fabs(v) < 1e30f;
   a.vec = vec ? 1 : 0;
