@@ -215,7 +215,10 @@ extern "C" tm_status tm_merge_exposures(int32_t n, const uint8_t *const *ldr, co
     TM_MERGE(2) TM_MERGE(3) TM_MERGE(4)
 #undef TM_MERGE
     default:
-      if (cudaFuncSetAttribute(k_merge<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      // the kernel's limit is shared by every thread of the process: always
+      // the largest, so that no call lowers it under another's launch
+      if (cudaFuncSetAttribute(k_merge<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)(sizeof(float2) * 768 * kMaxExposures)) != cudaSuccess)
         return fail_noctx(TM_ECUDA, "tm_merge_exposures: shared-memory attribute");
       k_merge<0><<<blocks, kMT, smem, st>>>(a, o);
   }
