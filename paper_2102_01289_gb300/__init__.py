@@ -385,7 +385,7 @@ class _CtxCache:
         self.ctxs = {}
 
     def get(self, t):
-        key = tuple([round(x, 9) for x in t.detach().cpu().reshape(-1).tolist()])
+        key = t.detach().cpu().float().reshape(-1).numpy().tobytes()  # the context's own 32-bit values
         if key not in self.ctxs:
             c = tm_create(params_from_tensor(self.template, t))
             # the autograd function keeps its input saved and unchanged between
