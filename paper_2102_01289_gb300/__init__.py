@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 from typing import Optional, Sequence
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -377,27 +378,52 @@ def params_from_tensor(template: TmParams, t) -> TmParams:
     return p
 
 
+class _Ctx(ctypes.c_void_p):
+    """A tm_ctx that is destroyed with its last reference (or by close)."""
+
+    def close(self):
+        h, self.value = self.value, None
+        if h:
+            tm_destroy(ctypes.c_void_p(h))
+
+    def __del__(self):
+        try:
+            self.close()
+        except Exception:
+            pass
+
+
 class _CtxCache:
-    """tm_ctx per distinct parameter values (the C context copies them)."""
+    """tm_ctx per distinct parameter values (the C context copies them), the
+    `limit` most recently used ones: a program that trains the parameters comes
+    with new values at every step, and each context holds its workspaces. A
+    context in use elsewhere lives until that reference goes."""
+
+    limit = 8
 
     def __init__(self, template: TmParams):
         self.template = template
-        self.ctxs = {}
+        self.ctxs = {}  # least recently used first
+        self._lock = threading.Lock()
 
     def get(self, t):
         key = t.detach().cpu().float().reshape(-1).numpy().tobytes()  # the context's own 32-bit values
-        if key not in self.ctxs:
-            c = tm_create(params_from_tensor(self.template, t))
-            # the autograd function keeps its input saved and unchanged between
-            # forward and backward, so the backward may take the forward's
-            # intermediates from the context (it checks they are that input's)
-            tm_set_option(c, TM_OPT_BACKWARD_REUSE, 1)
+        with self._lock:
+            c = self.ctxs.pop(key, None)
+            if c is None:
+                c = _Ctx(tm_create(params_from_tensor(self.template, t)).value)
+                # the autograd function keeps its input saved and unchanged between
+                # forward and backward, so the backward may take the forward's
+                # intermediates from the context (it checks they are that input's)
+                tm_set_option(c, TM_OPT_BACKWARD_REUSE, 1)
             self.ctxs[key] = c
-        return self.ctxs[key]
+            old = self.ctxs.pop(next(iter(self.ctxs))) if len(self.ctxs) > self.limit else None
+        del old  # (destroyed outside the lock)
+        return c
 
     def close(self):
         for c in self.ctxs.values():
-            tm_destroy(c)
+            c.close()
         self.ctxs.clear()
 
     def __del__(self):

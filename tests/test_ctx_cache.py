@@ -1,4 +1,6 @@
 """The contexts that the autograd function keeps per parameter vector."""
+import threading
+
 import pytest
 
 import paper_2102_01289_gb300 as tm
@@ -32,6 +34,59 @@ def test_a_context_per_distinct_value():
         assert cache.get(_theta(p, i2=0.6)).value != cache.get(_theta(p, i2=0.6 + 2.0 ** -24)).value
     finally:
         cache.close()
+
+
+def test_contexts_are_bounded(monkeypatch):
+    """Parameters that change at every step leave `limit` contexts, the most
+    recently used; the others are destroyed, one still referenced elsewhere
+    with its last reference, and close destroys the rest."""
+    destroyed = []
+    real = tm.tm_destroy
+
+    def record(ctx):
+        destroyed.append(ctx.value)
+        real(ctx)
+
+    monkeypatch.setattr(tm, "tm_destroy", record)
+    p = tm.make_params(8, [2, 5])
+    cache = tm._CtxCache(p)
+    first = cache.get(_theta(p, i2=0.5))
+    handle = first.value
+    held = cache.get(_theta(p, i2=0.25))
+    for k in range(3 * cache.limit):
+        cache.get(_theta(p, i3=0.1 + k))
+        assert cache.get(_theta(p, i2=0.5)).value == handle  # used again: stays
+        assert len(cache.ctxs) <= cache.limit
+    assert len(destroyed) == 2 * cache.limit + 1 and handle not in destroyed and held.value not in destroyed
+    old = held.value
+    del held
+    assert destroyed[-1] == old
+    cache.close()
+    assert handle in destroyed and first.value is None and not cache.ctxs
+    del first
+    assert len(destroyed) == 3 * cache.limit + 2  # each context once
+
+
+def test_threads_get_their_own_contexts():
+    """Threads with parameters of their own, more of them than the cache keeps:
+    each context holds the values it was asked for while it is in use."""
+    p = tm.make_params(8, [2, 5])
+    cache = tm._CtxCache(p)
+    bad = []
+
+    def work(k):
+        for i in range(50):
+            c = cache.get(_theta(p, i3=0.1 * (k + 1)))
+            if not c.value or tm.lib().tm_last_launch_count(c) != 0:
+                bad.append(k)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2 * cache.limit)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    cache.close()
+    assert not bad
 
 
 @pytest.mark.gpu
