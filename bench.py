@@ -333,11 +333,11 @@ def run_ours(args):
     e2e_sync_s = max_over_ranks(time.perf_counter() - t0, world, dev)
 
     peak, peak_kind = load_peaks()
-    hist_path = "fused" if "fused_sweep" in stages else "compact" if args.hist_path == "auto" else "materialised"
+    hist_path = path_of(stages)
     # the integral images run beside the sweep or the compact histogram's build
     # (two launches): those stage times overlap and are not one kernel's, so
     # the dominant kernel is taken among the others
-    beside = {"fused": ("integral_image",), "compact": ("integral_image", "integral_histogram")}.get(hist_path, ())
+    beside = {"fused": ("integral_image",), "compact": ("integral_image", "compact_histogram")}.get(hist_path, ())
     own = {k: v for k, v in stages.items() if k not in beside}
     dominant = max(own.items(), key=lambda kv: kv[1])[0] if own else None
     dom_ms = stages.get(dominant, 0.0) / args.steps if dominant else 0.0
@@ -460,15 +460,12 @@ def leg_batch(args, dev, kind, steps=None, warmup=None):
     for _ in range(warmup):
         tm.tm_forward_batch(ctx, xs, ys, stream)
     launches = tm.tm_last_launch_count(ctx)
-    # which batched pass(es) the images took: the compact integral histogram
-    # (automatic path), the fused sweep and/or the materialised one
+    # which batched pass(es) the images took: the compact integral histogram,
+    # the fused sweep and/or the materialised one
     tm.tm_set_option(ctx, tm.TM_OPT_STAGE_TIMING, 1)
     tm.tm_stage_times(ctx)
     tm.tm_forward_batch(ctx, xs, ys, stream)
-    names = {"batch": "fused", "batch_materialised": "materialised"}
-    if args.hist_path == "auto":
-        names = dict.fromkeys(names, "compact")
-    passes = sorted({names[k] for k in tm.tm_stage_times(ctx) if k in names})
+    passes = batch_passes(tm.tm_stage_times(ctx))
     tm.tm_set_option(ctx, tm.TM_OPT_STAGE_TIMING, 0)
     clocks.start()
     time.sleep(0.3)
@@ -614,8 +611,7 @@ def leg_paper_preset(args, dev, steps=None, warmup=None):
         "dtype": "f32",
         "config": {"workload": "wdr-12mp-paper-preset", "height": H, "width": W, "n_bins": 5,
                    "fields": [[int(params.rx[f]), int(params.ry[f])] for f in range(5)],
-                   "hist_path": "fused" if "fused_sweep" in stages
-                   else "compact" if args.hist_path == "auto" else "materialised",
+                   "hist_path": path_of(stages),
                    "l2": "inputs larger than L2 (two 144 MB images alternated)",
                    "inputs": "rendered on the device (synth.wdr_device)"},
         "stages_ms_per_step": {k: v / steps for k, v in stages.items()},
@@ -668,6 +664,18 @@ def load_traffic(kernel):
 
 
 HIST_PATHS = {"auto": 0, "fused": 1, "materialised": 2}
+
+
+def path_of(stages):
+    """The histogram path of single-image forwards, from the stages they reported."""
+    return "fused" if "fused_sweep" in stages else "compact" if "compact_histogram" in stages else "materialised"
+
+
+def batch_passes(stages):
+    """The pass(es) one batched forward took, from the stages it reported."""
+    if "batch_compact" in stages:
+        return ["compact"]
+    return [v for k, v in (("batch", "fused"), ("batch_materialised", "materialised")) if k in stages]
 
 
 def kernel_source_hash(kernel):

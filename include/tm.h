@@ -391,8 +391,15 @@ tm_status tm_set_option(tm_ctx *ctx, int32_t key, int64_t value);
 
 /* Per-stage device time, summed over every call since the previous read,
  * with stage timing on. Writes up to `cap` entries: ms[i] milliseconds and
- * names[i] a static stage name. Synchronises with the last recorded event
- * and resets the sums. Returns the number of stages written, or -1 on error
+ * names[i] a static stage name. A single image and a backward report what
+ * they run: "range", "prep", "integral_image", then "fused_sweep" (the sweep),
+ * "integral_histogram" (whole planes) or "compact_histogram" (the build of the
+ * compact integral histogram), and "lookup"; "bwd_pixel", "bwd_adjoint",
+ * "bwd_input". A batch reports its passes: "batch" on the fused sweep, and
+ * "batch_materialised" on a stored integral histogram, whole planes or
+ * compact; "batch_compact" is the part of the latter on the compact one (so
+ * its time is in both). Synchronises with the last recorded event and resets
+ * the sums. Returns the number of stages written, or -1 on error
  * (message in tm_last_error). */
 int32_t tm_stage_times(tm_ctx *ctx, float *ms, const char **names, int32_t cap);
 

@@ -253,10 +253,11 @@ tm_status validate_params(const tm_params *p, std::string &why) {
 }
 
 enum Stage { ST_RANGE, ST_PREP, ST_INTEGRAL, ST_HIST, ST_LOOKUP, ST_SWEEP, ST_BATCH,
-             ST_BWD_PIXEL, ST_BWD_ADJOINT, ST_BWD_INPUT, ST_BATCH_MAT, ST_COUNT };
+             ST_BWD_PIXEL, ST_BWD_ADJOINT, ST_BWD_INPUT, ST_BATCH_MAT, ST_COMPACT, ST_BATCH_COMPACT, ST_COUNT };
 const char *const kStageNames[ST_COUNT] = {"range", "prep", "integral_image", "integral_histogram",
                                           "lookup", "fused_sweep", "batch", "bwd_pixel",
-                                          "bwd_adjoint", "bwd_input", "batch_materialised"};
+                                          "bwd_adjoint", "bwd_input", "batch_materialised",
+                                          "compact_histogram", "batch_compact"};
 
 // Record a stage boundary on stream s (stage < 0 opens a new call).
 // Record a stage boundary on stream s (stage -1 opens a new call; kNoStage
@@ -900,7 +901,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   };
   int ls = compact ? build(0, c->sweep_stream)
                    : launch_sweep(P, dj, nimg, nitems, queue, smem, ctas, width, c->sweep_stream);
-  if (!graph) mark(c, c->sweep_stream, compact ? ST_HIST : ST_SWEEP, m_prep);
+  if (!graph) mark(c, c->sweep_stream, compact ? ST_COMPACT : ST_SWEEP, m_prep);
   n += std::max(ls, 0) + launch_integral_jobs(dj, nimg, b_rows, b_cols, c->int_stream);
   if (!graph) mark(c, c->int_stream, ST_INTEGRAL, m_prep);
   n += run_range ? 2 : 1;
@@ -1456,9 +1457,8 @@ tm_status choose_batch_path(tm_ctx *c, int n, const tm_image *in, const tm_image
 }
 
 // tm_forward_batch on validated arguments, n >= 1. With TM_OPT_HIST_PATH = 0
-// the batch runs on the compact integral histogram as one pass (stage "batch",
-// or "batch_materialised" if some image's fields are too wide for the sweep)
-// where every image fits it. Otherwise images whose fields do not fit the
+// the batch runs on the compact integral histogram as one pass (stages
+// "batch_materialised" and "batch_compact") where every image fits it. Otherwise images whose fields do not fit the
 // sweep take the materialised path, and the others the path measured faster
 // for this batch (cached per context by the images' sizes and dtype pairs),
 // each path's images as one batched pass. Every pass is captured in a graph.
@@ -1481,9 +1481,12 @@ tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *ou
   if ((s = ensure_stats(c, n))) return s;
   if (compact) {
     ++c->calls;
-    mark(c, st, -1);
+    const int m0 = mark(c, st, -1);
     s = forward_fused(c, n, in, out, st, true, kPathCompact);
-    if (!s) mark(c, st, min_.empty() ? ST_BATCH : ST_BATCH_MAT);
+    if (!s) {  // a stored histogram, and the compact one: both names from the call's start
+      mark(c, st, ST_BATCH_MAT, m0);
+      mark(c, st, ST_BATCH_COMPACT, m0);
+    }
     if (s != TM_ENOMEM) return s;
     c->no_compact = true;  // the other paths need less memory
   }

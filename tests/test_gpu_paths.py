@@ -1,0 +1,113 @@
+"""Which histogram path a forward takes, as its stages say, and the batched
+passes that the automatic path no longer takes by itself."""
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2102_01289_gb300 as tm  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    tm.build()
+
+
+def _stages(ctx, call):
+    """The stages that `call` reports."""
+    tm.tm_set_option(ctx, tm.TM_OPT_STAGE_TIMING, 1)
+    tm.tm_stage_times(ctx)
+    call()
+    names = set(tm.tm_stage_times(ctx))
+    tm.tm_set_option(ctx, tm.TM_OPT_STAGE_TIMING, 0)
+    return names
+
+
+def _forward(x, p, path):
+    y = torch.empty_like(x)
+    ctx = tm.tm_create(p)
+    try:
+        tm.tm_set_option(ctx, tm.TM_OPT_HIST_PATH, path)
+        tm.tm_forward(ctx, x, y)
+        torch.cuda.synchronize()
+    finally:
+        tm.tm_destroy(ctx)
+    return y
+
+
+def _images(sizes, seed):
+    return [synth.wdr_device(h, w, seed=seed + i, device="cuda") for i, (w, h) in enumerate(sizes)]
+
+
+def test_stage_names_say_the_path():
+    """One image, and batches with and without an image whose fields are too
+    wide for the sweep: the names tell the compact histogram from the others."""
+    p = tm.make_params(16, [4, (700, 600)])
+    wide, small = _images([(1600, 1200), (300, 200)], 1)
+    for path, single, batch in ((0, "compact_histogram", "batch_compact"), (2, "integral_histogram", None),
+                                (1, "fused_sweep", None)):
+        ctx = tm.tm_create(p)
+        try:
+            tm.tm_set_option(ctx, tm.TM_OPT_HIST_PATH, path)
+            names = _stages(ctx, lambda: tm.tm_forward(ctx, small, torch.empty_like(small)))
+            assert names & {"compact_histogram", "integral_histogram", "fused_sweep"} == {single}
+            for xs in ([small, small.clone()], [small, wide]):
+                if path == 1 and wide is xs[1]:
+                    continue  # refused
+                ys = [torch.empty_like(x) for x in xs]
+                names = _stages(ctx, lambda: tm.tm_forward_batch(ctx, xs, ys))
+                if path == 1:
+                    assert names == {"batch"}
+                else:
+                    assert names == {"batch_materialised"} | ({batch} if batch else set())
+        finally:
+            tm.tm_destroy(ctx)
+
+
+def test_uneven_batch_on_the_materialised_path():
+    """The paper's preset over uneven sizes with the materialised path asked
+    for: one batched pass, captured and then replayed, each output that of the
+    image's own call."""
+    p = tm.tm_params_pyramid(2000, 1500, 5, 5)
+    xs = _images([(2000, 1500), (1024, 768), (640, 480), (97, 61)], 300)
+    refs = [_forward(x, p, 2) for x in xs]
+    ys = [torch.empty_like(x) for x in xs]
+    ctx = tm.tm_create(p)
+    try:
+        tm.tm_set_option(ctx, tm.TM_OPT_HIST_PATH, 2)
+        for _ in range(3):
+            for y in ys:
+                y.zero_()
+            assert _stages(ctx, lambda: tm.tm_forward_batch(ctx, xs, ys)) == {"batch_materialised"}
+            torch.cuda.synchronize()
+            for y, r in zip(ys, refs):
+                assert torch.equal(y, r)
+    finally:
+        tm.tm_destroy(ctx)
+
+
+def test_batch_splits_over_two_passes():
+    """A batch that the compact histogram refuses (an image of 66000 rows) with
+    one image whose fields are too wide for the sweep: the automatic path runs
+    a sweep pass and a materialised pass, each image equal to its own call."""
+    p = tm.make_params(64, [4, (700, 600)])
+    xs = _images([(1600, 1200), (300, 1900), (3, 66000), (900, 1500), (1400, 1000)], 400)
+    refs = [_forward(x, p, 2) for x in xs]
+    ys = [torch.empty_like(x) for x in xs]
+    ctx = tm.tm_create(p)
+    try:
+        for _ in range(3):
+            for y in ys:
+                y.zero_()
+            names = _stages(ctx, lambda: tm.tm_forward_batch(ctx, xs, ys))
+            torch.cuda.synchronize()
+            assert {"batch", "batch_materialised"} <= names and "batch_compact" not in names, names
+            for y, r in zip(ys, refs):
+                assert torch.equal(y, r)
+    finally:
+        tm.tm_destroy(ctx)
