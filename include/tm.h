@@ -330,9 +330,11 @@ tm_status tm_debug_export(tm_ctx *ctx, int32_t what, void *dst, size_t bytes,
  *                        16 bins, 1.8 GB with 64). For others, for strips
  *                        that the sweep takes faster (one image: width > 128
  *                        heights, or height > 32 widths from 4096 rows; more:
- *                        every width >= 256 heights), and once its memory
- *                        could not be had, the first single-image
- *                        forward of each (width, height, input dtype, output
+ *                        every width >= 256 heights), and where its memory
+ *                        could not be had (that much or more: not tried
+ *                        again for 256 calls, or until this option is set;
+ *                        a batch is first tried one image at a time), the
+ *                        first single-image forward of each (width, height, input dtype, output
  *                        dtype) on a context runs paths 1 and 2 twice, timing
  *                        the second runs (it synchronises its stream once),
  *                        and keeps the faster. All paths give the same

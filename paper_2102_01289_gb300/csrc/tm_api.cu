@@ -72,7 +72,10 @@ struct tm_ctx {
   int hist_path = 0;
   int sweep_tiles = 0;  // TM_OPT_SWEEP_TILES (0: one wave of the sweep's CTAs per image share)
   int sweep_width = 0;  // TM_OPT_SWEEP_WIDTH (0: automatic)
-  bool no_compact = false;  // the compact integral histogram's memory could not be had
+  // the compact integral histogram's bytes that could not be had, at which call
+  // (a smaller request is tried, and any after kCompactRetry calls)
+  size_t compact_failed = SIZE_MAX;
+  uint64_t compact_failed_at = 0;
   int64_t launches = 0;
   int num_sms = 0;
   size_t smem_optin = 0;
@@ -617,11 +620,59 @@ bool sweep_fits(tm_ctx *c, const tm_image *in) {
                     std::min(c->smem_optin - 2048, (size_t)110 * 1024), 256, plan);
 }
 
-// Whether the compact integral histogram takes image `im` under the context's
-// fields and bins.
-bool compact_fits(const tm_ctx *c, const tm_image *im) {
-  CompactPlan C;
-  return !c->no_compact && plan_compact(dev_params(c->p, 0), im->width, im->height, C) && compact_bytes(C) <= kCompactMax;
+// A request that failed is tried again after this many forward calls: the
+// shortage may have passed (a failing one costs the workspace's reallocation).
+constexpr uint64_t kCompactRetry = 256;
+
+// How the compact integral histograms of a call's images are held: images are
+// grouped up to `limit` bytes (or one image), the largest group takes `bytes`.
+struct CompactLayout {
+  std::vector<CompactPlan> plans;  // per image, with the vector width of the call
+  bool wide = false;               // 32-bit vectors for every image if one needs them
+  std::vector<int> first;          // the groups' first images
+  std::vector<size_t> offs;        // per image, its offset in the groups' buffer
+  size_t bytes = 0;
+};
+
+bool compact_layout(const tm_ctx *c, int n, const tm_image *in, size_t limit, CompactLayout &L) {
+  const DevParams P = dev_params(c->p, 0);
+  L = CompactLayout{};
+  L.plans.resize((size_t)n);
+  L.offs.resize((size_t)n);
+  for (int i = 0; i < n; ++i) {
+    if (!plan_compact(P, in[i].width, in[i].height, L.plans[(size_t)i])) return false;
+    L.wide = L.wide || L.plans[(size_t)i].wide;
+  }
+  size_t used = 0;
+  for (int i = 0; i < n; ++i) {
+    CompactPlan &C = L.plans[(size_t)i];
+    if (L.wide && !C.wide) C.vec_bytes *= 2;
+    const size_t b = compact_bytes(C);
+    if (b > kCompactMax) return false;
+    if (L.first.empty() || used + b > limit || i - L.first.back() >= kCompactImages) {
+      L.first.push_back(i);
+      used = 0;
+    }
+    L.offs[(size_t)i] = used;
+    used += b;
+    L.bytes = std::max(L.bytes, used);
+  }
+  return true;
+}
+
+// Whether the compact integral histogram takes a call's images under the
+// context's fields, bins and memory; L: in groups of up to kCompactGroup bytes,
+// or of one image where such a group's memory could not be had.
+bool compact_fits(const tm_ctx *c, int n, const tm_image *in, CompactLayout &L) {
+  const bool failed = c->calls - c->compact_failed_at < kCompactRetry;
+  const size_t most = failed ? c->compact_failed : SIZE_MAX;
+  return compact_layout(c, n, in, kCompactGroup, L) &&
+         (L.bytes < most || (n > 1 && compact_layout(c, n, in, 0, L) && L.bytes < most));
+}
+
+void compact_nomem(tm_ctx *c, const CompactLayout &L) {
+  c->compact_failed = L.bytes;
+  c->compact_failed_at = c->calls;
 }
 
 // Whether the images of a call are strips that the sweep takes faster than the
@@ -642,18 +693,20 @@ bool strips(tm_ctx *c, int n, const tm_image *im) {
 }
 
 // The batched path over images that share it: one launch per stage for the
-// whole batch. path: kPathSweep, the sweep as a persistent kernel over a queue
-// of (image, strip, row band) tiles (TM_EUNSUPPORTED if some image cannot be
-// swept); or kPathCompact, the compact integral histogram, built and looked
-// up per group of images (every image has to fit it). `graph`: capture the
+// whole batch. Without a `layout`, the sweep as a persistent kernel over a
+// queue of (image, strip, row band) tiles (TM_EUNSUPPORTED if some image cannot
+// be swept); with one (compact_fits), the compact integral histogram, built and
+// looked up per group of images. `graph`: capture the
 // batch into a CUDA graph of the context's cache and replay it while the batch
 // is unchanged.
 tm_status finish_fused(tm_ctx *c, int nimg, const tm_image *in, const std::vector<Job> &jobs, int64_t n,
                        bool run_range, std::vector<Job> *jobs_out);
 
 tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image *out, cudaStream_t s,
-                        bool graph, Path path, bool do_lookup = true, std::vector<Job> *jobs_out = nullptr) {
-  const bool compact = path == kPathCompact;
+                        bool graph, const CompactLayout *layout = nullptr, bool do_lookup = true,
+                        std::vector<Job> *jobs_out = nullptr) {
+  const bool compact = layout != nullptr;
+  const Path path = compact ? kPathCompact : kPathSweep;
   tm_status st;
   if (graph)
     for (auto &G : c->graphs) {
@@ -669,7 +722,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   for (int i = 0; i < nimg; ++i) total_px += (double)in[i].width * in[i].height;
   std::vector<Job> jobs((size_t)nimg);
   std::vector<JobLayout> lays((size_t)nimg);
-  std::vector<size_t> offs((size_t)nimg), coffs((size_t)nimg);
+  std::vector<size_t> offs((size_t)nimg);
   // strips of 512 own columns (one CTA per SM, with all of its shared memory)
   // where every image fits them, else 256 (two CTAs per SM)
   const DevParams P0 = dev_params(c->p, 0);
@@ -696,15 +749,8 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     int first, rows, cols, look, tall;
   };
   std::vector<Group> groups;
-  std::vector<CompactPlan> cplans((size_t)nimg);
-  size_t c_used = 0, c_total = 0;
-  bool c_wide = false;  // 32-bit vectors for every image if one needs them
-  for (int i = 0; i < nimg && compact; ++i) {
-    CompactPlan &C = cplans[(size_t)i];
-    if (!plan_compact(P0, in[i].width, in[i].height, C))
-      return fail(c, TM_EUNSUPPORTED, "image %d is outside the compact path", i);
-    c_wide = c_wide || C.wide;
-  }
+  const bool c_wide = compact && layout->wide;
+  const size_t c_total = compact ? layout->bytes : 0;
   // under TM_OPT_BACKWARD_REUSE the lookup also keeps the window moments; a
   // recomputation for the backward keeps them where the compact lookup's plain
   // variant forms them beside the counts
@@ -729,16 +775,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     integral_layout(W, H, SIZE_MAX, (int)(2 * c->num_sms * share), J.nseg, J.seg_rows);
     size_t cnt_bytes = 0;
     if (compact) {
-      CompactPlan &C = cplans[(size_t)i];
-      if (c_wide && !C.wide) C.vec_bytes *= 2;
-      const size_t b = compact_bytes(C);
-      if (groups.empty() || c_used + b > kCompactGroup || i - groups.back().first >= kCompactImages) {
-        groups.push_back({i, 0, 0, 0, 0});
-        c_used = 0;
-      }
-      coffs[(size_t)i] = c_used;
-      c_used += b;
-      c_total = std::max(c_total, c_used);
+      if (groups.size() < layout->first.size() && layout->first[groups.size()] == i) groups.push_back({i, 0, 0, 0, 0});
       Group &g = groups.back();
       g.tall = std::max(g.tall, H);
       J.b0[kStCRows] = g.rows;
@@ -747,7 +784,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
       g.cols += compact_col_units(W, K);
       J.b0[kStLook] = g.look;
       g.look += compact_look_blocks(W, H, look_rows);
-      J.c_shift = C.shift;
+      J.c_shift = layout->plans[(size_t)i].shift;
       // count planes only for the backward
       J.plan.W = W, J.plan.H = H, J.plan.cnt_wide = (1 << c->p.n_fields) - 1;
       J.cnt_wide = J.plan.cnt_wide;
@@ -838,11 +875,11 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     J.s_pair = 1;
     J.segtot = reinterpret_cast<long long *>(b + L.segtot);
     if (compact) {
-      char *cb = ws + ws_total + coffs[(size_t)i];
+      const CompactPlan &C = layout->plans[(size_t)i];
+      char *cb = ws + ws_total + layout->offs[(size_t)i];
       J.c_rec = reinterpret_cast<uint2 *>(cb);
-      J.c_vec = cb + align256(cplans[(size_t)i].rec_bytes);
-      J.c_row = reinterpret_cast<uint16_t *>(cb + align256(cplans[(size_t)i].rec_bytes) +
-                                             align256(cplans[(size_t)i].vec_bytes));
+      J.c_vec = cb + align256(C.rec_bytes);
+      J.c_row = reinterpret_cast<uint16_t *>(cb + align256(C.rec_bytes) + align256(C.vec_bytes));
     }
     // (the compact path has count planes only where the backward reads them)
     J.cnt = !compact || keep_mom || !do_lookup ? reinterpret_cast<unsigned char *>(b + L.cnt) : nullptr;
@@ -1118,7 +1155,7 @@ tm_status choose_path(tm_ctx *c, const tm_image *in, const tm_image *out, cudaSt
   for (int path = 1; path <= 2 && !st; ++path) {
     for (int rep = 0; rep < 2 && !st; ++rep) {
       cudaEventRecord(e0, s);
-      st = path == 1 ? forward_fused(c, 1, in, out, s, false, kPathSweep) : forward_materialised(c, in, out, s);
+      st = path == 1 ? forward_fused(c, 1, in, out, s, false) : forward_materialised(c, in, out, s);
       if (path == 1 && st == TM_EUNSUPPORTED) {
         fused_ok = false;
         st = TM_OK;
@@ -1178,11 +1215,12 @@ tm_status forward_device(tm_ctx *c, const tm_image *in, const tm_image *out, cud
   ++c->calls;
   int path = c->hist_path;
   if (c->p.n_bins < 2) path = kPathMaterialised;  // no thresholds: nothing to count
-  if (path == 0 && compact_fits(c, in) && !strips(c, 1, in)) {
+  CompactLayout L;
+  if (path == 0 && !strips(c, 1, in) && compact_fits(c, 1, in, L)) {
     const bool graph = !c->stage_timing && !c->debug && !c->reuse_range && single_graph_ok(c, in, out, kPathCompact);
-    st = forward_fused(c, 1, in, out, s, graph, kPathCompact);
+    st = forward_fused(c, 1, in, out, s, graph, &L);
     if (st != TM_ENOMEM) return st;
-    c->no_compact = true;  // the other paths need less memory
+    compact_nomem(c, L);  // the other paths need less memory
   }
   if (path == 0) {
     const auto key = std::make_tuple((int)in->width, (int)in->height, (int)in->dtype, (int)out->dtype);
@@ -1196,7 +1234,7 @@ tm_status forward_device(tm_ctx *c, const tm_image *in, const tm_image *out, cud
   if (path == 1) {
     // a cached CUDA graph per image pair unless a per-call feature is on
     const bool graph = !c->stage_timing && !c->debug && !c->reuse_range && single_graph_ok(c, in, out, kPathSweep);
-    st = forward_fused(c, 1, in, out, s, graph, kPathSweep);
+    st = forward_fused(c, 1, in, out, s, graph);
     if (st != TM_EUNSUPPORTED) return st;
     if (c->hist_path == 1)
       return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit these fields (use the materialised path)");
@@ -1302,19 +1340,19 @@ tm_status backward_images(tm_ctx *c, int n, const tm_image *in, const tm_image *
   std::vector<Job> jobs;
   int64_t launches = 0;
   // the backward takes the fields that the sweep fits, whatever path counts
-  bool compact = c->hist_path == 0 && !strips(c, n, in);
-  for (int i = 0; i < n; ++i) {
+  for (int i = 0; i < n; ++i)
     if (!sweep_fits(c, &in[i])) return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit these fields");
-    compact = compact && compact_fits(c, &in[i]);
-  }
   if (c->bwd_reuse && c->fwd_valid && (int)c->fwd_in.size() == n && same_images(c->fwd_in, in, n)) {
     jobs = c->fwd_jobs;  // the last forward's intermediates of these images are in the workspace
   } else {
-    st = forward_fused(c, n, in, in, s, false, compact ? kPathCompact : kPathSweep, false, &jobs);
-    if (st == TM_ENOMEM && compact) {
-      c->no_compact = true;
-      st = forward_fused(c, n, in, in, s, false, kPathSweep, false, &jobs);
+    const bool compact = c->hist_path == 0 && !strips(c, n, in);
+    CompactLayout L;
+    st = TM_ENOMEM;
+    while (st == TM_ENOMEM && compact && compact_fits(c, n, in, L)) {
+      st = forward_fused(c, n, in, in, s, false, &L, false, &jobs);
+      if (st == TM_ENOMEM) compact_nomem(c, L);
     }
+    if (st == TM_ENOMEM) st = forward_fused(c, n, in, in, s, false, nullptr, false, &jobs);
     if (st) return st;
     launches = c->launches;
   }
@@ -1437,7 +1475,7 @@ tm_status choose_batch_path(tm_ctx *c, int n, const tm_image *in, const tm_image
   tm_status st = TM_OK;
   for (int rep = 0; rep < 2 && !st; ++rep) {
     cudaEventRecord(e[0], s);
-    st = forward_fused(c, n, in, out, s, false, kPathSweep);
+    st = forward_fused(c, n, in, out, s, false);
     cudaEventRecord(e[1], s);
     if (!st) st = forward_materialised_batch(c, n, in, out, s, false, stats0);
     cudaEventRecord(e[2], s);
@@ -1466,7 +1504,6 @@ tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *ou
   tm_status s = ensure_device_info(c);
   if (s) return s;
   std::vector<tm_image> fin, fout, min_, mout;
-  bool compact = c->hist_path == 0 && !strips(c, n, in);
   for (int i = 0; i < n; ++i) {
     bool fused = c->p.n_bins > 1 && c->hist_path != 2;
     if (fused && !sweep_fits(c, &in[i])) {
@@ -1474,21 +1511,20 @@ tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *ou
         return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit image %d's fields (use the materialised path)", i);
       fused = false;
     }
-    compact = compact && compact_fits(c, &in[i]);
     (fused ? fin : min_).push_back(in[i]);
     (fused ? fout : mout).push_back(out[i]);
   }
   if ((s = ensure_stats(c, n))) return s;
-  if (compact) {
+  const bool compact = c->hist_path == 0 && !strips(c, n, in);
+  for (CompactLayout L; compact && compact_fits(c, n, in, L); compact_nomem(c, L)) {
     ++c->calls;
     const int m0 = mark(c, st, -1);
-    s = forward_fused(c, n, in, out, st, true, kPathCompact);
+    s = forward_fused(c, n, in, out, st, true, &L);
     if (!s) {  // a stored histogram, and the compact one: both names from the call's start
       mark(c, st, ST_BATCH_MAT, m0);
       mark(c, st, ST_BATCH_COMPACT, m0);
     }
     if (s != TM_ENOMEM) return s;
-    c->no_compact = true;  // the other paths need less memory
   }
   if (!fin.empty() && c->hist_path == 0) {
     std::vector<std::tuple<int, int, int, int>> key;
@@ -1512,7 +1548,7 @@ tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *ou
   ++c->calls;
   if (!fin.empty()) {
     mark(c, st, -1);
-    s = forward_fused(c, (int)fin.size(), fin.data(), fout.data(), st, true, kPathSweep);
+    s = forward_fused(c, (int)fin.size(), fin.data(), fout.data(), st, true);
     if (s) return s;
     total += c->launches;
     mark(c, st, ST_BATCH);
@@ -1980,6 +2016,7 @@ tm_status tm_set_option(tm_ctx *c, int32_t key, int64_t value) {
     c->hist_path = (int)value;
     c->path_choice.clear();
     c->batch_choice.clear();
+    c->compact_failed = SIZE_MAX;
     return TM_OK;
   }
   return fail(c, TM_EINVAL, "unknown option %d", key);

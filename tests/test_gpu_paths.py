@@ -111,3 +111,82 @@ def test_batch_splits_over_two_passes():
                 assert torch.equal(y, r)
     finally:
         tm.tm_destroy(ctx)
+
+
+def _all_but(leave):
+    """Device memory held so that about `leave` bytes are free."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+
+
+def _path(ctx, x):
+    names = _stages(ctx, lambda: tm.tm_forward(ctx, x, torch.empty_like(x)))
+    return names & {"compact_histogram", "integral_histogram", "fused_sweep"}
+
+
+def test_short_memory_holds_for_what_did_not_fit():
+    """The compact histogram of a 12 MP image (1.8 GB) that cannot be had keeps
+    neither smaller images from it nor, once there is memory again, the same
+    image: after the option is set, or after 256 calls."""
+    p = tm.make_params(64, [4, 16])
+    big, small = _images([(4000, 3000), (300, 200)], 7)
+    for again in ("option", "calls"):
+        ctx = tm.tm_create(p)
+        hold = None
+        try:
+            torch.empty_like(big)  # (the caching allocator's block for the outputs)
+            hold = _all_but(900 << 20)
+            try:
+                assert "compact_histogram" not in _path(ctx, big)
+            except tm.TmError as e:
+                assert e.status == tm.TM_ENOMEM
+            assert _path(ctx, small) == {"compact_histogram"}
+            hold = None
+            torch.cuda.empty_cache()
+            if again == "option":
+                tm.tm_set_option(ctx, tm.TM_OPT_HIST_PATH, 0)
+            else:
+                y = torch.empty_like(small)
+                for _ in range(256):
+                    tm.tm_forward(ctx, small, y)
+            assert _path(ctx, big) == {"compact_histogram"}
+        finally:
+            tm.tm_destroy(ctx)
+            hold = None
+            torch.cuda.empty_cache()
+
+
+def test_batch_in_smaller_groups_when_memory_is_short():
+    """Sixteen images whose compact histograms (0.9 GB each) would run in two
+    groups: with 4 GB free they run one image at a time, the forward and the
+    backward's recomputation, and give the same outputs."""
+    p = tm.make_params(128, [8, 32])
+    xs = [synth.wdr_device(1536, 2048, seed=k, device="cuda") for k in range(16)]
+    gs = [torch.randn_like(x) for x in xs]
+    got = []
+    for short in (False, True):
+        ys, gin, gp = [torch.empty_like(x) for x in xs], [torch.empty_like(x) for x in xs], torch.empty(7, device="cuda")
+        ctx = tm.tm_create(p)
+        hold = None
+        try:
+            if short:
+                hold = _all_but(4 << 30)
+            for _ in range(2):
+                assert "batch_compact" in _stages(ctx, lambda: tm.tm_forward_batch(ctx, xs, ys))
+            if not short:
+                tm.tm_backward_batch(ctx, xs, gs, gin, gp)
+            else:  # (four images: the backward's own workspace takes the rest)
+                tm.tm_destroy(ctx)
+                ctx = tm.tm_create(p)
+                tm.tm_backward_batch(ctx, xs[:4], gs[:4], gin[:4], gp)
+            torch.cuda.synchronize()
+        finally:
+            tm.tm_destroy(ctx)
+            del hold
+            torch.cuda.empty_cache()
+        got.append((ys, gin))
+    for a, b in zip(*[g[0] for g in got]):
+        assert torch.equal(a, b)
+    for a, b in zip(got[0][1][:4], got[1][1][:4]):
+        assert torch.equal(a, b)
