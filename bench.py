@@ -472,8 +472,7 @@ def leg_batch(args, dev, kind, steps=None, warmup=None):
     ms_batch = _timed(lambda i: tm.tm_forward_batch(ctx, xs, ys, stream), steps, stream)
     clk = clocks.stop()
 
-    # per-image forward on the same images, after one untimed pass over all of
-    # them (the first forward of each image size measures both histogram paths)
+    # per-image forward on the same images, after one untimed pass over all of them
     def per_image(i):
         for x, y in zip(xs, ys):
             tm.tm_forward(ctx, x, y, stream)

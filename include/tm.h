@@ -141,12 +141,8 @@ const char *tm_status_string(tm_status s);
  *   in   device image, dtype TM_F32 or TM_F16.
  *   out  device image of the same width/height, dtype TM_F32, TM_F16 or TM_U8;
  *        must not overlap in.
- * Asynchronous on `stream`, except that with the automatic histogram path
- * (TM_OPT_HIST_PATH = 0, the default) the first call for an image size and
- * dtype pair that the compact integral histogram does not take (see there)
- * times the two other paths and synchronises `stream` once. The context's
- * workspace is reused, so calls on one context must be ordered (same stream,
- * or synchronised). On the fused and compact paths, an (in, out) pair of
+ * Asynchronous on `stream`. The context's workspace is reused, so calls on one
+ * context must be ordered (same stream, or synchronised). On the fused and compact paths, an (in, out) pair of
  * descriptors that comes back is captured in a CUDA graph of the context and
  * replayed while the same descriptors are passed (a replay reads the current
  * pixel contents); not with debug exports, stage timing or streaming range
@@ -180,25 +176,21 @@ tm_status tm_forward_host(tm_ctx *ctx, const tm_image *in_host,
 tm_status tm_forward_host_async(tm_ctx *ctx, const tm_image *in_host,
                                 const tm_image *out_host, void *stream);
 
-/* Forward over n images of possibly different sizes. With the automatic
- * histogram path a batch whose images all fit the compact integral histogram
- * (and are not all wide strips, see TM_OPT_HIST_PATH) runs on it as one batched pass: the range, bin and integral-image stages
- * once for all of them, then the histograms and lookups of a group of images
- * at a time (32 images, 8 GiB). Otherwise, images whose fields do not fit the
- * fused sweep take the materialised integral histogram; the others take
- * TM_OPT_HIST_PATH's path (automatic: the first batch of a given list of sizes
- * and dtype pairs times both batched passes on those images, synchronising
- * `stream` once, and keeps the faster for later batches).
- * The images on the fused path run as one batched pass: one launch per
- * stage, the sweep as one persistent launch over a shared queue of (image,
- * strip, row band) tiles. Those on the materialised path run as another:
- * the range, bin and integral-image stages once for all of them, then each
- * image's integral histogram and lookup. in[i], out[i] as for tm_forward
+/* Forward over n images of possibly different sizes, by TM_OPT_HIST_PATH's
+ * path for the whole batch. Compact (automatic path only, where every image
+ * fits it): one batched pass, the range, bin and integral-image stages once
+ * for all images, then the histograms and lookups of a group of images at a
+ * time (32 images, 8 GiB). Fused: the images whose fields fit the sweep run as
+ * one batched pass, one launch per stage, the sweep as one persistent launch
+ * over a shared queue of (image, strip, row band) tiles; the others (with the
+ * automatic path; TM_EUNSUPPORTED with TM_OPT_HIST_PATH = 1) as a materialised
+ * pass. Materialised: the range, bin and integral-image stages once for all
+ * images, then each image's integral histogram and lookup. in[i], out[i] as for tm_forward
  * (host arrays of descriptors; the pixel data is on the device). n == 0 is a
  * no-op. Each pass is captured in a CUDA graph and replayed while the same
  * descriptors (pointers, sizes, pitches, dtypes) are passed; a replay reads
  * the current pixel contents. Results are bit-identical to per-image
- * tm_forward calls (both paths give the same outputs bit for bit). */
+ * tm_forward calls (all paths give the same outputs bit for bit). */
 tm_status tm_forward_batch(tm_ctx *ctx, int32_t n, const tm_image *in,
                            const tm_image *out, void *stream);
 
@@ -327,19 +319,23 @@ tm_status tm_debug_export(tm_ctx *ctx, int32_t what, void *dst, size_t bytes,
  *                        32-column chunk instead of per column) for images
  *                        of at least two bins, at most 65535 columns and
  *                        rows and under 24 GiB of it (0.4 GB for 12 MP with
- *                        16 bins, 1.8 GB with 64). For others, for strips
- *                        that the sweep takes faster (one image: width > 128
- *                        heights, or height > 32 widths from 4096 rows; more:
- *                        every width >= 256 heights), and where its memory
- *                        could not be had (that much or more: not tried
- *                        again for 256 calls, or until this option is set;
- *                        a batch is first tried one image at a time), the
- *                        first single-image forward of each (width, height, input dtype, output
- *                        dtype) on a context runs paths 1 and 2 twice, timing
- *                        the second runs (it synchronises its stream once),
- *                        and keeps the faster. All paths give the same
- *                        outputs bit for bit. tm_backward takes the fields
- *                        that fit the fused sweep.
+ *                        16 bins, 1.8 GB with 64). Calls that it does not
+ *                        take, with images at least 16 times as long as wide
+ *                        (or the reverse), or whose last call's images were
+ *                        rough (the bins of a 32-pixel run spanned more than
+ *                        6, or 0.7 of them, on average, e.g. white noise) are
+ *                        measured: three calls each go to the compact path,
+ *                        path 1 and path 2, as far as they take them, the
+ *                        last of each timed with events on `stream` (nothing
+ *                        is synchronised), and then all to the fastest, per
+ *                        list of sizes and dtype pairs (64 are kept). Not
+ *                        while `stream` is being captured. Memory for the
+ *                        compact path that could not be had is not asked for
+ *                        again, or more of it, for 256 calls (a batch is
+ *                        first tried one image at a time). Setting the option
+ *                        forgets all this. All paths give the same outputs
+ *                        bit for bit. tm_backward takes the fields that fit
+ *                        the fused sweep.
  *   TM_OPT_STAGE_TIMING  1 = record a CUDA event after every stage of each
  *                        forward/backward call on its stream (see
  *                        tm_stage_times); 0 = off (default).
@@ -358,7 +354,8 @@ tm_status tm_debug_export(tm_ctx *ctx, int32_t what, void *dst, size_t bytes,
  *                        intermediates (bin map, quantised log, integral
  *                        images, count planes) from the context's workspace
  *                        instead of recomputing them, when the last forward
- *                        call on the context ran the fused path, each image
+ *                        call on the context ran the fused or the compact
+ *                        path for all its images, each image
  *                        over its own range, on the same image descriptors
  *                        (pointers, sizes, pitches, dtypes) in the same order.
  *                        The caller guarantees that the pixels of `in` have

@@ -8,7 +8,6 @@
 #include <cstring>
 #include <map>
 #include <mutex>
-#include <tuple>
 #include <string>
 #include <utility>
 #include <vector>
@@ -171,10 +170,28 @@ struct tm_ctx {
   bool fwd_valid = false;
   std::vector<Job> fwd_jobs;
   std::vector<tm_image> fwd_in;
-  // automatic histogram path: the measured choice per (width, height, in dtype, out dtype),
-  // and per batch of images that fit the sweep (their sizes and dtype pairs)
-  std::map<std::tuple<int, int, int, int>, int> path_choice;
-  std::map<std::vector<std::tuple<int, int, int, int>>, int> batch_choice;
+  // automatic histogram path: per kind of call and its images' sizes and dtype
+  // pairs, the paths that take it and what is known of them
+  struct Trial {
+    uint32_t id = 0;    // tag of its reports in hints[slot]
+    int slot = 0;
+    uint64_t used = 0;  // the call that asked last
+    int n = 0;
+    int cand[3] = {};   // candidate paths; the first is the one by the rules
+    size_t bytes[2] = {};      // of the compact histogram: in groups, and of one image at a time
+    int passes = 0;     // of the measurement so far, kTrialPasses per candidate
+    cudaEvent_t e[3][2] = {};  // around each candidate's last pass
+    float ms[3] = {};          // its time (0: not known yet; -1: left out)
+    int best = -1;             // the measured choice
+    float span = 0.f;          // mean bin span of the chunk rows, as last reported
+  };
+  std::map<std::vector<int>, Trial> trials;
+  uint64_t trial_asks = 0;
+  uint32_t trial_ids = 0;
+  unsigned long long *hints = nullptr;  // page-locked, kTrials slots, written by the device
+  unsigned long long *hint = nullptr;   // the current call's slot (null: none) and tag
+  unsigned hint_tag = 0;
+  cudaEvent_t pass_begin = nullptr;     // to be recorded before the call's first launch (null: no)
   // stage timing: events recorded on the call's stream after each stage
   int stage_timing = 0;
   // per call, its stage marks: the event, the stage it ends (or kNoStage),
@@ -519,6 +536,18 @@ JobLayout job_layout(const tm_params &p, int W, int H, int nseg, size_t cnt_byte
   return L;
 }
 
+// Before the first launch of a call.
+void first_launch(tm_ctx *c, cudaStream_t s) {
+  if (c->pass_begin) cudaEventRecord(c->pass_begin, s);
+  c->pass_begin = nullptr;
+}
+
+// Where a call's first job has to report how rough the images are.
+void set_hint(const tm_ctx *c, Job &J, int i) {
+  J.hint = i == 0 ? c->hint : nullptr;
+  J.hint_tag = c->hint_tag;
+}
+
 // The materialised path for one image: range, bins, integral images,
 // bin-major cumulative integral histogram, lookup. Used when the fused sweep
 // does not fit the fields, or on request (TM_OPT_HIST_PATH = 2).
@@ -546,6 +575,7 @@ tm_status forward_materialised(tm_ctx *c, const tm_image *in, const tm_image *ou
   J.in = to_image(in);
   J.out = to_image(out);
   J.st = c->stats;
+  set_hint(c, J, 0);
   bool run_range = true;
   if (c->reuse_range) {
     bool own = true;
@@ -558,6 +588,7 @@ tm_status forward_materialised(tm_ctx *c, const tm_image *in, const tm_image *ou
   J.s2 = J.s1 + 1;
   J.s_pair = 1;
   J.segtot = reinterpret_cast<long long *>(ws + L.segtot);
+  if (J.hint) J.grp = reinterpret_cast<uint16_t *>(ws + L.grp);
   J.qbits = qbits;
   J.nseg = nseg;
   J.seg_rows = seg_rows;
@@ -570,6 +601,7 @@ tm_status forward_materialised(tm_ctx *c, const tm_image *in, const tm_image *ou
   }
   const int rb = range_blocks(W, H, c->num_sms, 1.0), pb = prep_blocks(W, H, c->num_sms, 1.0);
   J.b0[kStRange] = J.b0[kStPrep] = J.b0[kStRows] = J.b0[kStCols] = J.b0[kStLook] = 0;
+  first_launch(c, s);
   int64_t n = put_jobs(&J, 1, c->djobs, s);
   mark(c, s, -1);
   if (run_range) launch_range(c->djobs, 1, rb, c->p.n_bins, J.in.dtype, s);
@@ -578,6 +610,7 @@ tm_status forward_materialised(tm_ctx *c, const tm_image *in, const tm_image *ou
   mark(c, s, ST_PREP);
   n += (run_range ? 2 : 1) +
        launch_integral_jobs(c->djobs, 1, integral_tile_blocks(W, nseg), integral_col_blocks(W), s);
+  if (J.hint) n += launch_span(c->djobs, 1, s);
   mark(c, s, ST_INTEGRAL);
   uint32_t *cpl = nullptr;
   if (c->p.n_bins > 1) {
@@ -660,21 +693,6 @@ bool compact_layout(const tm_ctx *c, int n, const tm_image *in, size_t limit, Co
   return true;
 }
 
-// Whether the compact integral histogram takes a call's images under the
-// context's fields, bins and memory; L: in groups of up to kCompactGroup bytes,
-// or of one image where such a group's memory could not be had.
-bool compact_fits(const tm_ctx *c, int n, const tm_image *in, CompactLayout &L) {
-  const bool failed = c->calls - c->compact_failed_at < kCompactRetry;
-  const size_t most = failed ? c->compact_failed : SIZE_MAX;
-  return compact_layout(c, n, in, kCompactGroup, L) &&
-         (L.bytes < most || (n > 1 && compact_layout(c, n, in, 0, L) && L.bytes < most));
-}
-
-void compact_nomem(tm_ctx *c, const CompactLayout &L) {
-  c->compact_failed = L.bytes;
-  c->compact_failed_at = c->calls;
-}
-
 // Whether the images of a call are strips that the sweep takes faster than the
 // compact integral histogram, whose row pass is a chain along each row and
 // whose column pass, with at most 128 warps per 32 columns, one down each
@@ -693,30 +711,34 @@ bool strips(tm_ctx *c, int n, const tm_image *im) {
 }
 
 // The batched path over images that share it: one launch per stage for the
-// whole batch. Without a `layout`, the sweep as a persistent kernel over a
-// queue of (image, strip, row band) tiles (TM_EUNSUPPORTED if some image cannot
-// be swept); with one (compact_fits), the compact integral histogram, built and
-// looked up per group of images. `graph`: capture the
+// whole batch. path: kPathSweep, the sweep as a persistent kernel over a queue
+// of (image, strip, row band) tiles (TM_EUNSUPPORTED if some image cannot be
+// swept); or kPathCompact, the compact integral histogram, built and looked up
+// per group of images of up to group_bytes (every image has to fit it).
+// `graph`: capture the
 // batch into a CUDA graph of the context's cache and replay it while the batch
 // is unchanged.
 tm_status finish_fused(tm_ctx *c, int nimg, const tm_image *in, const std::vector<Job> &jobs, int64_t n,
                        bool run_range, std::vector<Job> *jobs_out);
 
 tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image *out, cudaStream_t s,
-                        bool graph, const CompactLayout *layout = nullptr, bool do_lookup = true,
+                        bool graph, Path path, size_t group_bytes = kCompactGroup, bool do_lookup = true,
                         std::vector<Job> *jobs_out = nullptr) {
-  const bool compact = layout != nullptr;
-  const Path path = compact ? kPathCompact : kPathSweep;
+  const bool compact = path == kPathCompact;
   tm_status st;
   if (graph)
     for (auto &G : c->graphs) {
       if (G.path != path || !same_images(G.in, in, nimg) || !same_images(G.out, out, nimg)) continue;
       c->fwd_valid = false;
+      first_launch(c, s);
       TM_CUDA(c, cudaGraphLaunch(G.exec, s));
       G.used = c->calls;
       return finish_fused(c, nimg, in, G.jobs, G.launches, true, jobs_out);
     }
   c->fwd_valid = false;  // the workspace is rewritten below
+  CompactLayout layout;
+  if (compact && !compact_layout(c, nimg, in, group_bytes, layout))
+    return fail(c, TM_EUNSUPPORTED, "an image is outside the compact path");
   const bool debug = c->debug != 0 && nimg == 1 && !graph;
   double total_px = 0;
   for (int i = 0; i < nimg; ++i) total_px += (double)in[i].width * in[i].height;
@@ -749,8 +771,8 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     int first, rows, cols, look, tall;
   };
   std::vector<Group> groups;
-  const bool c_wide = compact && layout->wide;
-  const size_t c_total = compact ? layout->bytes : 0;
+  const bool c_wide = layout.wide;
+  const size_t c_total = layout.bytes;
   // under TM_OPT_BACKWARD_REUSE the lookup also keeps the window moments; a
   // recomputation for the backward keeps them where the compact lookup's plain
   // variant forms them beside the counts
@@ -775,7 +797,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     integral_layout(W, H, SIZE_MAX, (int)(2 * c->num_sms * share), J.nseg, J.seg_rows);
     size_t cnt_bytes = 0;
     if (compact) {
-      if (groups.size() < layout->first.size() && layout->first[groups.size()] == i) groups.push_back({i, 0, 0, 0, 0});
+      if (groups.size() < layout.first.size() && layout.first[groups.size()] == i) groups.push_back({i, 0, 0, 0, 0});
       Group &g = groups.back();
       g.tall = std::max(g.tall, H);
       J.b0[kStCRows] = g.rows;
@@ -784,7 +806,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
       g.cols += compact_col_units(W, K);
       J.b0[kStLook] = g.look;
       g.look += compact_look_blocks(W, H, look_rows);
-      J.c_shift = layout->plans[(size_t)i].shift;
+      J.c_shift = layout.plans[(size_t)i].shift;
       // count planes only for the backward
       J.plan.W = W, J.plan.H = H, J.plan.cnt_wide = (1 << c->p.n_fields) - 1;
       J.cnt_wide = J.plan.cnt_wide;
@@ -868,6 +890,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     J.out = to_image(&out[i]);
     J.st = c->stats + i;
     J.st_next = nullptr;
+    set_hint(c, J, i);
     J.bins = reinterpret_cast<uint8_t *>(b + L.bins);
     J.q = reinterpret_cast<int32_t *>(b + L.q);
     J.s1 = reinterpret_cast<long long *>(b + L.s12);
@@ -875,8 +898,8 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     J.s_pair = 1;
     J.segtot = reinterpret_cast<long long *>(b + L.segtot);
     if (compact) {
-      const CompactPlan &C = layout->plans[(size_t)i];
-      char *cb = ws + ws_total + layout->offs[(size_t)i];
+      const CompactPlan &C = layout.plans[(size_t)i];
+      char *cb = ws + ws_total + layout.offs[(size_t)i];
       J.c_rec = reinterpret_cast<uint2 *>(cb);
       J.c_vec = cb + align256(C.rec_bytes);
       J.c_row = reinterpret_cast<uint16_t *>(cb + align256(C.rec_bytes) + align256(C.vec_bytes));
@@ -911,6 +934,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   if ((st = ensure_side_streams(c))) return st;  // before any capture begins
   // a graph's descriptors are written once, ahead of it (a replay saves the
   // launch: 2 us of a forward's 41 at 512 x 384)
+  if (!graph) first_launch(c, s);
   const int64_t puts = put_jobs(jobs.data(), nimg, dj, s);
   if (graph) {
     if (!c->graph_stream) TM_CUDA(c, cudaStreamCreateWithFlags(&c->graph_stream, cudaStreamNonBlocking));
@@ -934,12 +958,14 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   const auto group_end = [&](size_t k) { return k + 1 < groups.size() ? groups[k + 1].first : nimg; };
   const auto build = [&](size_t k, cudaStream_t q) {
     const Group &g = groups[k];
-    return launch_compact_build(dj + g.first, group_end(k) - g.first, g.rows, g.cols, g.tall, K, c_wide, q);
+    return launch_compact_build(dj + g.first, group_end(k) - g.first, g.rows, g.cols, g.tall, K, c_wide,
+                                jobs[(size_t)g.first].hint != nullptr, q);
   };
   int ls = compact ? build(0, c->sweep_stream)
                    : launch_sweep(P, dj, nimg, nitems, queue, smem, ctas, width, c->sweep_stream);
   if (!graph) mark(c, c->sweep_stream, compact ? ST_COMPACT : ST_SWEEP, m_prep);
   n += std::max(ls, 0) + launch_integral_jobs(dj, nimg, b_rows, b_cols, c->int_stream);
+  if (!compact && jobs[0].hint) n += launch_span(dj, std::min(nimg, kCompactImages), c->int_stream);
   if (!graph) mark(c, c->int_stream, ST_INTEGRAL, m_prep);
   n += run_range ? 2 : 1;
   TM_CUDA(c, cudaEventRecord(c->ov_sweep, c->sweep_stream));
@@ -995,6 +1021,7 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     c->gspare = nullptr;
     c->gspare_n = 0;
     c->graphs.push_back(std::move(G));
+    first_launch(c, caller);
     TM_CUDA(c, cudaGraphLaunch(c->graphs.back().exec, caller));
   } else if (ls < 0) {
     return check_launch(c, "histogram shared-memory attribute");
@@ -1033,12 +1060,13 @@ tm_status finish_fused(tm_ctx *c, int nimg, const tm_image *in, const std::vecto
 // and integral-image stages run once for the whole batch; then each image's
 // cumulative integral histogram and lookup, on one shared set of planes (the
 // launches are stream-ordered). The stats of image i are c->stats[stats0 + i].
-// `graph`: capture into the context's materialised-batch graph and replay it
+// Captured into the context's materialised-batch graph, which is replayed
 // while the images are unchanged.
 tm_status forward_materialised_batch(tm_ctx *c, int nimg, const tm_image *in, const tm_image *out, cudaStream_t s,
-                                     bool graph, int stats0) {
+                                     int stats0) {
   tm_status st;
-  if (graph && c->mgraph && same_images(c->mgraph_in, in, nimg) && same_images(c->mgraph_out, out, nimg)) {
+  if (c->mgraph && same_images(c->mgraph_in, in, nimg) && same_images(c->mgraph_out, out, nimg)) {
+    first_launch(c, s);
     TM_CUDA(c, cudaGraphLaunch(c->mgraph, s));
     c->launches = c->mgraph_launches;
     return TM_OK;
@@ -1077,7 +1105,7 @@ tm_status forward_materialised_batch(tm_ctx *c, int nimg, const tm_image *in, co
   if ((st = ensure_stats(c, stats0 + nimg))) return st;
   if ((st = grow_device(c, &c->mws, &c->mws_bytes, ws_total + planes_bytes + scratch_bytes))) return st;
   if ((st = grow_device(c, (void **)&c->mdjobs, &c->mdjobs_bytes, sizeof(Job) * nimg))) return st;
-  if (graph && c->mgraph) {
+  if (c->mgraph) {
     cudaGraphExecDestroy(c->mgraph);  // re-captured below
     c->mgraph = nullptr;
   }
@@ -1091,89 +1119,269 @@ tm_status forward_materialised_batch(tm_ctx *c, int nimg, const tm_image *in, co
     J.in = to_image(&in[i]);
     J.out = to_image(&out[i]);
     J.st = c->stats + stats0 + i;
+    set_hint(c, J, i);
     J.bins = reinterpret_cast<uint8_t *>(b + L.bins);
     J.q = reinterpret_cast<int32_t *>(b + L.q);
     J.s1 = reinterpret_cast<long long *>(b + L.s12);
     J.s2 = J.s1 + 1;
     J.s_pair = 1;
     J.segtot = reinterpret_cast<long long *>(b + L.segtot);
+    if (c->hint) J.grp = reinterpret_cast<uint16_t *>(b + L.grp);
   }
   const cudaStream_t caller = s;
-  if (graph) {
-    if (!c->graph_stream) TM_CUDA(c, cudaStreamCreateWithFlags(&c->graph_stream, cudaStreamNonBlocking));
-    s = c->graph_stream;
-    TM_CUDA(c, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  }
+  if (!c->graph_stream) TM_CUDA(c, cudaStreamCreateWithFlags(&c->graph_stream, cudaStreamNonBlocking));
+  s = c->graph_stream;
+  TM_CUDA(c, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
   int64_t n = put_jobs(jobs.data(), nimg, c->mdjobs, s);
   const int in_dt = input_dtype(jobs.data(), nimg);
   launch_range(c->mdjobs, nimg, b_range, c->p.n_bins, in_dt, s);
   launch_prep(c->mdjobs, nimg, b_prep, c->p.n_bins, c->p.flags, c->p.n_fields, in_dt, s);
   n += 2 + launch_integral_jobs(c->mdjobs, nimg, b_rows, b_cols, s);
+  if (jobs[0].hint) n += launch_span(c->mdjobs, std::min(nimg, kCompactImages), s);
   for (int i = 0; i < nimg; ++i) {
     const Job &J = jobs[(size_t)i];
     if (planes) n += launch_integral_histogram(J.bins, J.in.W, J.in.H, c->p.n_bins, true, planes, scratch, s);
     n += launch_lookup_materialised(J.in, J.out, dev_params(c->p, J.qbits), J.bins, planes,
                                     reinterpret_cast<int64_t *>(J.s1), DebugPlanes{}, s);
   }
-  if (graph) {
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(s, &g);
-    if (e != cudaSuccess) {
-      if (g) cudaGraphDestroy(g);
-      cudaGetLastError();
-      return fail(c, TM_ECUDA, "materialised batch capture failed: %s", cudaGetErrorString(e));
-    }
-    e = cudaGraphInstantiate(&c->mgraph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-      c->mgraph = nullptr;
-      return cuda_fail(c, e, "cudaGraphInstantiate");
-    }
-    c->mgraph_in.assign(in, in + nimg);
-    c->mgraph_out.assign(out, out + nimg);
-    c->mgraph_launches = n;
-    TM_CUDA(c, cudaGraphLaunch(c->mgraph, caller));
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamEndCapture(s, &g);
+  if (e != cudaSuccess) {
+    if (g) cudaGraphDestroy(g);
+    cudaGetLastError();
+    return fail(c, TM_ECUDA, "materialised batch capture failed: %s", cudaGetErrorString(e));
   }
+  e = cudaGraphInstantiate(&c->mgraph, g, 0);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) {
+    c->mgraph = nullptr;
+    return cuda_fail(c, e, "cudaGraphInstantiate");
+  }
+  c->mgraph_in.assign(in, in + nimg);
+  c->mgraph_out.assign(out, out + nimg);
+  c->mgraph_launches = n;
+  first_launch(c, caller);
+  TM_CUDA(c, cudaGraphLaunch(c->mgraph, caller));
   if ((st = check_launch(c, "materialised batch launch"))) return st;
   c->launches = n;
   return TM_OK;
 }
 
-// Automatic histogram path: run each path twice on this image and time the
-// second run with events (synchronising the stream); 1 = fused, 2 = materialised.
-tm_status choose_path(tm_ctx *c, const tm_image *in, const tm_image *out, cudaStream_t s, int *choice) {
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  TM_CUDA(c, cudaEventCreate(&e0));
-  if (cudaEventCreate(&e1) != cudaSuccess) {
-    cudaEventDestroy(e0);
-    cudaGetLastError();
-    return fail(c, TM_ECUDA, "cudaEventCreate");
+// The automatic path. The first candidate is taken by the rules: the compact
+// integral histogram where it fits, but the sweep for strips(), else the sweep.
+// Where the rules are not sure, the candidates are measured on the calls
+// themselves: each runs three of them (so that calls that replay a graph are
+// timed on a replay: rough 64 x 4095 with 256 bins take 228 us in launches and
+// 300 in replays on the compact path, 233 and 209 on the sweep), the last
+// between events that are read when a later call finds them complete (nothing
+// is synchronised), and the fastest takes the calls from then on. That is where
+//   - the compact histogram does not take the call;
+//   - some image is at least 16 times as long as wide, or the reverse (the
+//     compact build's chains along rows and columns: 512 x 60000, 64 bins,
+//     1968 against the sweep's 2229 us; 2048 x 16 37 and 51, batches of 100
+//     of them 328 and 597);
+//   - the images are rough: in their last call the 32-column chunk rows spanned
+//     more than 6 bins, or 0.7 of them, on average (what the compact build and
+//     its vectors cost by). 12 MP, 64 bins, white noise, span 60: 2560 against
+//     1738 us; 128 bins, noise of a decade, span 35: 1823 against 1357; batches
+//     of 100 images of 256 x 256, 256 bins, span 23 and more: 1178 against 928.
+//     Of 1961 kinds of calls timed, those with shorter spans and sides were at
+//     most 5 % slower on the compact path. Photograph-like scenes with 64 bins
+//     span 0.5 to 6.
+// The span comes from the device (report_span) through host memory, so a call
+// goes by the last one that has run.
+constexpr size_t kTrials = 64;  // the most recently asked for are kept
+constexpr int kTrialPasses = 3; // launches, a graph's capture, its replay
+
+void drop_trial_events(tm_ctx::Trial &T) {
+  for (auto &e : T.e)
+    for (cudaEvent_t &ev : e) {
+      if (ev) cudaEventDestroy(ev);
+      ev = nullptr;
+    }
+}
+
+void drop_trials(tm_ctx *c) {
+  for (auto &t : c->trials) drop_trial_events(t.second);
+  c->trials.clear();
+}
+
+// A new trial of a call of `kind` on n images; compact: with that path, where it fits.
+enum TrialKind { kTrialSingle, kTrialBatch, kTrialBackward };
+tm_ctx::Trial new_trial(tm_ctx *c, TrialKind kind, int n, const tm_image *in, bool compact) {
+  tm_ctx::Trial T;
+  CompactLayout L;
+  bool sweep = kind == kTrialBackward;
+  for (int i = 0; i < n && !sweep; ++i) sweep = sweep_fits(c, &in[i]);
+  const bool strip = sweep && strips(c, n, in);
+  if (strip) T.cand[T.n++] = kPathSweep;
+  if (compact && compact_layout(c, n, in, kCompactGroup, L)) {
+    T.cand[T.n++] = kPathCompact;
+    T.bytes[0] = L.bytes;
+    compact_layout(c, n, in, 0, L);
+    T.bytes[1] = L.bytes;
   }
-  float ms[3] = {0.f, 0.f, 0.f};
-  tm_status st = TM_OK;
-  bool fused_ok = true;
-  for (int path = 1; path <= 2 && !st; ++path) {
-    for (int rep = 0; rep < 2 && !st; ++rep) {
-      cudaEventRecord(e0, s);
-      st = path == 1 ? forward_fused(c, 1, in, out, s, false) : forward_materialised(c, in, out, s);
-      if (path == 1 && st == TM_EUNSUPPORTED) {
-        fused_ok = false;
-        st = TM_OK;
-        break;
+  if (sweep && !strip) T.cand[T.n++] = kPathSweep;
+  if (kind != kTrialBackward) T.cand[T.n++] = kPathMaterialised;
+  return T;
+}
+
+// The trial of a call on n images (out null: none); the call's reports go to
+// its slot. Without the compact path where its memory could not be had; else
+// group_bytes is the limit of its groups.
+tm_ctx::Trial &trial_for(tm_ctx *c, TrialKind kind, int n, const tm_image *in, const tm_image *out,
+                         size_t &group_bytes) {
+  std::vector<int> key;
+  key.reserve(2 + 4 * (size_t)n);
+  key.push_back(kind);
+  key.push_back(1);
+  for (int i = 0; i < n; ++i) {
+    key.push_back(in[i].width);
+    key.push_back(in[i].height);
+    key.push_back(in[i].dtype);
+    key.push_back(out ? out[i].dtype : -1);
+  }
+  auto it = c->trials.end();
+  for (;;) {
+    it = c->trials.find(key);
+    if (it == c->trials.end()) {
+      tm_ctx::Trial T = new_trial(c, kind, n, in, key[1] != 0);
+      T.id = ++c->trial_ids;
+      T.slot = (int)c->trials.size();
+      if (c->trials.size() >= kTrials) {
+        auto old = std::min_element(c->trials.begin(), c->trials.end(),
+                                    [](const auto &a, const auto &b) { return a.second.used < b.second.used; });
+        T.slot = old->second.slot;
+        drop_trial_events(old->second);
+        c->trials.erase(old);
       }
-      cudaEventRecord(e1, s);
+      it = c->trials.emplace(key, T).first;
     }
-    if (!st && (path == 2 || fused_ok)) {
-      cudaError_t e = cudaEventSynchronize(e1);
-      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms[path], e0, e1);
-      if (e != cudaSuccess) st = cuda_fail(c, e, "timing the histogram paths");
+    const size_t most = c->calls - c->compact_failed_at < kCompactRetry ? c->compact_failed : SIZE_MAX;
+    group_bytes = it->second.bytes[0] < most ? kCompactGroup : 0;
+    if (it->second.bytes[1] < most || !key[1]) break;
+    key[1] = 0;
+  }
+  tm_ctx::Trial &T = it->second;
+  T.used = ++c->trial_asks;
+  if (!c->hints) {
+    if (cudaHostAlloc(&c->hints, kTrials * sizeof *c->hints, cudaHostAllocMapped) == cudaSuccess) {
+      memset(c->hints, 0, kTrials * sizeof *c->hints);
+    } else {
+      cudaGetLastError();
+      c->hints = nullptr;
     }
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  if (st) return st;
-  *choice = fused_ok && ms[1] <= ms[2] ? 1 : 2;
-  return TM_OK;
+  if (c->hints) {
+    const unsigned long long v = reinterpret_cast<const volatile unsigned long long *>(c->hints)[T.slot];
+    const uint32_t bits = (uint32_t)v;
+    if ((uint32_t)(v >> 32) == T.id) memcpy(&T.span, &bits, sizeof bits);
+  }
+  c->hint = c->hints ? c->hints + T.slot : nullptr;
+  c->hint_tag = T.id;
+  return T;
+}
+
+// The compact path's memory could not be had in groups of group_bytes.
+void compact_nomem(tm_ctx *c, const tm_ctx::Trial &T, size_t group_bytes) {
+  c->compact_failed = T.bytes[group_bytes ? 0 : 1];
+  c->compact_failed_at = c->calls;
+}
+
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
+// Whether the times of the first k candidates are known (or left out).
+bool trial_times(tm_ctx::Trial &T, int k) {
+  bool all = true;
+  for (int i = 0; i < k; ++i) {
+    if (T.ms[i] != 0.f) continue;
+    const cudaError_t e = cudaEventQuery(T.e[i][1]);
+    if (e == cudaErrorNotReady) {
+      cudaGetLastError();
+      all = false;
+    } else if (e != cudaSuccess || cudaEventElapsedTime(&T.ms[i], T.e[i][0], T.e[i][1]) != cudaSuccess) {
+      cudaGetLastError();
+      T.ms[i] = -1.f;
+    }
+  }
+  return all;
+}
+
+// The candidate (an index) that takes this call; pass: as a pass of the
+// measurement.
+int trial_next(tm_ctx *c, tm_ctx::Trial &T, int n, const tm_image *in, cudaStream_t s, bool &pass) {
+  pass = false;
+  if (T.n == 1) return 0;
+  const int K = c->p.n_bins - 1;
+  bool unsure = T.span > 6.f || T.span > 0.7f * K || std::find(T.cand, T.cand + T.n, kPathCompact) == T.cand + T.n;
+  for (int i = 0; i < n && !unsure; ++i) {
+    const long long W = in[i].width, H = in[i].height;
+    unsure = W >= 16 * H || H >= 16 * W;
+  }
+  if (!unsure) return 0;
+  if (T.best >= 0) return T.best;
+  if (capturing(s)) return 0;
+  int k = T.passes / kTrialPasses;
+  if (k < T.n && T.cand[k] == kPathMaterialised && k > 0 && T.passes % kTrialPasses == 0) {
+    // planes that are written and read once at the copy rate take longer than
+    // another candidate does: left out, with their memory
+    if (!trial_times(T, k)) return 0;
+    double bytes = 0;
+    for (int i = 0; i < n; ++i) bytes += 8.0 * K * (in[i].width + 1.0) * (in[i].height + 1.0);
+    for (int i = 0; i < k; ++i)
+      if (T.ms[i] > 0.f && bytes / 6.8e9 > T.ms[i]) T.ms[k] = -1.f;
+    if (T.ms[k] < 0.f) {
+      T.passes += kTrialPasses;
+      ++k;
+    }
+  }
+  if (k < T.n) {
+    for (cudaEvent_t &ev : T.e[k])
+      if (!ev && cudaEventCreate(&ev) != cudaSuccess) {
+        cudaGetLastError();
+        ev = nullptr;
+        return 0;
+      }
+    pass = true;
+    return k;
+  }
+  if (!trial_times(T, T.n)) return 0;
+  int best = 0;  // (a little faster is not enough)
+  for (int i = 1; i < T.n; ++i)
+    if (T.ms[i] > 0.f && (T.ms[best] <= 0.f || T.ms[i] < 0.97f * T.ms[best])) best = i;
+  T.best = best;
+  drop_trial_events(T);
+  return best;
+}
+
+// Around a call by candidate k (pass: of the measurement): the last pass is
+// timed from its first launch on, after a graph's capture.
+void trial_begin(tm_ctx *c, tm_ctx::Trial &T, int k, bool pass) {
+  c->pass_begin = pass && T.passes % kTrialPasses == kTrialPasses - 1 ? T.e[k][0] : nullptr;
+}
+
+void trial_end(tm_ctx::Trial &T, int k, cudaStream_t s) {
+  if (T.passes % kTrialPasses == kTrialPasses - 1) cudaEventRecord(T.e[k][1], s);
+  ++T.passes;
+}
+
+// Candidate k cannot be had for want of memory: out of the trial, if another is left.
+bool trial_drop(tm_ctx::Trial &T, int k) {
+  if (T.n < 2) return false;
+  drop_trial_events(T);
+  for (int i = k; i + 1 < T.n; ++i) T.cand[i] = T.cand[i + 1];
+  --T.n;
+  T.passes = 0;
+  T.best = -1;
+  for (float &ms : T.ms) ms = 0.f;
+  return true;
 }
 
 // Whether a single-image forward on (in, out) runs from a CUDA graph: yes
@@ -1208,38 +1416,38 @@ bool single_graph_ok(tm_ctx *c, const tm_image *in, const tm_image *out, Path pa
   return false;
 }
 
+// One image by `path`, from a cached CUDA graph per image pair unless a per-call
+// feature is on.
+tm_status forward_single(tm_ctx *c, Path path, const tm_image *in, const tm_image *out, cudaStream_t s) {
+  if (path == kPathMaterialised) return forward_materialised(c, in, out, s);
+  const bool graph = !c->stage_timing && !c->debug && !c->reuse_range && single_graph_ok(c, in, out, path);
+  return forward_fused(c, 1, in, out, s, graph, path);
+}
+
 // The forward launch sequence on one image (device buffers already checked).
 tm_status forward_device(tm_ctx *c, const tm_image *in, const tm_image *out, cudaStream_t s) {
   tm_status st = ensure_device_info(c);
   if (st) return st;
   ++c->calls;
-  int path = c->hist_path;
-  if (c->p.n_bins < 2) path = kPathMaterialised;  // no thresholds: nothing to count
-  CompactLayout L;
-  if (path == 0 && !strips(c, 1, in) && compact_fits(c, 1, in, L)) {
-    const bool graph = !c->stage_timing && !c->debug && !c->reuse_range && single_graph_ok(c, in, out, kPathCompact);
-    st = forward_fused(c, 1, in, out, s, graph, &L);
+  c->hint = nullptr;
+  c->pass_begin = nullptr;
+  if (c->p.n_bins < 2) return forward_materialised(c, in, out, s);  // no thresholds: nothing to count
+  if (c->hist_path != 0) {
+    st = forward_single(c, (Path)c->hist_path, in, out, s);
+    return st == TM_EUNSUPPORTED ? fail(c, st, "fused sweep does not fit these fields (use the materialised path)") : st;
+  }
+  for (;;) {
+    size_t group_bytes;
+    tm_ctx::Trial &T = trial_for(c, kTrialSingle, 1, in, out, group_bytes);
+    bool pass;
+    const int k = trial_next(c, T, 1, in, s, pass);
+    trial_begin(c, T, k, pass);
+    st = forward_single(c, (Path)T.cand[k], in, out, s);
+    if (!st && pass) trial_end(T, k, s);
     if (st != TM_ENOMEM) return st;
-    compact_nomem(c, L);  // the other paths need less memory
+    if (T.cand[k] == kPathCompact) compact_nomem(c, T, 0);  // the other paths need less memory
+    else if (!trial_drop(T, k)) return st;
   }
-  if (path == 0) {
-    const auto key = std::make_tuple((int)in->width, (int)in->height, (int)in->dtype, (int)out->dtype);
-    auto it = c->path_choice.find(key);
-    if (it == c->path_choice.end()) {
-      if ((st = choose_path(c, in, out, s, &path))) return st;
-      it = c->path_choice.emplace(key, path).first;
-    }
-    path = it->second;
-  }
-  if (path == 1) {
-    // a cached CUDA graph per image pair unless a per-call feature is on
-    const bool graph = !c->stage_timing && !c->debug && !c->reuse_range && single_graph_ok(c, in, out, kPathSweep);
-    st = forward_fused(c, 1, in, out, s, graph);
-    if (st != TM_EUNSUPPORTED) return st;
-    if (c->hist_path == 1)
-      return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit these fields (use the materialised path)");
-  }
-  return forward_materialised(c, in, out, s);
 }
 
 // The backward's device workspace: a header of the per-image accumulators,
@@ -1342,18 +1550,28 @@ tm_status backward_images(tm_ctx *c, int n, const tm_image *in, const tm_image *
   // the backward takes the fields that the sweep fits, whatever path counts
   for (int i = 0; i < n; ++i)
     if (!sweep_fits(c, &in[i])) return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit these fields");
+  tm_ctx::Trial *trial = nullptr;  // of which this call is a pass, measured as a whole
+  int trial_k = 0;
+  c->hint = nullptr;
+  c->pass_begin = nullptr;
   if (c->bwd_reuse && c->fwd_valid && (int)c->fwd_in.size() == n && same_images(c->fwd_in, in, n)) {
     jobs = c->fwd_jobs;  // the last forward's intermediates of these images are in the workspace
+  } else if (c->hist_path != 0) {
+    if ((st = forward_fused(c, n, in, in, s, false, kPathSweep, 0, false, &jobs))) return st;
+    launches = c->launches;
   } else {
-    const bool compact = c->hist_path == 0 && !strips(c, n, in);
-    CompactLayout L;
-    st = TM_ENOMEM;
-    while (st == TM_ENOMEM && compact && compact_fits(c, n, in, L)) {
-      st = forward_fused(c, n, in, in, s, false, &L, false, &jobs);
-      if (st == TM_ENOMEM) compact_nomem(c, L);
+    for (;;) {
+      size_t group_bytes;
+      tm_ctx::Trial &T = trial_for(c, kTrialBackward, n, in, nullptr, group_bytes);
+      bool pass;
+      trial_k = trial_next(c, T, n, in, s, pass);
+      trial_begin(c, T, trial_k, pass);
+      trial = pass ? &T : nullptr;
+      st = forward_fused(c, n, in, in, s, false, (Path)T.cand[trial_k], group_bytes, false, &jobs);
+      if (!st) break;
+      if (st != TM_ENOMEM || T.cand[trial_k] != kPathCompact) return st;
+      compact_nomem(c, T, group_bytes);
     }
-    if (st == TM_ENOMEM) st = forward_fused(c, n, in, in, s, false, nullptr, false, &jobs);
-    if (st) return st;
     launches = c->launches;
   }
   if ((st = grow_device(c, &c->bws, &c->bws_bytes, need))) return st;
@@ -1438,6 +1656,7 @@ tm_status backward_images(tm_ctx *c, int n, const tm_image *in, const tm_image *
     mark(c, s, ST_BWD_INPUT);
   }
   if ((st = check_launch(c, "backward launch"))) return st;
+  if (trial) trial_end(*trial, trial_k, s);
   c->launches = launches;
   return TM_OK;
 }
@@ -1463,105 +1682,72 @@ tm_status leave_caller(tm_ctx *c, cudaStream_t s, tm_status st) {
   return TM_OK;
 }
 
-// Automatic path of a batch's images that fit the sweep: run the batched
-// fused pass and the batched materialised pass twice each on them (without
-// graphs) and time the second runs with events (synchronising the stream);
-// 1 = fused, 2 = materialised. Both passes give bit-identical outputs (the
-// counts are exact and the lookups share their arithmetic).
-tm_status choose_batch_path(tm_ctx *c, int n, const tm_image *in, const tm_image *out, cudaStream_t s, int stats0,
-                            int *choice) {
-  cudaEvent_t e[4] = {nullptr, nullptr, nullptr, nullptr};
-  for (auto &ev : e) TM_CUDA(c, cudaEventCreate(&ev));
-  tm_status st = TM_OK;
-  for (int rep = 0; rep < 2 && !st; ++rep) {
-    cudaEventRecord(e[0], s);
-    st = forward_fused(c, n, in, out, s, false);
-    cudaEventRecord(e[1], s);
-    if (!st) st = forward_materialised_batch(c, n, in, out, s, false, stats0);
-    cudaEventRecord(e[2], s);
+// A batch by `path`: kPathCompact, all images as one pass (stages
+// "batch_materialised" and "batch_compact"); kPathSweep, those whose fields fit
+// the sweep as one pass (stage "batch") and the others as a materialised one
+// (stage "batch_materialised"); kPathMaterialised, all as a materialised pass.
+// Each pass runs from a CUDA graph.
+tm_status forward_passes(tm_ctx *c, Path path, size_t group_bytes, int n, const tm_image *in, const tm_image *out,
+                         cudaStream_t st) {
+  tm_status s;
+  if (path == kPathCompact) {
+    const int m0 = mark(c, st, -1);
+    if ((s = forward_fused(c, n, in, out, st, true, kPathCompact, group_bytes))) return s;
+    mark(c, st, ST_BATCH_MAT, m0);  // a stored histogram, and the compact one: both from the call's start
+    mark(c, st, ST_BATCH_COMPACT, m0);
+    return TM_OK;
   }
-  float ms_f = 0.f, ms_m = 0.f;
-  if (!st) {
-    cudaError_t r = cudaEventSynchronize(e[2]);
-    if (r == cudaSuccess) r = cudaEventElapsedTime(&ms_f, e[0], e[1]);
-    if (r == cudaSuccess) r = cudaEventElapsedTime(&ms_m, e[1], e[2]);
-    if (r != cudaSuccess) st = cuda_fail(c, r, "timing the batch histogram paths");
-  }
-  for (auto &ev : e)
-    if (ev) cudaEventDestroy(ev);
-  if (st) return st;
-  *choice = ms_f <= ms_m ? 1 : 2;
-  return TM_OK;
-}
-
-// tm_forward_batch on validated arguments, n >= 1. With TM_OPT_HIST_PATH = 0
-// the batch runs on the compact integral histogram as one pass (stages
-// "batch_materialised" and "batch_compact") where every image fits it. Otherwise images whose fields do not fit the
-// sweep take the materialised path, and the others the path measured faster
-// for this batch (cached per context by the images' sizes and dtype pairs),
-// each path's images as one batched pass. Every pass is captured in a graph.
-tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *out, cudaStream_t st) {
-  tm_status s = ensure_device_info(c);
-  if (s) return s;
   std::vector<tm_image> fin, fout, min_, mout;
   for (int i = 0; i < n; ++i) {
-    bool fused = c->p.n_bins > 1 && c->hist_path != 2;
-    if (fused && !sweep_fits(c, &in[i])) {
-      if (c->hist_path == 1)
-        return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit image %d's fields (use the materialised path)", i);
-      fused = false;
-    }
+    const bool fused = path == kPathSweep && sweep_fits(c, &in[i]);
     (fused ? fin : min_).push_back(in[i]);
     (fused ? fout : mout).push_back(out[i]);
   }
-  if ((s = ensure_stats(c, n))) return s;
-  const bool compact = c->hist_path == 0 && !strips(c, n, in);
-  for (CompactLayout L; compact && compact_fits(c, n, in, L); compact_nomem(c, L)) {
-    ++c->calls;
-    const int m0 = mark(c, st, -1);
-    s = forward_fused(c, n, in, out, st, true, &L);
-    if (!s) {  // a stored histogram, and the compact one: both names from the call's start
-      mark(c, st, ST_BATCH_MAT, m0);
-      mark(c, st, ST_BATCH_COMPACT, m0);
-    }
-    if (s != TM_ENOMEM) return s;
-  }
-  if (!fin.empty() && c->hist_path == 0) {
-    std::vector<std::tuple<int, int, int, int>> key;
-    for (size_t i = 0; i < fin.size(); ++i)
-      key.emplace_back((int)fin[i].width, (int)fin[i].height, (int)fin[i].dtype, (int)fout[i].dtype);
-    auto it = c->batch_choice.find(key);
-    if (it == c->batch_choice.end()) {
-      int choice = 1;
-      if ((s = choose_batch_path(c, (int)fin.size(), fin.data(), fout.data(), st, (int)min_.size(), &choice)))
-        return s;
-      it = c->batch_choice.emplace(key, choice).first;
-    }
-    if (it->second == 2) {
-      min_.insert(min_.end(), fin.begin(), fin.end());
-      mout.insert(mout.end(), fout.begin(), fout.end());
-      fin.clear();
-      fout.clear();
-    }
-  }
   int64_t total = 0;
-  ++c->calls;
   if (!fin.empty()) {
     mark(c, st, -1);
-    s = forward_fused(c, (int)fin.size(), fin.data(), fout.data(), st, true);
-    if (s) return s;
+    if ((s = forward_fused(c, (int)fin.size(), fin.data(), fout.data(), st, true, kPathSweep))) return s;
     total += c->launches;
     mark(c, st, ST_BATCH);
+    c->hint = nullptr;  // (one report per call)
   }
   if (!min_.empty()) {
     mark(c, st, -1);
-    s = forward_materialised_batch(c, (int)min_.size(), min_.data(), mout.data(), st, true, (int)fin.size());
+    s = forward_materialised_batch(c, (int)min_.size(), min_.data(), mout.data(), st, (int)fin.size());
     if (s) return s;
     total += c->launches;
     mark(c, st, ST_BATCH_MAT);
   }
   c->launches = total;
   return TM_OK;
+}
+
+// tm_forward_batch on validated arguments, n >= 1.
+tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *out, cudaStream_t st) {
+  tm_status s = ensure_device_info(c);
+  if (s) return s;
+  if (c->hist_path == 1 && c->p.n_bins > 1)
+    for (int i = 0; i < n; ++i)
+      if (!sweep_fits(c, &in[i]))
+        return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit image %d's fields (use the materialised path)", i);
+  if ((s = ensure_stats(c, n))) return s;
+  ++c->calls;
+  c->hint = nullptr;
+  c->pass_begin = nullptr;
+  if (c->p.n_bins < 2) return forward_passes(c, kPathMaterialised, 0, n, in, out, st);
+  if (c->hist_path != 0) return forward_passes(c, (Path)c->hist_path, 0, n, in, out, st);
+  for (;;) {
+    size_t group_bytes;
+    tm_ctx::Trial &T = trial_for(c, kTrialBatch, n, in, out, group_bytes);
+    bool pass;
+    const int k = trial_next(c, T, n, in, st, pass);
+    trial_begin(c, T, k, pass);
+    s = forward_passes(c, (Path)T.cand[k], group_bytes, n, in, out, st);
+    if (!s && pass) trial_end(T, k, st);
+    if (s != TM_ENOMEM) return s;
+    if (T.cand[k] == kPathCompact) compact_nomem(c, T, group_bytes);  // smaller groups, then the other paths
+    else if (!trial_drop(T, k)) return s;
+  }
 }
 
 extern "C" {
@@ -1617,6 +1803,8 @@ void tm_destroy(tm_ctx *c) {
       c->hslot[0])
     cudaDeviceSynchronize();
   drop_graph(c);
+  drop_trials(c);
+  if (c->hints) cudaFreeHost(c->hints);
   for (auto &call : c->marks)
     for (auto &m : call) cudaEventDestroy(m.e);
   for (cudaEvent_t e : c->event_pool) cudaEventDestroy(e);
@@ -2005,8 +2193,7 @@ tm_status tm_set_option(tm_ctx *c, int32_t key, int64_t value) {
       return fail(c, TM_EINVAL, "TM_OPT_SWEEP_WIDTH value %lld (0, 256 or 512)", (long long)value);
     if (c->sweep_width != (int)value) {
       drop_graph(c);
-      c->path_choice.clear();  // the timed path choices saw the other width
-      c->batch_choice.clear();
+      drop_trials(c);  // the measured choices saw the other width
     }
     c->sweep_width = (int)value;
     return TM_OK;
@@ -2014,8 +2201,7 @@ tm_status tm_set_option(tm_ctx *c, int32_t key, int64_t value) {
   if (key == TM_OPT_HIST_PATH) {
     if (value < 0 || value > 2) return fail(c, TM_EINVAL, "TM_OPT_HIST_PATH value %lld", (long long)value);
     c->hist_path = (int)value;
-    c->path_choice.clear();
-    c->batch_choice.clear();
+    drop_trials(c);
     c->compact_failed = SIZE_MAX;
     return TM_OK;
   }
