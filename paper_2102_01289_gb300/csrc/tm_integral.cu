@@ -15,6 +15,7 @@
 // histogram planes), so box sums (Eq. 6, Eq. 9) are exact whatever the image
 // size or summation order.
 #include <algorithm>
+#include <type_traits>
 #include <cstdint>
 
 #include "tm_kernels.cuh"
@@ -551,14 +552,21 @@ __global__ void __launch_bounds__(kINT, 4) k_fix_write(const FixJob *__restrict_
 //      indicator masks and the popcounts of their low bits the row prefixes.
 //      What lies left of a strip comes from the strips' row totals, exchanged
 //      once per 32 rows.
+// Where segments x planes leave SMs idle and the rows are long, a segment is
+// divided into parts of whole passes, a block each; more blocks of launch 1
+// then give the strips' row totals and their sums over a segment, from which a
+// part takes what lies left of it (hist_parts has the rule). With one block for
+// the whole width 64 x 16384 with 2 bins took 182 us, 256 x 16384 189 and 2160
+// x 3840 78 (55, 61 and 72 over the int64 tiles); now 30, 32 and 46.
 // Bound by the writes (4 bytes per element; the bin map stays in L2) and by
 // issue (105 warp instructions per strip row and plane). 32 planes of 1080p
-// (265 MB) took 230 us over the int64 tiles of the integral images and take 100
-// (counts 13, mid 10, writes 77).
+// (265 MB) took 230 us over the int64 tiles of the integral images and take 90
+// (counts 13, writes 77).
 constexpr int kHW = 8;                  // strips (warps) of a block's pass
 constexpr int kHStrip = 128;            // columns of a strip
 constexpr int kHCols = kHW * kHStrip;   // columns of a pass
 constexpr int kHDirect = 32;            // segments whose counts the write pass adds up
+constexpr int kHBlocks = 152;           // fewer blocks of the write pass than SMs: their segments are divided
 
 struct HistPlanes {
   const uint8_t *bins;
@@ -568,9 +576,56 @@ struct HistPlanes {
   int summed;        // the counts have been replaced by those of the segments above
 };
 
+// With more than one part of `cols` columns (a multiple of kHCols) per segment.
+struct HistParts : HistPlanes {
+  int cols;
+  uint32_t *segtot;  // nseg x n_planes x strips: the plane's pixels of a segment's strip
+  uint8_t *rowtot;   // strips x n_planes x H: of a strip's row
+};
+
+// Launch 1's other blocks: the totals of strip s in segment seg, per row and
+// over the segment. Plane p as in k_hist_cols.
+__device__ __forceinline__ void hist_strip_totals(const HistParts &Q, int s, int seg, unsigned *sum) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, strips = (Q.W + kHStrip - 1) / kHStrip;
+  const int r0 = seg * Q.seg_rows, r1 = min(r0 + Q.seg_rows, Q.H);
+  const int c = s * kHStrip + lane;
+  for (int p = threadIdx.x; p < Q.n_planes; p += kHStrip) sum[p] = 0;
+  __syncthreads();
+  for (int r = r0 + 4 * wid; r < r1; r += kHStrip / 8) {  // four rows per warp and step
+    int v[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        v[u][m] = r + u < r1 && c + 32 * m < Q.W ? (int)__ldg(Q.bins + (size_t)(r + u) * Q.W + c + 32 * m) : 256;
+    for (int p = 0; p < Q.n_planes; ++p) {
+      const int k = Q.k_begin + p;
+      unsigned t = 0;  // the rows' totals, a byte each
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        unsigned n = 0;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) n += Q.eq ? v[u][m] == k : v[u][m] < k;
+        t |= n << (8 * u);
+      }
+      t = __reduce_add_sync(0xffffffffu, t);  // at most 128 each
+      if (lane < 4 && r + lane < r1) Q.rowtot[((size_t)s * Q.n_planes + p) * Q.H + r + lane] = (uint8_t)(t >> (8 * lane));
+      if (lane == 0) atomicAdd(&sum[p], (t & 0xffu) + ((t >> 8) & 0xffu) + ((t >> 16) & 0xffu) + (t >> 24));
+    }
+  }
+  __syncthreads();
+  for (int p = threadIdx.x; p < Q.n_planes; p += kHStrip) Q.segtot[((size_t)seg * Q.n_planes + p) * strips + s] = sum[p];
+}
+
 // Plane p indicates [b == k] (eq) or [b < k], k = k_begin + p.
-__global__ void __launch_bounds__(kHStrip) k_hist_cols(const __grid_constant__ HistPlanes Q) {
+template <class Args>
+__global__ void __launch_bounds__(kHStrip) k_hist_cols(const __grid_constant__ Args Q) {
   extern __shared__ unsigned hcount[];  // [n_planes][kHStrip]
+  if constexpr (std::is_same<Args, HistParts>::value)
+    if ((int)blockIdx.y >= Q.nseg) {
+      hist_strip_totals(Q, blockIdx.x, blockIdx.y - Q.nseg, hcount);
+      return;
+    }
   const int c = blockIdx.x * kHStrip + threadIdx.x, seg = blockIdx.y;
   for (int p = 0; p < Q.n_planes; ++p) hcount[p * kHStrip + threadIdx.x] = 0;
   if (c >= Q.W) return;  // (a thread only touches its own column)
@@ -620,9 +675,10 @@ __device__ __forceinline__ unsigned warp_inclusive(unsigned v) {
   return v;
 }
 
-// kEq: Q.eq.
-template <bool kEq>
-__global__ void __launch_bounds__(32 * kHW, 5) k_hist_write(const __grid_constant__ HistPlanes Q) {
+// kEq: Q.eq. Args: HistPlanes, or HistParts (undivided segments take 3 to 5 %
+// longer with the parts compiled in: 3000 x 4000, 8 bins, 138 and 145 us).
+template <bool kEq, class Args>
+__global__ void __launch_bounds__(32 * kHW, 5) k_hist_write(const __grid_constant__ Args Q) {
   // [2][seg_rows]: the rows' totals of the passes before, read by one pass
   // while it writes the next one's (only where the image takes several)
   extern __shared__ unsigned left[];
@@ -637,14 +693,40 @@ __global__ void __launch_bounds__(32 * kHW, 5) k_hist_write(const __grid_constan
   const size_t W1 = (size_t)W + 1;
   uint32_t *const plane = Q.planes + (size_t)p * W1 * ((size_t)H + 1);
   const bool passes = W > kHCols;
-  for (int r = threadIdx.x; r < Q.seg_rows && passes; r += 32 * kHW) left[r] = 0;
-  if (seg == 0)
-    for (int c = threadIdx.x; c <= W; c += 32 * kHW) plane[c] = 0;
-  for (int r = r0 + (int)threadIdx.x; r < r1; r += 32 * kHW) plane[(size_t)(r + 1) * W1] = 0;
   unsigned carry = 0;  // the passes before: their columns' total in the segments above
+  int Cs = 0, Ce = W;  // the block's columns
+  if constexpr (std::is_same<Args, HistParts>::value) {
+    Cs = (int)blockIdx.y * Q.cols;
+    Ce = W - Cs > Q.cols ? Cs + Q.cols : W;
+    const int strips = (W + kHStrip - 1) / kHStrip, s1 = Cs / kHStrip;
+    if (seg == 0)
+      for (int c = Cs + (int)threadIdx.x; c < Ce; c += 32 * kHW) plane[c + 1] = 0;
+    if (seg == 0 && Cs == 0 && threadIdx.x == 0) plane[0] = 0;
+    for (int r = r0 + (int)threadIdx.x; r < r1; r += 32 * kHW) {
+      if (Cs == 0) plane[(size_t)(r + 1) * W1] = 0;
+      const uint8_t *t = Q.rowtot + (size_t)p * H + r;
+      unsigned n = 0;
+#pragma unroll 16
+      for (int s = 0; s < s1; ++s) n += __ldg(t + (size_t)s * Q.n_planes * H);
+      left[r - r0] = n;
+    }
+    for (int q = wid; q < seg; q += kHW)
+#pragma unroll 4
+      for (int s = lane; s < s1; s += 32) carry += __ldg(Q.segtot + ((size_t)q * Q.n_planes + p) * strips + s);
+    carry = __reduce_add_sync(0xffffffffu, carry);
+    if (lane == 0) above[wid] = carry;
+    __syncthreads();
+    carry = 0;
+    for (int w = 0; w < kHW; ++w) carry += above[w];
+  } else {
+    for (int r = threadIdx.x; r < Q.seg_rows && passes; r += 32 * kHW) left[r] = 0;
+    if (seg == 0)
+      for (int c = threadIdx.x; c <= W; c += 32 * kHW) plane[c] = 0;
+    for (int r = r0 + (int)threadIdx.x; r < r1; r += 32 * kHW) plane[(size_t)(r + 1) * W1] = 0;
+  }
   const unsigned le = 0xffffffffu >> (31 - lane);
   int flip = 0, par = 0;
-  for (int C0 = 0; C0 < W; C0 += kHCols, par ^= 1) {
+  for (int C0 = Cs; C0 < Ce; C0 += kHCols, par ^= 1) {
     const int c0 = C0 + wid * kHStrip;  // the warp's strip
     unsigned acc[4];                    // columns c0 + 32 m + lane
     bool ok[4];
@@ -796,15 +878,49 @@ static void hist_layout(int H, int &nseg, int &seg_rows) {
   nseg = (H + seg_rows - 1) / seg_rows;
 }
 
+// The parts of a segment, of whole passes: where there are fewer blocks than
+// SMs, as many as give two per SM, if the passes that a block is spared (about
+// 1 us + 0.16 us per row each) take longer than the strips' totals (0.6 us per
+// plane). 64 rows of 2048 columns, undivided and in parts, us: 8 bins 34.6 and
+// 27.9, 16 34.9 and 32.1, 32 35.5 and 40.1, 64 36 and 56; of 16384 columns, 64
+// bins 254 and 131, 256 bins 330 and 445. With 256 blocks (512 x 4096, 32 bins)
+// 105 undivided and 110.
+static void hist_parts(int W, int H, int nseg, int seg_rows, int planes, int &parts, int &cols) {
+  const long long pass = ((long long)W + kHCols - 1) / kHCols, blocks = (long long)nseg * planes;
+  const long long want = blocks < kHBlocks ? std::min(pass, (2 * kHBlocks + blocks - 1) / blocks) : 1;
+  long long per = (pass + want - 1) / want;
+  if ((pass - per) * (1.0 + 0.16 * std::min(seg_rows, H)) < 0.6 * planes) per = pass;
+  cols = (int)std::min<long long>(per * kHCols, W);
+  parts = (int)((W + (long long)cols - 1) / cols);
+}
+
 size_t hist_scratch_bytes(int W, int H, int planes) {
-  int nseg, seg_rows;
+  int nseg, seg_rows, parts, cols;
   hist_layout(H, nseg, seg_rows);
-  return sizeof(uint32_t) * (size_t)std::max(planes, 1) * nseg * W;
+  planes = std::max(planes, 1);
+  hist_parts(W, H, nseg, seg_rows, planes, parts, cols);
+  const size_t counts = sizeof(uint32_t) * (size_t)planes * nseg * W, strips = ((size_t)W + kHStrip - 1) / kHStrip;
+  return counts + (parts > 1 ? strips * planes * (sizeof(uint32_t) * nseg + H) : 0);
+}
+
+template <class Args>
+static int launch_hist(Args Q, int parts, cudaStream_t s) {
+  const size_t smem = sizeof(unsigned) * kHStrip * (size_t)Q.n_planes;  // at most 128 KB
+  cudaFuncSetAttribute(k_hist_cols<Args>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)(sizeof(unsigned) * kHStrip * kMaxBins));
+  k_hist_cols<Args><<<dim3((unsigned)((Q.W + kHStrip - 1) / kHStrip), (unsigned)(parts > 1 ? 2 * Q.nseg : Q.nseg)),
+                      kHStrip, smem, s>>>(Q);
+  Q.summed = Q.nseg > kHDirect ? 1 : 0;
+  if (Q.summed) k_hist_mid<<<(unsigned)(((size_t)Q.n_planes * Q.W + 127) / 128), 128, 0, s>>>(Q);
+  auto *const write = Q.eq ? k_hist_write<true, Args> : k_hist_write<false, Args>;
+  write<<<dim3((unsigned)(Q.nseg * Q.n_planes), (unsigned)parts), 32 * kHW,
+          Q.W > kHCols ? 2 * sizeof(unsigned) * Q.seg_rows : 0, s>>>(Q);
+  return 2 + Q.summed;
 }
 
 int launch_integral_histogram(const uint8_t *bins, int W, int H, int n_bins, bool cumulative,
                               uint32_t *planes, void *scratch, cudaStream_t s) {
-  HistPlanes Q{};
+  HistParts Q{};
   Q.bins = bins;
   Q.planes = planes;
   Q.counts = static_cast<uint32_t *>(scratch);
@@ -815,15 +931,15 @@ int launch_integral_histogram(const uint8_t *bins, int W, int H, int n_bins, boo
   Q.eq = cumulative ? 0 : 1;
   if (Q.n_planes <= 0) return 0;
   hist_layout(H, Q.nseg, Q.seg_rows);
-  const size_t smem = sizeof(unsigned) * kHStrip * (size_t)Q.n_planes;  // at most 128 KB
-  cudaFuncSetAttribute(k_hist_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)(sizeof(unsigned) * kHStrip * kMaxBins));
-  k_hist_cols<<<dim3((unsigned)((W + kHStrip - 1) / kHStrip), (unsigned)Q.nseg), kHStrip, smem, s>>>(Q);
-  Q.summed = Q.nseg > kHDirect ? 1 : 0;
-  if (Q.summed) k_hist_mid<<<(unsigned)(((size_t)Q.n_planes * W + 127) / 128), 128, 0, s>>>(Q);
-  auto *const write = cumulative ? k_hist_write<false> : k_hist_write<true>;
-  write<<<(unsigned)(Q.nseg * Q.n_planes), 32 * kHW, W > kHCols ? 2 * sizeof(unsigned) * Q.seg_rows : 0, s>>>(Q);
-  return 2 + Q.summed;
+  int parts;
+  hist_parts(W, H, Q.nseg, Q.seg_rows, Q.n_planes, parts, Q.cols);
+  if (parts > 1) {
+    const size_t strips = ((size_t)W + kHStrip - 1) / kHStrip;
+    Q.segtot = Q.counts + (size_t)Q.nseg * Q.n_planes * W;
+    Q.rowtot = reinterpret_cast<uint8_t *>(Q.segtot + (size_t)Q.nseg * Q.n_planes * strips);
+    return launch_hist(Q, parts, s);
+  }
+  return launch_hist<HistPlanes>(Q, 1, s);
 }
 
 }  // namespace tmk
