@@ -502,12 +502,22 @@ size_t sweep_count_bytes(const DevParams &P, const SweepPlan &S, long long *off)
   return o;
 }
 
+// The dynamic shared memory that plans stay within. A kernel's limit is state
+// shared by every thread of the process: always this, not the call's own size,
+// so that no context lowers it under another's launch.
+static int smem_most() {
+  int dev = 0, v = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return v - 2048;
+}
+
 template <int NF, int TX>
 static int launch_nf(const DevParams &P, const Job *jobs, int njobs, int nitems, int *queue, size_t smem,
                      int ctas, cudaStream_t s) {
   const bool incl = (P.flags & kFlagCdfIncl) != 0;
   auto *k = incl ? k_sweep<NF, TX, true> : k_sweep<NF, TX, false>;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_most()) != cudaSuccess) return -1;
   k<<<ctas, Shape<TX>::NT, smem, s>>>(P, jobs, njobs, nitems, queue);
   return 1;
 }
@@ -517,9 +527,9 @@ static int ctas_per_sm(int n_fields, size_t smem) {
   int per = 0;
   cudaError_t e;
   switch (n_fields) {
-#define TM_OCC(nf)                                                                                          \
+#define TM_OCC(nf)                                                                                            \
   case nf:                                                                                                  \
-    e = cudaFuncSetAttribute(k_sweep<nf, TX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+    e = cudaFuncSetAttribute(k_sweep<nf, TX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_most()); \
     if (e == cudaSuccess)                                                                                   \
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sweep<nf, TX, false>, Shape<TX>::NT, smem); \
     break;
