@@ -71,8 +71,8 @@ struct tm_ctx {
   int hist_path = 0;
   int sweep_tiles = 0;  // TM_OPT_SWEEP_TILES (0: one wave of the sweep's CTAs per image share)
   int sweep_width = 0;  // TM_OPT_SWEEP_WIDTH (0: automatic)
-  // the compact integral histogram's bytes that could not be had, at which call
-  // (a smaller request is tried, and any after kCompactRetry calls)
+  // the compact integral histogram's bytes that could not be had, at which of the
+  // trial_asks (a smaller request is tried, and any after kCompactRetry of them)
   size_t compact_failed = SIZE_MAX;
   uint64_t compact_failed_at = 0;
   int64_t launches = 0;
@@ -653,8 +653,8 @@ bool sweep_fits(tm_ctx *c, const tm_image *in) {
                     std::min(c->smem_optin - 2048, (size_t)110 * 1024), 256, plan);
 }
 
-// A request that failed is tried again after this many forward calls: the
-// shortage may have passed (a failing one costs the workspace's reallocation).
+// A request that failed is tried again after this many calls: the shortage may
+// have passed (a failing one costs the workspace's reallocation).
 constexpr uint64_t kCompactRetry = 256;
 
 // How the compact integral histograms of a call's images are held: images are
@@ -1257,7 +1257,7 @@ tm_ctx::Trial &trial_for(tm_ctx *c, TrialKind kind, int n, const tm_image *in, c
       }
       it = c->trials.emplace(key, T).first;
     }
-    const size_t most = c->calls - c->compact_failed_at < kCompactRetry ? c->compact_failed : SIZE_MAX;
+    const size_t most = c->trial_asks - c->compact_failed_at < kCompactRetry ? c->compact_failed : SIZE_MAX;
     group_bytes = it->second.bytes[0] < most ? kCompactGroup : 0;
     if (it->second.bytes[1] < most || !key[1]) break;
     key[1] = 0;
@@ -1285,7 +1285,7 @@ tm_ctx::Trial &trial_for(tm_ctx *c, TrialKind kind, int n, const tm_image *in, c
 // The compact path's memory could not be had in groups of group_bytes.
 void compact_nomem(tm_ctx *c, const tm_ctx::Trial &T, size_t group_bytes) {
   c->compact_failed = T.bytes[group_bytes ? 0 : 1];
-  c->compact_failed_at = c->calls;
+  c->compact_failed_at = c->trial_asks;
 }
 
 bool capturing(cudaStream_t s) {

@@ -284,3 +284,38 @@ def test_more_sizes_than_are_kept():
                     assert torch.equal(y, r)
     finally:
         tm.tm_destroy(ctx)
+
+
+def test_short_memory_in_the_backward_passes_too():
+    """The backward's recomputation of a 12 MP image without the memory for the
+    compact histogram, and 256 calls later with it: the gradients of the sweep."""
+    p = tm.make_params(64, [4])
+    x, small = _images([(4000, 3000), (300, 200)], 9)
+    g, gin, gp = torch.randn_like(x), torch.empty_like(x), torch.empty(5, device="cuda")
+    gs, gsin = torch.randn_like(small), torch.empty_like(small)
+    got = []
+    for path in (1, 0):
+        ctx = tm.tm_create(p)
+        hold = None
+        try:
+            tm.tm_set_option(ctx, tm.TM_OPT_HIST_PATH, path)
+            if path == 0:
+                hold = _all_but(2000 << 20)  # (the backward's own workspace takes 0.8 GB)
+            names = _stages(ctx, lambda: tm.tm_backward(ctx, x, g, gin, gp))
+            torch.cuda.synchronize()
+            assert "fused_sweep" in names
+            got.append(gin.clone() if path else gin)
+            if path == 0:
+                assert torch.equal(*got)
+                hold = None
+                torch.cuda.empty_cache()
+                assert "compact_histogram" in _stages(ctx, lambda: tm.tm_backward(ctx, small, gs, gsin, gp))
+                for _ in range(256):
+                    tm.tm_backward(ctx, small, gs, gsin, gp)
+                assert "compact_histogram" in _stages(ctx, lambda: tm.tm_backward(ctx, x, g, gin, gp))
+                torch.cuda.synchronize()
+                assert torch.equal(*got)
+        finally:
+            tm.tm_destroy(ctx)
+            hold = None
+            torch.cuda.empty_cache()
