@@ -15,6 +15,7 @@
 // histogram planes), so box sums (Eq. 6, Eq. 9) are exact whatever the image
 // size or summation order.
 #include <algorithm>
+#include <climits>
 #include <type_traits>
 #include <cstdint>
 
@@ -576,28 +577,43 @@ struct HistPlanes {
   int summed;        // the counts have been replaced by those of the segments above
 };
 
-// With more than one part of `cols` columns (a multiple of kHCols) per segment.
+// With more than one part of `cols` columns (a multiple of kHCols) per segment,
+// or with a side near 2^31: its kernels count columns and rows in unsigned
+// (Index), which the ordinary ones would pay for (256 x 256, 8 bins, 22.0 and
+// 23.8 us; 100000 x 16, 64 bins, 3910 and 3994).
 struct HistParts : HistPlanes {
   int cols;
   uint32_t *segtot;  // nseg x n_planes x strips: the plane's pixels of a segment's strip
   uint8_t *rowtot;   // strips x n_planes x H: of a strip's row
 };
 
+template <class Args>
+constexpr bool kHParts = std::is_same<Args, HistParts>::value;
+template <class Args>
+using Index = typename std::conditional<kHParts<Args>, unsigned, int>::type;
+
+// The end of the segment of rows that begins at r0.
+template <class Args>
+__device__ __forceinline__ int segment_end(const Args &Q, int r0) {
+  if (kHParts<Args>) return Q.H - r0 > Q.seg_rows ? r0 + Q.seg_rows : Q.H;
+  return min(r0 + Q.seg_rows, Q.H);
+}
+
 // Launch 1's other blocks: the totals of strip s in segment seg, per row and
 // over the segment. Plane p as in k_hist_cols.
 __device__ __forceinline__ void hist_strip_totals(const HistParts &Q, int s, int seg, unsigned *sum) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, strips = (Q.W + kHStrip - 1) / kHStrip;
-  const int r0 = seg * Q.seg_rows, r1 = min(r0 + Q.seg_rows, Q.H);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, strips = (Q.W - 1) / kHStrip + 1;
+  const int r0 = seg * Q.seg_rows, r1 = segment_end(Q, r0);
   const int c = s * kHStrip + lane;
   for (int p = threadIdx.x; p < Q.n_planes; p += kHStrip) sum[p] = 0;
   __syncthreads();
-  for (int r = r0 + 4 * wid; r < r1; r += kHStrip / 8) {  // four rows per warp and step
+  for (unsigned r = r0 + 4 * wid; r < (unsigned)r1; r += kHStrip / 8) {  // four rows per warp and step
     int v[4][4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
       for (int m = 0; m < 4; ++m)
-        v[u][m] = r + u < r1 && c + 32 * m < Q.W ? (int)__ldg(Q.bins + (size_t)(r + u) * Q.W + c + 32 * m) : 256;
+        v[u][m] = r + u < (unsigned)r1 && c + 32 * m < Q.W ? (int)__ldg(Q.bins + (size_t)(r + u) * Q.W + c + 32 * m) : 256;
     for (int p = 0; p < Q.n_planes; ++p) {
       const int k = Q.k_begin + p;
       unsigned t = 0;  // the rows' totals, a byte each
@@ -609,7 +625,8 @@ __device__ __forceinline__ void hist_strip_totals(const HistParts &Q, int s, int
         t |= n << (8 * u);
       }
       t = __reduce_add_sync(0xffffffffu, t);  // at most 128 each
-      if (lane < 4 && r + lane < r1) Q.rowtot[((size_t)s * Q.n_planes + p) * Q.H + r + lane] = (uint8_t)(t >> (8 * lane));
+      if (lane < 4 && r + lane < (unsigned)r1)
+        Q.rowtot[((size_t)s * Q.n_planes + p) * Q.H + r + lane] = (uint8_t)(t >> (8 * lane));
       if (lane == 0) atomicAdd(&sum[p], (t & 0xffu) + ((t >> 8) & 0xffu) + ((t >> 16) & 0xffu) + (t >> 24));
     }
   }
@@ -621,7 +638,7 @@ __device__ __forceinline__ void hist_strip_totals(const HistParts &Q, int s, int
 template <class Args>
 __global__ void __launch_bounds__(kHStrip) k_hist_cols(const __grid_constant__ Args Q) {
   extern __shared__ unsigned hcount[];  // [n_planes][kHStrip]
-  if constexpr (std::is_same<Args, HistParts>::value)
+  if constexpr (kHParts<Args>)
     if ((int)blockIdx.y >= Q.nseg) {
       hist_strip_totals(Q, blockIdx.x, blockIdx.y - Q.nseg, hcount);
       return;
@@ -629,12 +646,12 @@ __global__ void __launch_bounds__(kHStrip) k_hist_cols(const __grid_constant__ A
   const int c = blockIdx.x * kHStrip + threadIdx.x, seg = blockIdx.y;
   for (int p = 0; p < Q.n_planes; ++p) hcount[p * kHStrip + threadIdx.x] = 0;
   if (c >= Q.W) return;  // (a thread only touches its own column)
-  const int r0 = seg * Q.seg_rows, r1 = min(r0 + Q.seg_rows, Q.H);
+  const int r0 = seg * Q.seg_rows, r1 = segment_end(Q, r0);
   const uint8_t *b = Q.bins + (size_t)r0 * Q.W + c;
-  for (int r = r0; r < r1; r += 8) {
+  for (Index<Args> r = r0; r < (Index<Args>)r1; r += 8) {
     int v[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = r + u < r1 ? (int)__ldg(b + (size_t)u * Q.W) : 256;
+    for (int u = 0; u < 8; ++u) v[u] = r + u < (Index<Args>)r1 ? (int)__ldg(b + (size_t)u * Q.W) : 256;
 #pragma unroll
     for (int u = 0; u < 8; ++u)
       if (v[u] < Q.n_planes) ++hcount[v[u] * kHStrip + threadIdx.x];
@@ -689,26 +706,28 @@ __global__ void __launch_bounds__(32 * kHW, 5) k_hist_write(const __grid_constan
   const int W = Q.W, H = Q.H, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int p = blockIdx.x % Q.n_planes, seg = blockIdx.x / Q.n_planes;
   const int k = Q.k_begin + p;
-  const int r0 = seg * Q.seg_rows, r1 = min(r0 + Q.seg_rows, H);
+  const int r0 = seg * Q.seg_rows, r1 = segment_end(Q, r0);
   const size_t W1 = (size_t)W + 1;
   uint32_t *const plane = Q.planes + (size_t)p * W1 * ((size_t)H + 1);
   const bool passes = W > kHCols;
   unsigned carry = 0;  // the passes before: their columns' total in the segments above
   int Cs = 0, Ce = W;  // the block's columns
-  if constexpr (std::is_same<Args, HistParts>::value) {
+  if constexpr (kHParts<Args>) {
     Cs = (int)blockIdx.y * Q.cols;
     Ce = W - Cs > Q.cols ? Cs + Q.cols : W;
-    const int strips = (W + kHStrip - 1) / kHStrip, s1 = Cs / kHStrip;
+    const int strips = (W - 1) / kHStrip + 1, s1 = Cs / kHStrip;
     if (seg == 0)
-      for (int c = Cs + (int)threadIdx.x; c < Ce; c += 32 * kHW) plane[c + 1] = 0;
+      for (unsigned c = Cs + threadIdx.x; c < (unsigned)Ce; c += 32 * kHW) plane[c + 1] = 0;
     if (seg == 0 && Cs == 0 && threadIdx.x == 0) plane[0] = 0;
-    for (int r = r0 + (int)threadIdx.x; r < r1; r += 32 * kHW) {
-      if (Cs == 0) plane[(size_t)(r + 1) * W1] = 0;
+    if (Cs == 0)
+      for (unsigned r = r0 + threadIdx.x; r < (unsigned)r1; r += 32 * kHW) plane[(size_t)(r + 1) * W1] = 0;
+    for (unsigned r = r0 + wid; r < (unsigned)r1 && passes; r += kHW) {  // a warp per row (more parts: more passes)
       const uint8_t *t = Q.rowtot + (size_t)p * H + r;
       unsigned n = 0;
-#pragma unroll 16
-      for (int s = 0; s < s1; ++s) n += __ldg(t + (size_t)s * Q.n_planes * H);
-      left[r - r0] = n;
+#pragma unroll 8
+      for (int s = lane; s < s1; s += 32) n += __ldg(t + (size_t)s * Q.n_planes * H);
+      n = __reduce_add_sync(0xffffffffu, n);
+      if (lane == 0) left[r - r0] = n;
     }
     for (int q = wid; q < seg; q += kHW)
 #pragma unroll 4
@@ -726,8 +745,8 @@ __global__ void __launch_bounds__(32 * kHW, 5) k_hist_write(const __grid_constan
   }
   const unsigned le = 0xffffffffu >> (31 - lane);
   int flip = 0, par = 0;
-  for (int C0 = Cs; C0 < Ce; C0 += kHCols, par ^= 1) {
-    const int c0 = C0 + wid * kHStrip;  // the warp's strip
+  for (Index<Args> C0 = Cs; C0 < (Index<Args>)Ce; C0 += kHCols, par ^= 1) {
+    const int c0 = (int)C0 + wid * kHStrip;  // the warp's strip
     unsigned acc[4];                    // columns c0 + 32 m + lane
     bool ok[4];
 #pragma unroll
@@ -756,8 +775,8 @@ __global__ void __launch_bounds__(32 * kHW, 5) k_hist_write(const __grid_constan
       if (w < wid) base += above[w];
       carry += above[w];
     }
-    for (int rb = r0; rb < r1; rb += 32, flip ^= 1) {
-      const int n = min(32, r1 - rb);
+    for (Index<Args> rb = r0; rb < (Index<Args>)r1; rb += 32, flip ^= 1) {
+      const int n = min(32, r1 - (int)rb);
       const uint8_t *b = Q.bins + (size_t)rb * W + c0 + lane;
       uint4 rw = make_uint4(0u, 0u, 0u, 0u);  // lane = row: its masks
       for (int i = 0; i < n; i += 4) {
@@ -875,7 +894,7 @@ static void hist_layout(int H, int &nseg, int &seg_rows) {
   seg_rows = 64;
   const long long most = 4096LL * 64;
   if (H > most) seg_rows = (int)(((long long)H + 4095) / 4096 + 31) / 32 * 32;
-  nseg = (H + seg_rows - 1) / seg_rows;
+  nseg = (int)(((long long)H + seg_rows - 1) / seg_rows);
 }
 
 // The parts of a segment, of whole passes: where there are fewer blocks than
@@ -908,13 +927,15 @@ static int launch_hist(Args Q, int parts, cudaStream_t s) {
   const size_t smem = sizeof(unsigned) * kHStrip * (size_t)Q.n_planes;  // at most 128 KB
   cudaFuncSetAttribute(k_hist_cols<Args>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)(sizeof(unsigned) * kHStrip * kMaxBins));
-  k_hist_cols<Args><<<dim3((unsigned)((Q.W + kHStrip - 1) / kHStrip), (unsigned)(parts > 1 ? 2 * Q.nseg : Q.nseg)),
+  k_hist_cols<Args><<<dim3((unsigned)((Q.W - 1) / kHStrip + 1), (unsigned)(parts > 1 ? 2 * Q.nseg : Q.nseg)),
                       kHStrip, smem, s>>>(Q);
   Q.summed = Q.nseg > kHDirect ? 1 : 0;
   if (Q.summed) k_hist_mid<<<(unsigned)(((size_t)Q.n_planes * Q.W + 127) / 128), 128, 0, s>>>(Q);
   auto *const write = Q.eq ? k_hist_write<true, Args> : k_hist_write<false, Args>;
-  write<<<dim3((unsigned)(Q.nseg * Q.n_planes), (unsigned)parts), 32 * kHW,
-          Q.W > kHCols ? 2 * sizeof(unsigned) * Q.seg_rows : 0, s>>>(Q);
+  const size_t left = Q.W > kHCols ? 2 * sizeof(unsigned) * (size_t)Q.seg_rows : 0;
+  if (left > 40 * 1024)  // (more than 20 M rows)
+    cudaFuncSetAttribute(write, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  write<<<dim3((unsigned)(Q.nseg * Q.n_planes), (unsigned)parts), 32 * kHW, left, s>>>(Q);
   return 2 + Q.summed;
 }
 
@@ -933,11 +954,12 @@ int launch_integral_histogram(const uint8_t *bins, int W, int H, int n_bins, boo
   hist_layout(H, Q.nseg, Q.seg_rows);
   int parts;
   hist_parts(W, H, Q.nseg, Q.seg_rows, Q.n_planes, parts, Q.cols);
-  if (parts > 1) {
+  constexpr int kFar = INT_MAX - (1 << 20);  // (int counters may not pass a side by a step)
+  if (parts > 1 || W > kFar || H > kFar) {
     const size_t strips = ((size_t)W + kHStrip - 1) / kHStrip;
     Q.segtot = Q.counts + (size_t)Q.nseg * Q.n_planes * W;
     Q.rowtot = reinterpret_cast<uint8_t *>(Q.segtot + (size_t)Q.nseg * Q.n_planes * strips);
-    return launch_hist(Q, parts, s);
+    return launch_hist<HistParts>(Q, parts, s);
   }
   return launch_hist<HistPlanes>(Q, 1, s);
 }

@@ -54,6 +54,28 @@ def test_cumulative_planes_in_parts(H, W, n):
     assert torch.equal(*got)
 
 
+@pytest.mark.parametrize("H,W", [(1, 2 ** 31 - 1), (2 ** 31 - 1, 1), (2 ** 21, 1025)])
+def test_sides_up_to_the_largest(H, W):
+    """Maps of 2^31 pixels, one row, one column and two passes: one plane."""
+    if torch.cuda.mem_get_info()[0] < 120 * 2 ** 30:
+        pytest.skip("needs 120 GB of device memory")
+    bins = torch.zeros((H, W), dtype=torch.uint8, device="cuda")
+    bins.view(-1)[::3] = 1
+    hk = torch.full((2, H + 1, W + 1), -1, dtype=torch.int32, device="cuda")
+    tm.tm_integral_histogram(bins, 2, hk)
+    assert int(hk[:, 0].abs().max()) == 0 and int(hk[:, :, 0].abs().max()) == 0
+    row = min(H, 5)  # the first rows, and the last row: (entries are modulo 2^32)
+    ones = (bins[:row] == 1).to(torch.int64).cumsum(1).cumsum(0)
+    assert torch.equal(hk[1, 1:row + 1, 1:].to(torch.int64), ones)
+    del ones
+    cols = torch.zeros(W, dtype=torch.int64, device="cuda")
+    for part in bins.split(1 << 18):
+        cols += (part == 1).sum(0)
+    assert torch.equal(hk[1, H, 1:].to(torch.int64) & 0xffffffff, cols.cumsum(0))
+    area = torch.arange(1, W + 1, dtype=torch.int64, device="cuda") * H
+    assert torch.equal((hk[0, H, 1:].to(torch.int64) + hk[1, H, 1:].to(torch.int64)) & 0xffffffff, area & 0xffffffff)
+
+
 def test_long_rows_use_the_whole_chip():
     """Five planes of 16384 x 64 (1 Mi pixels) take less than four times as long
     as five planes of 1024 x 1024: one block per plane takes ten times as long."""
