@@ -184,6 +184,7 @@ struct tm_ctx {
     float ms[3] = {};          // its time (0: not known yet; -1: left out)
     int best = -1;             // the measured choice
     float span = 0.f;          // mean bin span of the chunk rows, as last reported
+    uint64_t renew = 0;        // candidates are missing for want of memory until then (0: none are)
   };
   std::map<std::vector<int>, Trial> trials;
   uint64_t trial_asks = 0;
@@ -797,7 +798,8 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
     integral_layout(W, H, SIZE_MAX, (int)(2 * c->num_sms * share), J.nseg, J.seg_rows);
     size_t cnt_bytes = 0;
     if (compact) {
-      if (groups.size() < layout.first.size() && layout.first[groups.size()] == i) groups.push_back({i, 0, 0, 0, 0});
+      if (groups.size() < layout.first.size() && layout.first[groups.size()] == i)
+        groups.push_back({i, 0, 0, 0, 0});
       Group &g = groups.back();
       g.tall = std::max(g.tall, H);
       J.b0[kStCRows] = g.rows;
@@ -990,8 +992,8 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
           ls = std::min(ls, r);
           n += std::max(r, 0);
         }
-        n += launch_lookup_compact(P, jobs.data() + g.first, group_end(k) - g.first, g.look, look_rows, c_wide, !debug, keep_mom,
-                                   !do_lookup, dt, s);
+        n += launch_lookup_compact(P, jobs.data() + g.first, group_end(k) - g.first, g.look, look_rows, c_wide,
+                                   !debug, keep_mom, !do_lookup, dt, s);
       }
     } else {
       n += launch_lookup_counts(P, dj, nimg, b_look, !debug && wide, keep_mom, dt, s);
@@ -1177,9 +1179,9 @@ tm_status forward_materialised_batch(tm_ctx *c, int nimg, const tm_image *in, co
 // is synchronised), and the fastest takes the calls from then on. That is where
 //   - the compact histogram does not take the call;
 //   - some image is at least 16 times as long as wide, or the reverse (the
-//     compact build's chains along rows and columns: 512 x 60000, 64 bins,
-//     1968 against the sweep's 2229 us; 2048 x 16 37 and 51, batches of 100
-//     of them 328 and 597);
+//     compact build's chains along rows and columns: 512 x 60000 with 64 bins
+//     2229 us, 1968 on the sweep; 2048 x 16 51 and 37, 100 of them 597 and
+//     328);
 //   - the images are rough: in their last call the 32-column chunk rows spanned
 //     more than 6 bins, or 0.7 of them, on average (what the compact build and
 //     its vectors cost by). 12 MP, 64 bins, white noise, span 60: 2560 against
@@ -1256,6 +1258,13 @@ tm_ctx::Trial &trial_for(tm_ctx *c, TrialKind kind, int n, const tm_image *in, c
         c->trials.erase(old);
       }
       it = c->trials.emplace(key, T).first;
+    } else if (it->second.renew && c->trial_asks >= it->second.renew) {
+      tm_ctx::Trial T = new_trial(c, kind, n, in, key[1] != 0);
+      T.id = it->second.id;
+      T.slot = it->second.slot;
+      T.span = it->second.span;
+      drop_trial_events(it->second);
+      it->second = T;
     }
     const size_t most = c->trial_asks - c->compact_failed_at < kCompactRetry ? c->compact_failed : SIZE_MAX;
     group_bytes = it->second.bytes[0] < most ? kCompactGroup : 0;
@@ -1372,8 +1381,10 @@ void trial_end(tm_ctx::Trial &T, int k, cudaStream_t s) {
   ++T.passes;
 }
 
-// Candidate k cannot be had for want of memory: out of the trial, if another is left.
-bool trial_drop(tm_ctx::Trial &T, int k) {
+// Candidate k cannot be had for want of memory: out of the trial for a while,
+// if another is left (else all are back at the next call).
+bool trial_drop(tm_ctx *c, tm_ctx::Trial &T, int k) {
+  T.renew = T.n < 2 ? 1 : c->trial_asks + kCompactRetry;
   if (T.n < 2) return false;
   drop_trial_events(T);
   for (int i = k; i + 1 < T.n; ++i) T.cand[i] = T.cand[i + 1];
@@ -1446,7 +1457,7 @@ tm_status forward_device(tm_ctx *c, const tm_image *in, const tm_image *out, cud
     if (!st && pass) trial_end(T, k, s);
     if (st != TM_ENOMEM) return st;
     if (T.cand[k] == kPathCompact) compact_nomem(c, T, 0);  // the other paths need less memory
-    else if (!trial_drop(T, k)) return st;
+    else if (!trial_drop(c, T, k)) return st;
   }
 }
 
@@ -1746,7 +1757,7 @@ tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *ou
     if (!s && pass) trial_end(T, k, st);
     if (s != TM_ENOMEM) return s;
     if (T.cand[k] == kPathCompact) compact_nomem(c, T, group_bytes);  // smaller groups, then the other paths
-    else if (!trial_drop(T, k)) return s;
+    else if (!trial_drop(c, T, k)) return s;
   }
 }
 
@@ -1799,8 +1810,8 @@ tm_status tm_create(const tm_params *params, tm_ctx **out) {
 
 void tm_destroy(tm_ctx *c) {
   if (!c) return;
-  if (c->ws || c->mws || c->stats || c->rr_stats || c->stage || c->djobs || c->gspare || !c->graphs.empty() || c->mgraph ||
-      c->hslot[0])
+  if (c->ws || c->mws || c->stats || c->rr_stats || c->stage || c->djobs || c->gspare || !c->graphs.empty() ||
+      c->mgraph || c->hslot[0])
     cudaDeviceSynchronize();
   drop_graph(c);
   drop_trials(c);
@@ -2075,7 +2086,10 @@ tm_status tm_integral_image(const int32_t *q, int32_t width, int32_t height, int
   J.q = const_cast<int32_t *>(q);
   J.s1 = reinterpret_cast<long long *>(s1);
   J.s2 = reinterpret_cast<long long *>(s2);
-  integral_layout(width, height, SIZE_MAX, 304, J.nseg, J.seg_rows);
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  integral_layout(width, height, SIZE_MAX, 2 * sms, J.nseg, J.seg_rows);
   const size_t seg_bytes = 8 * integral_scratch_elems(width, height, J.nseg);
   void *scr = nullptr;
   cudaError_t e = cudaMallocAsync(&scr, align256(sizeof(Job)) + seg_bytes, st);

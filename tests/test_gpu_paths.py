@@ -155,6 +155,30 @@ def test_short_memory_holds_for_what_did_not_fit():
             torch.cuda.empty_cache()
 
 
+def test_calls_that_failed_for_memory_have_all_paths_again():
+    """A 12 MP image for which no path's memory can be had: the call fails, and
+    the next one with memory takes the sweep (the compact histogram is tried
+    again later), not whatever path was tried last."""
+    p = tm.make_params(64, [4, 16])
+    (x,) = _images([(4000, 3000)], 7)
+    ctx = tm.tm_create(p)
+    hold = None
+    try:
+        y = torch.empty_like(x)
+        hold = _all_but(100 << 20)
+        for _ in range(2):
+            with pytest.raises(tm.TmError) as e:
+                tm.tm_forward(ctx, x, y)
+            assert e.value.status == tm.TM_ENOMEM
+        hold = None
+        torch.cuda.empty_cache()
+        assert _path(ctx, x) == {"fused_sweep"}
+    finally:
+        tm.tm_destroy(ctx)
+        hold = None
+        torch.cuda.empty_cache()
+
+
 def test_batch_in_smaller_groups_when_memory_is_short():
     """Sixteen images whose compact histograms (0.9 GB each) would run in two
     groups: with 4 GB free they run one image at a time, the forward and the
@@ -164,7 +188,8 @@ def test_batch_in_smaller_groups_when_memory_is_short():
     gs = [torch.randn_like(x) for x in xs]
     got = []
     for short in (False, True):
-        ys, gin, gp = [torch.empty_like(x) for x in xs], [torch.empty_like(x) for x in xs], torch.empty(7, device="cuda")
+        ys, gin = [torch.empty_like(x) for x in xs], [torch.empty_like(x) for x in xs]
+        gp = torch.empty(7, device="cuda")
         ctx = tm.tm_create(p)
         hold = None
         try:
