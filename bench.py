@@ -678,18 +678,24 @@ def batch_passes(stages):
 
 
 def kernel_source_hash(kernel):
+    """The sha256 prefix of a kernel's source: its file and every kernel header."""
+    import glob
     import hashlib
 
     import paper_2102_01289_gb300 as tm
 
-    srcs = {"fused_sweep": "tm_sweep.cu", "lookup": "tm_lookup.cu", "lookup_compact": "tm_compact.cu", "bwd_pixel": "tm_backward.cu",
-            "bwd_input": "tm_backward.cu", "fix_stats": "tm_integral.cu", "fix_write": "tm_integral.cu",
-            "integral_histogram": "tm_integral.cu", "integral_image": "tm_integral.cu",
-            "prep": "tm_prepass.cu", "range": "tm_prepass.cu"}
+    srcs = {"fused_sweep": "tm_sweep.cu", "lookup": "tm_lookup.cu", "lookup_compact": "tm_compact.cu",
+            "bwd_pixel": "tm_backward.cu", "bwd_input": "tm_backward.cu", "fix_stats": "tm_integral.cu",
+            "fix_write": "tm_integral.cu", "integral_histogram": "tm_integral.cu", "integral_image": "tm_integral.cu",
+            "compact_histogram": "tm_compact.cu", "prep": "tm_prepass.cu", "range": "tm_prepass.cu"}
     f = os.path.join(tm.PKG, "csrc", srcs.get(kernel, ""))
     if not os.path.isfile(f):
         return None
-    return hashlib.sha256(open(f, "rb").read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for name in [f] + sorted(glob.glob(os.path.join(tm.PKG, "csrc", "*.cuh"))):
+        with open(name, "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:16]
 
 
 def main():

@@ -257,10 +257,10 @@ __device__ __forceinline__ void store_rgb(const Image &im, int x, int y, float r
   }
 }
 
-// 1 / x, log2 x and 2^x on the special-function unit for arguments and results
-// in the normal range: the flush-to-zero forms of the approximations behind
-// __fdividef, __log2f and exp2f, without the instructions that rescale
-// denormals (the same bits there).
+// 1 / x, log2 x and 2^x on the special-function unit: the PTX instructions
+// rcp.approx.ftz.f32, lg2.approx.ftz.f32 and ex2.approx.ftz.f32, which take and
+// give subnormal numbers as zero. For arguments and results in the normal range
+// (there they were measured equal to __fdividef, __log2f and exp2f).
 __device__ __forceinline__ float rcp_normal(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

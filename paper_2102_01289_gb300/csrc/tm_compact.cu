@@ -19,7 +19,8 @@
 // vectors of one photograph-like scene about 40 MB. Forwards, against the
 // sweep: 12 MP, 64 bins, 736 -> 502 us; with noise of 0.3 decades 1006 -> 709;
 // 1080p, 32 bins, 199 -> 116. White noise (every chunk row mixed for every
-// threshold) is its worst case: 1080p 281 -> 238, but 12 MP 1733 -> 2538.
+// threshold) is its worst case: 1080p 281 -> 238, but 12 MP 1733 -> 2538 (the
+// automatic path measures such images and leaves them to the sweep).
 // Differences between two rows are taken modulo the width of m and B, so B is
 // 16 bits wide unless a window is taller than 65535 / 31 rows.
 //
@@ -226,7 +227,8 @@ __device__ __forceinline__ void col_pass(const Job &J, int c, int kg, int K, int
         for (int z = 0; z < T; ++z) rp[u][z] = 0;
         if (own && i + u < n) load_prefix<T>(row + (i + u) * KL, rp[u]);
         b[u] = 256;
-        if (i + u < 32 && ((mixed >> ((i + u) & 31)) & 1u) && colok) b[u] = (int)__ldg(bins + (size_t)(unsigned)(i + u) * W);
+        if (i + u < 32 && ((mixed >> ((i + u) & 31)) & 1u) && colok)
+          b[u] = (int)__ldg(bins + (size_t)(unsigned)(i + u) * W);
       }
     };
     unsigned nrp[S::Step][T];
@@ -682,7 +684,8 @@ static void launch_look_dtype(const DevParams &P, const LookPack &L, int blocks,
 
 int launch_lookup_compact(const DevParams &P, const Job *jobs, int njobs, int blocks, int rows, bool wide,
                           bool plain, bool keep, bool counts_only, int dtype, cudaStream_t s) {
-  const bool general = !plain || !P.fast || (P.flags & kFlagAreaLit) || (keep && (wide || !P.small_win || dtype != kF32));
+  const bool general =
+      !plain || !P.fast || (P.flags & kFlagAreaLit) || (keep && (wide || !P.small_win || dtype != kF32));
   LookPack L{};
   L.n = njobs;
   L.rows = rows;

@@ -613,7 +613,8 @@ __device__ __forceinline__ void hist_strip_totals(const HistParts &Q, int s, int
     for (int u = 0; u < 4; ++u)
 #pragma unroll
       for (int m = 0; m < 4; ++m)
-        v[u][m] = r + u < (unsigned)r1 && c + 32 * m < Q.W ? (int)__ldg(Q.bins + (size_t)(r + u) * Q.W + c + 32 * m) : 256;
+        v[u][m] = r + u < (unsigned)r1 && c + 32 * m < Q.W ? (int)__ldg(Q.bins + (size_t)(r + u) * Q.W + c + 32 * m)
+                                                          : 256;
     for (int p = 0; p < Q.n_planes; ++p) {
       const int k = Q.k_begin + p;
       unsigned t = 0;  // the rows' totals, a byte each
@@ -631,7 +632,8 @@ __device__ __forceinline__ void hist_strip_totals(const HistParts &Q, int s, int
     }
   }
   __syncthreads();
-  for (int p = threadIdx.x; p < Q.n_planes; p += kHStrip) Q.segtot[((size_t)seg * Q.n_planes + p) * strips + s] = sum[p];
+  for (int p = threadIdx.x; p < Q.n_planes; p += kHStrip)
+    Q.segtot[((size_t)seg * Q.n_planes + p) * strips + s] = sum[p];
 }
 
 // Plane p indicates [b == k] (eq) or [b < k], k = k_begin + p.

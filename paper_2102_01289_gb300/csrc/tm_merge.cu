@@ -66,7 +66,8 @@ __device__ __forceinline__ float quotient(float num, float den, float rden) {
 
 // kN: the number of exposures when known at compile time (0: read from a).
 template <int kN>
-__global__ void __launch_bounds__(kMT, kMB) k_merge(const __grid_constant__ MergeArgs a, const __grid_constant__ Image out) {
+__global__ void __launch_bounds__(kMT, kMB)
+    k_merge(const __grid_constant__ MergeArgs a, const __grid_constant__ Image out) {
   extern __shared__ float2 tab[];  // [n][3][256]: (g(z) - ln dt_j, w(z))
   __shared__ float rcp[kRecips];
   const int ne = kN ? kN : a.n;
@@ -99,7 +100,8 @@ __global__ void __launch_bounds__(kMT, kMB) k_merge(const __grid_constant__ Merg
         for (int s = 0; s < 12; ++s) {
           // the byte's value times 8, the entry's offset
           const unsigned at = (s & 3 ? w[s >> 2] >> (8 * (s & 3) - 3) : w[s >> 2] << 3) & 0x7f8u;
-          const float2 t = *reinterpret_cast<const float2 *>(reinterpret_cast<const char *>(tab + (j * 3 + s % 3) * 256) + at);
+          const char *row = reinterpret_cast<const char *>(tab + (j * 3 + s % 3) * 256);
+          const float2 t = *reinterpret_cast<const float2 *>(row + at);
           num[s] = fmaf(t.y, t.x, num[s]);
           den[s] += t.y;
         }
@@ -213,7 +215,8 @@ extern "C" tm_status tm_merge_exposures(int32_t n, const uint8_t *const *ldr, co
   // the table reads, and the general one took 230 us for 12 MP of white noise
   // (217 a pixel per thread; 223 now, photographs 151 -> 122). With variants
   // for five to seven 2 MP took up to 5 % longer.
-  auto *const kernel = n == 2 ? k_merge<2> : n == 3 ? k_merge<3> : n == 4 ? k_merge<4> : n == 8 ? k_merge<8> : k_merge<0>;
+  auto *const kernel = n == 2 ? k_merge<2> : n == 3 ? k_merge<3> : n == 4 ? k_merge<4> : n == 8 ? k_merge<8>
+                                                                                                : k_merge<0>;
   // the limit is state of the kernel shared by every thread of the process:
   // always the largest, so that no call lowers it under another's launch
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

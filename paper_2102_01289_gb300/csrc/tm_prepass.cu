@@ -119,7 +119,8 @@ __device__ void commit_range(Stats *st, unsigned bmin, unsigned bmax, int nb, in
   const unsigned bits = __float_as_uint(imin);
   if (wid == 0 && lane < 2) lg[lane] = log((double)(lane ? imax : imin));
   if (wid == 1 && lane < 3)
-    lg[2 + lane] = log2((double)(lane == 0 ? imin : lane == 1 ? imax : __uint_as_float((bits & 0x7fffffu) | 0x3f800000u)));
+    lg[2 + lane] =
+        log2((double)(lane == 0 ? imin : lane == 1 ? imax : __uint_as_float((bits & 0x7fffffu) | 0x3f800000u)));
   __syncthreads();
   const double lmin = lg[0], lmax = lg[1];
   const int last_warp = (int)(blockDim.x >> 5) - 1;

@@ -56,7 +56,8 @@ def test_cumulative_planes_in_parts(H, W, n):
 
 @pytest.mark.parametrize("H,W", [(1, 2 ** 31 - 1), (2 ** 31 - 1, 1), (2 ** 21, 1025)])
 def test_sides_up_to_the_largest(H, W):
-    """Maps of 2^31 pixels, one row, one column and two passes: one plane."""
+    """Maps of 2^31 pixels, one row, one column and two passes: two planes."""
+    torch.cuda.empty_cache()
     if torch.cuda.mem_get_info()[0] < 120 * 2 ** 30:
         pytest.skip("needs 120 GB of device memory")
     bins = torch.zeros((H, W), dtype=torch.uint8, device="cuda")
