@@ -324,10 +324,10 @@ tm_status tm_debug_export(tm_ctx *ctx, int32_t what, void *dst, size_t bytes,
  *                        (or the reverse), or whose last call's images were
  *                        rough (the bins of a 32-pixel run spanned more than
  *                        6, or 0.7 of them, on average, e.g. white noise) are
- *                        measured: three calls each go to the compact path,
+ *                        measured: four calls each go to the compact path,
  *                        path 1 and path 2, as far as they take them, the
- *                        last of each timed with events on `stream` (nothing
- *                        is synchronised), and then all to the fastest, per
+ *                        last two timed with events on `stream` (nothing is
+ *                        synchronised), and then all to the fastest, per
  *                        list of sizes and dtype pairs (64 are kept). Not
  *                        while `stream` is being captured. Memory for the
  *                        compact path that could not be had is not asked for

@@ -180,17 +180,18 @@ struct tm_ctx {
     int cand[3] = {};   // candidate paths; the first is the one by the rules
     size_t bytes[2] = {};      // of the compact histogram: in groups, and of one image at a time
     int passes = 0;     // of the measurement so far, kTrialPasses per candidate
-    cudaEvent_t e[3][2] = {};  // around each candidate's last pass
-    float ms[3] = {};          // its time (0: not known yet; -1: left out)
+    cudaEvent_t e[3][2][2] = {};  // around each candidate's last two passes
+    float ms[3] = {};          // the shorter one's time (0: not known yet; -1: left out)
     int best = -1;             // the measured choice
-    float span = 0.f;          // mean bin span of the chunk rows, as last reported
+    bool rough = false;        // the images, as last reported (report_span)
     uint64_t renew = 0;        // candidates are missing for want of memory until then (0: none are)
   };
   std::map<std::vector<int>, Trial> trials;
   uint64_t trial_asks = 0;
   uint32_t trial_ids = 0;
   unsigned long long *hints = nullptr;  // page-locked, kTrials slots, written by the device
-  unsigned long long *hint = nullptr;   // the current call's slot (null: none) and tag
+  unsigned long long *said = nullptr;   // on the device: what it last wrote there
+  int hint_slot = -1;                   // the current call's slot (-1: none) and tag
   unsigned hint_tag = 0;
   cudaEvent_t pass_begin = nullptr;     // to be recorded before the call's first launch (null: no)
   // stage timing: events recorded on the call's stream after each stage
@@ -545,8 +546,11 @@ void first_launch(tm_ctx *c, cudaStream_t s) {
 
 // Where a call's first job has to report how rough the images are.
 void set_hint(const tm_ctx *c, Job &J, int i) {
-  J.hint = i == 0 ? c->hint : nullptr;
+  const bool on = i == 0 && c->hint_slot >= 0;
+  J.hint = on ? c->hints + c->hint_slot : nullptr;
+  J.said = on ? c->said + c->hint_slot : nullptr;
   J.hint_tag = c->hint_tag;
+  J.rough = std::min(6.f, 0.7f * (float)(c->p.n_bins - 1));
 }
 
 // The materialised path for one image: range, bins, integral images,
@@ -610,8 +614,7 @@ tm_status forward_materialised(tm_ctx *c, const tm_image *in, const tm_image *ou
   launch_prep(c->djobs, 1, pb, c->p.n_bins, c->p.flags, c->p.n_fields, J.in.dtype, s);
   mark(c, s, ST_PREP);
   n += (run_range ? 2 : 1) +
-       launch_integral_jobs(c->djobs, 1, integral_tile_blocks(W, nseg), integral_col_blocks(W), s);
-  if (J.hint) n += launch_span(c->djobs, 1, s);
+       launch_integral_jobs(c->djobs, 1, integral_tile_blocks(W, nseg), integral_col_blocks(W), J.hint != nullptr, s);
   mark(c, s, ST_INTEGRAL);
   uint32_t *cpl = nullptr;
   if (c->p.n_bins > 1) {
@@ -960,14 +963,12 @@ tm_status forward_fused(tm_ctx *c, int nimg, const tm_image *in, const tm_image 
   const auto group_end = [&](size_t k) { return k + 1 < groups.size() ? groups[k + 1].first : nimg; };
   const auto build = [&](size_t k, cudaStream_t q) {
     const Group &g = groups[k];
-    return launch_compact_build(dj + g.first, group_end(k) - g.first, g.rows, g.cols, g.tall, K, c_wide,
-                                jobs[(size_t)g.first].hint != nullptr, q);
+    return launch_compact_build(dj + g.first, group_end(k) - g.first, g.rows, g.cols, g.tall, K, c_wide, q);
   };
   int ls = compact ? build(0, c->sweep_stream)
                    : launch_sweep(P, dj, nimg, nitems, queue, smem, ctas, width, c->sweep_stream);
   if (!graph) mark(c, c->sweep_stream, compact ? ST_COMPACT : ST_SWEEP, m_prep);
-  n += std::max(ls, 0) + launch_integral_jobs(dj, nimg, b_rows, b_cols, c->int_stream);
-  if (!compact && jobs[0].hint) n += launch_span(dj, std::min(nimg, kCompactImages), c->int_stream);
+  n += std::max(ls, 0) + launch_integral_jobs(dj, nimg, b_rows, b_cols, jobs[0].hint != nullptr, c->int_stream);
   if (!graph) mark(c, c->int_stream, ST_INTEGRAL, m_prep);
   n += run_range ? 2 : 1;
   TM_CUDA(c, cudaEventRecord(c->ov_sweep, c->sweep_stream));
@@ -1128,7 +1129,7 @@ tm_status forward_materialised_batch(tm_ctx *c, int nimg, const tm_image *in, co
     J.s2 = J.s1 + 1;
     J.s_pair = 1;
     J.segtot = reinterpret_cast<long long *>(b + L.segtot);
-    if (c->hint) J.grp = reinterpret_cast<uint16_t *>(b + L.grp);
+    if (c->hint_slot >= 0) J.grp = reinterpret_cast<uint16_t *>(b + L.grp);
   }
   const cudaStream_t caller = s;
   if (!c->graph_stream) TM_CUDA(c, cudaStreamCreateWithFlags(&c->graph_stream, cudaStreamNonBlocking));
@@ -1138,8 +1139,7 @@ tm_status forward_materialised_batch(tm_ctx *c, int nimg, const tm_image *in, co
   const int in_dt = input_dtype(jobs.data(), nimg);
   launch_range(c->mdjobs, nimg, b_range, c->p.n_bins, in_dt, s);
   launch_prep(c->mdjobs, nimg, b_prep, c->p.n_bins, c->p.flags, c->p.n_fields, in_dt, s);
-  n += 2 + launch_integral_jobs(c->mdjobs, nimg, b_rows, b_cols, s);
-  if (jobs[0].hint) n += launch_span(c->mdjobs, std::min(nimg, kCompactImages), s);
+  n += 2 + launch_integral_jobs(c->mdjobs, nimg, b_rows, b_cols, jobs[0].hint != nullptr, s);
   for (int i = 0; i < nimg; ++i) {
     const Job &J = jobs[(size_t)i];
     if (planes) n += launch_integral_histogram(J.bins, J.in.W, J.in.H, c->p.n_bins, true, planes, scratch, s);
@@ -1172,11 +1172,13 @@ tm_status forward_materialised_batch(tm_ctx *c, int nimg, const tm_image *in, co
 // The automatic path. The first candidate is taken by the rules: the compact
 // integral histogram where it fits, but the sweep for strips(), else the sweep.
 // Where the rules are not sure, the candidates are measured on the calls
-// themselves: each runs three of them (so that calls that replay a graph are
-// timed on a replay: rough 64 x 4095 with 256 bins take 228 us in launches and
-// 300 in replays on the compact path, 233 and 209 on the sweep), the last
-// between events that are read when a later call finds them complete (nothing
-// is synchronised), and the fastest takes the calls from then on. That is where
+// themselves: each runs four of them, the last two between events that are read
+// when a later call finds them complete (nothing is synchronised), and the one
+// with the shortest takes the calls from then on. (Two passes before them, so
+// that calls that replay a graph are timed on replays: rough 64 x 4095 with 256
+// bins take 228 us in launches and 300 in replays on the compact path, 233 and
+// 209 on the sweep. Two timed: 1024 x 32768 with 256 bins took 2990 us and once
+// 3730.) That is where
 //   - the compact histogram does not take the call;
 //   - some image is at least 16 times as long as wide, or the reverse (the
 //     compact build's chains along rows and columns: 512 x 60000 with 64 bins
@@ -1190,17 +1192,18 @@ tm_status forward_materialised_batch(tm_ctx *c, int nimg, const tm_image *in, co
 //     Of 1961 kinds of calls timed, those with shorter spans and sides were at
 //     most 5 % slower on the compact path. Photograph-like scenes with 64 bins
 //     span 0.5 to 6.
-// The span comes from the device (report_span) through host memory, so a call
-// goes by the last one that has run.
+// That comes from the device (report_span) through host memory, so a call goes
+// by the last one that has run.
 constexpr size_t kTrials = 64;  // the most recently asked for are kept
-constexpr int kTrialPasses = 3; // launches, a graph's capture, its replay
+constexpr int kTrialPasses = 4; // launches, a graph's capture, its replay twice
 
 void drop_trial_events(tm_ctx::Trial &T) {
-  for (auto &e : T.e)
-    for (cudaEvent_t &ev : e) {
-      if (ev) cudaEventDestroy(ev);
-      ev = nullptr;
-    }
+  for (auto &passes : T.e)
+    for (auto &e : passes)
+      for (cudaEvent_t &ev : e) {
+        if (ev) cudaEventDestroy(ev);
+        ev = nullptr;
+      }
 }
 
 void drop_trials(tm_ctx *c) {
@@ -1262,7 +1265,7 @@ tm_ctx::Trial &trial_for(tm_ctx *c, TrialKind kind, int n, const tm_image *in, c
       tm_ctx::Trial T = new_trial(c, kind, n, in, key[1] != 0);
       T.id = it->second.id;
       T.slot = it->second.slot;
-      T.span = it->second.span;
+      T.rough = it->second.rough;
       drop_trial_events(it->second);
       it->second = T;
     }
@@ -1274,19 +1277,23 @@ tm_ctx::Trial &trial_for(tm_ctx *c, TrialKind kind, int n, const tm_image *in, c
   tm_ctx::Trial &T = it->second;
   T.used = ++c->trial_asks;
   if (!c->hints) {
-    if (cudaHostAlloc(&c->hints, kTrials * sizeof *c->hints, cudaHostAllocMapped) == cudaSuccess) {
-      memset(c->hints, 0, kTrials * sizeof *c->hints);
+    const size_t bytes = kTrials * sizeof *c->hints;
+    if (cudaHostAlloc(&c->hints, bytes, cudaHostAllocMapped) == cudaSuccess &&
+        cudaMalloc(&c->said, bytes) == cudaSuccess && cudaMemset(c->said, 0, bytes) == cudaSuccess) {
+      memset(c->hints, 0, bytes);
     } else {
       cudaGetLastError();
-      c->hints = nullptr;
+      if (c->said) cudaFree(c->said);
+      if (c->hints) cudaFreeHost(c->hints);
+  if (c->said) cudaFree(c->said);
+      c->said = c->hints = nullptr;
     }
   }
   if (c->hints) {
     const unsigned long long v = reinterpret_cast<const volatile unsigned long long *>(c->hints)[T.slot];
-    const uint32_t bits = (uint32_t)v;
-    if ((uint32_t)(v >> 32) == T.id) memcpy(&T.span, &bits, sizeof bits);
+    if ((uint32_t)(v >> 32) == T.id) T.rough = (v & 1) != 0;
   }
-  c->hint = c->hints ? c->hints + T.slot : nullptr;
+  c->hint_slot = c->hints ? T.slot : -1;
   c->hint_tag = T.id;
   return T;
 }
@@ -1311,13 +1318,19 @@ bool trial_times(tm_ctx::Trial &T, int k) {
   bool all = true;
   for (int i = 0; i < k; ++i) {
     if (T.ms[i] != 0.f) continue;
-    const cudaError_t e = cudaEventQuery(T.e[i][1]);
+    const cudaError_t e = cudaEventQuery(T.e[i][1][1]);
     if (e == cudaErrorNotReady) {
       cudaGetLastError();
       all = false;
-    } else if (e != cudaSuccess || cudaEventElapsedTime(&T.ms[i], T.e[i][0], T.e[i][1]) != cudaSuccess) {
-      cudaGetLastError();
-      T.ms[i] = -1.f;
+      continue;
+    }
+    T.ms[i] = -1.f;
+    for (const auto &ev : T.e[i]) {
+      float ms = 0.f;
+      if (cudaEventElapsedTime(&ms, ev[0], ev[1]) == cudaSuccess && ms > 0.f)
+        T.ms[i] = T.ms[i] > 0.f ? std::min(T.ms[i], ms) : ms;
+      else
+        cudaGetLastError();
     }
   }
   return all;
@@ -1329,7 +1342,7 @@ int trial_next(tm_ctx *c, tm_ctx::Trial &T, int n, const tm_image *in, cudaStrea
   pass = false;
   if (T.n == 1) return 0;
   const int K = c->p.n_bins - 1;
-  bool unsure = T.span > 6.f || T.span > 0.7f * K || std::find(T.cand, T.cand + T.n, kPathCompact) == T.cand + T.n;
+  bool unsure = T.rough || std::find(T.cand, T.cand + T.n, kPathCompact) == T.cand + T.n;
   for (int i = 0; i < n && !unsure; ++i) {
     const long long W = in[i].width, H = in[i].height;
     unsure = W >= 16 * H || H >= 16 * W;
@@ -1352,12 +1365,13 @@ int trial_next(tm_ctx *c, tm_ctx::Trial &T, int n, const tm_image *in, cudaStrea
     }
   }
   if (k < T.n) {
-    for (cudaEvent_t &ev : T.e[k])
-      if (!ev && cudaEventCreate(&ev) != cudaSuccess) {
-        cudaGetLastError();
-        ev = nullptr;
-        return 0;
-      }
+    for (auto &e : T.e[k])
+      for (cudaEvent_t &ev : e)
+        if (!ev && cudaEventCreate(&ev) != cudaSuccess) {
+          cudaGetLastError();
+          ev = nullptr;
+          return 0;
+        }
     pass = true;
     return k;
   }
@@ -1370,14 +1384,16 @@ int trial_next(tm_ctx *c, tm_ctx::Trial &T, int n, const tm_image *in, cudaStrea
   return best;
 }
 
-// Around a call by candidate k (pass: of the measurement): the last pass is
-// timed from its first launch on, after a graph's capture.
+// Around a call by candidate k (pass: of the measurement): its last passes are
+// timed from their first launch on, after a graph's capture.
 void trial_begin(tm_ctx *c, tm_ctx::Trial &T, int k, bool pass) {
-  c->pass_begin = pass && T.passes % kTrialPasses == kTrialPasses - 1 ? T.e[k][0] : nullptr;
+  const int timed = T.passes % kTrialPasses - (kTrialPasses - 2);
+  c->pass_begin = pass && timed >= 0 ? T.e[k][timed][0] : nullptr;
 }
 
 void trial_end(tm_ctx::Trial &T, int k, cudaStream_t s) {
-  if (T.passes % kTrialPasses == kTrialPasses - 1) cudaEventRecord(T.e[k][1], s);
+  const int timed = T.passes % kTrialPasses - (kTrialPasses - 2);
+  if (timed >= 0) cudaEventRecord(T.e[k][timed][1], s);
   ++T.passes;
 }
 
@@ -1440,7 +1456,7 @@ tm_status forward_device(tm_ctx *c, const tm_image *in, const tm_image *out, cud
   tm_status st = ensure_device_info(c);
   if (st) return st;
   ++c->calls;
-  c->hint = nullptr;
+  c->hint_slot = -1;
   c->pass_begin = nullptr;
   if (c->p.n_bins < 2) return forward_materialised(c, in, out, s);  // no thresholds: nothing to count
   if (c->hist_path != 0) {
@@ -1563,7 +1579,7 @@ tm_status backward_images(tm_ctx *c, int n, const tm_image *in, const tm_image *
     if (!sweep_fits(c, &in[i])) return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit these fields");
   tm_ctx::Trial *trial = nullptr;  // of which this call is a pass, measured as a whole
   int trial_k = 0;
-  c->hint = nullptr;
+  c->hint_slot = -1;
   c->pass_begin = nullptr;
   if (c->bwd_reuse && c->fwd_valid && (int)c->fwd_in.size() == n && same_images(c->fwd_in, in, n)) {
     jobs = c->fwd_jobs;  // the last forward's intermediates of these images are in the workspace
@@ -1720,7 +1736,7 @@ tm_status forward_passes(tm_ctx *c, Path path, size_t group_bytes, int n, const 
     if ((s = forward_fused(c, (int)fin.size(), fin.data(), fout.data(), st, true, kPathSweep))) return s;
     total += c->launches;
     mark(c, st, ST_BATCH);
-    c->hint = nullptr;  // (one report per call)
+    c->hint_slot = -1;  // (one report per call)
   }
   if (!min_.empty()) {
     mark(c, st, -1);
@@ -1743,7 +1759,7 @@ tm_status forward_batch(tm_ctx *c, int n, const tm_image *in, const tm_image *ou
         return fail(c, TM_EUNSUPPORTED, "fused sweep does not fit image %d's fields (use the materialised path)", i);
   if ((s = ensure_stats(c, n))) return s;
   ++c->calls;
-  c->hint = nullptr;
+  c->hint_slot = -1;
   c->pass_begin = nullptr;
   if (c->p.n_bins < 2) return forward_passes(c, kPathMaterialised, 0, n, in, out, st);
   if (c->hist_path != 0) return forward_passes(c, (Path)c->hist_path, 0, n, in, out, st);
@@ -1816,6 +1832,7 @@ void tm_destroy(tm_ctx *c) {
   drop_graph(c);
   drop_trials(c);
   if (c->hints) cudaFreeHost(c->hints);
+  if (c->said) cudaFree(c->said);
   for (auto &call : c->marks)
     for (auto &m : call) cudaEventDestroy(m.e);
   for (cudaEvent_t e : c->event_pool) cudaEventDestroy(e);
@@ -2097,7 +2114,7 @@ tm_status tm_integral_image(const int32_t *q, int32_t width, int32_t height, int
   J.segtot = reinterpret_cast<long long *>(static_cast<char *>(scr) + align256(sizeof(Job)));
   put_jobs(&J, 1, static_cast<Job *>(scr), st);
   launch_integral_jobs(static_cast<Job *>(scr), 1, integral_tile_blocks(width, J.nseg),
-                       integral_col_blocks(width), st);
+                       integral_col_blocks(width), false, st);
   e = cudaGetLastError();
   cudaFreeAsync(scr, st);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "tm_integral_image");

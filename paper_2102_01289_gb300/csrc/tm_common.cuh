@@ -134,43 +134,15 @@ struct alignas(16) Job {
   void *c_vec;              // in-chunk vectors, (W / 32 + 1) x (n - 1) x (H + 1) slots x 32 columns
   uint16_t *c_row;          // row prefixes over the chunks, groups x (W / 32 + 1) x H x 2^c_shift
   int c_shift;              // log2 of the thresholds per group
-  unsigned hint_tag;        // first job: report_span writes hint_tag << 32 | the mean bin span of the
-  unsigned long long *hint; //   images' chunk rows (float bits) here, in host memory (null: not asked for)
+  // the first job's, for the report of the integral images (hint null: not asked for)
+  unsigned long long *hint;  // in host memory: hint_tag << 32 | whether the call's images are rough
+  unsigned long long *said;  // in device memory: what it last stored there
+  unsigned hint_tag;
+  float rough;               // the mean bin span above which they are
   SweepPlan plan;           // sweep tiling of this image
 };
 
 static_assert(sizeof(Job) % 16 == 0, "jobs are copied in 16-byte words");
-
-// How rough a launch's images are, by one block: the mean bin span (largest -
-// smallest) of up to 1024 of their 32-column chunk rows, spread over all of
-// them, to the first job's hint (at most 1024 jobs). Short: at 512 x 384 the
-// block would otherwise outlast the others of its launch (4096 rows: 41.8 us a
-// forward against 38.2).
-inline __device__ __noinline__ void report_span(const Job *__restrict__ jobs, int njobs) {
-  __shared__ unsigned long long part[32];
-  unsigned rows = 0, spans = 0;
-  const int lg = 10 - (32 - __clz(njobs - 1));  // 2^lg rows of each job
-#pragma unroll 4
-  for (int i = threadIdx.x; i < njobs << lg; i += blockDim.x) {
-    const Job &J = jobs[i >> lg];
-    const unsigned total = (unsigned)((J.in.W + 31) >> 5) * (unsigned)J.in.H;
-    const unsigned q = (unsigned)i & ((1u << lg) - 1u);
-    const unsigned v = __ldg(J.grp + ((unsigned long long)q * total >> lg));  // (some repeat where there are fewer)
-    ++rows;
-    spans += (v >> 8) - (v & 0xffu);
-  }
-  rows = __reduce_add_sync(0xffffffffu, rows);
-  spans = __reduce_add_sync(0xffffffffu, spans);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = (unsigned long long)rows << 32 | spans;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long t = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += part[w];
-    const float span = (float)(unsigned)t / (float)(unsigned)(t >> 32);
-    *reinterpret_cast<volatile unsigned long long *>(jobs[0].hint) =
-        (unsigned long long)jobs[0].hint_tag << 32 | __float_as_uint(span);
-  }
-}
 
 // Index of the job owning block `blk` of stage `st` (jobs sorted by b0).
 __device__ __forceinline__ int find_job(const Job *jobs, int njobs, int st, int blk) {

@@ -109,16 +109,10 @@ __device__ __forceinline__ void store_records(uint2 *p, const unsigned *pt, cons
 }
 
 // Rows: a warp per row, lane = T thresholds, walking along the row's chunks.
-// span: one more block, the last, reports how rough the images are.
 template <int KL>
-__global__ void __launch_bounds__(32 * kRowWarps)
-    k_compact_rows(const Job *__restrict__ jobs, int njobs, int K, bool span) {
+__global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(const Job *__restrict__ jobs, int njobs, int K) {
   using S = Shape<KL>;
   constexpr int T = S::T;
-  if (span && blockIdx.x == gridDim.x - 1) {
-    report_span(jobs, njobs);
-    return;
-  }
   const Job &J = jobs[find_job(jobs, njobs, kStCRows, blockIdx.x)];
   const int lane = threadIdx.x & 31;
   const int W = J.in.W, H = J.in.H, G = (W + 31) >> 5, Gp = (W >> 5) + 1;
@@ -611,9 +605,9 @@ int launch_cols(const Job *jobs, int njobs, int blocks, int tall, int K, cudaStr
 }
 
 template <int KL>
-int launch_build(const Job *jobs, int njobs, int row_blocks, int col_blocks, int tall, int K, bool wide, bool span,
+int launch_build(const Job *jobs, int njobs, int row_blocks, int col_blocks, int tall, int K, bool wide,
                  cudaStream_t s) {
-  k_compact_rows<KL><<<row_blocks + (span ? 1 : 0), 32 * kRowWarps, 0, s>>>(jobs, njobs, K, span);
+  k_compact_rows<KL><<<row_blocks, 32 * kRowWarps, 0, s>>>(jobs, njobs, K);
   const int r = wide ? launch_cols<KL, uint32_t>(jobs, njobs, col_blocks, tall, K, s)
                      : launch_cols<KL, uint16_t>(jobs, njobs, col_blocks, tall, K, s);
   return r < 0 ? -1 : 2;
@@ -651,13 +645,13 @@ int compact_col_units(int W, int K) {
 }
 
 int launch_compact_build(const Job *jobs, int njobs, int row_blocks, int col_blocks, int tall, int K, bool wide,
-                         bool span, cudaStream_t s) {
+                         cudaStream_t s) {
   switch (group_shift(K)) {
-    case 2: return launch_build<4>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, span, s);
-    case 3: return launch_build<8>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, span, s);
-    case 4: return launch_build<16>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, span, s);
-    case 5: return launch_build<32>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, span, s);
-    default: return launch_build<64>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, span, s);
+    case 2: return launch_build<4>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, s);
+    case 3: return launch_build<8>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, s);
+    case 4: return launch_build<16>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, s);
+    case 5: return launch_build<32>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, s);
+    default: return launch_build<64>(jobs, njobs, row_blocks, col_blocks, tall, K, wide, s);
   }
 }
 

@@ -23,9 +23,6 @@ int input_dtype(const Job *jobs, int njobs);
 int range_blocks(int W, int H, int num_sms, double share);
 int prep_blocks(int W, int H, int num_sms, double share);
 
-// report_span over the jobs of a launch (the compact build has it built in).
-int launch_span(const Job *jobs, int njobs, cudaStream_t s);
-
 // Stage a2 (Eq. 5): integral images of q and q^2, (H+1) x (W+1) int64, over
 // tiles of row segments x column chunks. integral_layout picks the segments
 // (J.nseg of J.seg_rows rows) whose scratch fits max_scratch_elems (the
@@ -34,12 +31,13 @@ int launch_span(const Job *jobs, int njobs, cudaStream_t s);
 // integral_tile_blocks(W, nseg) blocks of the tile launches (first block
 // J.b0[kStRows]), integral_col_blocks(W) of the column-prefix launch
 // (J.b0[kStCols]), and integral_scratch_elems(W, H, nseg) int64 elements of
-// scratch at J.segtot. Returns the number of launches.
+// scratch at J.segtot. span: also report_span over the jobs (at most 32 of
+// them). Returns the number of launches.
 void integral_layout(int W, int H, size_t max_scratch_elems, int tiles, int &nseg, int &seg_rows);
 size_t integral_scratch_elems(int W, int H, int nseg);
 int integral_tile_blocks(int W, int nseg);
 int integral_col_blocks(int W);
-int launch_integral_jobs(const Job *jobs, int njobs, int tile_blocks, int col_blocks, cudaStream_t s);
+int launch_integral_jobs(const Job *jobs, int njobs, int tile_blocks, int col_blocks, bool span, cudaStream_t s);
 
 // The backward's integral planes (64-bit fixed point) of one image's `np`
 // float plane pairs (u_p, v_p), each W x H in rows of `pitch` floats: u_p scaled by 2^fix_shift(amax[p],
@@ -98,13 +96,12 @@ int launch_sweep(const DevParams &P, const Job *jobs, int njobs, int nitems, int
 // build over a group of jobs of n - 1 = K thresholds, from their bin maps and
 // group summaries (J.b0[kStCRows], J.b0[kStCCols]: the job's first block and
 // its first unit of the column launch; wide: CompactPlan::wide of any job; tall:
-// the tallest image's rows; span: report_span for the group; returns its
-// launches, -1 on error).
+// the tallest image's rows; returns its launches, -1 on error).
 bool plan_compact(const DevParams &P, int W, int H, CompactPlan &C);
 int compact_row_blocks(int H, int K);
 int compact_col_units(int W, int K);
 int launch_compact_build(const Job *jobs, int njobs, int row_blocks, int col_units, int tall, int K, bool wide,
-                         bool span, cudaStream_t s);
+                         cudaStream_t s);
 // The lookup from it (jobs: HOST descriptors of at most kCompactImages images,
 // which travel as kernel parameters): blocks of `rows` rows (compact_look_blocks of an image,
 // first block J.b0[kStLook]). plain: no job has debug planes

@@ -65,7 +65,7 @@ extern "C" tm_status tm_integral_image_noalloc(const int32_t *q, int32_t width, 
   // needs clearing.
   put_jobs(&J, 1, static_cast<Job *>(base), st);
   launch_integral_jobs(static_cast<const Job *>(base), 1, integral_tile_blocks(width, nseg), integral_col_blocks(width),
-                       st);
+                       false, st);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail_noctx(TM_ECUDA, "tm_integral_image_noalloc: kernel launch failed");
   return TM_OK;

@@ -287,13 +287,6 @@ __global__ void __launch_bounds__(256) k_prep(const Job *__restrict__ jobs, int 
   if (J.st_next) commit_range(J.st_next, bmin, bmax, nb, n_bins, qbits);
 }
 
-__global__ void __launch_bounds__(256) k_span(const Job *__restrict__ jobs, int njobs) { report_span(jobs, njobs); }
-
-int launch_span(const Job *jobs, int njobs, cudaStream_t s) {
-  k_span<<<1, 256, 0, s>>>(jobs, njobs);
-  return 1;
-}
-
 int range_blocks(int W, int H, int num_sms, double share) {
   const long long groups = (long long)((W + 3) / 4) * H;
   long long b = (groups + 511) / 512;

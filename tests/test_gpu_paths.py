@@ -102,7 +102,7 @@ def test_batch_splits_over_two_passes():
     ys = [torch.empty_like(x) for x in xs]
     ctx = tm.tm_create(p)
     try:
-        for rep in range(8):
+        for rep in range(10):
             for y in ys:
                 y.zero_()
             names = _stages(ctx, lambda: tm.tm_forward_batch(ctx, xs, ys))
@@ -240,9 +240,9 @@ def test_rough_images_take_the_measured_path():
             assert torch.equal(y, refs[id(x)])
 
     try:
-        run(photo, 12)
+        run(photo, 15)
         assert _path(ctx, photo) == {"compact_histogram"}
-        run(noise, 12)
+        run(noise, 15)
         assert _path(ctx, noise) == {"fused_sweep"}
         run(photo, 1)
         assert _path(ctx, photo) == {"compact_histogram"}
@@ -263,7 +263,7 @@ def test_rough_backward_equals_the_sweeps():
         ctx = tm.tm_create(p)
         try:
             tm.tm_set_option(ctx, tm.TM_OPT_HIST_PATH, path)
-            for _ in range(1 if path else 8):
+            for _ in range(1 if path else 12):
                 gin, gp = [torch.empty_like(x) for x in xs], torch.empty(7, device="cuda")
                 tm.tm_backward_batch(ctx, xs, gs, gin, gp)
                 torch.cuda.synchronize()
@@ -282,7 +282,7 @@ def test_long_images_take_the_measured_path():
     refs = [_forward(x, p, 2) for x in xs[:7]]
     ctx = tm.tm_create(p)
     try:
-        for _ in range(12):
+        for _ in range(15):
             for y in ys:
                 y.zero_()
             tm.tm_forward_batch(ctx, xs, ys)
