@@ -407,7 +407,7 @@ class _CtxCache:
         self._lock = threading.Lock()
 
     def get(self, t):
-        key = t.detach().cpu().float().reshape(-1).numpy().tobytes()  # the context's own 32-bit values
+        key = tuple((t if t.dim() == 1 else t.reshape(-1)).tolist())  # (exact)
         with self._lock:
             c = self.ctxs.pop(key, None)
             if c is None:

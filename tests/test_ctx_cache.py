@@ -31,6 +31,7 @@ def test_a_context_per_distinct_value():
         assert a.value != b.value
         assert cache.get(_theta(p, i3=1e-10, i4=1e-10)).value == a.value
         assert cache.get(_theta(p, i3=3e-10, i4=1e-10).double()).value == b.value
+        assert cache.get(_theta(p, i3=3e-10, i4=1e-10)[None].requires_grad_(True)).value == b.value  # any shape
         assert cache.get(_theta(p, i2=0.6)).value != cache.get(_theta(p, i2=0.6 + 2.0 ** -24)).value
     finally:
         cache.close()
